@@ -1265,10 +1265,15 @@ k_clear_dead_rows(int64_t n, const uint32_t *__restrict__ om, const int64_t *__r
 // neighbours that carry label(q) are ever scanned.
 // -------------------------------------------------------------------------
 
-// A partial embedding of a search plan: positions 0..depth-1 placed.
-constexpr int kItemMaxDepth = 7;
+// A partial embedding of a search plan: positions 0..depth-1 placed.  An item
+// handed on by a long search may hold a part of the next position's candidates
+// only: entries [lo, hi) of the label group its level scans, counted from the
+// group's start (hi = 0: all of them).
+constexpr int kItemMaxDepth = 10;
 struct __align__(16) SearchItem {
     int32_t psi[kItemMaxDepth];
+    int64_t entry;            // edge pass: CSR entry (psi[0], psi[1]) the item asks about
+    uint32_t lo, hi;
     int32_t hd;               // head | depth << 8
 };
 
@@ -1301,6 +1306,8 @@ struct SearchArgs {
     SearchItem *spill;        // a search that has scanned spill_after windows hands its
     int64_t spill_cap;        // untried candidates on here as new items (0: never)
     uint64_t spill_after;
+    int starve;               // also hand on when the item list has run dry (idle warps)
+    int item_batch;           // items a warp takes at a time
     int enum_heads;           // k_expand: 1 = final search (one head), 0 = NLCC
     const uint32_t *sat_seed; // existence passes: heads already known satisfied (nullable)
     // listing (mode kList): every match found gets an index from list_count;
@@ -1320,6 +1327,7 @@ struct WarpSearch {
     int32_t psi[kMaxT];
     int64_t pos[kMaxT];       // next window start inside the chosen label range
     int64_t end[kMaxT];
+    int64_t base[kMaxT];      // start of the scanned label group
     int64_t wbase[kMaxT];     // start of the window the mask refers to
     uint32_t mask[kMaxT];     // untried valid candidates of that window
     uint32_t chk[kMaxT];      // further joins, looked up from scratch per candidate
@@ -1328,10 +1336,12 @@ struct WarpSearch {
     const uint32_t *done_word;  // existence: the answer is known once this bit is set
     uint32_t done_bit;          // (by another warp's embedding); nullptr: never
     int head;                   // plan slot of the running item (spilled items keep it)
-    // the first kJoinCache stored join groups of one level, copied to shared
-    // memory when they are short: join tests at that level search them there
+    int64_t entry;              // edge pass: the running item's CSR entry
+    // the first kJoinCache stored join groups of one level in shared memory:
+    // whole when they hold at most kJoinCacheLen ids, else every jc_step-th
+    // id, which leaves a join test the search of one stretch of jc_step ids
     int jc_level;
-    int jc_len[2];
+    int jc_n[2], jc_step[2];
     int32_t jc[2][128];
     // the last match this warp marked (by plan position) and its plan: a
     // match found next in depth-first order usually differs from it only at
@@ -1379,15 +1389,34 @@ __device__ __forceinline__ bool adjacent(const SearchArgs &a, int32_t x, int32_t
     return lo < stop && __ldg(a.lcol + lo) == u;
 }
 
-// CSR entry index of (x, y) in the id-sorted rows, or -1.
-__device__ __forceinline__ int64_t find_entry(const int64_t *rp, const int32_t *col, int32_t x, int32_t y) {
-    int64_t lo = rp[x], hi = rp[x + 1];
-    const int64_t stop = hi;
-    while (lo < hi) {
-        int64_t mid = (lo + hi) >> 1;
-        if (__ldg(col + mid) < y) lo = mid + 1; else hi = mid;
+// CSR entries e1 of (x, y) and e2 of (y, x) in the id-sorted rows, or -1.  The
+// two binary searches run side by side, so their loads overlap.
+__device__ __forceinline__ void find_entries(const int64_t *rp, const int32_t *col, int32_t x, int32_t y, int64_t &e1,
+                                             int64_t &e2) {
+    int64_t l1 = rp[x], h1 = rp[x + 1], l2 = rp[y], h2 = rp[y + 1];
+    const int64_t s1 = h1, s2 = h2;
+    while (l1 < h1 || l2 < h2) {
+        const int64_t m1 = (l1 + h1) >> 1, m2 = (l2 + h2) >> 1;
+        const int32_t c1 = l1 < h1 ? __ldg(col + m1) : 0;
+        const int32_t c2 = l2 < h2 ? __ldg(col + m2) : 0;
+        if (l1 < h1) { if (c1 < y) l1 = m1 + 1; else h1 = m1; }
+        if (l2 < h2) { if (c2 < x) l2 = m2 + 1; else h2 = m2; }
     }
-    return (lo < stop && __ldg(col + lo) == y) ? lo : -1;
+    e1 = (l1 < s1 && __ldg(col + l1) == y) ? l1 : -1;
+    e2 = (l2 < s2 && __ldg(col + l2) == x) ? l2 : -1;
+}
+
+__device__ __forceinline__ void set_bit(uint32_t *bits, int64_t e) {
+    const uint32_t b = 1u << (uint32_t)(e & 31);
+    if (!(bits[e >> 5] & b)) atomicOr(&bits[e >> 5], b);
+}
+
+// Both entries of the edge (x, y) get their bit in the output edge map.
+__device__ __forceinline__ void mark_edge(const SearchArgs &a, int32_t x, int32_t y) {
+    int64_t e1, e2;
+    find_entries(a.rp, a.col, x, y, e1, e2);
+    if (e1 >= 0) set_bit(a.eb_out, e1);
+    if (e2 >= 0) set_bit(a.eb_out, e2);
 }
 
 // Open level d: among the placed neighbours of position d pick the one whose
@@ -1422,6 +1451,7 @@ __device__ __forceinline__ void open_level(const SearchArgs &a, const DevPlan &P
     }
     const uint32_t extra = __reduce_or_sync(FULL_MASK, (join && slot >= kMaxBack) ? (1u << j) : 0u);
     if (lane == best) {
+        W.base[d] = lo;
         W.pos[d] = lo;
         W.end[d] = hi;
         W.mask[d] = 0u;
@@ -1431,72 +1461,75 @@ __device__ __forceinline__ void open_level(const SearchArgs &a, const DevPlan &P
     __syncwarp();
 }
 
-// Returns true if an embedding exists (ENUM = false) / after enumerating all
-// embeddings from this root (ENUM = true).  `over` is set when the window
-// budget ran out; for existence the root is then reported as satisfied, which
-// keeps the result a superset of the exact answer.
 // Both directions of every template edge of the embedding in W.psi get their
 // bit in the output edge map (id-sorted entry indices).
 __device__ __forceinline__ void mark_edges(const SearchArgs &a, const DevPlan &P, const WarpSearch &W) {
-    const int lane = (int)lane_id();
-    for (int t = lane; t < P.n_marks; t += 32) {
-        int32_t x = W.psi[P.mark_a[t]], y = W.psi[P.mark_b[t]];
-        int64_t e1 = find_entry(a.rp, a.col, x, y);
-        int64_t e2 = find_entry(a.rp, a.col, y, x);
-        if (e1 >= 0) {
-            uint32_t b1 = 1u << (uint32_t)(e1 & 31);
-            if (!(a.eb_out[e1 >> 5] & b1)) atomicOr(&a.eb_out[e1 >> 5], b1);
+    for (int t = (int)lane_id(); t < P.n_marks; t += 32) mark_edge(a, W.psi[P.mark_a[t]], W.psi[P.mark_b[t]]);
+    __syncwarp();
+}
+
+// `n` matches use the edge (x, y): counted on both of its entries.
+__device__ __forceinline__ void count_edge(const SearchArgs &a, int32_t x, int32_t y, unsigned long long n) {
+    int64_t e1, e2;
+    find_entries(a.rp, a.col, x, y, e1, e2);
+    if (e1 >= 0) atomicAdd(&a.ecnt[e1], n);
+    if (e2 >= 0) atomicAdd(&a.ecnt[e2], n);
+}
+
+// Matches found by a listing search: positions 0..k-2 in W.psi, and in the
+// lanes of vm one image u each of the last position.  Every match is stored
+// (if its index is below the cap) and counted on every vertex and on both
+// entries of every edge it uses; what the matches share is counted once for
+// all of them.
+__device__ __forceinline__ void list_window(const SearchArgs &a, const DevPlan &P, const WarpSearch &W, uint32_t vm,
+                                            int32_t u) {
+    const int lane = (int)lane_id(), last = P.k - 1;
+    const unsigned long long n = (unsigned long long)__popc(vm);
+    const bool ok = (vm >> lane) & 1u;
+    unsigned long long idx = 0;
+    if (lane == 0) idx = atomicAdd(a.list_count, n);
+    idx = __shfl_sync(FULL_MASK, idx, 0) + (unsigned long long)__popc(vm & ((1u << lane) - 1u));
+    if (ok && idx < a.list_cap) {
+        int32_t *row = a.list_out + idx * (unsigned long long)a.list_n0;
+        for (int j = 0; j < last; j++) row[P.q[j]] = W.psi[j];
+        row[P.q[last]] = u;
+    }
+    if (a.vcnt) {
+        if (lane < last) atomicAdd(&a.vcnt[W.psi[lane]], n);
+        if (ok) atomicAdd(&a.vcnt[u], 1ull);
+    }
+    if (a.ecnt) {
+        for (int t = lane; t < P.n_marks; t += 32) {
+            const int pa = P.mark_a[t], pb = P.mark_b[t];
+            if (pa != last && pb != last) count_edge(a, W.psi[pa], W.psi[pb], n);
         }
-        if (e2 >= 0) {
-            uint32_t b2 = 1u << (uint32_t)(e2 & 31);
-            if (!(a.eb_out[e2 >> 5] & b2)) atomicOr(&a.eb_out[e2 >> 5], b2);
+        for (int t = 0; t < P.n_marks; t++) {
+            const int pa = P.mark_a[t], pb = P.mark_b[t];
+            if ((pa == last || pb == last) && ok) count_edge(a, W.psi[pa == last ? pb : pa], u, 1ull);
         }
     }
     __syncwarp();
 }
 
-// A match found by a listing search: stored (if its index is below the cap)
-// and counted on every vertex and on both entries of every edge it uses.
-__device__ __forceinline__ void list_embedding(const SearchArgs &a, const DevPlan &P, const WarpSearch &W) {
+// Warp-uniform: make the join cache hold level d's first stored groups.
+__device__ __forceinline__ void join_cache(const SearchArgs &a, WarpSearch &W, int d) {
+    if (W.jc_level == d) return;
     const int lane = (int)lane_id();
-    unsigned long long idx = 0;
-    if (lane == 0) idx = atomicAdd(a.list_count, 1ull);
-    idx = __shfl_sync(FULL_MASK, idx, 0);
-    if (lane < P.k) {
-        const int32_t x = W.psi[lane];
-        if (idx < a.list_cap) a.list_out[idx * (unsigned long long)a.list_n0 + (unsigned long long)P.q[lane]] = x;
-        if (a.vcnt) atomicAdd(&a.vcnt[x], 1ull);
+    const int nb = min(W.nb[d], kJoinCache);
+    for (int b = 0; b < nb; b++) {
+        const int64_t lo = W.blo[d][b], len = W.bhi[d][b] - lo;
+        const int64_t step = len <= kJoinCacheLen ? 1 : (len + kJoinCacheLen - 1) / kJoinCacheLen;
+        const int n = (int)((len + step - 1) / step);
+        for (int i = lane; i < n; i += 32) W.jc[b][i] = __ldg(a.lcol + lo + i * step);
+        if (lane == 0) { W.jc_n[b] = n; W.jc_step[b] = (int)step; }
     }
-    if (a.ecnt) {
-        for (int t = lane; t < P.n_marks; t += 32) {
-            const int32_t x = W.psi[P.mark_a[t]], y = W.psi[P.mark_b[t]];
-            const int64_t e1 = find_entry(a.rp, a.col, x, y), e2 = find_entry(a.rp, a.col, y, x);
-            if (e1 >= 0) atomicAdd(&a.ecnt[e1], 1ull);
-            if (e2 >= 0) atomicAdd(&a.ecnt[e2], 1ull);
-        }
-    }
+    if (lane == 0) W.jc_level = d;
     __syncwarp();
 }
 
 // Is the entry e of the scanned label group a valid image u for position d?
 // Its omega must hold q_d, it must differ from earlier same-label images, and
 // it must be joined to every other placed neighbour of position d.
-// Warp-uniform: make the join cache hold level d's first stored groups.
-__device__ __forceinline__ void join_cache(const SearchArgs &a, WarpSearch &W, int d) {
-    if (W.jc_level == d) return;
-    const int lane = (int)lane_id();
-    const int nb = min(W.nb[d], kJoinCache);
-    for (int b = 0; b < kJoinCache; b++) {
-        const int64_t lo = W.blo[d][b], len = W.bhi[d][b] - lo;
-        const bool fits = b < nb && len <= kJoinCacheLen;
-        if (fits)
-            for (int i = lane; i < (int)len; i += 32) W.jc[b][i] = __ldg(a.lcol + lo + i);
-        if (lane == 0) W.jc_len[b] = fits ? (int)len : -1;
-    }
-    if (lane == 0) W.jc_level = d;
-    __syncwarp();
-}
-
 __device__ __forceinline__ bool test_candidate(const SearchArgs &a, const DevPlan &P, WarpSearch &W,
                                                int d, int64_t e, int64_t end, int32_t &u) {
     if (W.nb[d] > 0) join_cache(a, W, d);
@@ -1507,17 +1540,20 @@ __device__ __forceinline__ bool test_candidate(const SearchArgs &a, const DevPla
     for (uint32_t sm = P.same[d]; sm; sm &= sm - 1u)
         if (W.psi[__ffs(sm) - 1] == u) return false;
     for (int b = 0; b < W.nb[d]; b++) {
-        if (b < kJoinCache && W.jc_len[b] >= 0) {
-            int lo = 0, hi = W.jc_len[b];
-            const int stop = hi;
-            while (lo < hi) {
-                const int m2 = (lo + hi) >> 1;
-                if (W.jc[b][m2] < u) lo = m2 + 1; else hi = m2;
-            }
-            if (!(lo < stop && W.jc[b][lo] == u)) return false;
-            continue;
-        }
         int64_t lo = W.blo[d][b], hi = W.bhi[d][b];
+        if (b < kJoinCache) {
+            int i = 0, h = W.jc_n[b];                // i: ids of the cache that are <= u
+            while (i < h) {
+                const int m2 = (i + h) >> 1;
+                if (W.jc[b][m2] <= u) i = m2 + 1; else h = m2;
+            }
+            if (i == 0) return false;
+            if (W.jc[b][i - 1] == u) continue;
+            const int step = W.jc_step[b];
+            if (step == 1) return false;
+            hi = min(hi, lo + (int64_t)i * step);
+            lo += (int64_t)(i - 1) * step + 1;
+        }
         const int64_t stop = hi;
         while (lo < hi) {
             int64_t m2 = (lo + hi) >> 1;
@@ -1530,26 +1566,21 @@ __device__ __forceinline__ bool test_candidate(const SearchArgs &a, const DevPla
     return true;
 }
 
-// omega*(psi(i)) gets q_i for every position of the match in W.psi.
-__device__ __forceinline__ void mark_vertices(const SearchArgs &a, const DevPlan &P, const WarpSearch &W) {
-    const int lane = (int)lane_id();
-    if (lane < P.k) {
-        const int32_t x = W.psi[lane];
-        const uint32_t bit = 1u << P.q[lane];
-        if (!(a.om_out[x] & bit)) atomicOr(&a.om_out[x], bit);
-    }
-    __syncwarp();
-}
-
-// Mark a match found by a marking enumeration: every (vertex, template
-// vertex) pair and both entries of every template edge, skipping those the
-// warp's previous match (same plan) already marked: marks are only ever set,
-// so a pair or an edge whose positions hold the same vertices as in that
-// match is marked already.
-__device__ __forceinline__ void mark_match(const SearchArgs &a, const DevPlan &P, WarpSearch &W) {
-    const int lane = (int)lane_id();
+// Mark the matches found by a marking enumeration (positions 0..k-2 in W.psi,
+// the images u of the last position in the lanes of vm): every (vertex,
+// template vertex) pair and both entries of every template edge.  What the
+// matches of a window share is marked by one lane each, and only where it
+// differs from what the warp marked last (same plan): marks are only ever set,
+// and a pair or an edge whose positions hold the same vertices as then is
+// marked already.  What hangs on the last position is marked by the match's
+// own lane: each edge costs two binary searches of up to 17 dependent loads, so
+// marking match by match kept 31 of 32 lanes idle (a marking pass of up to 2^16
+// matches took 18.7 ms on one template over 4M vertices, 0.7 ms now).
+__device__ __forceinline__ void mark_window(const SearchArgs &a, const DevPlan &P, WarpSearch &W, uint32_t vm,
+                                            int32_t u) {
+    const int lane = (int)lane_id(), last = P.k - 1;
     const bool same_plan = W.last_plan == &P;
-    if (lane < P.k) {
+    if (lane < last) {
         const int32_t x = W.psi[lane];
         if (!(same_plan && W.last[lane] == x)) {
             const uint32_t bit = 1u << P.q[lane];
@@ -1558,21 +1589,20 @@ __device__ __forceinline__ void mark_match(const SearchArgs &a, const DevPlan &P
     }
     for (int t = lane; t < P.n_marks; t += 32) {
         const int pa = P.mark_a[t], pb = P.mark_b[t];
+        if (pa == last || pb == last) continue;
         const int32_t x = W.psi[pa], y = W.psi[pb];
-        if (same_plan && W.last[pa] == x && W.last[pb] == y) continue;
-        const int64_t e1 = find_entry(a.rp, a.col, x, y);
-        const int64_t e2 = find_entry(a.rp, a.col, y, x);
-        if (e1 >= 0) {
-            const uint32_t b1 = 1u << (uint32_t)(e1 & 31);
-            if (!(a.eb_out[e1 >> 5] & b1)) atomicOr(&a.eb_out[e1 >> 5], b1);
-        }
-        if (e2 >= 0) {
-            const uint32_t b2 = 1u << (uint32_t)(e2 & 31);
-            if (!(a.eb_out[e2 >> 5] & b2)) atomicOr(&a.eb_out[e2 >> 5], b2);
+        if (!(same_plan && W.last[pa] == x && W.last[pb] == y)) mark_edge(a, x, y);
+    }
+    if ((vm >> lane) & 1u) {
+        const uint32_t bit = 1u << P.q[last];
+        if (!(a.om_out[u] & bit)) atomicOr(&a.om_out[u], bit);
+        for (int t = 0; t < P.n_marks; t++) {
+            const int pa = P.mark_a[t], pb = P.mark_b[t];
+            if (pa == last || pb == last) mark_edge(a, W.psi[pa == last ? pb : pa], u);
         }
     }
     __syncwarp();
-    if (lane < P.k) W.last[lane] = W.psi[lane];
+    if (lane < last) W.last[lane] = W.psi[lane];
     if (lane == 0) W.last_plan = &P;
     __syncwarp();
 }
@@ -1581,41 +1611,42 @@ __device__ __forceinline__ void mark_match(const SearchArgs &a, const DevPlan &P
 // and mark the vertices and edges of every one / count them and list them.
 constexpr int kExist = 0, kCount = 1, kMark = 2, kList = 3;
 
-// Hand the rest of a long search to other warps: for every open level L
-// (d0..d) each untried candidate c -- the remaining bits of the level's
-// tested window and every valid entry of its untested range -- becomes an item
-// (psi[0..L-1], c) of depth L+1 in the spill list; for counting, candidates
-// of the last position are counted here instead.  The items are counted
-// first and written only if they all fit.  Returns false (the search goes on
-// where it is) when they do not.  Reservations only ever add to the counter:
-// the successful ones are exactly those ending at or below the capacity, and
-// they fill the list up to the lowest start of a failed one (spill_stop), so
-// the list is valid below min(counter, spill_stop).
-template <int MODE>
-__device__ bool spill(const SearchArgs &a, const DevPlan &P, WarpSearch &W, int d0, int d,
-                      unsigned long long &matches) {
+// Windows a search scans at least before it hands work on to idle warps, and
+// between its looks at what the other warps do.
+constexpr uint64_t kLook = 16;
+constexpr int kSpillParts = 32;      // items one open level's untested candidates become, at most
+
+// Hand the rest of a long search to other warps.  Every open level L (d0..d)
+// gives one item (psi[0..L-1], c) of depth L+1 per tested and untried
+// candidate c, and up to kSpillParts items of depth L that each hold a stretch
+// of its untested candidates.  No candidate is tested here: handing on costs a
+// few dozen stores, so a search can do it as soon as other warps are idle.
+// That is what bounds these kernels: a window is a chain of dependent loads (a
+// microsecond or more), so a pass lasts as long as its longest search.  Handing
+// on only after 2048 windows, 16M vertices / 5*10^8 entries / 5-cycle template:
+// 50 ms in 10 passes of k_nlcc_items and 18.6 ms in 3 of k_edge_search; handing
+// on when the list is empty: 2.1 ms in 32 passes and 0.5 ms in 8 (the whole
+// prune 75.7 -> 7.7 ms; a batch of 24 templates on 4M vertices 105 -> 27 ms).
+// Returns false (the search goes on where it is) when the list is full.
+// Reservations only ever add to the counter: the successful ones are exactly
+// those ending at or below the capacity, and they fill the list up to the
+// lowest start of a failed one (spill_stop), so the list is valid below
+// min(counter, spill_stop).
+__device__ bool spill(const SearchArgs &a, const WarpSearch &W, int d0, int d) {
     const int lane = (int)lane_id();
-    const uint32_t below = (1u << lane) - 1u;
-    const int k = P.k;
-    unsigned long long total = 0, direct = 0;
+    unsigned int total = 0;
     for (int L = d0; L <= d; L++) {
-        unsigned long long cnt = (unsigned long long)__popc(W.mask[L]);
-        for (int64_t pos = W.pos[L]; pos < W.end[L]; pos += 32) {
-            int32_t u;
-            const bool ok = test_candidate(a, P, W, L, pos + lane, W.end[L], u);
-            cnt += (unsigned long long)__popc(__ballot_sync(FULL_MASK, ok));
-        }
-        if (MODE == kCount && L == k - 1) direct += cnt; else total += cnt;
+        const int64_t wins = (W.end[L] - W.pos[L] + 31) >> 5;
+        total += (unsigned int)__popc(W.mask[L]) + (unsigned int)max((int64_t)0, min(wins, (int64_t)kSpillParts));
     }
-    unsigned long long base = 0;
-    unsigned int fits = 1;
+    unsigned int base = 0, fits = 1;
     if (lane == 0 && total) {
-        if (*(volatile const unsigned int *)&a.st->n_spill >= (unsigned long long)a.spill_cap) {
+        if ((int64_t)*(volatile const unsigned int *)&a.st->n_spill >= a.spill_cap) {
             fits = 0;                               // full already: do not grow the counter
         } else {
-            base = atomicAdd(&a.st->n_spill, (unsigned int)total);
-            if (base + total > (unsigned long long)a.spill_cap) {
-                atomicMin(&a.st->spill_stop, (unsigned int)base);
+            base = atomicAdd(&a.st->n_spill, total);
+            if ((int64_t)base + total > a.spill_cap) {
+                atomicMin(&a.st->spill_stop, base);
                 fits = 0;
             }
         }
@@ -1623,47 +1654,68 @@ __device__ bool spill(const SearchArgs &a, const DevPlan &P, WarpSearch &W, int 
     if (!__shfl_sync(FULL_MASK, fits, 0)) return false;
     base = __shfl_sync(FULL_MASK, base, 0);
     for (int L = d0; L <= d; L++) {
-        if (MODE == kCount && L == k - 1) continue;
         SearchItem si;
+#pragma unroll
         for (int j = 0; j < kItemMaxDepth; j++) si.psi[j] = j < L ? W.psi[j] : 0;
-        si.hd = W.head | ((L + 1) << 8);
+        si.entry = W.entry;
+        si.lo = si.hi = 0u;
         const uint32_t m = W.mask[L];
         if ((m >> lane) & 1u) {
-            si.psi[L] = __ldg(a.lcol + W.wbase[L] + lane);
-            a.spill[base + __popc(m & below)] = si;
+            const int32_t c = __ldg(a.lcol + W.wbase[L] + lane);
+#pragma unroll
+            for (int j = 0; j < kItemMaxDepth; j++)
+                if (j == L) si.psi[j] = c;
+            si.hd = W.head | ((L + 1) << 8);
+            a.spill[base + __popc(m & ((1u << lane) - 1u))] = si;
+#pragma unroll
+            for (int j = 0; j < kItemMaxDepth; j++)
+                if (j == L) si.psi[j] = 0;
         }
-        base += (unsigned long long)__popc(m);
-        for (int64_t pos = W.pos[L]; pos < W.end[L]; pos += 32) {
-            int32_t u;
-            const bool ok = test_candidate(a, P, W, L, pos + lane, W.end[L], u);
-            const uint32_t vm = __ballot_sync(FULL_MASK, ok);
-            if (ok) {
-                si.psi[L] = u;
-                a.spill[base + __popc(vm & below)] = si;
-            }
-            base += (unsigned long long)__popc(vm);
+        base += (unsigned int)__popc(m);
+        const int64_t from = W.pos[L] - W.base[L], to = W.end[L] - W.base[L], wins = (to - from + 31) >> 5;
+        if (wins <= 0) continue;
+        const int parts = (int)min(wins, (int64_t)kSpillParts);
+        if (lane < parts) {
+            si.lo = (uint32_t)(from + 32 * (wins * lane / parts));
+            si.hi = (uint32_t)min(to, from + 32 * (wins * (lane + 1) / parts));
+            si.hd = W.head | (L << 8);
+            a.spill[base + lane] = si;
         }
+        base += (unsigned int)parts;
     }
-    matches += direct;
     __syncwarp();
     return true;
 }
 
-// Depth-first search from positions 0..d0-1 already placed in W.psi.
+// Depth-first search from positions 0..d0-1 already placed in W.psi (part_hi:
+// over entries [part_lo, part_hi) of position d0's label group only).  kExist:
+// true if an embedding exists; the other modes enumerate every embedding.
+// `over` is set when the window budget ran out; for existence the root is then
+// reported as satisfied, which keeps the result a superset of the exact answer.
 template <int MODE>
 __device__ bool search_from(const SearchArgs &a, const DevPlan &P, int d0, WarpSearch &W,
-                            unsigned long long &entries, unsigned long long &matches, bool &over) {
+                            unsigned long long &entries, unsigned long long &matches, bool &over,
+                            uint32_t part_lo = 0u, uint32_t part_hi = 0u) {
     const int lane = (int)lane_id();
     const int k = P.k;
     uint64_t used = 0;
+    unsigned long long pub = (MODE == kCount || MODE == kMark) ? W.pub : 0;   // matches published so far
     if (d0 >= k) {                                  // the placed prefix is already a full map
         if (MODE == kExist) return true;
         matches++;
-        if (MODE == kMark) mark_match(a, P, W);
-        if (MODE == kList) list_embedding(a, P, W);
+        const int32_t x = W.psi[k - 1];
+        if (MODE == kMark) mark_window(a, P, W, 1u, x);
+        if (MODE == kList) list_window(a, P, W, 1u, x);
         return false;
     }
     open_level(a, P, W, d0);
+    if (part_hi) {
+        if (lane == 0) {
+            W.end[d0] = W.base[d0] + part_hi;
+            W.pos[d0] = W.base[d0] + part_lo;
+        }
+        __syncwarp();
+    }
     int d = d0;
     while (d >= d0) {
         const uint32_t m = W.mask[d];
@@ -1671,10 +1723,12 @@ __device__ bool search_from(const SearchArgs &a, const DevPlan &P, int d0, WarpS
             const int64_t pos = W.pos[d], end = W.end[d];
             if (pos >= end) { d--; continue; }
             if (++used > a.budget) { over = true; return MODE == kExist; }
-            if ((used & 31u) == 0u) {
-                // every 32 windows: has another warp answered this existence
-                // question already, or has the count run past its cap?
-                unsigned int stop = 0;
+            // every kLook windows (marking: and every 128 matches): has another
+            // warp answered this existence question already, has the count run
+            // past its cap, are other warps out of work?
+            const bool look = (used & (kLook - 1)) == 0u || (MODE == kMark && matches - pub >= 128u);
+            if (look) {
+                unsigned int stop = 0, hand = 0;
                 if (lane == 0) {
                     if (MODE == kExist) {
                         stop = W.done_word && (*(volatile const uint32_t *)W.done_word & W.done_bit);
@@ -1682,50 +1736,60 @@ __device__ bool search_from(const SearchArgs &a, const DevPlan &P, int d0, WarpS
                         // counting (and marking) stops as soon as the total passes
                         // the cap: publish this warp's new matches and read the
                         // total, so that no warp runs on to the cap by itself
-                        const unsigned long long d = matches - W.pub;
+                        const unsigned long long dm = matches - pub;
                         const unsigned long long tot =
-                            d ? atomicAdd(&a.st->matches, d) + d : *(volatile const unsigned long long *)&a.st->matches;
+                            dm ? atomicAdd(&a.st->matches, dm) + dm : *(volatile const unsigned long long *)&a.st->matches;
                         W.pub = matches;
                         stop = tot > a.cap || *(volatile const unsigned int *)&a.st->overflow;
                     } else {
                         stop = matches > a.cap || *(volatile const unsigned int *)&a.st->overflow;
                     }
+                    if (a.starve && used >= kLook)
+                        hand = *(volatile const unsigned long long *)a.next_root >= (unsigned long long)a.n_items;
                 }
+                pub = matches;
                 if (__shfl_sync(FULL_MASK, stop, 0)) {
                     // past the cap (the matches are published already, so the
                     // caller's batch-end check would not see it)
                     if (MODE == kCount || MODE == kMark) over = true;
                     return false;
                 }
+                hand = __shfl_sync(FULL_MASK, hand, 0);
+                if (hand && d < kItemMaxDepth && spill(a, W, d0, d)) return false;
             }
-            if (a.spill_after && used > a.spill_after && d < kItemMaxDepth &&
-                spill<MODE>(a, P, W, d0, d, matches))
+            if (a.spill_after && used > a.spill_after && d < kItemMaxDepth && spill(a, W, d0, d))
                 return false;                       // the rest runs as new items
             entries += (unsigned long long)min((int64_t)32, end - pos);
             int32_t u;
             const bool ok = test_candidate(a, P, W, d, pos + lane, end, u);
             const uint32_t vm = __ballot_sync(FULL_MASK, ok);
-            if (MODE == kCount && d == k - 1) {
-                // counting: every valid image of the last position completes a match
-                matches += (unsigned long long)__popc(vm);
-                if (lane == 0) { W.mask[d] = 0u; W.pos[d] = pos + 32; }
+            if (d == k - 1) {
+                // every valid image of the last position completes a match
+                if (MODE == kExist) {
+                    if (vm) {
+                        if (lane == __ffs(vm) - 1) W.psi[d] = u;
+                        __syncwarp();
+                        return true;
+                    }
+                } else if (vm) {
+                    matches += (unsigned long long)__popc(vm);
+                    if (MODE == kMark) mark_window(a, P, W, vm, u);
+                    if (MODE == kList) list_window(a, P, W, vm, u);
+                }
+                __syncwarp();
+                if (lane == 0) W.pos[d] = pos + 32;
                 __syncwarp();
                 continue;
             }
+            __syncwarp();
             if (lane == 0) { W.mask[d] = vm; W.wbase[d] = pos; W.pos[d] = pos + 32; }
             __syncwarp();
             continue;
         }
         const int b = __ffs(m) - 1;
+        __syncwarp();
         if (lane == 0) { W.mask[d] = m & (m - 1u); W.psi[d] = __ldg(a.lcol + W.wbase[d] + b); }
         __syncwarp();
-        if (d == k - 1) {
-            if (MODE == kExist) return true;
-            matches++;                              // kMark / kList (counting never stores last-level masks)
-            if (MODE == kList) list_embedding(a, P, W);
-            else mark_match(a, P, W);
-            continue;
-        }
         d++;
         open_level(a, P, W, d);
     }
@@ -1844,8 +1908,12 @@ k_expand(SearchArgs a) {
                     ok = ((__ldg(a.om + u) >> q1) & 1u) && !((P.same[1] & 1u) && u == v);
                 }
                 SearchItem si;
+#pragma unroll
+                for (int j = 2; j < kItemMaxDepth; j++) si.psi[j] = 0;
                 si.psi[0] = v;
                 si.psi[1] = u;
+                si.entry = 0;
+                si.lo = si.hi = 0u;
                 si.hd = h | (2 << 8);
                 b.push(ok, si);
             }
@@ -1893,7 +1961,9 @@ k_expand_next(SearchArgs a, const SearchItem *in, int64_t n_in) {
             int32_t u;
             const bool ok = test_candidate(a, P, W, depth, base + lane, hi, u);
             SearchItem si = item;
-            si.psi[depth] = u;
+#pragma unroll
+            for (int j = 0; j < kItemMaxDepth; j++)
+                if (j == depth) si.psi[j] = u;
             si.hd = h | ((depth + 1) << 8);
             b.push(ok, si);
         }
@@ -1908,7 +1978,6 @@ __device__ __forceinline__ int64_t grab_items(const SearchArgs &a, int batch) {
     return (int64_t)__shfl_sync(FULL_MASK, r, 0);
 }
 
-constexpr int kItemBatch = 4;
 constexpr int kMaxPlans = 64;      // plan slots (heads, or oriented template edges)
 constexpr uint64_t kMarkCap = 1ull << 20;   // matches one marking enumeration handles
 constexpr uint64_t kFewMatches = 1ull << 16;   // marked during the first enumeration itself
@@ -1923,8 +1992,8 @@ k_nlcc_items(SearchArgs a) {
     WarpSearch &W = ws[wib];
     unsigned long long entries = 0, matches = 0;
     bool over = false;
-    for (int64_t it0 = grab_items(a, kItemBatch); it0 < a.n_items; it0 = grab_items(a, kItemBatch)) {
-        const int64_t it1 = min(a.n_items, it0 + kItemBatch);
+    for (int64_t it0 = grab_items(a, a.item_batch); it0 < a.n_items; it0 = grab_items(a, a.item_batch)) {
+        const int64_t it1 = min(a.n_items, it0 + a.item_batch);
         for (int64_t it = it0; it < it1; it++) {
             const SearchItem item = a.items[it];
             const int h = item.hd & 0xff, depth = item.hd >> 8;
@@ -1933,10 +2002,10 @@ k_nlcc_items(SearchArgs a) {
             if (lane == 0) done = *(volatile uint32_t *)&a.sat[item.psi[0]] & bit;
             if (__shfl_sync(FULL_MASK, done, 0)) continue;
             if (lane < depth) W.psi[lane] = item.psi[lane];
-            if (lane == 0) { W.done_word = &a.sat[item.psi[0]]; W.done_bit = bit; W.head = h; }
+            if (lane == 0) { W.done_word = &a.sat[item.psi[0]]; W.done_bit = bit; W.head = h; W.entry = 0; }
             __syncwarp();
             bool ran_out = false;
-            if (search_from<kExist>(a, a.plans[h], depth, W, entries, matches, ran_out)) {
+            if (search_from<kExist>(a, a.plans[h], depth, W, entries, matches, ran_out, item.lo, item.hi)) {
                 const DevPlan &P = a.plans[h];
                 if (ran_out) {
                     // budget exhausted: keep the head (a superset of the exact answer)
@@ -1971,18 +2040,18 @@ k_final_items(SearchArgs a) {
     __syncwarp();
     unsigned long long entries = 0, matches = 0;
     bool over = false;
-    for (int64_t it0 = grab_items(a, kItemBatch); it0 < a.n_items; it0 = grab_items(a, kItemBatch)) {
+    for (int64_t it0 = grab_items(a, a.item_batch); it0 < a.n_items; it0 = grab_items(a, a.item_batch)) {
         unsigned int stop = 0;
         if (lane == 0) stop = *(volatile unsigned int *)&a.st->overflow;
         if (__shfl_sync(FULL_MASK, stop, 0)) break;
-        const int64_t it1 = min(a.n_items, it0 + kItemBatch);
+        const int64_t it1 = min(a.n_items, it0 + a.item_batch);
         for (int64_t it = it0; it < it1 && !over; it++) {
             const SearchItem item = a.items[it];
             const int depth = item.hd >> 8;
             if (lane < depth) W.psi[lane] = item.psi[lane];
-            if (lane == 0) { W.done_word = nullptr; W.head = item.hd & 0xff; }
+            if (lane == 0) { W.done_word = nullptr; W.head = item.hd & 0xff; W.entry = 0; }
             __syncwarp();
-            search_from<MODE>(a, a.plans[0], depth, W, entries, matches, over);
+            search_from<MODE>(a, a.plans[0], depth, W, entries, matches, over, item.lo, item.hi);
             __syncwarp();
         }
         const unsigned long long pub = W.pub;     // read by every lane before lane 0 moves it
@@ -2044,9 +2113,12 @@ k_edge_items(SearchArgs a, EdgeTab tab) {
             for (int o = 0; o < tab.n; o++) {
                 const bool ok = wy && ((wx >> tab.a[o]) & 1u) && ((wy >> tab.b[o]) & 1u);
                 SearchItem si;
-                for (int j = 0; j < kItemMaxDepth; j++) si.psi[j] = 0;
+#pragma unroll
+                for (int j = 2; j < kItemMaxDepth; j++) si.psi[j] = 0;
                 si.psi[0] = x;
                 si.psi[1] = y;
+                si.entry = e;
+                si.lo = si.hi = 0u;
                 si.hd = o | (2 << 8);
                 b.push(ok, si);
             }
@@ -2063,32 +2135,33 @@ k_edge_search(SearchArgs a) {
     WarpSearch &W = ws[wib];
     unsigned long long entries = 0, matches = 0;
     bool over = false;
-    for (int64_t it0 = grab_items(a, kItemBatch); it0 < a.n_items; it0 = grab_items(a, kItemBatch)) {
-        const int64_t it1 = min(a.n_items, it0 + kItemBatch);
+    for (int64_t it0 = grab_items(a, a.item_batch); it0 < a.n_items; it0 = grab_items(a, a.item_batch)) {
+        const int64_t it1 = min(a.n_items, it0 + a.item_batch);
         for (int64_t it = it0; it < it1; it++) {
             const SearchItem item = a.items[it];
             const int o = item.hd & 0xff, depth = item.hd >> 8;
-            // the entry of the item's template edge: psi[0], psi[1] are its
-            // ends (items handed on by long searches keep them)
-            int64_t e = 0;
-            if (lane == 0) e = find_entry(a.rp, a.col, item.psi[0], item.psi[1]);
-            e = __shfl_sync(FULL_MASK, e, 0);
+            // the entry of the item's template edge (items handed on by long
+            // searches keep it)
+            const int64_t e = item.entry;
             uint32_t done = 0;                          // marked by an embedding found meanwhile?
             if (lane == 0) done = (*(volatile uint32_t *)&a.eb_out[e >> 5] >> (uint32_t)(e & 31)) & 1u;
             if (__shfl_sync(FULL_MASK, done, 0)) continue;
             if (lane < depth) W.psi[lane] = item.psi[lane];
-            if (lane == 0) { W.done_word = &a.eb_out[e >> 5]; W.done_bit = 1u << (uint32_t)(e & 31); W.head = o; }
+            if (lane == 0) {
+                W.done_word = &a.eb_out[e >> 5];
+                W.done_bit = 1u << (uint32_t)(e & 31);
+                W.head = o;
+                W.entry = e;
+            }
             __syncwarp();
             const DevPlan &P = a.plans[o];
             bool ran_out = false;
-            if (search_from<kExist>(a, P, depth, W, entries, matches, ran_out)) {
+            if (search_from<kExist>(a, P, depth, W, entries, matches, ran_out, item.lo, item.hi)) {
                 if (!ran_out) {
                     mark_edges(a, P, W);
                 } else if (lane == 0) {
                     // budget exhausted: keep the edge (a superset of the exact answer)
-                    const int64_t e2 = find_entry(a.rp, a.col, item.psi[1], item.psi[0]);
-                    atomicOr(&a.eb_out[e >> 5], 1u << (uint32_t)(e & 31));
-                    if (e2 >= 0) atomicOr(&a.eb_out[e2 >> 5], 1u << (uint32_t)(e2 & 31));
+                    mark_edge(a, item.psi[0], item.psi[1]);
                 }
             }
             over = over || ran_out;
@@ -2702,7 +2775,8 @@ int ensure_entry_labels(ccpm_ctx *ctx, ccpm_graph *g) {
     return CCPM_OK;
 }
 
-// Split search work level by level while there is too little of it to fill
+// For searches that do not hand work on to idle warps (a caller's own budget,
+// search_split < 0): split the work level by level while there is too little to fill
 // the GPU (and the items still leave positions to place).
 int expand_more(ccpm_ctx *ctx, Workspace &w, SearchArgs &a, int max_depth, int64_t &launches) {
     for (int depth = 2; depth < max_depth && depth < kItemMaxDepth; depth++) {
@@ -2744,13 +2818,13 @@ int grid_for(ccpm_ctx *ctx, int64_t work_items, int per_block, int blocks_per_sm
 constexpr uint64_t kSpillAfter = 2048;
 
 // Run an item kernel, then again over the items long searches handed on, until
-// none are left (each round of items is strictly deeper, so at most one pass
-// per template position).  kind 0: NLCC existence (k_nlcc_items), 1: final
+// none are left (an item handed on is deeper, or holds fewer candidates of the
+// same position, than the one it came from, so the passes end).  kind 0: NLCC existence (k_nlcc_items), 1: final
 // count, 2: final count and mark, 3: count and list, 4: per-entry existence
 // (k_edge_search).  Counting (and marking) stops once the cap
 // is passed.
-int item_passes(ccpm_ctx *ctx, Workspace &w, SearchArgs &a, int kind, uint64_t split, int64_t &launches,
-                int64_t &passes) {
+int item_passes(ccpm_ctx *ctx, Workspace &w, SearchArgs &a, int kind, uint64_t split, bool starve,
+                int64_t &launches, int64_t &passes) {
     cudaStream_t s = ctx->stream;
     SearchItem *bufs[2] = {w.items, w.spill_items};
     const int64_t caps[2] = {w.items_cap, w.spill_cap};
@@ -2760,10 +2834,14 @@ int item_passes(ccpm_ctx *ctx, Workspace &w, SearchArgs &a, int kind, uint64_t s
         a.spill = bufs[cur ^ 1];
         a.spill_cap = caps[cur ^ 1];
         a.spill_after = split;
+        a.starve = starve ? 1 : 0;
         CU(ctx, cudaMemsetAsync(w.next_root, 0, sizeof(unsigned long long), s));
         CU(ctx, cudaMemsetAsync(&w.st->n_spill, 0, sizeof(unsigned int), s));
         CU(ctx, cudaMemsetAsync(&w.st->spill_stop, 0xFF, sizeof(unsigned int), s));
-        const int gi = grid_for(ctx, (a.n_items + kItemBatch - 1) / kItemBatch * 32, 128, 16);
+        // few items: one at a time, so that none waits behind a long one
+        const int64_t warps = (int64_t)grid_sms(ctx) * 64;
+        a.item_batch = (int)std::max<int64_t>(1, std::min<int64_t>(16, a.n_items / (8 * warps)));
+        const int gi = grid_for(ctx, (a.n_items + a.item_batch - 1) / a.item_batch * 32, 128, 16);
         launches++;
         passes++;
         if (kind == 0) k_nlcc_items<<<gi, 128, 0, s>>>(a);
@@ -2786,6 +2864,7 @@ int item_passes(ccpm_ctx *ctx, Workspace &w, SearchArgs &a, int kind, uint64_t s
     a.items = w.items;
     a.spill = nullptr;
     a.spill_after = 0;
+    a.starve = 0;
     return CCPM_OK;
 }
 
@@ -3470,6 +3549,12 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
     const int hub_deg = opt.hub_degree > 0 ? std::min(opt.hub_degree, kMaxHubDeg) : kDefaultHubDeg;
     const uint64_t budget = opt.search_budget ? opt.search_budget : kDefaultSearchBudget;
     const uint64_t split = opt.search_split < 0 ? 0 : (opt.search_split == 0 ? kSpillAfter : (uint64_t)opt.search_split);
+    // a caller's own budget counts windows as one search scans them: no handing
+    // on to idle warps, which would restart its count.  Those searches are
+    // spread up front instead (expand_more: a kernel and a host round trip per
+    // level), which is slower where both work: 8.3 against 7.7 ms on the 5-cycle
+    // template over 16M vertices, 32 against 27 ms for a batch over 4M
+    const bool starve = opt.search_split >= 0 && opt.search_budget == 0;
     int rc = ws_ensure(ctx, g, hub_deg);
     if (rc) return rc;
     Workspace &w = ctx->ws;
@@ -3708,13 +3793,13 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
             CUF(cudaGetLastError());
             RCF(P.read_stats());
             a.n_items = w.st_h->n_items;
-            if (a.n_items <= w.items_cap) RCF(expand_more(ctx, w, a, __builtin_popcount(c.vmask), P.launches));
+            if (!starve && a.n_items <= w.items_cap) RCF(expand_more(ctx, w, a, __builtin_popcount(c.vmask), P.launches));
             CUF(cudaMemsetAsync(w.next_root, 0, sizeof(unsigned long long), s));
             P.search_launches++;
             CUF(cudaMemcpyAsync(w.aux_h, &w.st->windows, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
             CUF(cudaEventRecord(w.ev[10], s));
             if (a.n_items <= w.items_cap) {
-                RCF(item_passes(ctx, w, a, 0, split, P.launches, P.item_passes));
+                RCF(item_passes(ctx, w, a, 0, split, starve, P.launches, P.item_passes));
             } else {
                 P.launches++;
                 k_nlcc_search<<<grid_for(ctx, n_roots * 32, 128, 16), 128, 0, s>>>(a);
@@ -3790,7 +3875,7 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
         a.items = w.items;
         a.items_cap = w.items_cap;
         auto run_items = [&](bool edge_pass) -> int {
-            int rc2 = item_passes(ctx, w, a, edge_pass ? 4 : 0, split, P.launches, P.item_passes);
+            int rc2 = item_passes(ctx, w, a, edge_pass ? 4 : 0, split, starve, P.launches, P.item_passes);
             return rc2 ? rc2 : P.read_stats();
         };
         // the final enumeration keeps the background label frequencies (measured
@@ -3828,12 +3913,12 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
             CU(ctx, cudaGetLastError());
             if ((rc2 = P.read_stats())) return rc2;
             a.n_items = w.st_h->n_items;
-            if (a.n_items <= w.items_cap && (rc2 = expand_more(ctx, w, a, t.n0, P.launches))) return rc2;
+            if (!starve && a.n_items <= w.items_cap && (rc2 = expand_more(ctx, w, a, t.n0, P.launches))) return rc2;
             CU(ctx, cudaMemsetAsync(w.next_root, 0, sizeof(unsigned long long), s));
             const bool use_items = a.n_items <= w.items_cap;
             const int gr = grid_for(ctx, nr * 32, 128, 16);
             if (use_items) {
-                if ((rc2 = item_passes(ctx, w, a, mode == kMark ? 2 : 1, split, P.launches, P.item_passes))) return rc2;
+                if ((rc2 = item_passes(ctx, w, a, mode == kMark ? 2 : 1, split, starve, P.launches, P.item_passes))) return rc2;
             } else if (mode == kMark) {
                 P.launches++;
                 k_final_search<kMark><<<gr, 128, 0, s>>>(a);
@@ -3904,7 +3989,7 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
                 CUF(cudaGetLastError());
                 RCF(P.read_stats());
                 a.n_items = w.st_h->n_items;
-                if (a.n_items <= w.items_cap) RCF(expand_more(ctx, w, a, t.n0, P.launches));
+                if (!starve && a.n_items <= w.items_cap) RCF(expand_more(ctx, w, a, t.n0, P.launches));
                 if (a.n_items <= w.items_cap) {
                     RCF(run_items(false));
                 } else {
@@ -4479,6 +4564,12 @@ int ccpm_result_matches(ccpm_ctx_t ctx, ccpm_result_t r, ccpm_tmpl_t tm, const c
     const int hub_deg = opt.hub_degree > 0 ? std::min(opt.hub_degree, kMaxHubDeg) : kDefaultHubDeg;
     const uint64_t budget = opt.search_budget ? opt.search_budget : ~0ull;
     const uint64_t split = opt.search_split < 0 ? 0 : (opt.search_split == 0 ? kSpillAfter : (uint64_t)opt.search_split);
+    // a caller's own budget counts windows as one search scans them: no handing
+    // on to idle warps, which would restart its count.  Those searches are
+    // spread up front instead (expand_more: a kernel and a host round trip per
+    // level), which is slower where both work: 8.3 against 7.7 ms on the 5-cycle
+    // template over 16M vertices, 32 against 27 ms for a batch over 4M
+    const bool starve = opt.search_split >= 0 && opt.search_budget == 0;
     int rc = ws_ensure(ctx, g, hub_deg);
     if (rc) return rc;
     if ((rc = ensure_label_rows(ctx, g))) return rc;
@@ -4558,10 +4649,10 @@ int ccpm_result_matches(ccpm_ctx_t ctx, ccpm_result_t r, ccpm_tmpl_t tm, const c
         CUR(cudaMemcpyAsync(w.st_h, w.st, sizeof(RoundStats), cudaMemcpyDeviceToHost, s));
         CUR(cudaStreamSynchronize(s));
         a.n_items = w.st_h->n_items;
-        if (a.n_items <= w.items_cap && (rc = expand_more(ctx, w, a, t.n0, launches))) { release(); return rc; }
+        if (!starve && a.n_items <= w.items_cap && (rc = expand_more(ctx, w, a, t.n0, launches))) { release(); return rc; }
         CUR(cudaMemsetAsync(w.next_root, 0, sizeof(unsigned long long), s));
         if (a.n_items <= w.items_cap) {
-            if ((rc = item_passes(ctx, w, a, 3, split, launches, passes))) { release(); return rc; }
+            if ((rc = item_passes(ctx, w, a, 3, split, starve, launches, passes))) { release(); return rc; }
         } else {
             k_final_search<kList><<<grid_for(ctx, n_roots * 32, 128, 16), 128, 0, s>>>(a);
             CUR(cudaGetLastError());
