@@ -337,7 +337,6 @@ void build_dev_tmpl(const Template &t, DevTmpl &d) {
     std::memset(&d, 0, sizeof(d));
     d.n0 = t.n0;
     for (int q = 0; q < t.n0; q++) d.adj[q] = t.adj[q];
-    int n = 0;
     for (int q = 0; q < t.n0; q++) {
         uint32_t done = 0;
         for (int b = 0; b < t.n0; b++) {
@@ -346,15 +345,23 @@ void build_dev_tmpl(const Template &t, DevTmpl &d) {
             for (int c = 0; c < t.n0; c++)
                 if (((t.adj[q] >> c) & 1u) && t.labels[c] == t.labels[b]) grp |= 1u << c;
             done |= grp;
-            if (popc(grp) >= 2 && n < kMaxCls) {
-                d.cls_mask[n] = grp;
-                d.cls_need[n] = (uint32_t)popc(grp);
-                d.cls_q[n] = (uint32_t)q;
-                n++;
-            }
+            if (popc(grp) >= 2) add_class(d, q, grp);
         }
     }
-    d.n_cls = n;
+}
+
+// Template vertex q needs popc(grp) neighbours meeting grp.  The number needed
+// is the mask's size, so vertices with the same mask share one class, and the
+// rounds count each mask once (a 5-clique of labels 6,7,6,7,8 has six such
+// pairs and two masks).
+void add_class(DevTmpl &d, int q, uint32_t grp) {
+    int c = 0;
+    while (c < d.n_cls && d.cls_mask[c] != grp) c++;
+    if (c == kMaxCls) return;                        // never: at most kMaxCls pairs are accepted
+    d.cls_mask[c] = grp;
+    d.cls_need[c] = (uint32_t)popc(grp);
+    d.cls_q[c] |= 1u << q;
+    d.n_cls = std::max(d.n_cls, c + 1);
 }
 
 void build_plan(const Template &t, uint32_t svert, const uint32_t *sadj, int root,

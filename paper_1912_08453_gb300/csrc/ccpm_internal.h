@@ -18,9 +18,10 @@ constexpr int kMaxHubDeg = 1 << 24; // larger hub_degree options are clamped to 
 constexpr int64_t kEntryLabelRows = (int64_t)1 << 22;   // first-round rows that pay for the entry labels
 constexpr uint64_t kDefaultSearchBudget = 1ull << 22;
 
-// Template tables for the LCC kernels.  A "class" is (q, L) with
-// |adj_L(q)| >= 2: vertex q of the template needs at least `need` distinct
-// active neighbours whose omega meets `mask` = adj_L(q) (Section 4.1 / Section 4.3).
+// Template tables for the LCC kernels.  A "class" is a set adj_L(q) of two or
+// more equally labelled neighbours: every template vertex that has this set
+// (cls_q, a mask) needs at least `need` distinct active neighbours whose omega
+// meets `mask` = adj_L(q) (Section 4.1 / Section 4.3).
 struct DevTmpl {
     int n0;
     int n_cls;
@@ -104,6 +105,7 @@ int  template_build(Template &t, int n0, const uint8_t *labels, int m0, const in
 int  constraints_generate(Template &t, std::string &err);
 uint64_t count_automorphisms(const Template &t);
 void build_dev_tmpl(const Template &t, DevTmpl &d);
+void add_class(DevTmpl &d, int q, uint32_t grp);
 // order[] of S's vertices from `root`: greedy, most back edges first, then
 // fewest live candidates (qlive[q]: vertices whose omega holds q, when given;
 // otherwise the background frequency of q's label), then lowest id.

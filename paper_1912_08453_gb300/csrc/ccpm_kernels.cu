@@ -133,6 +133,30 @@ struct WarpBuf {
     }
 };
 
+// The leftovers of a block's warp buffers (at most 32 items each, counts in
+// cnt[0..8)): appended with one atomic for the block.  Called by every thread
+// after a __syncthreads.
+template <typename T>
+__device__ __forceinline__ void block_flush(const WarpBuf<T> &b, const int *cnt, int wib) {
+    __shared__ unsigned int base;
+    int before = 0, total = 0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); w++) {
+        if (w < wib) before += cnt[w];
+        total += cnt[w];
+    }
+    if (total == 0) return;                          // block-uniform
+    if (threadIdx.x == 0) base = atomicAdd(b.gcount, (unsigned int)total);
+    __syncthreads();
+    if ((int)lane_id() < cnt[wib]) b.out[base + before + lane_id()] = b.buf[lane_id()];
+    __syncthreads();                                 // base is reused by the next list
+}
+
+__device__ __forceinline__ unsigned long long warp_total(unsigned long long x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(FULL_MASK, x, o);
+    return x;
+}
+
 // Zero the bits of CSR entries [beg, end); `G` lanes cooperate.  Words fully
 // inside the range belong to this row alone and are stored; the two boundary
 // words are shared with neighbouring rows and are cleared atomically.
@@ -247,7 +271,6 @@ struct LccArgs {
     int hub_deg;
     int64_t *deg;                 // entries each listed vertex keeps (0 if it dies), or nullptr
     int med_chunk;                // medium vertices a warp prefetches together (1..16)
-    int small_chunk;              // unused by the short-row path (32 rows per batch)
     // first round after a fresh init: omega(u) is the initial mask of u's
     // label, so the neighbour gather reads the 1-byte label instead of the
     // 4-byte omega word (lab0 = labels, lmask = label -> initial omega)
@@ -528,7 +551,7 @@ __device__ __forceinline__ uint32_t decide(uint32_t wv, const Partial<MAXC> &p, 
     }
 #pragma unroll
     for (int c = 0; c < MAXC; c++)
-        if (c < s.n_cls && p.cnt[c] < s.cls_need[c]) keep &= ~(1u << s.cls_q[c]);
+        if (c < s.n_cls && p.cnt[c] < s.cls_need[c]) keep &= ~s.cls_q[c];
     if (p.nN == 0u) keep = 0u;
     return keep;
 }
@@ -546,7 +569,7 @@ struct LccTally {
     uint32_t changed = 0;
 };
 
-// Short rows, 32 per warp batch (lane i owns row i of the batch).  The rows'
+// Short rows, up to 32 per warp batch (lane i owns row i of the batch).  The rows'
 // entries are walked as one stream, 32 per step with one entry per lane, so
 // lanes stay busy whatever the row lengths.  A step holds pieces of several
 // rows: every lane finds its row from the piece starts, and per-row sums are
@@ -602,10 +625,16 @@ __device__ __forceinline__ void short_rows(const LccArgs &a, const SmemTmpl &s, 
                                            const uint32_t (&cm)[4], ShortRows &sr, int64_t first, int64_t stride,
                                            int64_t n_small, WarpBuf<int32_t> &bs, LccTally &tl) {
     const int lane = (int)lane_id();
-    const int64_t n_batch = (n_small + 31) / 32;
+    // A batch is one serial walk over its rows' entries: 32 rows of 50 entries
+    // take 50 steps of a microsecond each.  A frontier that gives the resident
+    // warps less than 32 rows each is dealt out in smaller batches (a round over
+    // 3000 such rows of an 8192-vertex graph: 55 us with 32 rows to a warp, 10 us
+    // with one).
+    const int per = (int)max((int64_t)1, min((int64_t)32, n_small / stride));
+    const int64_t n_batch = (n_small + per - 1) / per;
     auto load_v = [&](int64_t ch) -> int32_t {
-        const int64_t idx = ch * 32 + lane;
-        return (ch < n_batch && idx < n_small) ? a.small_in[idx] : -1;
+        const int64_t idx = ch * per + lane;
+        return (ch < n_batch && lane < per && idx < n_small) ? a.small_in[idx] : -1;
     };
     int32_t v_nx = load_v(first);
     uint32_t wv_nx = 0u;
@@ -753,6 +782,8 @@ k_lcc_round(LccArgs a, DevTmpl t) {
     __shared__ ChunkItem cbuf[8][32];
     __shared__ ShortRows srows[8];
     __shared__ int scnt[3][8];
+    __shared__ unsigned long long totals[6];
+    if (threadIdx.x < 6) totals[threadIdx.x] = 0ull;
     load_tmpl(s, t);
     if (a.lab0)
         for (int i = threadIdx.x; i < 256; i += blockDim.x) slm[i] = a.lmask.m[i];
@@ -882,27 +913,28 @@ k_lcc_round(LccArgs a, DevTmpl t) {
     // (3) short rows: 32 vertices per warp batch, entries streamed flat
     short_rows<MAXC, DENSE>(a, s, slm, cm, srows[wib], gwarp, nwarps, n_small, bs, tl);
 
-    bs.flush();
-    bm.flush();
-    bc.flush();
-    // warp totals
-    unsigned long long scanned64 = tl.scanned;
-    for (int o = 16; o > 0; o >>= 1) {
-        scanned64 += __shfl_xor_sync(FULL_MASK, scanned64, o);
-        tl.rows += __shfl_xor_sync(FULL_MASK, tl.rows, o);
-        tl.alive += __shfl_xor_sync(FULL_MASK, tl.alive, o);
-        tl.kept += __shfl_xor_sync(FULL_MASK, tl.kept, o);
-        tl.rows_next += __shfl_xor_sync(FULL_MASK, tl.rows_next, o);
-        tl.changed |= __shfl_xor_sync(FULL_MASK, tl.changed, o);
-    }
+    // what is left in the warps' buffers and their totals go out once per block:
+    // with a warp each, the thousands of atomics on one address lasted longer
+    // than the round itself on small frontiers
+    __syncthreads();
+    block_flush(bs, &scnt[0][0], wib);
+    block_flush(bm, &scnt[1][0], wib);
+    block_flush(bc, &scnt[2][0], wib);
+    const unsigned long long warp_sum[5] = {warp_total(tl.scanned), warp_total(tl.rows), warp_total(tl.alive),
+                                            warp_total(tl.kept), warp_total(tl.rows_next)};
+    const bool changed = __any_sync(FULL_MASK, tl.changed != 0u);
     if (lane == 0) {
-        if (scanned64) atomicAdd(&a.st->scanned, scanned64);
-        if (tl.rows) atomicAdd(&a.st->row_entries, tl.rows);
-        if (tl.alive) atomicAdd(&a.st->alive, tl.alive);
-        if (tl.kept) atomicAdd(&a.st->kept, tl.kept);
-        if (tl.rows_next) atomicAdd(&a.st->rows_next, tl.rows_next);
-        if (tl.changed) atomicOr(&a.st->changed, 1u);
+#pragma unroll
+        for (int i = 0; i < 5; i++)
+            if (warp_sum[i]) atomicAdd(&totals[i], warp_sum[i]);
+        if (changed) totals[5] = 1ull;
     }
+    __syncthreads();
+    if (threadIdx.x < 5 && totals[threadIdx.x]) {
+        // row_entries, alive, kept and rows_next follow one another
+        atomicAdd(threadIdx.x == 0 ? &a.st->scanned : &a.st->row_entries + (threadIdx.x - 1), totals[threadIdx.x]);
+    }
+    if (threadIdx.x == 5 && totals[5]) atomicOr(&a.st->changed, 1u);
 }
 
 // -------------------------------------------------------------------------
@@ -3039,10 +3071,9 @@ struct Pipeline {
         // enough that every resident warp gets several of them
         const int64_t resident = (int64_t)grid_sms(ctx) * 32;
         a.med_chunk = (int)std::max<int64_t>(1, std::min<int64_t>(16, n_med / (4 * resident)));
-        a.small_chunk = n_small >= 32 * 4 * resident ? 32 : (n_small >= 16 * 4 * resident ? 16 : 8);
         // a queued round does not know its sizes: one full resident wave
         int64_t warps = prev ? ((int64_t)1 << 40)
-                             : n_chunk + (n_med + a.med_chunk - 1) / a.med_chunk + (n_small + a.small_chunk - 1) / a.small_chunk;
+                             : n_chunk + (n_med + a.med_chunk - 1) / a.med_chunk + n_small;
         launches++;
         lcc_launches++;
         // one resident wave: grid-stride work is split evenly over warps that all run at once
@@ -4952,6 +4983,7 @@ const char *noalloc_template(int n0, const uint8_t *labels, int m0, const int32_
         d.adj[a] |= 1u << b;
         d.adj[b] |= 1u << a;
     }
+    int n_pairs = 0;
     uint32_t seen = 1u, fr = 1u;
     while (fr) {
         uint32_t nx = 0;
@@ -4971,11 +5003,8 @@ const char *noalloc_template(int n0, const uint8_t *labels, int m0, const int32_
                 if (((d.adj[q] >> c) & 1u) && labels[c] == labels[b]) grp |= 1u << c;
             done |= grp;
             if (__builtin_popcount(grp) >= 2) {
-                if (d.n_cls >= kMaxCls) return "template has more than 32 label-multiplicity classes";
-                d.cls_mask[d.n_cls] = grp;
-                d.cls_need[d.n_cls] = (uint32_t)__builtin_popcount(grp);
-                d.cls_q[d.n_cls] = (uint32_t)q;
-                d.n_cls++;
+                if (++n_pairs > kMaxCls) return "template has more than 32 label-multiplicity classes";
+                add_class(d, q, grp);
             }
         }
     }
@@ -5097,7 +5126,6 @@ int lcc_fixpoint_noalloc_body(int device, void *cuda_stream, int64_t n, int64_t 
         a.hub_deg = hub;
         a.deg = nullptr;
         a.med_chunk = 1;
-        a.small_chunk = 8;
         a.lab0 = nullptr;
         a.elab = nullptr;
         a.sparse = 0;
@@ -5107,7 +5135,8 @@ int lcc_fixpoint_noalloc_body(int device, void *cuda_stream, int64_t n, int64_t 
         a.nw_bytes = 0;
         a.nw_cur = nullptr;
         a.nw_next = nullptr;
-        const int g = grid((n_chunk + n_med + (n_small + 7) / 8) * 32, 256);
+        // at most one resident wave (four blocks an SM): the rows are dealt out evenly over the warps
+        const int g = std::min(grid((n_chunk + n_med + n_small) * 32, 256), 4 * num_sms);
         if (dt.n_cls == 0) k_lcc_round<0, false><<<g, 256, 0, s>>>(a, dt);
         else if (dt.n_cls <= 4) k_lcc_round<4, false><<<g, 256, 0, s>>>(a, dt);
         else k_lcc_round<32, false><<<g, 256, 0, s>>>(a, dt);
