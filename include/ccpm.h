@@ -186,9 +186,10 @@ typedef struct {
     double   ms_search_kernel;     /* device time of the NLCC search kernels  */
     int64_t  search_launches;      /* their launches                          */
     int64_t  search_entries_nlcc;  /* row entries those kernels examined      */
-    /* what the kernel itself reads and writes per round: 24 B per active
-     * vertex (two int64 offsets, omega read and write) + 4.125 B per entry of
-     * an active row (column index, edge bit) + 4 B per active entry (gather) */
+    /* what the kernel itself reads and writes per round: 24 B per vertex it
+     * evaluates (two int64 offsets, omega read and write) + 4.125 B per entry
+     * of such a row (column index, edge bit) + 4 B per active entry (gather);
+     * later rounds over large rows evaluate only the vertices near a change   */
     int64_t  lcc_kernel_bytes;
     int64_t  lcc_first_entries;    /* M_a of the first round after init       */
     double   ms_lcc_first;         /* device time of that round               */

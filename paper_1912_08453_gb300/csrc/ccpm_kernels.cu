@@ -9,8 +9,8 @@
 // Edge bits are kept exact for rows of active vertices only.  A bit in the row
 // of an active v that points to a vertex u eliminated in the previous round is
 // cleared lazily: the next round sees omega(u) = 0, treats the entry as
-// inactive and clears the bit.  Rows of eliminated vertices are zeroed when
-// they die; rows of vertices that never become active are zeroed only when
+// inactive and clears the bit.  Rows of eliminated vertices, and of vertices
+// that never become active, keep bits that no round reads; they are zeroed when
 // the edge bitmap is handed back without the final search.  Once the rows are
 // compacted (K4) the rounds read the compacted rows and their own bitmap; the
 // full bitmap is then frozen and handed back in its fixpoint form (bit, both
@@ -60,7 +60,19 @@ struct RoundStats {
     unsigned int n_spill;         // items handed on by searches that ran long (reserved)
     unsigned int spill_stop;      // the spill list is valid below this index (see spill)
     unsigned int skipped;         // LCC round queued after the fixpoint: did nothing
+    // changes of omega waiting to be passed on to the neighbours (Change list,
+    // and the pieces of their long rows); for a delta round also what its
+    // vertices had before: entries active after their last evaluation, and the
+    // vertices it eliminates with the entries in their rows
+    unsigned int n_chg, n_chg_piece;
+    unsigned int died;            // full rounds: survivors are alive - died
+    unsigned long long old_kept, died_rows;
 };
+
+// A vertex whose omega a round (or a non-local check) has changed, and its new
+// omega; a piece of its row if that is long.
+struct Change { int32_t v; uint32_t w; };
+struct ChangePiece { int32_t v, c; };
 
 struct HubAcc {                   // partial LCC state of one split row
     uint32_t U, nN, flags, done;
@@ -202,10 +214,17 @@ __device__ __forceinline__ uint32_t grp_sum(uint32_t x) {
 
 struct LabelMask { uint32_t m[256]; };
 
+// The narrow copy of omega the LCC gathers read (1 or 2 bytes per vertex; 0: none).
+__device__ __forceinline__ void store_narrow(void *nw, int bytes, int64_t v, uint32_t w) {
+    if (bytes == 1) ((uint8_t *)nw)[v] = (uint8_t)w;
+    else if (bytes == 2) ((uint16_t *)nw)[v] = (uint16_t)w;
+}
+
 __global__ void __launch_bounds__(256)
 k_init(int64_t n, const int64_t *__restrict__ rp, const uint8_t *__restrict__ lab, LabelMask lm,
-       const uint32_t *__restrict__ om_in, uint32_t *om0, uint32_t *om1, int32_t *small_out, int32_t *med_out,
-       ChunkItem *chunk_out, HubAcc *acc, RoundStats *st, int hub_deg, int short_max) {
+       const uint32_t *__restrict__ om_in, uint32_t *om0, uint32_t *om1, void *nw0, void *nw1, int nw_bytes,
+       int32_t *small_out, int32_t *med_out, ChunkItem *chunk_out, HubAcc *acc, RoundStats *st, int hub_deg,
+       int short_max, unsigned int set_changed) {
     __shared__ uint32_t slm[256];
     __shared__ int32_t sbuf[2][8][32];
     __shared__ int scnt[2][8];
@@ -226,6 +245,8 @@ k_init(int64_t n, const int64_t *__restrict__ rp, const uint8_t *__restrict__ la
             if (om_in) w &= om_in[v];     // resumed state, kept inside the initial one
             om0[v] = w;
             om1[v] = w;
+            store_narrow(nw0, nw_bytes, v, w);
+            store_narrow(nw1, nw_bytes, v, w);
             if (w) deg = rp[v + 1] - rp[v];
         }
         rows += (unsigned long long)deg;
@@ -247,6 +268,8 @@ k_init(int64_t n, const int64_t *__restrict__ rp, const uint8_t *__restrict__ la
     bm.flush();
     for (int o = 16; o > 0; o >>= 1) rows += __shfl_xor_sync(FULL_MASK, rows, o);
     if (lane_id() == 0 && rows) atomicAdd(&st->row_entries, rows);
+    // the first round reads these counters as those of a round before it
+    if (blockIdx.x == 0 && threadIdx.x == 0 && set_changed) st->changed = 1u;
 }
 
 // -------------------------------------------------------------------------
@@ -269,7 +292,13 @@ struct LccArgs {
     HubAcc *acc;
     RoundStats *st;
     int hub_deg;
-    int64_t *deg;                 // entries each listed vertex keeps (0 if it dies), or nullptr
+    uint32_t *deg;                // entries each evaluated vertex keeps (0 if it dies), or nullptr
+    // delta rounds (kDelta): the lists hold the vertices to look at again (their
+    // bit in `dirty` is set), omega is read and not written: what changes goes
+    // to the Change list
+    uint32_t *dirty;
+    Change *chg;
+    ChangePiece *chg_piece;
     int med_chunk;                // medium vertices a warp prefetches together (1..16)
     // first round after a fresh init: omega(u) is the initial mask of u's
     // label, so the neighbour gather reads the 1-byte label instead of the
@@ -308,9 +337,12 @@ __device__ __forceinline__ uint32_t gather_om(const uint32_t *__restrict__ om, c
 // omega'(v) of the next round, and its narrow copy.
 __device__ __forceinline__ void store_om(const LccArgs &a, int32_t v, uint32_t w) {
     a.om_next[v] = w;
-    if (a.nw_bytes == 1) ((uint8_t *)a.nw_next)[v] = (uint8_t)w;
-    else if (a.nw_bytes == 2) ((uint16_t *)a.nw_next)[v] = (uint16_t)w;
+    store_narrow(a.nw_next, a.nw_bytes, v, w);
 }
+
+// Rounds: the first after init (every edge bit of its rows set), over every
+// active vertex, and over the vertices near a change only.
+constexpr int kDense = 0, kFull = 1, kDelta = 2;
 
 template <int MAXC>
 struct Partial {
@@ -350,6 +382,50 @@ __device__ __forceinline__ void tally_entry(uint32_t w, uint32_t nbr_v, const Sm
 #pragma unroll
             for (int c = 0; c < MAXC; c++)
                 if (c < s.n_cls) p.cnt[c] += (w & s.cls_mask[c]) ? 1u : 0u;
+        }
+    }
+}
+
+// Visit the entries of [beg, end) whose bit is set, 32 at a time and in
+// ascending order: f(e, valid) is called by all lanes, lane i with the i-th
+// set entry of the batch (valid) or none.  The bits are read 32 words
+// (1024 entries) per load, so long runs of inactive entries cost little.
+template <typename F>
+__device__ __forceinline__ void for_set_bits(const uint32_t *bits, int64_t beg, int64_t end, F &&f) {
+    const int lane = (int)lane_id();
+    const int64_t wb = beg >> 5, we = (end + 31) >> 5;
+    for (int64_t w0 = wb; w0 < we; w0 += 32) {
+        const int64_t wi = w0 + lane;
+        uint32_t word = 0u;
+        if (wi < we) {
+            word = bits[wi];
+            const int64_t e0 = wi << 5;
+            if (e0 < beg) word &= ~0u << (uint32_t)(beg - e0);
+            if (end - e0 < 32) word &= (1u << (uint32_t)(end - e0)) - 1u;
+        }
+        const uint32_t c = __popc(word);
+        uint32_t incl = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(FULL_MASK, incl, o);
+            if (lane >= o) incl += t;
+        }
+        const uint32_t total = __shfl_sync(FULL_MASK, incl, 31);
+        const uint32_t excl = incl - c;
+        for (uint32_t k0 = 0; k0 < total; k0 += 32) {
+            const uint32_t k = k0 + (uint32_t)lane;
+            int i = 0;                                // last word whose prefix is <= k
+#pragma unroll
+            for (int step = 16; step > 0; step >>= 1) {
+                const uint32_t ex = __shfl_sync(FULL_MASK, excl, i + step);
+                if (ex <= k) i += step;
+            }
+            const uint32_t wd = __shfl_sync(FULL_MASK, word, i);
+            const uint32_t ex_i = __shfl_sync(FULL_MASK, excl, i);
+            const bool valid = k < total;
+            int64_t e = -1;
+            if (valid) e = ((w0 + i) << 5) + (int64_t)select_bit(wd, k - ex_i);
+            f(e, valid);
         }
     }
 }
@@ -566,8 +642,46 @@ __device__ __forceinline__ uint32_t nbr_mask(uint32_t wv, const SmemTmpl &s) {
 struct LccTally {
     uint32_t scanned = 0;          // per lane
     unsigned long long rows = 0, alive = 0, kept = 0, rows_next = 0;   // lane 0 (or the row lanes)
-    uint32_t changed = 0;
+    unsigned long long old_kept = 0, died_rows = 0;                    // delta rounds
+    uint32_t changed = 0, died = 0;
 };
+
+// What a round decided for vertex v (one lane): its omega was wv and is now
+// `keep`, `kept` of the `len` entries of its row stay active.  A full round
+// writes omega'; a delta round lists the change (long: the row is longer than
+// hub_deg, its pieces are listed too).
+template <int MODE>
+__device__ __forceinline__ void settle(const LccArgs &a, int32_t v, uint32_t wv, uint32_t keep, uint32_t kept,
+                                       int64_t len, bool is_long, LccTally &tl) {
+    if (keep) { tl.kept += kept; tl.rows_next += (unsigned long long)len; }
+    else tl.died++;
+    if (MODE == kDelta) {
+        tl.old_kept += a.deg[v];
+        if (keep == 0u) tl.died_rows += (unsigned long long)len;
+        if (keep != wv && is_long) {
+            const unsigned int np = (unsigned int)((len + a.hub_deg - 1) / a.hub_deg);
+            const unsigned int b = atomicAdd(&a.st->n_chg_piece, np);
+            for (unsigned int c = 0; c < np; c++)
+                a.chg_piece[b + c] = ChangePiece{v, (int32_t)c};
+        }
+    } else {
+        store_om(a, v, keep);
+    }
+    if (a.deg) a.deg[v] = keep ? kept : 0u;
+}
+
+// A listed vertex that died in an earlier round.
+template <int MODE>
+__device__ __forceinline__ void settle_dead(const LccArgs &a, int32_t v) {
+    if (MODE == kDelta) return;
+    store_om(a, v, 0u);
+    if (a.deg) a.deg[v] = 0u;
+}
+
+__device__ __forceinline__ void clear_dirty(const LccArgs &a, int32_t v) {
+    atomicAnd(&a.dirty[v >> 5], ~(1u << (v & 31)));
+}
+
 
 // Short rows, up to 32 per warp batch (lane i owns row i of the batch).  The rows'
 // entries are walked as one stream, 32 per step with one entry per lane, so
@@ -620,10 +734,11 @@ __device__ __forceinline__ void short_locate(const LccArgs &a, ShortRows &sr, in
     __syncwarp();                                // sr.row is rewritten by the next step
 }
 
-template <int MAXC, bool DENSE>
+template <int MAXC, int MODE>
 __device__ __forceinline__ void short_rows(const LccArgs &a, const SmemTmpl &s, const uint32_t *slm,
                                            const uint32_t (&cm)[4], ShortRows &sr, int64_t first, int64_t stride,
-                                           int64_t n_small, WarpBuf<int32_t> &bs, LccTally &tl) {
+                                           int64_t n_small, WarpBuf<int32_t> &bs, WarpBuf<Change> &bg, LccTally &tl) {
+    constexpr bool DENSE = MODE == kDense;
     const int lane = (int)lane_id();
     // A batch is one serial walk over its rows' entries: 32 rows of 50 entries
     // take 50 steps of a microsecond each.  A frontier that gives the resident
@@ -737,8 +852,8 @@ __device__ __forceinline__ void short_rows(const LccArgs &a, const SmemTmpl &s, 
             }
             cur = nx;
         }
+        uint32_t keep = 0u;
         if (v >= 0) {
-            uint32_t keep = 0u;
             if (wv) {
                 Partial<MAXC> p;
                 p.U = U;
@@ -748,22 +863,25 @@ __device__ __forceinline__ void short_rows(const LccArgs &a, const SmemTmpl &s, 
                 keep = decide<MAXC>(wv, p, s);
                 tl.rows += (unsigned long long)d;
                 tl.alive++;
-                if (keep) { tl.kept += N; tl.rows_next += (unsigned long long)d; }
                 if (keep != wv) tl.changed = 1u;
-                if (keep == 0u) clear_row<1>(a.ebits, b, b + d, 0);
+                settle<MODE>(a, v, wv, keep, N, d, d > a.hub_deg, tl);
+            } else {
+                settle_dead<MODE>(a, v);
             }
-            store_om(a, v, keep);
-            if (a.deg) a.deg[v] = keep ? (int64_t)N : 0;
+            if (MODE == kDelta) clear_dirty(a, v);
         }
-        // the batch's vertices that were active at the start of the round
-        bs.push(v >= 0 && wv != 0u, v);
+        // the batch's vertices that were active at the start of the round (delta:
+        // those whose omega changes)
+        if (MODE == kDelta) bg.push(v >= 0 && keep != wv, Change{v, keep});
+        else bs.push(v >= 0 && wv != 0u, v);
         __syncwarp();                            // sr.off / sr.nbr are rewritten by the next batch
     }
 }
 
-template <int MAXC, bool DENSE>
+template <int MAXC, int MODE>
 __global__ void __launch_bounds__(256, 4)
 k_lcc_round(LccArgs a, DevTmpl t) {
+    constexpr bool DENSE = MODE == kDense;
     int64_t n_small = a.n_small, n_med = a.n_med, n_chunk = a.n_chunk;
     int MB = a.med_chunk;
     if (a.prev) {
@@ -771,9 +889,12 @@ k_lcc_round(LccArgs a, DevTmpl t) {
             if (blockIdx.x == 0 && threadIdx.x == 0) a.st->skipped = 1u;
             return;
         }
-        n_small = a.prev->n_small;
-        n_med = a.prev->n_med;
-        n_chunk = a.prev->n_chunk;
+        // a full round's lists were written by the round before, a delta
+        // round's by k_push into its own counters
+        const RoundStats *sizes = MODE == kDelta ? a.st : a.prev;
+        n_small = sizes->n_small;
+        n_med = sizes->n_med;
+        n_chunk = sizes->n_chunk;
         MB = (int)max((int64_t)1, min((int64_t)16, n_med / (4 * (int64_t)a.resident_warps)));
     }
     __shared__ SmemTmpl s;
@@ -781,16 +902,18 @@ k_lcc_round(LccArgs a, DevTmpl t) {
     __shared__ int32_t sbuf[2][8][32];
     __shared__ ChunkItem cbuf[8][32];
     __shared__ ShortRows srows[8];
-    __shared__ int scnt[3][8];
-    __shared__ unsigned long long totals[6];
-    if (threadIdx.x < 6) totals[threadIdx.x] = 0ull;
+    __shared__ Change gbuf[MODE == kDelta ? 8 : 1][32];
+    __shared__ int scnt[4][8];
+    __shared__ unsigned long long totals[9];
+    if (threadIdx.x < 9) totals[threadIdx.x] = 0ull;
     load_tmpl(s, t);
     if (a.lab0)
         for (int i = threadIdx.x; i < 256; i += blockDim.x) slm[i] = a.lmask.m[i];
     const int wib = threadIdx.x >> 5;
     const int lane = (int)lane_id();
-    if (lane == 0) { scnt[0][wib] = 0; scnt[1][wib] = 0; scnt[2][wib] = 0; }
+    if (lane == 0) { scnt[0][wib] = 0; scnt[1][wib] = 0; scnt[2][wib] = 0; scnt[3][wib] = 0; }
     __syncthreads();
+    WarpBuf<Change> bg{gbuf[MODE == kDelta ? wib : 0], &scnt[3][wib], a.chg, &a.st->n_chg};
     WarpBuf<int32_t> bs{sbuf[0][wib], &scnt[0][wib], a.small_out, &a.st->n_small};
     WarpBuf<int32_t> bm{sbuf[1][wib], &scnt[1][wib], a.med_out, &a.st->n_med};
     WarpBuf<ChunkItem> bc{cbuf[wib], &scnt[2][wib], a.chunk_out, &a.st->n_chunk};
@@ -810,8 +933,8 @@ k_lcc_round(LccArgs a, DevTmpl t) {
         const uint32_t wv = __ldg(a.om_cur + ci.v);
         if (wv == 0u) {
             if (ci.c == 0 && lane == 0) {
-                store_om(a, ci.v, 0u);
-                if (a.deg) a.deg[ci.v] = 0;
+                settle_dead<MODE>(a, ci.v);
+                if (MODE == kDelta) clear_dirty(a, ci.v);
             }
             continue;
         }
@@ -828,6 +951,7 @@ k_lcc_round(LccArgs a, DevTmpl t) {
 #pragma unroll
         for (int c = 0; c < MAXC; c++) p.cnt[c] = grp_sum<32>(p.cnt[c]);
         HubAcc *h = a.acc + ci.slot;
+        Change change{ci.v, wv};
         unsigned int ticket = 0;
         if (lane == 0) {
             if (p.U) atomicOr(&h->U, p.U);
@@ -850,19 +974,19 @@ k_lcc_round(LccArgs a, DevTmpl t) {
             for (int c = 0; c < MAXC; c++) tot.cnt[c] = atomicAdd(&h->cnt[c], 0u);
             uint32_t keep = decide<MAXC>(wv, tot, s);
             if (lane == 0) {
-                store_om(a, ci.v, keep);
-                if (a.deg) a.deg[ci.v] = keep ? (int64_t)tot.nN : 0;
+                settle<MODE>(a, ci.v, wv, keep, tot.nN, rend - rbeg, true, tl);
+                if (MODE == kDelta) clear_dirty(a, ci.v);
             }
-            if (lane == 0 && keep) { tl.kept += tot.nN; tl.rows_next += (unsigned long long)(rend - rbeg); }
+            change.w = keep;
             if (keep != wv || tot.achg) tl.changed = 1u;
-            if (keep == 0u) clear_row<32>(a.ebits, rbeg, rend, lane);
             __syncwarp();
             if (lane == 0) {
                 h->U = 0u; h->nN = 0u; h->flags = 0u; h->done = 0u;
                 for (int c = 0; c < MAXC; c++) h->cnt[c] = 0u;
             }
         }
-        bc.push(lane == 0, ci);
+        if (MODE == kDelta) bg.push(lane == 0 && change.w != wv, change);
+        else bc.push(lane == 0, ci);
     }
 
     // (2) medium rows: one warp per vertex, taken 16 at a time: the list
@@ -879,12 +1003,12 @@ k_lcc_round(LccArgs a, DevTmpl t) {
             wl = __ldg(a.om_cur + vl);
             if (wl) { bl = a.rp[vl]; el = a.rp[vl + 1]; }
         }
+        uint32_t wnew = wl;
         for (int j = 0; j < MB; j++) {
             const int32_t v = __shfl_sync(FULL_MASK, vl, j);
             if (v < 0) break;
             const uint32_t wv = __shfl_sync(FULL_MASK, wl, j);
             const int64_t beg = __shfl_sync(FULL_MASK, bl, j), end = __shfl_sync(FULL_MASK, el, j);
-            uint32_t keep = 0u, p_nN = 0u;
             if (wv) {
                 if (lane == 0) { tl.rows += (unsigned long long)(end - beg); tl.alive++; }
                 Partial<MAXC> p;
@@ -895,46 +1019,214 @@ k_lcc_round(LccArgs a, DevTmpl t) {
                 p.achg = grp_or<32>(p.achg);
 #pragma unroll
                 for (int c = 0; c < MAXC; c++) p.cnt[c] = grp_sum<32>(p.cnt[c]);
-                keep = decide<MAXC>(wv, p, s);
-                p_nN = p.nN;
-                if (lane == 0 && keep) { tl.kept += p.nN; tl.rows_next += (unsigned long long)(end - beg); }
+                const uint32_t keep = decide<MAXC>(wv, p, s);
                 if (keep != wv || p.achg) tl.changed = 1u;
-                if (keep == 0u) clear_row<32>(a.ebits, beg, end, lane);
-            }
-            if (lane == 0) {
-                store_om(a, v, keep);
-                if (a.deg) a.deg[v] = keep ? (int64_t)p_nN : 0;
+                if (lane == 0) settle<MODE>(a, v, wv, keep, p.nN, end - beg, end - beg > a.hub_deg, tl);
+                if (lane == j) wnew = keep;
+            } else if (lane == 0) {
+                settle_dead<MODE>(a, v);
             }
         }
-        // the chunk's vertices that were active at the start of the round, in one push
-        bm.push(vl >= 0 && wl != 0u, vl);
+        // the chunk's vertices that were active at the start of the round (delta:
+        // those whose omega changes), in one push
+        if (MODE == kDelta) {
+            if (vl >= 0) clear_dirty(a, vl);
+            bg.push(vl >= 0 && wnew != wl, Change{vl, wnew});
+        } else {
+            bm.push(vl >= 0 && wl != 0u, vl);
+        }
     }
 
     // (3) short rows: 32 vertices per warp batch, entries streamed flat
-    short_rows<MAXC, DENSE>(a, s, slm, cm, srows[wib], gwarp, nwarps, n_small, bs, tl);
+    short_rows<MAXC, MODE>(a, s, slm, cm, srows[wib], gwarp, nwarps, n_small, bs, bg, tl);
 
     // what is left in the warps' buffers and their totals go out once per block:
     // with a warp each, the thousands of atomics on one address lasted longer
     // than the round itself on small frontiers
     __syncthreads();
-    block_flush(bs, &scnt[0][0], wib);
-    block_flush(bm, &scnt[1][0], wib);
-    block_flush(bc, &scnt[2][0], wib);
-    const unsigned long long warp_sum[5] = {warp_total(tl.scanned), warp_total(tl.rows), warp_total(tl.alive),
-                                            warp_total(tl.kept), warp_total(tl.rows_next)};
-    const bool changed = __any_sync(FULL_MASK, tl.changed != 0u);
-    if (lane == 0) {
-#pragma unroll
-        for (int i = 0; i < 5; i++)
-            if (warp_sum[i]) atomicAdd(&totals[i], warp_sum[i]);
-        if (changed) totals[5] = 1ull;
+    if (MODE == kDelta) {
+        block_flush(bg, &scnt[3][0], wib);
+    } else {
+        block_flush(bs, &scnt[0][0], wib);
+        block_flush(bm, &scnt[1][0], wib);
+        block_flush(bc, &scnt[2][0], wib);
+    }
+    auto add = [&](int i, unsigned long long x) {
+        x = warp_total(x);
+        if (lane == 0 && x) atomicAdd(&totals[i], x);
+    };
+    add(0, tl.scanned);
+    add(1, tl.rows);
+    add(2, tl.alive);
+    add(3, tl.kept);
+    add(4, tl.rows_next);
+    add(5, tl.changed);
+    add(6, tl.died);
+    if (MODE == kDelta) {
+        add(7, tl.old_kept);
+        add(8, tl.died_rows);
     }
     __syncthreads();
-    if (threadIdx.x < 5 && totals[threadIdx.x]) {
-        // row_entries, alive, kept and rows_next follow one another
-        atomicAdd(threadIdx.x == 0 ? &a.st->scanned : &a.st->row_entries + (threadIdx.x - 1), totals[threadIdx.x]);
+    const unsigned long long sum = threadIdx.x < 9 ? totals[threadIdx.x] : 0ull;
+    if (sum) {
+        switch (threadIdx.x) {
+            case 0: atomicAdd(&a.st->scanned, sum); break;
+            case 1: atomicAdd(&a.st->row_entries, sum); break;
+            case 2: atomicAdd(&a.st->alive, sum); break;
+            case 3: atomicAdd(&a.st->kept, sum); break;
+            case 4: atomicAdd(&a.st->rows_next, sum); break;
+            case 5: atomicOr(&a.st->changed, 1u); break;
+            case 6: atomicAdd(&a.st->died, (unsigned int)sum); break;
+            case 7: atomicAdd(&a.st->old_kept, sum); break;
+            default: atomicAdd(&a.st->died_rows, sum); break;
+        }
     }
-    if (threadIdx.x == 5 && totals[5]) atomicOr(&a.st->changed, 1u);
+}
+
+// -------------------------------------------------------------------------
+// Delta rounds.  What a round decides for a vertex depends on its own omega,
+// its neighbours' and the bits of its row, so a vertex can only be decided
+// otherwise than in the round before if its omega or a neighbour's changed
+// there.  k_push writes the changes (Jacobi: after the round that found them)
+// and lists the vertices to look at again: the changed ones and every
+// neighbour over an entry that was still active (a vertex that died keeps its
+// bits; no round reads them again).  k_lcc_round<., kDelta> evaluates these.  All
+// other active vertices would find what they found before: the entries they
+// scan are the entries they kept, so the counts of a round follow from the
+// totals and the evaluated vertices alone (Pipeline::lcc).
+//
+// An 8-vertex template over frequent labels on 32M vertices (10^9 entries)
+// eliminates 16M vertices in its first round and changes few after the second:
+// its rounds three to six took 3.2 ms each, nearly all of it gathers of
+// neighbours that had not changed, and take 1.6 ms together as delta rounds with
+// 0.3 ms of k_push (the LCC phase 22.7 -> 11.7 ms).
+// -------------------------------------------------------------------------
+
+struct PushArgs {
+    const int64_t *rp;
+    const int32_t *col;
+    const uint32_t *bits;
+    uint32_t *om;                 // the current omega and its narrow copy
+    void *nw;
+    int nw_bytes;
+    const uint32_t *om_old;       // after a full round: omega before it
+    const int32_t *small_in, *med_in;
+    const ChunkItem *chunk_in;
+    const Change *chg;
+    const ChangePiece *chg_piece;
+    const RoundStats *prev;       // the counters of the round (or check) that made the changes
+    uint32_t *dirty;
+    int32_t *small_out, *med_out;
+    ChunkItem *chunk_out;
+    RoundStats *st;               // list sizes of the round to come
+    int hub_deg, short_max;
+};
+
+// List the vertices u of the lanes with `want` that are not listed yet.
+__device__ __forceinline__ void list_dirty(const PushArgs &a, bool want, int32_t u, WarpBuf<int32_t> &bs,
+                                           WarpBuf<int32_t> &bm) {
+    if (want) {
+        const uint32_t m = 1u << (u & 31);
+        want = !(a.dirty[u >> 5] & m) && !(atomicOr(&a.dirty[u >> 5], m) & m);
+    }
+    int64_t deg = 0;
+    if (want) deg = a.rp[u + 1] - a.rp[u];
+    const int64_t small_max = a.hub_deg < a.short_max ? a.hub_deg : a.short_max;
+    bs.push(want && deg <= small_max, u);
+    bm.push(want && deg > small_max && deg <= a.hub_deg, u);
+    if (want && deg > a.hub_deg) {
+        const int nch = (int)((deg + a.hub_deg - 1) / a.hub_deg);
+        const int slot = (int)atomicAdd(&a.st->n_hub_slots, 1u);
+        const unsigned int base = atomicAdd(&a.st->n_chunk, (unsigned int)nch);
+        for (int c = 0; c < nch; c++) a.chunk_out[base + c] = ChunkItem{u, c, slot, nch};
+    }
+}
+
+// The neighbours over the active entries of [beg, end) in a changed vertex's row.
+__device__ __forceinline__ void push_row(const PushArgs &a, int64_t beg, int64_t end, WarpBuf<int32_t> &bs,
+                                         WarpBuf<int32_t> &bm) {
+    for_set_bits(a.bits, beg, end, [&](int64_t e, bool valid) {
+        int32_t u = 0;
+        if (valid) {
+            u = __ldg(a.col + e);
+            valid = a.om[u] != 0u;
+        }
+        list_dirty(a, valid, u, bs, bm);
+    });
+}
+
+// LISTS: the changes are those between om_old and om over the lists of a full
+// round; else they come from the Change list and are written to omega here.
+template <bool LISTS>
+__global__ void __launch_bounds__(256)
+k_push(PushArgs a) {
+    if (a.prev->changed == 0u) return;
+    __shared__ int32_t sbuf[2][8][32];
+    __shared__ int scnt[2][8];
+    const int wib = threadIdx.x >> 5;
+    const int lane = (int)lane_id();
+    if (lane == 0) { scnt[0][wib] = 0; scnt[1][wib] = 0; }
+    __syncthreads();
+    WarpBuf<int32_t> bs{sbuf[0][wib], &scnt[0][wib], a.small_out, &a.st->n_small};
+    WarpBuf<int32_t> bm{sbuf[1][wib], &scnt[1][wib], a.med_out, &a.st->n_med};
+    const int64_t gwarp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    // (1) pieces of long rows, one warp each
+    const int64_t n_piece = LISTS ? a.prev->n_chunk : a.prev->n_chg_piece;
+    for (int64_t it = gwarp; it < n_piece; it += nwarps) {
+        int32_t v, c;
+        if (LISTS) {
+            const ChunkItem ci = a.chunk_in[it];
+            v = ci.v;
+            c = ci.c;
+            const uint32_t w = a.om[v];
+            if (w == a.om_old[v]) continue;
+            if (c == 0) list_dirty(a, lane == 0 && w != 0u, v, bs, bm);
+        } else {
+            const ChangePiece cp = a.chg_piece[it];
+            v = cp.v;
+            c = cp.c;
+        }
+        const int64_t rend = a.rp[v + 1], beg = a.rp[v] + (int64_t)c * a.hub_deg;
+        push_row(a, beg, min(rend, beg + (int64_t)a.hub_deg), bs, bm);
+    }
+    // (2) the other rows, 32 vertices per warp step, each changed one walked by the warp
+    const int64_t n_small = LISTS ? a.prev->n_small : 0;
+    const int64_t n_rows = LISTS ? n_small + a.prev->n_med : a.prev->n_chg;
+    // few changes: fewer per warp, so that every warp gets some
+    const int per = (int)max((int64_t)1, min((int64_t)32, n_rows / nwarps));
+    for (int64_t b = gwarp * per; b < n_rows; b += nwarps * per) {
+        const int64_t idx = b + lane;
+        int32_t v = -1;
+        uint32_t w = 0u;
+        int64_t beg = 0, end = 0;
+        if (lane < per && idx < n_rows) {
+            if (LISTS) {
+                v = idx < n_small ? a.small_in[idx] : a.med_in[idx - n_small];
+                w = a.om[v];
+                if (w == a.om_old[v]) v = -1;
+            } else {
+                const Change ch = a.chg[idx];
+                v = ch.v;
+                w = ch.w;
+                a.om[v] = w;
+                store_narrow(a.nw, a.nw_bytes, v, w);
+            }
+            if (v >= 0) {
+                beg = a.rp[v];
+                end = a.rp[v + 1];
+            }
+        }
+        list_dirty(a, v >= 0 && w != 0u, v, bs, bm);
+        const bool walk = v >= 0 && (LISTS || end - beg <= a.hub_deg);   // long rows: (1)
+        for (uint32_t todo = __ballot_sync(FULL_MASK, walk); todo; todo &= todo - 1u) {
+            const int src = __ffs(todo) - 1;
+            push_row(a, __shfl_sync(FULL_MASK, beg, src), __shfl_sync(FULL_MASK, end, src), bs, bm);
+        }
+    }
+    __syncthreads();
+    block_flush(bs, &scnt[0][0], wib);
+    block_flush(bm, &scnt[1][0], wib);
 }
 
 // -------------------------------------------------------------------------
@@ -980,50 +1272,6 @@ struct CompactArgs {
     int64_t *gdir;                // per slot: start of each label group, then the row end
     unsigned int *n_slots;        // slot counter (zeroed before)
 };
-
-// Visit the entries of [beg, end) whose bit is set, 32 at a time and in
-// ascending order: f(e, valid) is called by all lanes, lane i with the i-th
-// set entry of the batch (valid) or none.  The bits are read 32 words
-// (1024 entries) per load, so long runs of inactive entries cost little.
-template <typename F>
-__device__ __forceinline__ void for_set_bits(const uint32_t *bits, int64_t beg, int64_t end, F &&f) {
-    const int lane = (int)lane_id();
-    const int64_t wb = beg >> 5, we = (end + 31) >> 5;
-    for (int64_t w0 = wb; w0 < we; w0 += 32) {
-        const int64_t wi = w0 + lane;
-        uint32_t word = 0u;
-        if (wi < we) {
-            word = bits[wi];
-            const int64_t e0 = wi << 5;
-            if (e0 < beg) word &= ~0u << (uint32_t)(beg - e0);
-            if (end - e0 < 32) word &= (1u << (uint32_t)(end - e0)) - 1u;
-        }
-        const uint32_t c = __popc(word);
-        uint32_t incl = c;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(FULL_MASK, incl, o);
-            if (lane >= o) incl += t;
-        }
-        const uint32_t total = __shfl_sync(FULL_MASK, incl, 31);
-        const uint32_t excl = incl - c;
-        for (uint32_t k0 = 0; k0 < total; k0 += 32) {
-            const uint32_t k = k0 + (uint32_t)lane;
-            int i = 0;                                // last word whose prefix is <= k
-#pragma unroll
-            for (int step = 16; step > 0; step >>= 1) {
-                const uint32_t ex = __shfl_sync(FULL_MASK, excl, i + step);
-                if (ex <= k) i += step;
-            }
-            const uint32_t wd = __shfl_sync(FULL_MASK, word, i);
-            const uint32_t ex_i = __shfl_sync(FULL_MASK, excl, i);
-            const bool valid = k < total;
-            int64_t e = -1;
-            if (valid) e = ((w0 + i) << 5) + (int64_t)select_bit(wd, k - ex_i);
-            f(e, valid);
-        }
-    }
-}
 
 __device__ __forceinline__ uint32_t lane_rank_count(int r, int n_rank) {
     uint32_t rc = 0;
@@ -1232,15 +1480,16 @@ k_compact_fill(CompactArgs a) {
 // costs one pass over omega.
 __global__ void __launch_bounds__(256)
 k_live_entries(int64_t n, const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
-               const uint32_t *__restrict__ om, const uint32_t *__restrict__ bits, uint32_t *out, int64_t *deg,
+               const uint32_t *__restrict__ om, const uint32_t *__restrict__ bits, uint32_t *out, uint32_t *deg,
                RoundStats *st) {
     const int64_t gwarp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int lane = (int)lane_id();
     unsigned long long total = 0;
-    for (int64_t b = gwarp * 32; b <= n; b += nwarps * 32) {
+    for (int64_t b = gwarp * 32; b < n; b += nwarps * 32) {
         const int64_t v = b + lane;
-        int64_t beg = 0, end = 0, mine = 0;
+        int64_t beg = 0, end = 0;
+        uint32_t mine = 0;
         const bool live = v < n && om[v] != 0u;
         if (live) { beg = rp[v]; end = rp[v + 1]; }
         for (uint32_t todo = __ballot_sync(FULL_MASK, live); todo; todo &= todo - 1u) {
@@ -1252,9 +1501,9 @@ k_live_entries(int64_t n, const int64_t *__restrict__ rp, const int32_t *__restr
                 if (keep) atomicOr(&out[e >> 5], 1u << (uint32_t)(e & 31));
                 c += (uint32_t)__popc(__ballot_sync(FULL_MASK, keep));
             });
-            if (lane == src) mine = (int64_t)c;
+            if (lane == src) mine = c;
         }
-        if (v <= n) deg[v] = mine;               // deg[n] = 0 closes the prefix sum
+        if (live) deg[v] = mine;
         total += (unsigned long long)mine;
     }
     for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(FULL_MASK, total, o);
@@ -2325,7 +2574,9 @@ k_label_sort(int64_t n, const int64_t *__restrict__ rp, const int32_t *__restric
     }
 }
 
-// Exclusive prefix sum of n int64 values, in three passes: each block scans
+// Row offsets of a compaction: exclusive prefix sum, over vertices 0..n (one
+// value past the last), of the entries each live vertex keeps (deg; vertices
+// whose omega is empty keep none), in three passes: each block scans
 // a tile of kScanTile values and writes its total, one block scans the tile
 // totals (in tiles of its own, carrying the running sum), and each tile adds
 // its offset.
@@ -2353,19 +2604,20 @@ __device__ __forceinline__ int64_t block_excl_scan(int64_t x, int64_t &total) {
 }
 
 __global__ void __launch_bounds__(256)
-k_scan_tiles(int64_t n, const int64_t *__restrict__ in, int64_t *out, int64_t *tile_sum) {
+k_scan_tiles(int64_t n, const uint32_t *__restrict__ deg, const uint32_t *__restrict__ om, int64_t *out,
+             int64_t *tile_sum) {
     const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * 8;
     int64_t v[8], s = 0;
 #pragma unroll
     for (int k = 0; k < 8; k++) {
-        v[k] = base + k < n ? in[base + k] : 0;
+        v[k] = base + k < n && om[base + k] ? (int64_t)deg[base + k] : 0;
         s += v[k];
     }
     int64_t total;
     int64_t run = block_excl_scan(s, total);
 #pragma unroll
     for (int k = 0; k < 8; k++) {
-        if (base + k < n) out[base + k] = run;
+        if (base + k <= n) out[base + k] = run;
         run += v[k];
     }
     if (threadIdx.x == 0) tile_sum[blockIdx.x] = total;
@@ -2398,7 +2650,7 @@ k_scan_add(int64_t n, int64_t *out, const int64_t *__restrict__ tile_off) {
     const int64_t off = tile_off[blockIdx.x];
     const int64_t base = (int64_t)blockIdx.x * kScanTile;
     for (int i = threadIdx.x; i < kScanTile; i += blockDim.x)
-        if (base + i < n) out[base + i] += off;
+        if (base + i <= n) out[base + i] += off;
 }
 
 // Roots of a search: every vertex whose omega meets `heads`.
@@ -2420,26 +2672,55 @@ k_collect_roots(int64_t n, const uint32_t *__restrict__ om, uint32_t heads, int3
 }
 
 // Alg. 6 lines 5-11: issuers whose token failed lose the head; a vertex whose
-// omega empties is eliminated with its edges.  Both omega buffers are kept
-// equal (they are equal at an LCC fixpoint).
+// omega empties is eliminated with its edges.  The changes are listed for the
+// LCC rounds that follow, and the totals of the state (entries kept, rows) lose
+// what the eliminated vertices held.  Both omega buffers are written: which
+// one the rounds continue from is the caller's matter.
 __global__ void __launch_bounds__(256)
 k_nlcc_apply(const int32_t *__restrict__ roots, int64_t n_roots, uint32_t heads,
-             const uint32_t *__restrict__ sat, uint32_t *om0, uint32_t *om1,
-             const int64_t *__restrict__ rp, uint32_t *ebits, RoundStats *st) {
+             const uint32_t *__restrict__ sat, const uint32_t *om, uint32_t *om0, uint32_t *om1, void *nw0, void *nw1,
+             int nw_bytes, const int64_t *__restrict__ rp, uint32_t *deg, Change *chg,
+             ChangePiece *chg_piece, int hub_deg, RoundStats *st) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    uint32_t changed = 0;
+    uint32_t changed = 0, died = 0;
+    unsigned long long old_kept = 0, died_rows = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_roots; i += stride) {
         const int32_t v = roots[i];
-        const uint32_t w = om0[v];
+        const uint32_t w = om[v];
         const uint32_t nw = w & ~(heads & ~sat[v]);
         if (nw != w) {
             om0[v] = nw;
             om1[v] = nw;
+            store_narrow(nw0, nw_bytes, v, nw);
+            store_narrow(nw1, nw_bytes, v, nw);
             changed = 1u;
-            if (nw == 0u) clear_row<1>(ebits, rp[v], rp[v + 1], 0);
+            const int64_t beg = rp[v], len = rp[v + 1] - beg;
+            if (nw == 0u) {
+                old_kept += deg[v];
+                deg[v] = 0u;
+                died_rows += (unsigned long long)len;
+                died++;
+            }
+            chg[atomicAdd(&st->n_chg, 1u)] = Change{v, nw};
+            if (len > hub_deg) {
+                const unsigned int np = (unsigned int)((len + hub_deg - 1) / hub_deg);
+                const unsigned int b = atomicAdd(&st->n_chg_piece, np);
+                for (unsigned int c = 0; c < np; c++) chg_piece[b + c] = ChangePiece{v, (int32_t)c};
+            }
         }
     }
-    if (__any_sync(FULL_MASK, changed) && lane_id() == 0) atomicOr(&st->changed, 1u);
+    changed = __any_sync(FULL_MASK, changed);
+    died = __reduce_add_sync(FULL_MASK, died);
+    old_kept = warp_total(old_kept);
+    died_rows = warp_total(died_rows);
+    if (lane_id() == 0 && changed) {
+        atomicOr(&st->changed, 1u);
+        if (died) {
+            atomicAdd(&st->died, died);
+            atomicAdd(&st->old_kept, old_kept);
+            atomicAdd(&st->died_rows, died_rows);
+        }
+    }
 }
 
 __device__ __forceinline__ bool ebit(const uint32_t *eb, int64_t e) {
@@ -2469,23 +2750,6 @@ k_materialize(int64_t n, const uint32_t *__restrict__ om, const int64_t *__restr
     }
 }
 
-// Both narrow copies of omega from the current omega (an LCC phase starts
-// with the two omega buffers equal).
-__global__ void __launch_bounds__(256)
-k_narrow(int64_t n, const uint32_t *__restrict__ om, void *nw0, void *nw1, int bytes) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-        const uint32_t w = om[v];
-        if (bytes == 1) {
-            ((uint8_t *)nw0)[v] = (uint8_t)w;
-            ((uint8_t *)nw1)[v] = (uint8_t)w;
-        } else {
-            ((uint16_t *)nw0)[v] = (uint16_t)w;
-            ((uint16_t *)nw1)[v] = (uint16_t)w;
-        }
-    }
-}
-
 __global__ void k_set_word(uint32_t *p, uint32_t v) { *p = v; }
 __global__ void k_and_word(uint32_t *p, uint32_t v) { *p &= v; }
 
@@ -2509,6 +2773,24 @@ k_omega_hist(int64_t n, const uint32_t *__restrict__ om, int n0, unsigned long l
         if (lane_id() == 0 && c) atomicAdd(&hist[q], (unsigned long long)c);
     }
     if (lane_id() == 0 && total) atomicAdd(&hist[kMaxT], total);
+}
+
+// Per label: vertices (out[0..255]) and the entries in their rows (out[256..511]).
+__global__ void __launch_bounds__(256)
+k_label_hist(int64_t n, const int64_t *__restrict__ rp, const uint8_t *__restrict__ lab, unsigned long long *out) {
+    __shared__ unsigned int cnt[256];
+    __shared__ unsigned long long rows[256];
+    cnt[threadIdx.x] = 0u;
+    rows[threadIdx.x] = 0ull;
+    __syncthreads();
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
+        atomicAdd(&cnt[lab[v]], 1u);
+        atomicAdd(&rows[lab[v]], (unsigned long long)(rp[v + 1] - rp[v]));
+    }
+    __syncthreads();
+    if (cnt[threadIdx.x]) atomicAdd(&out[threadIdx.x], (unsigned long long)cnt[threadIdx.x]);
+    if (rows[threadIdx.x]) atomicAdd(&out[256 + threadIdx.x], rows[threadIdx.x]);
 }
 
 // Population counts for the result summary.
@@ -2537,8 +2819,10 @@ k_count(int64_t n, const uint32_t *__restrict__ om, int64_t words, const uint32_
 
 using namespace ccpm;
 
-// LCC rounds queued per host round trip.
-constexpr int kLccGroup = 4;
+// LCC rounds queued per host round trip: the first group of a prune, and the
+// later ones.  A round queued past the fixpoint costs two launches that return
+// at once (3 us), a host round trip 20 us or more.
+constexpr int kLccFirstGroup = 6, kLccGroup = 4;
 
 struct Workspace {
     int64_t n = 0, m = 0, words = 0;
@@ -2561,7 +2845,12 @@ struct Workspace {
     int64_t spill_cap = 0;
     DevPlan *plans = nullptr;
     RoundStats *st = nullptr;        // device
-    RoundStats *st_ring = nullptr;   // counters of a group of queued LCC rounds
+    RoundStats *st_ring = nullptr;   // counters of two groups of queued LCC rounds
+    uint32_t *dirty = nullptr;       // delta rounds: one bit per listed vertex, all zero between rounds
+    int32_t *dsmall = nullptr, *dmed = nullptr;   // their lists
+    ChunkItem *dchunk = nullptr;
+    Change *chg = nullptr;           // changes of omega not passed on yet
+    ChangePiece *chg_piece = nullptr;
     RoundStats *st_ring_h = nullptr; // pinned host mirror
     unsigned long long *next_root = nullptr;   // dynamic root counter of the searches
     RoundStats *st_h = nullptr;      // pinned host mirror
@@ -2571,13 +2860,13 @@ struct Workspace {
     unsigned long long *hist_h = nullptr;
     DevPlan *plans_h = nullptr;      // pinned staging for plan uploads
     unsigned long long *aux_h = nullptr;     // pinned: counters snapshotted in stream order
-    cudaEvent_t ev[12] = {};
+    cudaEvent_t ev[13] = {};
     // compacted rows (K4), two generations; allocated at the first compaction
     int64_t *sub_rp[2] = {nullptr, nullptr};
     int32_t *sub_col[2] = {nullptr, nullptr};
     uint32_t *sub_bits[2] = {nullptr, nullptr};
     int64_t sub_cap[2] = {0, 0};     // entries sub_col / sub_bits can hold
-    int64_t *deg = nullptr;          // n + 1 kept-entry counts, scanned into sub_rp
+    uint32_t *deg = nullptr;         // entries each live vertex kept in its last evaluation
     uint8_t *sub_nlab[2] = {nullptr, nullptr};
     int32_t *sub_dslot[2] = {nullptr, nullptr};   // live vertex -> label-group directory slot
     int64_t *sub_gdir[2] = {nullptr, nullptr};
@@ -2621,6 +2910,7 @@ struct ccpm_graph {
     uint8_t *lab = nullptr;
     bool borrowed = false;
     int64_t label_freq[256] = {};
+    int64_t label_rows[256] = {};   // entries in the rows of each label's vertices
     int32_t *lcol = nullptr;      // rows grouped by neighbour label (built on first search)
     uint8_t *nlab = nullptr;
     std::mutex lrow_mu;           // concurrent batch workers build the grouped rows once
@@ -2720,6 +3010,7 @@ void ws_free(Workspace &w) {
     cudaFree(w.sat); cudaFree(w.items); cudaFree(w.items2); cudaFree(w.spill_items); cudaFree(w.plans); cudaFree(w.st); cudaFree(w.cnt); cudaFree(w.next_root);
     if (w.st_h) cudaFreeHost(w.st_h);
     cudaFree(w.st_ring);
+    cudaFree(w.dirty); cudaFree(w.dsmall); cudaFree(w.dmed); cudaFree(w.dchunk); cudaFree(w.chg); cudaFree(w.chg_piece);
     if (w.st_ring_h) cudaFreeHost(w.st_ring_h);
     if (w.cnt_h) cudaFreeHost(w.cnt_h);
     cudaFree(w.hist);
@@ -2766,8 +3057,15 @@ int ws_ensure(ccpm_ctx *ctx, ccpm_graph *g, int hub_deg) {
     if ((rc = dalloc(ctx, &w.spill_items, (size_t)w.spill_cap))) return rc;
     if ((rc = dalloc(ctx, &w.plans, (size_t)kMaxPlans))) return rc;
     if ((rc = dalloc(ctx, &w.st, 1))) return rc;
-    if ((rc = dalloc(ctx, &w.st_ring, (size_t)kLccGroup))) return rc;
-    CU(ctx, cudaMallocHost((void **)&w.st_ring_h, sizeof(RoundStats) * kLccGroup));
+    if ((rc = dalloc(ctx, &w.st_ring, (size_t)(2 * kLccFirstGroup)))) return rc;
+    CU(ctx, cudaMallocHost((void **)&w.st_ring_h, sizeof(RoundStats) * kLccFirstGroup));
+    if ((rc = dalloc(ctx, &w.dirty, (size_t)g->n / 32 + 1))) return rc;
+    if ((rc = dalloc(ctx, &w.dsmall, (size_t)g->n))) return rc;
+    if ((rc = dalloc(ctx, &w.dmed, (size_t)g->n))) return rc;
+    if ((rc = dalloc(ctx, &w.dchunk, (size_t)w.chunk_cap))) return rc;
+    if ((rc = dalloc(ctx, &w.chg, (size_t)g->n))) return rc;
+    if ((rc = dalloc(ctx, &w.chg_piece, (size_t)w.chunk_cap))) return rc;
+    if ((rc = dalloc(ctx, &w.deg, (size_t)g->n))) return rc;
     if ((rc = dalloc(ctx, &w.cnt, 2))) return rc;
     if ((rc = dalloc(ctx, &w.next_root, 1))) return rc;
     CU(ctx, cudaMallocHost((void **)&w.st_h, sizeof(RoundStats)));
@@ -3006,7 +3304,10 @@ struct Pipeline {
     const int64_t *lgdir = nullptr;
     int lnrank = 0;
     uint8_t llab_rank[256] = {};
-    int64_t last_kept = -1, last_rows = -1;   // the latest round: entries still active, rows of the survivors
+    // the state after the latest round: entries still active, entries in the
+    // rows of the active vertices, active vertices
+    int64_t last_kept = -1, last_rows = -1, last_alive = 0;
+    bool synced = true;             // the lists hold every live vertex, both omega buffers are equal
 
     // alive counts per template vertex (w.hist_h[0..31]) and total bits ([32])
     int omega_hist() {
@@ -3028,24 +3329,22 @@ struct Pipeline {
         return CCPM_OK;
     }
 
-    // One LCC round.  slot: its counters; prev (nullable): the previous
-    // round's counters, from which the round reads its list sizes on the
-    // device (a round queued without a host round trip).  step: its place in
-    // the group of queued rounds; round `step` of a group reads the omega and
-    // list buffers the previous one wrote (the host flips cur / li only once
-    // the group is done, by the number of rounds that ran).
-    int launch_round(RoundStats *slot, const RoundStats *prev, int step = 0) {
+    // One LCC round.  slot: its counters; prev (nullable): the counters of the
+    // round before, from which the round reads its list sizes and whether there
+    // is anything to do on the device (without: the host's sizes).  c, l: the
+    // omega and list buffers it reads (the host flips cur / li only once a
+    // group of queued rounds is done, by the number of rounds that ran).
+    int launch_round(RoundStats *slot, const RoundStats *prev, int c, int l, bool delta) {
         Workspace &w = ctx->ws;
-        const int c = cur ^ (step & 1), l = li ^ (step & 1);
         LccArgs a;
         a.rp = lrp;
         a.col = lcol;
         a.om_cur = w.om[c];
         a.om_next = w.om[c ^ 1];
         a.ebits = lbits;
-        a.small_in = w.small[l];
-        a.med_in = w.med[l];
-        a.chunk_in = w.chunk[l];
+        a.small_in = delta ? w.dsmall : w.small[l];
+        a.med_in = delta ? w.dmed : w.med[l];
+        a.chunk_in = delta ? w.dchunk : w.chunk[l];
         a.n_small = n_small;
         a.n_med = n_med;
         a.n_chunk = n_chunk;
@@ -3057,7 +3356,10 @@ struct Pipeline {
         a.prev = prev;
         a.resident_warps = grid_sms(ctx) * 32;
         a.hub_deg = w.hub_deg;
-        a.deg = compact_mode >= 0 ? w.deg : nullptr;
+        a.deg = w.deg;
+        a.dirty = w.dirty;
+        a.chg = w.chg;
+        a.chg_piece = w.chg_piece;
         a.lab0 = from_labels ? g->lab : nullptr;
         a.elab = from_labels ? elab : nullptr;
         a.sparse = (!dense && gen < 0) ? 1 : 0;
@@ -3077,88 +3379,181 @@ struct Pipeline {
         launches++;
         lcc_launches++;
         // one resident wave: grid-stride work is split evenly over warps that all run at once
-#define CCPM_LAUNCH_LCC(C, D) k_lcc_round<C, D><<<lcc_grid(ctx, k_lcc_round<C, D>, warps), 256, 0, ctx->stream>>>(a, dt)
-        if (dense) {
-            if (maxc == 0) CCPM_LAUNCH_LCC(0, true);
-            else if (maxc <= 4) CCPM_LAUNCH_LCC(4, true);
-            else CCPM_LAUNCH_LCC(32, true);
-        } else {
-            if (maxc == 0) CCPM_LAUNCH_LCC(0, false);
-            else if (maxc <= 4) CCPM_LAUNCH_LCC(4, false);
-            else CCPM_LAUNCH_LCC(32, false);
-        }
+#define CCPM_LAUNCH_LCC(C, M) k_lcc_round<C, M><<<lcc_grid(ctx, k_lcc_round<C, M>, warps), 256, 0, ctx->stream>>>(a, dt)
+#define CCPM_LAUNCH_MODE(M)                        \
+    do {                                           \
+        if (maxc == 0) CCPM_LAUNCH_LCC(0, M);      \
+        else if (maxc <= 4) CCPM_LAUNCH_LCC(4, M); \
+        else CCPM_LAUNCH_LCC(32, M);               \
+    } while (0)
+        if (delta) CCPM_LAUNCH_MODE(kDelta);
+        else if (dense) CCPM_LAUNCH_MODE(kDense);
+        else CCPM_LAUNCH_MODE(kFull);
+#undef CCPM_LAUNCH_MODE
 #undef CCPM_LAUNCH_LCC
         dense = false;      // only the first round after init sees every bit set
         CU(ctx, cudaGetLastError());
         return CCPM_OK;
     }
 
-    // LCC to fixpoint; returns rounds via *rounds.  Rounds are queued in
-    // groups of up to kLccGroup with one host round trip per group: each
-    // queued round reads its list sizes from the previous round's counters,
-    // and rounds queued after the fixpoint return at once.  The first round
-    // after init runs alone (its time is reported on its own, and a
-    // compaction may follow it).  Compaction is considered between groups.
-    int lcc(int64_t *rounds, bool first_alone = false) {
+    // Pass the changes of a round (prev) on: the lists of the delta round whose
+    // counters are `slot`.  lists: the round was a full one that read the omega
+    // buffer c ^ 1 and left its vertices in the lists l.
+    int launch_push(RoundStats *slot, const RoundStats *prev, int c, int l, bool lists) {
+        Workspace &w = ctx->ws;
+        PushArgs a;
+        a.rp = lrp;
+        a.col = lcol;
+        a.bits = lbits;
+        a.om = w.om[c];
+        a.nw = w.nw[c];
+        a.nw_bytes = nw_bytes;
+        a.om_old = w.om[c ^ 1];
+        a.small_in = w.small[l];
+        a.med_in = w.med[l];
+        a.chunk_in = w.chunk[l];
+        a.chg = w.chg;
+        a.chg_piece = w.chg_piece;
+        a.prev = prev;
+        a.dirty = w.dirty;
+        a.small_out = w.dsmall;
+        a.med_out = w.dmed;
+        a.chunk_out = w.dchunk;
+        a.st = slot;
+        a.hub_deg = w.hub_deg;
+        a.short_max = short_max;
+        launches++;
+        const int grid = grid_for(ctx, (int64_t)1 << 40, 256, 8);
+        if (lists) k_push<true><<<grid, 256, 0, ctx->stream>>>(a);
+        else k_push<false><<<grid, 256, 0, ctx->stream>>>(a);
+        CU(ctx, cudaGetLastError());
+        return CCPM_OK;
+    }
+
+    // LCC to fixpoint; returns rounds via *rounds.  Rounds are queued in groups
+    // with one host round trip per group: each reads what it needs from the
+    // counters of the round before (w.st: of the initialisation, or of the
+    // non-local check whose changes are in the Change list), and rounds queued
+    // after the fixpoint return at once.  A prune's first rounds (two, or one
+    // from a saved state) evaluate every active vertex, as nearly all of them
+    // change; where the rows are large (use_deltas) the later ones are delta
+    // rounds.  With options.compact > 0 every round is a full one and the rows
+    // may be compacted between groups.
+    int lcc(int64_t *rounds, bool initial) {
         Workspace &w = ctx->ws;
         int64_t r = 0;
-        if (nw_bytes) {
-            launches++;
-            k_narrow<<<grid_for(ctx, g->n, 256, 8), 256, 0, ctx->stream>>>(g->n, w.om[cur], w.nw[0], w.nw[1], nw_bytes);
-            CU(ctx, cudaGetLastError());
+        const bool deltas = use_deltas(initial ? first_rows : last_rows);
+        int full_left = initial ? (dense ? 2 : 1) : 0;
+        const RoundStats *src = (initial || deltas) ? w.st : nullptr;
+        if (!initial && !deltas && !synced) {
+            // earlier delta rounds left the lists and the other omega buffer
+            // behind: rebuild them (k_init marks its counters as changed)
+            int rc = rebucket(lrp, false, 1u);
+            if (rc) return rc;
+            src = w.st;
         }
-        bool alone = first_alone;
-        for (;;) {
-            const int G = alone ? 1 : kLccGroup;
-            alone = false;
-            CU(ctx, cudaMemsetAsync(w.st_ring, 0, sizeof(RoundStats) * (size_t)G, ctx->stream));
+        bool seed = false;                // the next delta round follows a full one
+        for (int group = 0;; group++) {
+            const bool first = initial && group == 0;
+            const int G = first ? (compact_mode > 0 ? 1 : kLccFirstGroup) : kLccGroup;
+            RoundStats *ring = w.st_ring + (group & 1) * kLccFirstGroup;
+            CU(ctx, cudaMemsetAsync(ring, 0, sizeof(RoundStats) * (size_t)G, ctx->stream));
             CU(ctx, cudaEventRecord(w.ev[4], ctx->stream));
+            int n_full = 0, c = cur, l = li, rc;
             for (int i = 0; i < G; i++) {
-                int rc = launch_round(w.st_ring + i, i ? w.st_ring + i - 1 : nullptr, i);
-                if (rc) return rc;
+                const RoundStats *prev = i ? ring + i - 1 : src;
+                if (!deltas || full_left > 0) {
+                    if (full_left > 0) full_left--;
+                    if ((rc = launch_round(ring + i, prev, c, l, false))) return rc;
+                    n_full++;
+                    c ^= 1;
+                    l ^= 1;
+                    seed = true;
+                    synced = true;
+                } else {
+                    if ((rc = launch_push(ring + i, prev, c, l, seed))) return rc;
+                    if ((rc = launch_round(ring + i, prev, c, l, true))) return rc;
+                    seed = false;
+                    synced = false;
+                }
+                if (first && i == 0) CU(ctx, cudaEventRecord(w.ev[12], ctx->stream));
             }
             CU(ctx, cudaEventRecord(w.ev[5], ctx->stream));
-            CU(ctx, cudaMemcpyAsync(w.st_ring_h, w.st_ring, sizeof(RoundStats) * (size_t)G, cudaMemcpyDeviceToHost,
+            CU(ctx, cudaMemcpyAsync(w.st_ring_h, ring, sizeof(RoundStats) * (size_t)G, cudaMemcpyDeviceToHost,
                                     ctx->stream));
+            if (first)
+                CU(ctx, cudaMemcpyAsync(w.st_h, w.st, sizeof(RoundStats), cudaMemcpyDeviceToHost, ctx->stream));
             CU(ctx, ctx_sync(ctx));
+            if (first && (w.st_h->n_hub_slots > (unsigned)w.acc_cap || (int64_t)w.st_h->n_chunk > w.chunk_cap))
+                return set_err(ctx, CCPM_EOVERFLOW, "hub bookkeeping overflow");
             float ms = 0.f;
             CU(ctx, cudaEventElapsedTime(&ms, w.ev[4], w.ev[5]));
             ms_lcc_kernel += ms;
+            if (first) {
+                CU(ctx, cudaEventElapsedTime(&ms, w.ev[4], w.ev[12]));
+                ms_first = ms;
+            }
             bool done = false;
             int ran = 0;
-            for (int i = 0; i < G; i++) {
+            for (int i = 0; i < G && !done; i++) {
                 const RoundStats &h = w.st_ring_h[i];
                 if (h.skipped) break;
                 ran++;
                 r++;
-                scanned += (int64_t)h.scanned;
-                rows += (int64_t)h.row_entries;
-                alive += (int64_t)h.alive;
-                alg_bytes += (33 * (int64_t)h.scanned) / 4 + 16 * (int64_t)h.alive;
-                kernel_bytes += 24 * (int64_t)h.alive + (33 * (int64_t)h.row_entries) / 8 + 4 * (int64_t)h.scanned;
-                if (lcc_rounds_run == 0) {
-                    first_entries = (int64_t)h.scanned;
-                    ms_first = ms;
+                int64_t sc, n_rows, n_alive;
+                if (i < n_full) {
+                    sc = (int64_t)h.scanned;
+                    n_rows = (int64_t)h.row_entries;
+                    n_alive = (int64_t)h.alive;
+                    last_kept = (int64_t)h.kept;
+                    last_rows = (int64_t)h.rows_next;
+                    last_alive = n_alive - (int64_t)h.died;
+                    n_small = h.n_small;
+                    n_med = h.n_med;
+                    n_chunk = h.n_chunk;
+                    li ^= 1;
+                    cur ^= 1;
+                } else {
+                    // the vertices not evaluated scan what they kept
+                    sc = last_kept - (int64_t)h.old_kept + (int64_t)h.scanned;
+                    n_rows = last_rows;
+                    n_alive = last_alive;
+                    last_kept += (int64_t)h.kept - (int64_t)h.old_kept;
+                    last_rows -= (int64_t)h.died_rows;
+                    last_alive -= (int64_t)h.died;
                 }
+                scanned += sc;
+                rows += n_rows;
+                alive += n_alive;
+                alg_bytes += (33 * sc) / 4 + 16 * n_alive;
+                // what the round itself reads: the vertices it evaluates
+                kernel_bytes += 24 * (int64_t)h.alive + (33 * (int64_t)h.row_entries) / 8 + 4 * (int64_t)h.scanned;
+                if (lcc_rounds_run == 0) first_entries = sc;
                 lcc_rounds_run++;
-                n_small = h.n_small;
-                n_med = h.n_med;
-                n_chunk = h.n_chunk;
-                last_kept = (int64_t)h.kept;
-                last_rows = (int64_t)h.rows_next;
-                li ^= 1;
-                cur ^= 1;
-                if (!h.changed) { done = true; break; }
+                done = !h.changed;
             }
             // launches that returned at once are not rounds
             lcc_launches -= G - ran;
             if (done) break;
             if (r > (int64_t)4 * (g->m + g->n) + 8)
                 return set_err(ctx, CCPM_ETIMEOUT, "LCC did not converge");
-            if (want_compact() && (rc_compact = compact())) return rc_compact;
+            src = ring + G - 1;
+            if (compact_mode > 0 && want_compact()) {
+                if ((rc_compact = compact())) return rc_compact;
+                src = nullptr;            // rebuilt lists: their sizes are the host's
+            }
         }
         *rounds = r;
         return CCPM_OK;
+    }
+
+    // The totals after a non-local check (its counters in w.st_h): the vertices
+    // it eliminated, and the entries they held, are gone.
+    void after_check() {
+        const RoundStats &h = *ctx->ws.st_h;
+        last_kept -= (int64_t)h.old_kept;
+        last_rows -= (int64_t)h.died_rows;
+        last_alive -= (int64_t)h.died;
     }
 
     // Label-group directory of the compacted rows for the searches (none on
@@ -3192,17 +3587,25 @@ struct Pipeline {
                last_kept < last_rows;
     }
 
+    // Delta rounds pay for their second kernel (5 us) once a full round has more
+    // than a few million entries to look over: exploring a clique on 8192
+    // vertices took 154 ms with full rounds and 177 with delta rounds, the LCC
+    // phase of 32M vertices with 350M entries in the live rows 22.7 and 11.7.
+    bool use_deltas(int64_t rows_now) const { return compact_mode <= 0 && rows_now >= ((int64_t)1 << 22); }
+
     // Frontier of the live vertices over rows rp (the pieces of a long row
     // consecutive and in order); also makes both omega buffers equal.
-    int rebucket(const int64_t *rp, bool sync = true) {
+    int rebucket(const int64_t *rp, bool sync = true, unsigned int set_changed = 0u) {
+        synced = true;
         Workspace &w = ctx->ws;
         LabelMask all;
         std::memset(&all, 0xFF, sizeof(all));
         CU(ctx, cudaMemsetAsync(w.st, 0, sizeof(RoundStats), ctx->stream));
         launches++;
         k_init<<<grid_for(ctx, g->n, 256, 8), 256, 0, ctx->stream>>>(g->n, rp, g->lab, all, w.om[cur], w.om[cur],
-                                                                     w.om[cur ^ 1], w.small[li], w.med[li],
-                                                                     w.chunk[li], w.acc, w.st, w.hub_deg, short_max);
+                                                                     w.om[cur ^ 1], w.nw[cur], w.nw[cur ^ 1], nw_bytes,
+                                                                     w.small[li], w.med[li], w.chunk[li], w.acc, w.st,
+                                                                     w.hub_deg, short_max, set_changed);
         CU(ctx, cudaGetLastError());
         if (!sync) return CCPM_OK;
         int rc = read_stats();
@@ -3295,7 +3698,7 @@ struct Pipeline {
         // round (0 for every vertex that is not live): exclusive prefix sum of
         // the kept counts (tile scans, a scan of the tile totals, the tile
         // offsets added)
-        const int64_t cnt = g->n + 1, tiles = (cnt + kScanTile - 1) / kScanTile;
+        const int64_t tiles = g->n / kScanTile + 1;
         const size_t tmp = sizeof(int64_t) * (size_t)tiles;
         if (tmp > w.scan_tmp_bytes) {
             cudaFree(w.scan_tmp);
@@ -3306,9 +3709,9 @@ struct Pipeline {
         }
         int64_t *tile_sum = (int64_t *)w.scan_tmp;
         launches += 3;
-        k_scan_tiles<<<(unsigned)tiles, 256, 0, s>>>(cnt, w.deg, w.sub_rp[nb], tile_sum);
+        k_scan_tiles<<<(unsigned)tiles, 256, 0, s>>>(g->n, w.deg, w.om[cur], w.sub_rp[nb], tile_sum);
         k_scan_sums<<<1, 256, 0, s>>>(tiles, tile_sum);
-        k_scan_add<<<(unsigned)tiles, 256, 0, s>>>(cnt, w.sub_rp[nb], tile_sum);
+        k_scan_add<<<(unsigned)tiles, 256, 0, s>>>(g->n, w.sub_rp[nb], tile_sum);
         CU(ctx, cudaGetLastError());
         if (n_chunk > 0) {
             launches++;
@@ -3456,10 +3859,24 @@ int ccpm_graph_load_csr(ccpm_ctx_t ctx, int64_t n, int64_t m, const int64_t *row
         g->rp = const_cast<int64_t *>(row_ptr);
         g->col = const_cast<int32_t *>(col);
         g->lab = const_cast<uint8_t *>(labels);
-        std::vector<uint8_t> h((size_t)n);
-        cudaError_t e = cudaMemcpy(h.data(), labels, (size_t)n, cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) { delete g; return set_err(ctx, CCPM_ECUDA, "graph: label readback"); }
-        for (int64_t v = 0; v < n; v++) g->label_freq[h[v]]++;
+        // label counts on the device; the arrays may still be in the making on
+        // the default stream, which the copy of the labels used to wait for
+        unsigned long long *d = nullptr, h[512];
+        cudaError_t e = cudaDeviceSynchronize();
+        if (e == cudaSuccess) e = cudaMalloc((void **)&d, sizeof(h));
+        if (e == cudaSuccess) e = cudaMemsetAsync(d, 0, sizeof(h), ctx->stream);
+        if (e == cudaSuccess) {
+            k_label_hist<<<grid_for(ctx, n, 256, 8), 256, 0, ctx->stream>>>(n, row_ptr, labels, d);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaMemcpyAsync(h, d, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+        cudaFree(d);
+        if (e != cudaSuccess) { delete g; return set_err(ctx, CCPM_ECUDA, "graph: label counts"); }
+        for (int L = 0; L < 256; L++) {
+            g->label_freq[L] = (int64_t)h[L];
+            g->label_rows[L] = (int64_t)h[256 + L];
+        }
     } else {
         int rc;
         if ((rc = dalloc(ctx, &g->rp, (size_t)n + 1)) || (rc = dalloc(ctx, &g->col, (size_t)m)) ||
@@ -3476,7 +3893,10 @@ int ccpm_graph_load_csr(ccpm_ctx_t ctx, int64_t n, int64_t m, const int64_t *row
         // the offsets' check and the label histogram run while the copies do
         bool monotone = true;
         for (int64_t v = 0; v < n && monotone; v++) monotone = row_ptr[v + 1] >= row_ptr[v];
-        for (int64_t v = 0; v < n; v++) g->label_freq[labels[v]]++;
+        for (int64_t v = 0; v < n; v++) {
+            g->label_freq[labels[v]]++;
+            g->label_rows[labels[v]] += row_ptr[v + 1] - row_ptr[v];
+        }
         const cudaError_t e2 = cudaStreamSynchronize(ctx->stream);
         if (e == cudaSuccess) e = e2;
         if (e != cudaSuccess || !monotone) {
@@ -3681,12 +4101,7 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
         if (rc_) return fail(rc_);    \
     } while (0)
 
-    if (P.compact_mode >= 0) {
-        // kept-entry counts the rounds leave for a compaction: 0 for every vertex
-        // no round has listed
-        if (!w.deg) RCF(dalloc(ctx, &w.deg, (size_t)g->n + 1));
-        CUF(cudaMemsetAsync(w.deg, 0, sizeof(int64_t) * (size_t)(g->n + 1), s));
-    }
+    CUF(cudaMemsetAsync(w.dirty, 0, sizeof(uint32_t) * (size_t)(g->n / 32 + 1), s));
     CUF(cudaEventRecord(w.ev[0], s));
     // ---- init (Alg. 3)
     LabelMask lm;
@@ -3713,9 +4128,9 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
     {
         int grid = grid_for(ctx, g->n, 256, 8);
         P.launches++;
-        k_init<<<grid, 256, 0, s>>>(g->n, g->rp, g->lab, lm, resume ? r->om : nullptr, w.om[0], w.om[1],
-                                    w.small[0], w.med[0],
-                                    w.chunk[0], w.acc, w.st, hub_deg, P.short_max);
+        k_init<<<grid, 256, 0, s>>>(g->n, g->rp, g->lab, lm, resume ? r->om : nullptr, w.om[0], w.om[1], w.nw[0],
+                                    w.nw[1], P.nw_bytes, w.small[0], w.med[0], w.chunk[0], w.acc, w.st, hub_deg,
+                                    P.short_max, 1u);
         CUF(cudaGetLastError());
     }
     if (resume) {
@@ -3725,15 +4140,10 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
         CUF(cudaGetLastError());
         P.dense = false;
     }
-    RCF(P.read_stats());
     P.cur = 0;
     P.li = 0;
-    P.n_small = w.st_h->n_small;
-    P.n_med = w.st_h->n_med;
-    P.n_chunk = w.st_h->n_chunk;
-    P.first_rows = (int64_t)w.st_h->row_entries;
-    if (w.st_h->n_hub_slots > (unsigned)w.acc_cap || P.n_chunk > w.chunk_cap)
-        return fail(set_err(ctx, CCPM_EOVERFLOW, "hub bookkeeping overflow"));
+    for (int L = 0; L < 256; L++)
+        if (lm.m[L]) P.first_rows += g->label_rows[L];
     // the first round reads the entry labels when its rows cover a large
     // share of the graph (building them is one pass over the entries)
     if (P.dense && (opt.entry_labels > 0 ||
@@ -3874,10 +4284,12 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
             CUF(cudaGetLastError());
             CUF(cudaEventRecord(w.ev[11], s));
             P.launches++;
-            k_nlcc_apply<<<grid_for(ctx, n_roots, 256, 8), 256, 0, s>>>(w.roots, n_roots, c.hmask, w.sat,
-                                                                        w.om[0], w.om[1], P.lrp, P.lbits, w.st);
+            k_nlcc_apply<<<grid_for(ctx, n_roots, 256, 8), 256, 0, s>>>(
+                w.roots, n_roots, c.hmask, w.sat, w.om[P.cur], w.om[0], w.om[1], w.nw[0], w.nw[1], P.nw_bytes, P.lrp,
+                w.deg, w.chg, w.chg_piece, hub_deg, w.st);
             CUF(cudaGetLastError());
             RCF(P.read_stats());
+            P.after_check();
             if (w.st_h->overflow) over = true;
             P.windows += (int64_t)w.st_h->windows;
             P.nlcc_entries += (int64_t)(w.st_h->windows - w.aux_h[0]);
@@ -3891,8 +4303,7 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
         CUF(cudaEventRecord(w.ev[7], s));
         int64_t rr = 0;
         if (changed) {
-            // the previous fixpoint's frontier holds every live vertex
-            RCF(P.lcc(&rr));
+            RCF(P.lcc(&rr, false));
         }
         CUF(cudaEventRecord(w.ev[8], s));
         r->phase_rounds.push_back((int32_t)rr);
@@ -4641,7 +5052,6 @@ int ccpm_result_matches(ccpm_ctx_t ctx, ccpm_result_t r, ccpm_tmpl_t tm, const c
     if (rc) return rc;
     Workspace &w = ctx->ws;
     cudaStream_t s = ctx->stream;
-    if (!w.deg && (rc = dalloc(ctx, &w.deg, (size_t)g->n + 1))) return rc;
     // host outputs are filled through device buffers of this call
     int32_t *d_list = list;
     unsigned long long *d_vc = (unsigned long long *)vertex_counts, *d_ec = (unsigned long long *)entry_counts;
@@ -4695,10 +5105,11 @@ int ccpm_result_matches(ccpm_ctx_t ctx, ccpm_result_t r, ccpm_tmpl_t tm, const c
     for (int q = 0; q < t.n0; q++) lm.m[t.labels[q]] |= 1u << q;
     CUR(cudaMemsetAsync(w.st, 0, sizeof(RoundStats), s));
     CUR(cudaMemsetAsync(w.ebits, 0, sizeof(uint32_t) * (size_t)(w.words + 1), s));
-    k_init<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, g->rp, g->lab, lm, r->om, w.om[0], w.om[1], w.small[0],
-                                                       w.med[0], w.chunk[0], w.acc, w.st, hub_deg, P.short_max);
+    k_init<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, g->rp, g->lab, lm, r->om, w.om[0], w.om[1], nullptr, nullptr,
+                                                       0, w.small[0], w.med[0], w.chunk[0], w.acc, w.st, hub_deg,
+                                                       P.short_max, 0u);
     CUR(cudaGetLastError());
-    k_live_entries<<<grid_for(ctx, g->n + 1, 256, 8), 256, 0, s>>>(g->n, g->rp, g->col, w.om[0], r->eb, w.ebits, w.deg,
+    k_live_entries<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, g->rp, g->col, w.om[0], r->eb, w.ebits, w.deg,
                                                                    w.st);
     CUR(cudaGetLastError());
     k_collect_roots<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, w.om[0], 1u << root, w.roots, w.st);
@@ -5095,8 +5506,8 @@ int lcc_fixpoint_noalloc_body(int device, void *cuda_stream, int64_t n, int64_t 
         NA_CU(cudaMemsetAsync(ebits, 0xFF, sizeof(uint32_t) * (size_t)words, s));
         if (m_dir & 31) k_set_word<<<1, 1, 0, s>>>(ebits + words - 1, (1u << (uint32_t)(m_dir & 31)) - 1u);
     }
-    k_init<<<grid(n, 256), 256, 0, s>>>(n, row_ptr, labels, lm, nullptr, om[0], om[1], small[0], med[0], chunk[0], acc,
-                                        st, hub, kSmallDeg);
+    k_init<<<grid(n, 256), 256, 0, s>>>(n, row_ptr, labels, lm, nullptr, om[0], om[1], nullptr, nullptr, 0, small[0],
+                                        med[0], chunk[0], acc, st, hub, kSmallDeg, 0u);
     NA_CU(cudaGetLastError());
     NA_CU(read_stats());
     if (hs.n_hub_slots > (unsigned)L.acc_cap || (int64_t)hs.n_chunk > L.chunk_cap)
@@ -5125,6 +5536,9 @@ int lcc_fixpoint_noalloc_body(int device, void *cuda_stream, int64_t n, int64_t 
         a.st = st;
         a.hub_deg = hub;
         a.deg = nullptr;
+        a.dirty = nullptr;
+        a.chg = nullptr;
+        a.chg_piece = nullptr;
         a.med_chunk = 1;
         a.lab0 = nullptr;
         a.elab = nullptr;
@@ -5137,9 +5551,9 @@ int lcc_fixpoint_noalloc_body(int device, void *cuda_stream, int64_t n, int64_t 
         a.nw_next = nullptr;
         // at most one resident wave (four blocks an SM): the rows are dealt out evenly over the warps
         const int g = std::min(grid((n_chunk + n_med + n_small) * 32, 256), 4 * num_sms);
-        if (dt.n_cls == 0) k_lcc_round<0, false><<<g, 256, 0, s>>>(a, dt);
-        else if (dt.n_cls <= 4) k_lcc_round<4, false><<<g, 256, 0, s>>>(a, dt);
-        else k_lcc_round<32, false><<<g, 256, 0, s>>>(a, dt);
+        if (dt.n_cls == 0) k_lcc_round<0, kFull><<<g, 256, 0, s>>>(a, dt);
+        else if (dt.n_cls <= 4) k_lcc_round<4, kFull><<<g, 256, 0, s>>>(a, dt);
+        else k_lcc_round<32, kFull><<<g, 256, 0, s>>>(a, dt);
         NA_CU(cudaGetLastError());
         NA_CU(read_stats());
         r++;
