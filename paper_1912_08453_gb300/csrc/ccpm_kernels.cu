@@ -45,6 +45,7 @@ namespace ccpm {
 struct RoundStats {
     unsigned long long scanned;   // active CSR entries read this round
     unsigned long long windows;   // CSR entries examined by searches
+    unsigned long long expanded;  // ... and while their items were listed
     unsigned long long matches;   // final search: matches found
     unsigned long long tokens;    // NLCC: (vertex, head) searches issued
     unsigned long long row_entries;   // CSR entries in rows of active vertices
@@ -57,8 +58,6 @@ struct RoundStats {
     unsigned int n_roots;
     unsigned int n_items;         // (root, head, first candidate) search items
     unsigned int overflow;        // a search hit its budget
-    unsigned int n_spill;         // items handed on by searches that ran long (reserved)
-    unsigned int spill_stop;      // the spill list is valid below this index (see spill)
     unsigned int skipped;         // LCC round queued after the fixpoint: did nothing
     // changes of omega waiting to be passed on to the neighbours (Change list,
     // and the pieces of their long rows); for a delta round also what its
@@ -67,6 +66,15 @@ struct RoundStats {
     unsigned int n_chg, n_chg_piece;
     unsigned int died;            // full rounds: survivors are alive - died
     unsigned long long old_kept, died_rows;
+};
+
+// Counters of one pass of a search over its items: the next item to take, the
+// items handed on by searches that ran long (reserved), and the complement of
+// the index below which that list is valid (see spill; zero: all of it).
+struct PassCtl {
+    unsigned long long next;
+    unsigned int n_out, stop_inv;
+    __device__ __host__ unsigned int handed_on() const { return n_out < ~stop_inv ? n_out : ~stop_inv; }
 };
 
 // A vertex whose omega a round (or a non-local check) has changed, and its new
@@ -224,7 +232,13 @@ __global__ void __launch_bounds__(256)
 k_init(int64_t n, const int64_t *__restrict__ rp, const uint8_t *__restrict__ lab, LabelMask lm,
        const uint32_t *__restrict__ om_in, uint32_t *om0, uint32_t *om1, void *nw0, void *nw1, int nw_bytes,
        int32_t *small_out, int32_t *med_out, ChunkItem *chunk_out, HubAcc *acc, RoundStats *st, int hub_deg,
-       int short_max, unsigned int set_changed) {
+       int short_max, unsigned int set_changed, const RoundStats *only_if, uint32_t *ebits, int64_t m) {
+    if (only_if && only_if->changed == 0u) return;
+    if (ebits && blockIdx.x == 0 && threadIdx.x == 0) {
+        // no entries past m: the padding bits of the last word and the guard word stay 0
+        if (m & 31) ebits[m >> 5] &= (1u << (uint32_t)(m & 31)) - 1u;
+        ebits[(m + 31) >> 5] = 0u;
+    }
     __shared__ uint32_t slm[256];
     __shared__ int32_t sbuf[2][8][32];
     __shared__ int scnt[2][8];
@@ -315,6 +329,7 @@ struct LccArgs {
     // rounds queued without a host round trip: the list sizes come from the
     // previous round's counters, and a round after the fixpoint does nothing
     const RoundStats *prev;       // nullable: sizes are the fields above
+    const RoundStats *gate;       // nullable: the round runs only if these counters say `changed`
     int resident_warps;           // warps of one resident wave (medium prefetch unit)
     uint32_t eta_off;             // ~0: ablation without edge elimination (every live
                                   // neighbour passes eta); 0: the method
@@ -884,11 +899,12 @@ k_lcc_round(LccArgs a, DevTmpl t) {
     constexpr bool DENSE = MODE == kDense;
     int64_t n_small = a.n_small, n_med = a.n_med, n_chunk = a.n_chunk;
     int MB = a.med_chunk;
+    const RoundStats *gate = a.prev ? a.prev : a.gate;
+    if (gate && gate->changed == 0u) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) a.st->skipped = 1u;
+        return;
+    }
     if (a.prev) {
-        if (a.prev->changed == 0u) {
-            if (blockIdx.x == 0 && threadIdx.x == 0) a.st->skipped = 1u;
-            return;
-        }
         // a full round's lists were written by the round before, a delta
         // round's by k_push into its own counters
         const RoundStats *sizes = MODE == kDelta ? a.st : a.prev;
@@ -1607,8 +1623,9 @@ struct SearchArgs {
                               // compacted rows (ids ascending) with nlab = nullptr
     const uint32_t *om;
     const int32_t *roots;
-    int64_t n_roots;
-    unsigned long long *next_root;   // dynamic work counter
+    int64_t n_roots;          // -1: st->n_roots
+    PassCtl *ctl;             // this pass
+    const PassCtl *ctl_prev;  // nullable: the items are those that pass handed on
     const DevPlan *plans;     // plans[h] for each head h (NLCC) or plans[0] (final)
     uint32_t heads;           // NLCC: heads of the constraint; final: 1 << plans[0].q[0]
     uint32_t *sat;            // NLCC output: satisfied heads per vertex
@@ -1618,13 +1635,12 @@ struct SearchArgs {
     uint64_t budget;          // windows per (root, head)
     uint64_t cap;             // final: stop past this many matches
     SearchItem *items;        // split search work: partial embeddings
-    int64_t n_items;
+    int64_t n_items;          // -1: st->n_items (none of them if they are more than items_cap)
     int64_t items_cap;
     SearchItem *spill;        // a search that has scanned spill_after windows hands its
     int64_t spill_cap;        // untried candidates on here as new items (0: never)
     uint64_t spill_after;
     int starve;               // also hand on when the item list has run dry (idle warps)
-    int item_batch;           // items a warp takes at a time
     int enum_heads;           // k_expand: 1 = final search (one head), 0 = NLCC
     const uint32_t *sat_seed; // existence passes: heads already known satisfied (nullable)
     // listing (mode kList): every match found gets an index from list_count;
@@ -1654,6 +1670,7 @@ struct WarpSearch {
     uint32_t done_bit;          // (by another warp's embedding); nullptr: never
     int head;                   // plan slot of the running item (spilled items keep it)
     int64_t entry;              // edge pass: the running item's CSR entry
+    int64_t n_items;            // items of this pass
     // the first kJoinCache stored join groups of one level in shared memory:
     // whole when they hold at most kJoinCacheLen ids, else every jc_step-th
     // id, which leaves a join test the search of one stretch of jc_step ids
@@ -1947,8 +1964,7 @@ constexpr int kSpillParts = 32;      // items one open level's untested candidat
 // Returns false (the search goes on where it is) when the list is full.
 // Reservations only ever add to the counter: the successful ones are exactly
 // those ending at or below the capacity, and they fill the list up to the
-// lowest start of a failed one (spill_stop), so the list is valid below
-// min(counter, spill_stop).
+// lowest start of a failed one (PassCtl::handed_on).
 __device__ bool spill(const SearchArgs &a, const WarpSearch &W, int d0, int d) {
     const int lane = (int)lane_id();
     unsigned int total = 0;
@@ -1958,12 +1974,12 @@ __device__ bool spill(const SearchArgs &a, const WarpSearch &W, int d0, int d) {
     }
     unsigned int base = 0, fits = 1;
     if (lane == 0 && total) {
-        if ((int64_t)*(volatile const unsigned int *)&a.st->n_spill >= a.spill_cap) {
+        if ((int64_t)*(volatile const unsigned int *)&a.ctl->n_out >= a.spill_cap) {
             fits = 0;                               // full already: do not grow the counter
         } else {
-            base = atomicAdd(&a.st->n_spill, total);
+            base = atomicAdd(&a.ctl->n_out, total);
             if ((int64_t)base + total > a.spill_cap) {
-                atomicMin(&a.st->spill_stop, base);
+                atomicMax(&a.ctl->stop_inv, ~base);
                 fits = 0;
             }
         }
@@ -2062,7 +2078,7 @@ __device__ bool search_from(const SearchArgs &a, const DevPlan &P, int d0, WarpS
                         stop = matches > a.cap || *(volatile const unsigned int *)&a.st->overflow;
                     }
                     if (a.starve && used >= kLook)
-                        hand = *(volatile const unsigned long long *)a.next_root >= (unsigned long long)a.n_items;
+                        hand = *(volatile const unsigned long long *)&a.ctl->next >= (unsigned long long)W.n_items;
                 }
                 pub = matches;
                 if (__shfl_sync(FULL_MASK, stop, 0)) {
@@ -2115,7 +2131,7 @@ __device__ bool search_from(const SearchArgs &a, const DevPlan &P, int d0, WarpS
 
 __device__ __forceinline__ int64_t grab_root(const SearchArgs &a) {
     unsigned long long r = 0;
-    if (lane_id() == 0) r = atomicAdd(a.next_root, 1ull);
+    if (lane_id() == 0) r = atomicAdd(&a.ctl->next, 1ull);
     return (int64_t)__shfl_sync(FULL_MASK, r, 0);
 }
 
@@ -2203,7 +2219,8 @@ k_expand(SearchArgs a) {
     const int64_t gwarp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     unsigned long long entries = 0, tokens = 0;
-    for (int64_t it = gwarp; it < a.n_roots; it += nwarps) {
+    const int64_t n_roots = a.n_roots >= 0 ? a.n_roots : (int64_t)a.st->n_roots;
+    for (int64_t it = gwarp; it < n_roots; it += nwarps) {
         const int32_t v = a.roots[it];
         const uint32_t seed = (!a.enum_heads && a.sat_seed) ? __ldg(a.sat_seed + v) : 0u;
         const uint32_t hv = a.enum_heads ? a.heads : (__ldg(a.om + v) & a.heads & ~seed);
@@ -2238,7 +2255,7 @@ k_expand(SearchArgs a) {
     }
     b.flush();
     if (lane == 0) {
-        if (entries) atomicAdd(&a.st->windows, entries);
+        if (entries) atomicAdd(&a.st->expanded, entries);
         if (tokens) atomicAdd(&a.st->tokens, tokens);
     }
 }
@@ -2286,13 +2303,24 @@ k_expand_next(SearchArgs a, const SearchItem *in, int64_t n_in) {
         }
     }
     b.flush();
-    if (lane == 0 && entries) atomicAdd(&a.st->windows, entries);
+    if (lane == 0 && entries) atomicAdd(&a.st->expanded, entries);
 }
 
 __device__ __forceinline__ int64_t grab_items(const SearchArgs &a, int batch) {
     unsigned long long r = 0;
-    if (lane_id() == 0) r = atomicAdd(a.next_root, (unsigned long long)batch);
+    if (lane_id() == 0) r = atomicAdd(&a.ctl->next, (unsigned long long)batch);
     return (int64_t)__shfl_sync(FULL_MASK, r, 0);
+}
+
+// Items of this pass, and how many of them a warp takes at a time: one where
+// there are few, so that none waits behind a long one.
+__device__ __forceinline__ int64_t pass_items(const SearchArgs &a, int &batch) {
+    int64_t n = a.n_items;
+    if (a.ctl_prev) n = a.ctl_prev->handed_on();
+    else if (n < 0) n = a.st->n_items <= a.items_cap ? (int64_t)a.st->n_items : 0;
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    batch = (int)max((int64_t)1, min((int64_t)16, n / (8 * warps)));
+    return n;
 }
 
 constexpr int kMaxPlans = 64;      // plan slots (heads, or oriented template edges)
@@ -2303,14 +2331,19 @@ constexpr int64_t kExpandBelow = 16384;
 
 __global__ void __launch_bounds__(128)
 k_nlcc_items(SearchArgs a) {
+    int batch;
+    const int64_t n_items = pass_items(a, batch);
+    if (n_items == 0) return;                        // a pass queued after the last one
     __shared__ WarpSearch ws[4];
     const int wib = threadIdx.x >> 5;
     const int lane = (int)lane_id();
     WarpSearch &W = ws[wib];
+    if (lane == 0) W.n_items = n_items;
+    __syncwarp();
     unsigned long long entries = 0, matches = 0;
     bool over = false;
-    for (int64_t it0 = grab_items(a, a.item_batch); it0 < a.n_items; it0 = grab_items(a, a.item_batch)) {
-        const int64_t it1 = min(a.n_items, it0 + a.item_batch);
+    for (int64_t it0 = grab_items(a, batch); it0 < n_items; it0 = grab_items(a, batch)) {
+        const int64_t it1 = min(n_items, it0 + batch);
         for (int64_t it = it0; it < it1; it++) {
             const SearchItem item = a.items[it];
             const int h = item.hd & 0xff, depth = item.hd >> 8;
@@ -2349,19 +2382,24 @@ k_nlcc_items(SearchArgs a) {
 template <int MODE>
 __global__ void __launch_bounds__(128)
 k_final_items(SearchArgs a) {
+    int batch;
+    const int64_t n_items = pass_items(a, batch);
+    if (n_items == 0) return;                        // a pass queued after the last one
     __shared__ WarpSearch ws[4];
     const int wib = threadIdx.x >> 5;
     const int lane = (int)lane_id();
     WarpSearch &W = ws[wib];
+    if (lane == 0) W.n_items = n_items;
+    __syncwarp();
     if (lane == 0) { W.last_plan = nullptr; W.pub = 0; }
     __syncwarp();
     unsigned long long entries = 0, matches = 0;
     bool over = false;
-    for (int64_t it0 = grab_items(a, a.item_batch); it0 < a.n_items; it0 = grab_items(a, a.item_batch)) {
+    for (int64_t it0 = grab_items(a, batch); it0 < n_items; it0 = grab_items(a, batch)) {
         unsigned int stop = 0;
         if (lane == 0) stop = *(volatile unsigned int *)&a.st->overflow;
         if (__shfl_sync(FULL_MASK, stop, 0)) break;
-        const int64_t it1 = min(a.n_items, it0 + a.item_batch);
+        const int64_t it1 = min(n_items, it0 + batch);
         for (int64_t it = it0; it < it1 && !over; it++) {
             const SearchItem item = a.items[it];
             const int depth = item.hd >> 8;
@@ -2413,7 +2451,8 @@ k_edge_items(SearchArgs a, EdgeTab tab) {
     // one block per root: its warps take every (blockDim/32)-th window of the
     // root's row, so the rows of hubs are split across the block
     const int nwb = (int)(blockDim.x >> 5);
-    for (int64_t it = blockIdx.x; it < a.n_roots; it += gridDim.x) {
+    const int64_t n_roots = a.n_roots >= 0 ? a.n_roots : (int64_t)a.st->n_roots;
+    for (int64_t it = blockIdx.x; it < n_roots; it += gridDim.x) {
         const int32_t x = a.roots[it];
         const uint32_t wx = __ldg(a.om + x);
         const int64_t beg = a.rp[x], end = a.rp[x + 1];
@@ -2446,14 +2485,19 @@ k_edge_items(SearchArgs a, EdgeTab tab) {
 
 __global__ void __launch_bounds__(128)
 k_edge_search(SearchArgs a) {
+    int batch;
+    const int64_t n_items = pass_items(a, batch);
+    if (n_items == 0) return;                        // a pass queued after the last one
     __shared__ WarpSearch ws[4];
     const int wib = threadIdx.x >> 5;
     const int lane = (int)lane_id();
     WarpSearch &W = ws[wib];
+    if (lane == 0) W.n_items = n_items;
+    __syncwarp();
     unsigned long long entries = 0, matches = 0;
     bool over = false;
-    for (int64_t it0 = grab_items(a, a.item_batch); it0 < a.n_items; it0 = grab_items(a, a.item_batch)) {
-        const int64_t it1 = min(a.n_items, it0 + a.item_batch);
+    for (int64_t it0 = grab_items(a, batch); it0 < n_items; it0 = grab_items(a, batch)) {
+        const int64_t it1 = min(n_items, it0 + batch);
         for (int64_t it = it0; it < it1; it++) {
             const SearchItem item = a.items[it];
             const int o = item.hd & 0xff, depth = item.hd >> 8;
@@ -2491,8 +2535,9 @@ k_edge_search(SearchArgs a) {
 }
 
 // omega* of the roots from their satisfied bits.
-__global__ void k_sat_to_omega(const int32_t *roots, int64_t n_roots, const uint32_t *sat, const uint32_t *om,
+__global__ void k_sat_to_omega(const int32_t *roots, const RoundStats *st, const uint32_t *sat, const uint32_t *om,
                                uint32_t *om_out) {
+    const int64_t n_roots = st->n_roots;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_roots; i += stride) {
         const int32_t v = roots[i];
@@ -2675,12 +2720,16 @@ k_collect_roots(int64_t n, const uint32_t *__restrict__ om, uint32_t heads, int3
 // omega empties is eliminated with its edges.  The changes are listed for the
 // LCC rounds that follow, and the totals of the state (entries kept, rows) lose
 // what the eliminated vertices held.  Both omega buffers are written: which
-// one the rounds continue from is the caller's matter.
+// one the rounds continue from is the caller's matter.  last: the last queued
+// pass of the search (NULL: the search is known to be complete).
 __global__ void __launch_bounds__(256)
-k_nlcc_apply(const int32_t *__restrict__ roots, int64_t n_roots, uint32_t heads,
+k_nlcc_apply(const int32_t *__restrict__ roots, const PassCtl *last, int64_t items_cap, uint32_t heads,
              const uint32_t *__restrict__ sat, const uint32_t *om, uint32_t *om0, uint32_t *om1, void *nw0, void *nw1,
              int nw_bytes, const int64_t *__restrict__ rp, uint32_t *deg, Change *chg,
              ChangePiece *chg_piece, int hub_deg, RoundStats *st) {
+    // queued behind the search's passes: does nothing if they did not finish it
+    if (last && (st->n_items > items_cap || last->handed_on())) return;
+    const int64_t n_roots = st->n_roots;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     uint32_t changed = 0, died = 0;
     unsigned long long old_kept = 0, died_rows = 0;
@@ -2751,28 +2800,44 @@ k_materialize(int64_t n, const uint32_t *__restrict__ om, const int64_t *__restr
 }
 
 __global__ void k_set_word(uint32_t *p, uint32_t v) { *p = v; }
-__global__ void k_and_word(uint32_t *p, uint32_t v) { *p &= v; }
 
 // Per template vertex q: number of vertices with q in omega(v); slot 32: the
-// total of |omega(v)|.  Inputs of the ordering features and the logs.
+// total of |omega(v)|.  Inputs of the ordering features and the logs, and what
+// says that a check has no root.  One pass over omega: lane q counts template
+// vertex q, and 32 empty words (most of them, once LCC has run) cost a load and
+// a vote (all 32 counters of every lane used to be added up for every word: 85
+// us over 16M vertices, 18 us now).
 __global__ void __launch_bounds__(256)
 k_omega_hist(int64_t n, const uint32_t *__restrict__ om, int n0, unsigned long long *hist) {
-    unsigned int cnt[kMaxT];
-#pragma unroll
-    for (int q = 0; q < kMaxT; q++) cnt[q] = 0u;
+    __shared__ unsigned int sh[kMaxT];
+    if (threadIdx.x < kMaxT) sh[threadIdx.x] = 0u;
+    __syncthreads();
+    const int lane = (int)lane_id();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-        const uint32_t w = __ldg(om + v);
+    unsigned int mine = 0;
+    constexpr int U = 4;                             // words in flight per lane
+    for (int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - lane; b < n; b += stride * U) {
+        uint32_t w[U];
 #pragma unroll
-        for (int q = 0; q < kMaxT; q++) cnt[q] += (w >> q) & 1u;
+        for (int j = 0; j < U; j++) {
+            const int64_t v = b + j * stride + lane;
+            w[j] = v < n ? __ldg(om + v) : 0u;
+        }
+#pragma unroll
+        for (int j = 0; j < U; j++) {
+            for (uint32_t any = __reduce_or_sync(FULL_MASK, w[j]); any; any &= any - 1u) {
+                const int q = __ffs(any) - 1;
+                const uint32_t m = __ballot_sync(FULL_MASK, (w[j] >> q) & 1u);
+                if (lane == q) mine += __popc(m);
+            }
+        }
     }
-    unsigned long long total = 0;
-    for (int q = 0; q < n0; q++) {
-        unsigned int c = __reduce_add_sync(FULL_MASK, cnt[q]);
-        total += c;
-        if (lane_id() == 0 && c) atomicAdd(&hist[q], (unsigned long long)c);
+    if (mine) atomicAdd(&sh[lane], mine);
+    __syncthreads();
+    if ((int)threadIdx.x < n0 && sh[threadIdx.x]) {
+        atomicAdd(&hist[threadIdx.x], (unsigned long long)sh[threadIdx.x]);
+        atomicAdd(&hist[kMaxT], (unsigned long long)sh[threadIdx.x]);
     }
-    if (lane_id() == 0 && total) atomicAdd(&hist[kMaxT], total);
 }
 
 // Per label: vertices (out[0..255]) and the entries in their rows (out[256..511]).
@@ -2824,6 +2889,24 @@ using namespace ccpm;
 // at once (3 us), a host round trip 20 us or more.
 constexpr int kLccFirstGroup = 6, kLccGroup = 4;
 
+// Passes of a search queued per host round trip (even: each batch of passes
+// starts with the same of the two item buffers).  A search rarely needs more
+// where the graph is small; a pass without items costs 3 us.
+constexpr int kChain = 4;
+
+// Device counters with a pinned host mirror, copied in one piece.
+struct RoundGroup {
+    RoundStats ring[kLccFirstGroup];
+    unsigned long long hist[kMaxT + 1];
+};
+struct Control {
+    RoundGroup grp[2];            // two groups of queued LCC rounds, and omega's histogram after each
+    RoundStats init;              // k_init: sizes of the lists it makes
+    RoundStats st;                // searches and checks
+    PassCtl pass[kChain];
+    unsigned long long cnt[2];    // population counts of the result
+};
+
 struct Workspace {
     int64_t n = 0, m = 0, words = 0;
     int hub_deg = 0;
@@ -2844,22 +2927,16 @@ struct Workspace {
     SearchItem *spill_items = nullptr;   // items handed on by long searches
     int64_t spill_cap = 0;
     DevPlan *plans = nullptr;
-    RoundStats *st = nullptr;        // device
-    RoundStats *st_ring = nullptr;   // counters of two groups of queued LCC rounds
+    Control *ctl = nullptr, *ctl_h = nullptr;     // device, pinned host mirror
+    RoundStats *st = nullptr, *st_h = nullptr;    // their search counters
+    unsigned long long *cnt = nullptr, *cnt_h = nullptr;
+    unsigned long long hist_h[kMaxT + 1] = {};    // the latest omega histogram
     uint32_t *dirty = nullptr;       // delta rounds: one bit per listed vertex, all zero between rounds
     int32_t *dsmall = nullptr, *dmed = nullptr;   // their lists
     ChunkItem *dchunk = nullptr;
     Change *chg = nullptr;           // changes of omega not passed on yet
     ChangePiece *chg_piece = nullptr;
-    RoundStats *st_ring_h = nullptr; // pinned host mirror
-    unsigned long long *next_root = nullptr;   // dynamic root counter of the searches
-    RoundStats *st_h = nullptr;      // pinned host mirror
-    unsigned long long *cnt = nullptr;
-    unsigned long long *cnt_h = nullptr;
-    unsigned long long *hist = nullptr;      // 33 counters (k_omega_hist)
-    unsigned long long *hist_h = nullptr;
     DevPlan *plans_h = nullptr;      // pinned staging for plan uploads
-    unsigned long long *aux_h = nullptr;     // pinned: counters snapshotted in stream order
     cudaEvent_t ev[13] = {};
     // compacted rows (K4), two generations; allocated at the first compaction
     int64_t *sub_rp[2] = {nullptr, nullptr};
@@ -3007,16 +3084,10 @@ void ws_free(Workspace &w) {
     cudaFree(w.om[0]); cudaFree(w.om[1]); cudaFree(w.nw[0]); cudaFree(w.nw[1]); cudaFree(w.ebits);
     cudaFree(w.small[0]); cudaFree(w.small[1]); cudaFree(w.med[0]); cudaFree(w.med[1]);
     cudaFree(w.chunk[0]); cudaFree(w.chunk[1]); cudaFree(w.acc); cudaFree(w.roots);
-    cudaFree(w.sat); cudaFree(w.items); cudaFree(w.items2); cudaFree(w.spill_items); cudaFree(w.plans); cudaFree(w.st); cudaFree(w.cnt); cudaFree(w.next_root);
-    if (w.st_h) cudaFreeHost(w.st_h);
-    cudaFree(w.st_ring);
+    cudaFree(w.sat); cudaFree(w.items); cudaFree(w.items2); cudaFree(w.spill_items); cudaFree(w.plans); cudaFree(w.ctl);
+    if (w.ctl_h) cudaFreeHost(w.ctl_h);
     cudaFree(w.dirty); cudaFree(w.dsmall); cudaFree(w.dmed); cudaFree(w.dchunk); cudaFree(w.chg); cudaFree(w.chg_piece);
-    if (w.st_ring_h) cudaFreeHost(w.st_ring_h);
-    if (w.cnt_h) cudaFreeHost(w.cnt_h);
-    cudaFree(w.hist);
-    if (w.hist_h) cudaFreeHost(w.hist_h);
     if (w.plans_h) cudaFreeHost(w.plans_h);
-    if (w.aux_h) cudaFreeHost(w.aux_h);
     for (auto &e : w.ev) if (e) cudaEventDestroy(e);
     for (int i = 0; i < 2; i++) { cudaFree(w.sub_rp[i]); cudaFree(w.sub_col[i]); cudaFree(w.sub_bits[i]); }
     for (int i = 0; i < 2; i++) { cudaFree(w.sub_nlab[i]); cudaFree(w.sub_dslot[i]); cudaFree(w.sub_gdir[i]); }
@@ -3056,9 +3127,12 @@ int ws_ensure(ccpm_ctx *ctx, ccpm_graph *g, int hub_deg) {
     w.spill_cap = std::max<int64_t>(w.items_cap / 4, (int64_t)1 << 20);
     if ((rc = dalloc(ctx, &w.spill_items, (size_t)w.spill_cap))) return rc;
     if ((rc = dalloc(ctx, &w.plans, (size_t)kMaxPlans))) return rc;
-    if ((rc = dalloc(ctx, &w.st, 1))) return rc;
-    if ((rc = dalloc(ctx, &w.st_ring, (size_t)(2 * kLccFirstGroup)))) return rc;
-    CU(ctx, cudaMallocHost((void **)&w.st_ring_h, sizeof(RoundStats) * kLccFirstGroup));
+    if ((rc = dalloc(ctx, &w.ctl, 1))) return rc;
+    CU(ctx, cudaMallocHost((void **)&w.ctl_h, sizeof(Control)));
+    w.st = &w.ctl->st;
+    w.st_h = &w.ctl_h->st;
+    w.cnt = w.ctl->cnt;
+    w.cnt_h = w.ctl_h->cnt;
     if ((rc = dalloc(ctx, &w.dirty, (size_t)g->n / 32 + 1))) return rc;
     if ((rc = dalloc(ctx, &w.dsmall, (size_t)g->n))) return rc;
     if ((rc = dalloc(ctx, &w.dmed, (size_t)g->n))) return rc;
@@ -3066,14 +3140,7 @@ int ws_ensure(ccpm_ctx *ctx, ccpm_graph *g, int hub_deg) {
     if ((rc = dalloc(ctx, &w.chg, (size_t)g->n))) return rc;
     if ((rc = dalloc(ctx, &w.chg_piece, (size_t)w.chunk_cap))) return rc;
     if ((rc = dalloc(ctx, &w.deg, (size_t)g->n))) return rc;
-    if ((rc = dalloc(ctx, &w.cnt, 2))) return rc;
-    if ((rc = dalloc(ctx, &w.next_root, 1))) return rc;
-    CU(ctx, cudaMallocHost((void **)&w.st_h, sizeof(RoundStats)));
-    CU(ctx, cudaMallocHost((void **)&w.cnt_h, 2 * sizeof(unsigned long long)));
-    CU(ctx, cudaMalloc((void **)&w.hist, (kMaxT + 1) * sizeof(unsigned long long)));
-    CU(ctx, cudaMallocHost((void **)&w.hist_h, (kMaxT + 1) * sizeof(unsigned long long)));
     CU(ctx, cudaMallocHost((void **)&w.plans_h, kMaxPlans * sizeof(DevPlan)));
-    CU(ctx, cudaMallocHost((void **)&w.aux_h, 4 * sizeof(unsigned long long)));
     CU(ctx, cudaMemsetAsync(w.acc, 0, sizeof(HubAcc) * (size_t)w.acc_cap, ctx->stream));
     for (auto &e : w.ev) CU(ctx, cudaEventCreate(&e));
     return CCPM_OK;
@@ -3154,9 +3221,9 @@ int expand_more(ccpm_ctx *ctx, Workspace &w, SearchArgs &a, int max_depth, int64
         int grid = (int)std::max<int64_t>(1, std::min<int64_t>((a.n_items + 3) / 4, (int64_t)grid_sms(ctx) * 16));
         k_expand_next<<<grid, 128, 0, ctx->stream>>>(a, w.items2, a.n_items);
         CU(ctx, cudaGetLastError());
-        unsigned int n2 = 0;
-        CU(ctx, cudaMemcpyAsync(&n2, &w.st->n_items, sizeof(unsigned int), cudaMemcpyDeviceToHost, ctx->stream));
+        CU(ctx, cudaMemcpyAsync(w.st_h, w.st, sizeof(RoundStats), cudaMemcpyDeviceToHost, ctx->stream));
         CU(ctx, ctx_sync(ctx));
+        const unsigned int n2 = w.st_h->n_items;
         if ((int64_t)n2 > w.items_cap) return set_err(ctx, CCPM_EOVERFLOW, "search items overflow");
         a.n_items = n2;
     }
@@ -3183,57 +3250,118 @@ int grid_for(ccpm_ctx *ctx, int64_t work_items, int per_block, int blocks_per_sm
 // Windows a search scans before it hands the rest of its work to other warps.
 constexpr uint64_t kSpillAfter = 2048;
 
-// Run an item kernel, then again over the items long searches handed on, until
-// none are left (an item handed on is deeper, or holds fewer candidates of the
-// same position, than the one it came from, so the passes end).  kind 0: NLCC existence (k_nlcc_items), 1: final
-// count, 2: final count and mark, 3: count and list, 4: per-entry existence
-// (k_edge_search).  Counting (and marking) stops once the cap
-// is passed.
-int item_passes(ccpm_ctx *ctx, Workspace &w, SearchArgs &a, int kind, uint64_t split, bool starve,
-                int64_t &launches, int64_t &passes) {
-    cudaStream_t s = ctx->stream;
+// Read all counters.
+int read_control(ccpm_ctx *ctx, Workspace &w) {
+    CU(ctx, cudaMemcpyAsync(w.ctl_h, w.ctl, sizeof(Control), cudaMemcpyDeviceToHost, ctx->stream));
+    CU(ctx, ctx_sync(ctx));
+    return CCPM_OK;
+}
+
+// Zero the counters of a search.
+int clear_search(ccpm_ctx *ctx, Workspace &w) {
+    CU(ctx, cudaMemsetAsync(w.st, 0, sizeof(RoundStats) + sizeof(PassCtl) * kChain, ctx->stream));
+    return CCPM_OK;
+}
+static_assert(offsetof(Control, pass) == offsetof(Control, st) + sizeof(RoundStats), "cleared together");
+
+// How a search runs.  kind 0: NLCC existence (k_nlcc_items), 1: final count, 2:
+// final count and mark, 3: count and list, 4: per-entry existence
+// (k_edge_search).  split: windows a search scans before it hands its rest on
+// in any case (0: never); starve: it also does when other warps are idle.
+struct SearchMode {
+    int kind;
+    uint64_t split;
+    bool starve;
+};
+
+// Queue kChain passes over the items in a.items (a.n_items, or on the device):
+// each but the first runs over what the one before handed on.
+int queue_passes(ccpm_ctx *ctx, Workspace &w, SearchArgs &a, const SearchMode &m, int64_t &launches) {
     SearchItem *bufs[2] = {w.items, w.spill_items};
     const int64_t caps[2] = {w.items_cap, w.spill_cap};
-    int cur = 0;
-    for (;;) {
-        a.items = bufs[cur];
-        a.spill = bufs[cur ^ 1];
-        a.spill_cap = caps[cur ^ 1];
-        a.spill_after = split;
-        a.starve = starve ? 1 : 0;
-        CU(ctx, cudaMemsetAsync(w.next_root, 0, sizeof(unsigned long long), s));
-        CU(ctx, cudaMemsetAsync(&w.st->n_spill, 0, sizeof(unsigned int), s));
-        CU(ctx, cudaMemsetAsync(&w.st->spill_stop, 0xFF, sizeof(unsigned int), s));
-        // few items: one at a time, so that none waits behind a long one
-        const int64_t warps = (int64_t)grid_sms(ctx) * 64;
-        a.item_batch = (int)std::max<int64_t>(1, std::min<int64_t>(16, a.n_items / (8 * warps)));
-        const int gi = grid_for(ctx, (a.n_items + a.item_batch - 1) / a.item_batch * 32, 128, 16);
+    a.spill_after = m.split;
+    a.starve = m.starve ? 1 : 0;
+    // known item counts: no more warps than items
+    const int gi = a.n_items >= 0 ? grid_for(ctx, a.n_items * 32, 128, 16) : grid_sms(ctx) * 16;
+    for (int p = 0; p < kChain; p++) {
+        a.items = bufs[p & 1];
+        a.spill = bufs[(p & 1) ^ 1];
+        a.spill_cap = caps[(p & 1) ^ 1];
+        a.ctl = w.ctl->pass + p;
+        a.ctl_prev = p ? a.ctl - 1 : nullptr;
+        const int grid = p ? grid_sms(ctx) * 16 : gi;
         launches++;
-        passes++;
-        if (kind == 0) k_nlcc_items<<<gi, 128, 0, s>>>(a);
-        else if (kind == 1) k_final_items<kCount><<<gi, 128, 0, s>>>(a);
-        else if (kind == 2) k_final_items<kMark><<<gi, 128, 0, s>>>(a);
-        else if (kind == 3) k_final_items<kList><<<gi, 128, 0, s>>>(a);
-        else k_edge_search<<<gi, 128, 0, s>>>(a);
+        if (m.kind == 0) k_nlcc_items<<<grid, 128, 0, ctx->stream>>>(a);
+        else if (m.kind == 1) k_final_items<kCount><<<grid, 128, 0, ctx->stream>>>(a);
+        else if (m.kind == 2) k_final_items<kMark><<<grid, 128, 0, ctx->stream>>>(a);
+        else if (m.kind == 3) k_final_items<kList><<<grid, 128, 0, ctx->stream>>>(a);
+        else k_edge_search<<<grid, 128, 0, ctx->stream>>>(a);
         CU(ctx, cudaGetLastError());
-        CU(ctx, cudaMemcpyAsync(&w.aux_h[1], &w.st->n_spill, sizeof(unsigned int), cudaMemcpyDeviceToHost, s));
-        CU(ctx, cudaMemcpyAsync(&w.aux_h[2], &w.st->overflow, sizeof(unsigned int), cudaMemcpyDeviceToHost, s));
-        CU(ctx, cudaMemcpyAsync(&w.aux_h[3], &w.st->spill_stop, sizeof(unsigned int), cudaMemcpyDeviceToHost, s));
-        CU(ctx, ctx_sync(ctx));
-        const unsigned int spilled = std::min((unsigned int)(w.aux_h[1] & 0xFFFFFFFFull),
-                                              (unsigned int)(w.aux_h[3] & 0xFFFFFFFFull));
-        const unsigned int over = (unsigned int)(w.aux_h[2] & 0xFFFFFFFFull);
-        if (spilled == 0 || (kind != 0 && kind != 4 && over)) break;
-        a.n_items = spilled;
-        cur ^= 1;
     }
     a.items = w.items;
     a.spill = nullptr;
     a.spill_after = 0;
     a.starve = 0;
+    a.ctl = w.ctl->pass;
+    a.ctl_prev = nullptr;
     return CCPM_OK;
 }
 
+// Queue the item list of a search over a.roots and its first passes, with no
+// host round trip (searches that do not hand on to idle warps: one per level
+// of the expansion).  The counters were cleared before.
+int queue_search(ccpm_ctx *ctx, Workspace &w, SearchArgs &a, const SearchMode &m, int max_depth, int64_t &launches) {
+    a.ctl = w.ctl->pass;
+    a.ctl_prev = nullptr;
+    launches++;
+    const int64_t most = a.n_roots >= 0 ? a.n_roots : (int64_t)1 << 40;
+    k_expand<<<grid_for(ctx, most * 32, 256, 8), 256, 0, ctx->stream>>>(a);
+    CU(ctx, cudaGetLastError());
+    a.n_items = -1;
+    if (!m.starve) {
+        int rc = read_control(ctx, w);
+        if (rc) return rc;
+        a.n_items = w.st_h->n_items;
+        if (a.n_items > w.items_cap) a.n_items = -1;         // more than fit: the passes do nothing
+        else if ((rc = expand_more(ctx, w, a, max_depth, launches))) return rc;
+    }
+    return queue_passes(ctx, w, a, m, launches);
+}
+
+// Was a queued search complete?  (Its counters have been read.)
+bool search_complete(const Workspace &w, const SearchMode &m) {
+    if (w.st_h->n_items > w.items_cap) return false;
+    if (m.kind >= 1 && m.kind <= 3 && w.st_h->overflow) return true;    // past the cap (or out of budget): stopped
+    return w.ctl_h->pass[kChain - 1].handed_on() == 0;
+}
+
+// Complete a queued search whose counters have been read: further passes over
+// what was handed on (an item handed on is deeper, or holds fewer candidates
+// of the same position, than the one it came from, so the passes end), or, if
+// its items did not fit, one warp per root.
+int finish_search(ccpm_ctx *ctx, Workspace &w, SearchArgs &a, const SearchMode &m, int64_t &launches) {
+    int rc;
+    if (w.st_h->n_items > w.items_cap && m.kind != 4) {
+        CU(ctx, cudaMemsetAsync(w.ctl->pass, 0, sizeof(PassCtl), ctx->stream));
+        launches++;
+        a.n_roots = w.st_h->n_roots;
+        a.ctl = w.ctl->pass;
+        const int grid = grid_for(ctx, a.n_roots * 32, 128, 16);
+        if (m.kind == 0) k_nlcc_search<<<grid, 128, 0, ctx->stream>>>(a);
+        else if (m.kind == 1) k_final_search<kCount><<<grid, 128, 0, ctx->stream>>>(a);
+        else if (m.kind == 2) k_final_search<kMark><<<grid, 128, 0, ctx->stream>>>(a);
+        else k_final_search<kList><<<grid, 128, 0, ctx->stream>>>(a);
+        CU(ctx, cudaGetLastError());
+        return read_control(ctx, w);
+    }
+    while (!search_complete(w, m)) {
+        a.n_items = w.ctl_h->pass[kChain - 1].handed_on();
+        CU(ctx, cudaMemsetAsync(w.ctl->pass, 0, sizeof(PassCtl) * kChain, ctx->stream));
+        if ((rc = queue_passes(ctx, w, a, m, launches))) return rc;
+        if ((rc = read_control(ctx, w))) return rc;
+    }
+    return CCPM_OK;
+}
 
 // Ordering features of one constraint in the current state (alive[q] =
 // vertices with q in omega, total = sum of |omega|), step = constraints run.
@@ -3284,7 +3412,7 @@ struct Pipeline {
     int rc_compact = 0;
     double ms_lcc_kernel = 0.0;
     double ms_search_kernel = 0.0;
-    int64_t search_launches = 0, nlcc_entries = 0, item_passes = 0;
+    int64_t search_launches = 0, nlcc_entries = 0;
     int maxc = 0;
     int short_max = kSmallDeg;      // rows up to this length take the flat short-row path
     bool eta_off = false;           // ablation: no edge elimination
@@ -3309,32 +3437,15 @@ struct Pipeline {
     int64_t last_kept = -1, last_rows = -1, last_alive = 0;
     bool synced = true;             // the lists hold every live vertex, both omega buffers are equal
 
-    // alive counts per template vertex (w.hist_h[0..31]) and total bits ([32])
-    int omega_hist() {
-        Workspace &w = ctx->ws;
-        CU(ctx, cudaMemsetAsync(w.hist, 0, (kMaxT + 1) * sizeof(unsigned long long), ctx->stream));
-        launches++;
-        k_omega_hist<<<grid_for(ctx, g->n, 256, 4), 256, 0, ctx->stream>>>(g->n, w.om[cur], t->n0, w.hist);
-        CU(ctx, cudaGetLastError());
-        CU(ctx, cudaMemcpyAsync(w.hist_h, w.hist, (kMaxT + 1) * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
-                                ctx->stream));
-        CU(ctx, ctx_sync(ctx));
-        return CCPM_OK;
-    }
-
-    int read_stats() {
-        Workspace &w = ctx->ws;
-        CU(ctx, cudaMemcpyAsync(w.st_h, w.st, sizeof(RoundStats), cudaMemcpyDeviceToHost, ctx->stream));
-        CU(ctx, ctx_sync(ctx));
-        return CCPM_OK;
-    }
+    int read_stats() { return read_control(ctx, ctx->ws); }
 
     // One LCC round.  slot: its counters; prev (nullable): the counters of the
     // round before, from which the round reads its list sizes and whether there
-    // is anything to do on the device (without: the host's sizes).  c, l: the
+    // is anything to do on the device (without: the host's sizes, and the round
+    // runs only if the counters `gate` (nullable) say that something changed).  c, l: the
     // omega and list buffers it reads (the host flips cur / li only once a
     // group of queued rounds is done, by the number of rounds that ran).
-    int launch_round(RoundStats *slot, const RoundStats *prev, int c, int l, bool delta) {
+    int launch_round(RoundStats *slot, const RoundStats *prev, const RoundStats *gate, int c, int l, bool delta) {
         Workspace &w = ctx->ws;
         LccArgs a;
         a.rp = lrp;
@@ -3354,6 +3465,7 @@ struct Pipeline {
         a.acc = w.acc;
         a.st = slot;
         a.prev = prev;
+        a.gate = gate;
         a.resident_warps = grid_sms(ctx) * 32;
         a.hub_deg = w.hub_deg;
         a.deg = w.deg;
@@ -3432,39 +3544,45 @@ struct Pipeline {
 
     // LCC to fixpoint; returns rounds via *rounds.  Rounds are queued in groups
     // with one host round trip per group: each reads what it needs from the
-    // counters of the round before (w.st: of the initialisation, or of the
-    // non-local check whose changes are in the Change list), and rounds queued
-    // after the fixpoint return at once.  A prune's first rounds (two, or one
+    // counters of the round before (the first: of the initialisation, or of the
+    // non-local check queued before it, whose changes are in the Change list),
+    // and rounds queued after the fixpoint, or after a check that changed
+    // nothing, return at once.  After each group omega's histogram is taken if
+    // asked for (w.hist_h).  A prune's first rounds (two, or one
     // from a saved state) evaluate every active vertex, as nearly all of them
     // change; where the rows are large (use_deltas) the later ones are delta
     // rounds.  With options.compact > 0 every round is a full one and the rows
     // may be compacted between groups.
-    int lcc(int64_t *rounds, bool initial) {
+    int lcc(int64_t *rounds, bool initial, bool want_hist) {
         Workspace &w = ctx->ws;
         int64_t r = 0;
         const bool deltas = use_deltas(initial ? first_rows : last_rows);
         int full_left = initial ? (dense ? 2 : 1) : 0;
-        const RoundStats *src = (initial || deltas) ? w.st : nullptr;
+        const RoundStats *src = initial ? &w.ctl->init : (deltas ? w.st : nullptr);
+        const RoundStats *gate = initial ? nullptr : w.st;
+        const bool was_synced = synced;
         if (!initial && !deltas && !synced) {
             // earlier delta rounds left the lists and the other omega buffer
-            // behind: rebuild them (k_init marks its counters as changed)
-            int rc = rebucket(lrp, false, 1u);
+            // behind: rebuild them if the check changed anything (k_init then
+            // marks its counters as changed)
+            int rc = rebucket(lrp, false, w.st);
             if (rc) return rc;
-            src = w.st;
+            src = &w.ctl->init;
         }
         bool seed = false;                // the next delta round follows a full one
         for (int group = 0;; group++) {
             const bool first = initial && group == 0;
             const int G = first ? (compact_mode > 0 ? 1 : kLccFirstGroup) : kLccGroup;
-            RoundStats *ring = w.st_ring + (group & 1) * kLccFirstGroup;
-            CU(ctx, cudaMemsetAsync(ring, 0, sizeof(RoundStats) * (size_t)G, ctx->stream));
+            RoundGroup *grp = w.ctl->grp + (group & 1);
+            RoundStats *ring = grp->ring;
+            CU(ctx, cudaMemsetAsync(grp, 0, sizeof(RoundGroup), ctx->stream));
             CU(ctx, cudaEventRecord(w.ev[4], ctx->stream));
             int n_full = 0, c = cur, l = li, rc;
             for (int i = 0; i < G; i++) {
                 const RoundStats *prev = i ? ring + i - 1 : src;
                 if (!deltas || full_left > 0) {
                     if (full_left > 0) full_left--;
-                    if ((rc = launch_round(ring + i, prev, c, l, false))) return rc;
+                    if ((rc = launch_round(ring + i, prev, i ? nullptr : gate, c, l, false))) return rc;
                     n_full++;
                     c ^= 1;
                     l ^= 1;
@@ -3472,20 +3590,32 @@ struct Pipeline {
                     synced = true;
                 } else {
                     if ((rc = launch_push(ring + i, prev, c, l, seed))) return rc;
-                    if ((rc = launch_round(ring + i, prev, c, l, true))) return rc;
+                    if ((rc = launch_round(ring + i, prev, nullptr, c, l, true))) return rc;
                     seed = false;
                     synced = false;
                 }
                 if (first && i == 0) CU(ctx, cudaEventRecord(w.ev[12], ctx->stream));
             }
             CU(ctx, cudaEventRecord(w.ev[5], ctx->stream));
-            CU(ctx, cudaMemcpyAsync(w.st_ring_h, ring, sizeof(RoundStats) * (size_t)G, cudaMemcpyDeviceToHost,
-                                    ctx->stream));
-            if (first)
-                CU(ctx, cudaMemcpyAsync(w.st_h, w.st, sizeof(RoundStats), cudaMemcpyDeviceToHost, ctx->stream));
-            CU(ctx, ctx_sync(ctx));
-            if (first && (w.st_h->n_hub_slots > (unsigned)w.acc_cap || (int64_t)w.st_h->n_chunk > w.chunk_cap))
+            if (want_hist) {
+                // the omega buffer the state is in if every queued round ran; any
+                // that did not leaves the two buffers equal (a fixpoint)
+                launches++;
+                k_omega_hist<<<grid_for(ctx, g->n, 256, 8), 256, 0, ctx->stream>>>(g->n, w.om[c], t->n0, grp->hist);
+                CU(ctx, cudaGetLastError());
+            }
+            if ((rc = read_control(ctx, w))) return rc;
+            if (group == 0 && !initial) after_check();
+            const RoundGroup &grp_h = w.ctl_h->grp[group & 1];
+            if (want_hist) std::memcpy(w.hist_h, grp_h.hist, sizeof(w.hist_h));
+            if (first && (w.ctl_h->init.n_hub_slots > (unsigned)w.acc_cap ||
+                          (int64_t)w.ctl_h->init.n_chunk > w.chunk_cap))
                 return set_err(ctx, CCPM_EOVERFLOW, "hub bookkeeping overflow");
+            if (!initial && group == 0 && !w.st_h->changed) {
+                synced = was_synced;                      // the check changed nothing: no round ran
+                break;
+            }
+            gate = nullptr;
             float ms = 0.f;
             CU(ctx, cudaEventElapsedTime(&ms, w.ev[4], w.ev[5]));
             ms_lcc_kernel += ms;
@@ -3496,7 +3626,7 @@ struct Pipeline {
             bool done = false;
             int ran = 0;
             for (int i = 0; i < G && !done; i++) {
-                const RoundStats &h = w.st_ring_h[i];
+                const RoundStats &h = grp_h.ring[i];
                 if (h.skipped) break;
                 ran++;
                 r++;
@@ -3595,25 +3725,28 @@ struct Pipeline {
 
     // Frontier of the live vertices over rows rp (the pieces of a long row
     // consecutive and in order); also makes both omega buffers equal.
-    int rebucket(const int64_t *rp, bool sync = true, unsigned int set_changed = 0u) {
+    // only_if (nullable): on the device, only if these counters say `changed`.
+    int rebucket(const int64_t *rp, bool sync = true, const RoundStats *only_if = nullptr) {
         synced = true;
         Workspace &w = ctx->ws;
         LabelMask all;
         std::memset(&all, 0xFF, sizeof(all));
-        CU(ctx, cudaMemsetAsync(w.st, 0, sizeof(RoundStats), ctx->stream));
+        CU(ctx, cudaMemsetAsync(&w.ctl->init, 0, sizeof(RoundStats), ctx->stream));
         launches++;
         k_init<<<grid_for(ctx, g->n, 256, 8), 256, 0, ctx->stream>>>(g->n, rp, g->lab, all, w.om[cur], w.om[cur],
                                                                      w.om[cur ^ 1], w.nw[cur], w.nw[cur ^ 1], nw_bytes,
-                                                                     w.small[li], w.med[li], w.chunk[li], w.acc, w.st,
-                                                                     w.hub_deg, short_max, set_changed);
+                                                                     w.small[li], w.med[li], w.chunk[li], w.acc,
+                                                                     &w.ctl->init, w.hub_deg, short_max,
+                                                                     only_if ? 1u : 0u, only_if, nullptr, 0);
         CU(ctx, cudaGetLastError());
         if (!sync) return CCPM_OK;
         int rc = read_stats();
         if (rc) return rc;
-        n_small = w.st_h->n_small;
-        n_med = w.st_h->n_med;
-        n_chunk = w.st_h->n_chunk;
-        if (w.st_h->n_hub_slots > (unsigned)w.acc_cap || n_chunk > w.chunk_cap)
+        const RoundStats &h = w.ctl_h->init;
+        n_small = h.n_small;
+        n_med = h.n_med;
+        n_chunk = h.n_chunk;
+        if (h.n_hub_slots > (unsigned)w.acc_cap || n_chunk > w.chunk_cap)
             return set_err(ctx, CCPM_EOVERFLOW, "hub bookkeeping overflow");
         return CCPM_OK;
     }
@@ -3685,7 +3818,7 @@ struct Pipeline {
         ca.med_in = w.med[li];
         ca.chunk_in = w.chunk[li];
         ca.acc = w.acc;
-        ca.lists = w.st;
+        ca.lists = &w.ctl->init;
         ca.hub_deg = w.hub_deg;
         ca.n_rank = nl;
         std::memset(ca.lab_rank, 0xFF, sizeof(ca.lab_rank));
@@ -4115,22 +4248,13 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
     } else {
         CUF(cudaMemsetAsync(w.ebits, 0xFF, sizeof(uint32_t) * (size_t)w.words, s));
     }
-    // no entries past m_dir: padding bits of the last word and the guard word stay 0
-    k_set_word<<<1, 1, 0, s>>>(w.ebits + w.words, 0u);
-    P.launches += 1 + ((g->m & 31) != 0);
-    if (g->m & 31) {
-        const uint32_t pad = (1u << (uint32_t)(g->m & 31)) - 1u;
-        if (resume) k_and_word<<<1, 1, 0, s>>>(w.ebits + w.words - 1, pad);
-        else k_set_word<<<1, 1, 0, s>>>(w.ebits + w.words - 1, pad);
-    }
-    CUF(cudaGetLastError());
-    CUF(cudaMemsetAsync(w.st, 0, sizeof(RoundStats), s));
+    CUF(cudaMemsetAsync(&w.ctl->init, 0, sizeof(RoundStats), s));
     {
         int grid = grid_for(ctx, g->n, 256, 8);
         P.launches++;
         k_init<<<grid, 256, 0, s>>>(g->n, g->rp, g->lab, lm, resume ? r->om : nullptr, w.om[0], w.om[1], w.nw[0],
-                                    w.nw[1], P.nw_bytes, w.small[0], w.med[0], w.chunk[0], w.acc, w.st, hub_deg,
-                                    P.short_max, 1u);
+                                    w.nw[1], P.nw_bytes, w.small[0], w.med[0], w.chunk[0], w.acc, &w.ctl->init,
+                                    hub_deg, P.short_max, 1u, nullptr, w.ebits, g->m);
         CUF(cudaGetLastError());
     }
     if (resume) {
@@ -4155,7 +4279,7 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
     // ---- LCC to fixpoint (Alg. 4)
     P.searches_ahead = opt.lcc_only ? 0 : (int)t.order.size();
     int64_t rounds = 0;
-    RCF(P.lcc(&rounds, true));
+    RCF(P.lcc(&rounds, true, P.searches_ahead > 0));
     r->phase_rounds.push_back((int32_t)rounds);
     int64_t total_rounds = rounds;
     CUF(cudaEventRecord(w.ev[1], s));
@@ -4174,7 +4298,6 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
     if (opt.order_mode == CCPM_ORDER_LEARNED && !opt.mlp)
         return fail(set_err(ctx, CCPM_EINVAL, "CCPM_ORDER_LEARNED needs options.mlp"));
     r->logs.clear();
-    if (n_constraints > 0) RCF(P.omega_hist());
     for (int step = 0; step < n_constraints; step++) {
         // features of every remaining constraint in the current state
         std::vector<float> feats(remaining.size() * CCPM_MLP_IN);
@@ -4235,86 +4358,73 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
         for (int h = 0; h < kMaxT; h++)
             if ((c.hmask >> h) & 1u) build_plan(t, c.vmask, sadj, h, g->label_freq, false, w.plans_h[h], -1, w.hist_h);
         CUF(cudaMemcpyAsync(w.plans, w.plans_h, sizeof(DevPlan) * kMaxT, cudaMemcpyHostToDevice, s));
-        CUF(cudaMemsetAsync(w.st, 0, sizeof(RoundStats), s));
+        // not a no-op: some live vertex is a root, so rows to search are needed
+        if (P.want_compact() || P.cheaper_than_label_rows()) RCF(P.compact());
+        if (P.gen < 0) RCF(ensure_label_rows(ctx, g));
+        RCF(clear_search(ctx, w));
         P.launches++;
         k_collect_roots<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, w.om[P.cur], c.hmask, w.roots, w.st);
         CUF(cudaGetLastError());
-        RCF(P.read_stats());
-        const int64_t n_roots = w.st_h->n_roots;
-        if (n_roots > 0) {
-            if (P.want_compact() || P.cheaper_than_label_rows()) RCF(P.compact());
-            if (P.gen < 0) RCF(ensure_label_rows(ctx, g));
-            CUF(cudaMemsetAsync(w.next_root, 0, sizeof(unsigned long long), s));
-            SearchArgs a{};
-            a.rp = g->rp;
-            a.col = g->col;
-            a.rl = P.gen >= 0 ? P.lrp : g->rp;
-            a.lcol = P.gen >= 0 ? P.lcol : g->lcol;
-            a.nlab = P.gen >= 0 ? P.lnlab : g->nlab;
-            P.directory(a);
-            a.om = w.om[P.cur];
-            a.roots = w.roots;
-            a.n_roots = n_roots;
-            a.next_root = w.next_root;
-            a.plans = w.plans;
-            a.heads = c.hmask;
-            a.sat = w.sat;
-            a.st = w.st;
-            a.budget = budget;
-            a.items = w.items;
-            a.items_cap = w.items_cap;
-            a.enum_heads = 0;
-            // one item per (root, head, candidate for position 1)
+        SearchArgs a{};
+        a.rp = g->rp;
+        a.col = g->col;
+        a.rl = P.gen >= 0 ? P.lrp : g->rp;
+        a.lcol = P.gen >= 0 ? P.lcol : g->lcol;
+        a.nlab = P.gen >= 0 ? P.lnlab : g->nlab;
+        P.directory(a);
+        a.om = w.om[P.cur];
+        a.roots = w.roots;
+        a.n_roots = -1;
+        a.plans = w.plans;
+        a.heads = c.hmask;
+        a.sat = w.sat;
+        a.st = w.st;
+        a.budget = budget;
+        a.items = w.items;
+        a.items_cap = w.items_cap;
+        a.enum_heads = 0;
+        const SearchMode mode{0, split, starve};
+        P.search_launches++;
+        // one item per (root, head, candidate for position 1); the search, the
+        // elimination of the issuers that failed and the LCC rounds after it are
+        // queued together, and one host round trip reads what became of them
+        CUF(cudaEventRecord(w.ev[10], s));
+        RCF(queue_search(ctx, w, a, mode, __builtin_popcount(c.vmask), P.launches));
+        CUF(cudaEventRecord(w.ev[11], s));
+        auto apply = [&](const PassCtl *last) {
             P.launches++;
-            k_expand<<<grid_for(ctx, n_roots * 32, 256, 8), 256, 0, s>>>(a);
-            CUF(cudaGetLastError());
-            RCF(P.read_stats());
-            a.n_items = w.st_h->n_items;
-            if (!starve && a.n_items <= w.items_cap) RCF(expand_more(ctx, w, a, __builtin_popcount(c.vmask), P.launches));
-            CUF(cudaMemsetAsync(w.next_root, 0, sizeof(unsigned long long), s));
-            P.search_launches++;
-            CUF(cudaMemcpyAsync(w.aux_h, &w.st->windows, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-            CUF(cudaEventRecord(w.ev[10], s));
-            if (a.n_items <= w.items_cap) {
-                RCF(item_passes(ctx, w, a, 0, split, starve, P.launches, P.item_passes));
-            } else {
-                P.launches++;
-                k_nlcc_search<<<grid_for(ctx, n_roots * 32, 128, 16), 128, 0, s>>>(a);
-            }
-            CUF(cudaGetLastError());
-            CUF(cudaEventRecord(w.ev[11], s));
-            P.launches++;
-            k_nlcc_apply<<<grid_for(ctx, n_roots, 256, 8), 256, 0, s>>>(
-                w.roots, n_roots, c.hmask, w.sat, w.om[P.cur], w.om[0], w.om[1], w.nw[0], w.nw[1], P.nw_bytes, P.lrp,
-                w.deg, w.chg, w.chg_piece, hub_deg, w.st);
-            CUF(cudaGetLastError());
-            RCF(P.read_stats());
-            P.after_check();
-            if (w.st_h->overflow) over = true;
-            P.windows += (int64_t)w.st_h->windows;
-            P.nlcc_entries += (int64_t)(w.st_h->windows - w.aux_h[0]);
-            tokens += (int64_t)w.st_h->tokens;
-            float ms_k = 0.f;
-            CUF(cudaEventElapsedTime(&ms_k, w.ev[10], w.ev[11]));
-            P.ms_search_kernel += ms_k;
-        }
-        bool changed = n_roots > 0 && w.st_h->changed;
-        P.searches_ahead = (int)remaining.size();
+            k_nlcc_apply<<<grid_for(ctx, g->n, 256, 4), 256, 0, s>>>(
+                w.roots, last, w.items_cap, c.hmask, w.sat, w.om[P.cur], w.om[0], w.om[1], w.nw[0], w.nw[1], P.nw_bytes,
+                P.lrp, w.deg, w.chg, w.chg_piece, hub_deg, w.st);
+            return cudaGetLastError();
+        };
+        CUF(apply(w.ctl->pass + kChain - 1));
         CUF(cudaEventRecord(w.ev[7], s));
+        P.searches_ahead = (int)remaining.size();
         int64_t rr = 0;
-        if (changed) {
-            RCF(P.lcc(&rr, false));
+        RCF(P.lcc(&rr, false, true));
+        if (!search_complete(w, mode)) {
+            // more passes than were queued: the elimination has not run yet
+            RCF(finish_search(ctx, w, a, mode, P.launches));
+            CUF(cudaEventRecord(w.ev[11], s));
+            CUF(apply(nullptr));
+            CUF(cudaEventRecord(w.ev[7], s));
+            RCF(P.lcc(&rr, false, true));
         }
-        CUF(cudaEventRecord(w.ev[8], s));
+        if (w.st_h->overflow) over = true;
+        P.windows += (int64_t)(w.st_h->windows + w.st_h->expanded);
+        P.nlcc_entries += (int64_t)w.st_h->windows;
+        tokens += (int64_t)w.st_h->tokens;
+        float ms_k = 0.f;
+        CUF(cudaEventElapsedTime(&ms_k, w.ev[10], w.ev[11]));
+        P.ms_search_kernel += ms_k;
         r->phase_rounds.push_back((int32_t)rr);
         total_rounds += rr;
-        if (changed) RCF(P.omega_hist());      // state for the next decision
-        else CUF(ctx_sync(ctx));
         float ms_a = 0.f, ms_b = 0.f;
         cudaEventElapsedTime(&ms_a, w.ev[6], w.ev[7]);
-        cudaEventElapsedTime(&ms_b, w.ev[7], w.ev[8]);
+        cudaEventElapsedTime(&ms_b, w.ev[7], w.ev[5]);
         lg.ms_search = ms_a;
-        lg.ms_lcc = ms_b;
+        lg.ms_lcc = rr ? ms_b : 0.0;
         lg.lcc_rounds = (int32_t)rr;
         lg.tokens = (int32_t)std::min<int64_t>(tokens - tokens_before, INT32_MAX);
         lg.bits_after = (int64_t)w.hist_h[kMaxT];
@@ -4329,6 +4439,16 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
     uint64_t matches = 0;
     bool final_done = false;
     float ms_fc = 0.f, ms_fv = 0.f, ms_fe = 0.f;
+    bool summary_done = false, existence = false;
+    // the end of the result's making, then its active vertices and entries
+    auto queue_summary = [&]() -> int {
+        CU(ctx, cudaEventRecord(w.ev[3], s));
+        CU(ctx, cudaMemsetAsync(w.cnt, 0, 2 * sizeof(unsigned long long), s));
+        P.launches++;
+        k_count<<<grid_for(ctx, std::max<int64_t>(g->n, w.words), 256, 8), 256, 0, s>>>(g->n, r->om, w.words, r->eb, w.cnt);
+        CU(ctx, cudaGetLastError());
+        return CCPM_OK;
+    };
     cudaEvent_t fev[4] = {w.ev[6], w.ev[7], w.ev[8], w.ev[9]};
     if (opt.run_final) {
         const uint32_t all = t.n0 == 32 ? 0xFFFFFFFFu : ((1u << t.n0) - 1u);
@@ -4344,7 +4464,6 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
         a.nlab = P.gen >= 0 ? P.lnlab : g->nlab;
         P.directory(a);
         a.roots = w.roots;
-        a.next_root = w.next_root;
         a.plans = w.plans;
         a.sat = w.sat;
         a.eb_out = r->eb;
@@ -4352,10 +4471,6 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
         a.budget = budget;
         a.items = w.items;
         a.items_cap = w.items_cap;
-        auto run_items = [&](bool edge_pass) -> int {
-            int rc2 = item_passes(ctx, w, a, edge_pass ? 4 : 0, split, starve, P.launches, P.item_passes);
-            return rc2 ? rc2 : P.read_stats();
-        };
         // the final enumeration keeps the background label frequencies (measured
         // faster than ordering by live candidates there)
         const unsigned long long *live = nullptr;
@@ -4369,44 +4484,28 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
         auto count_pass = [&](int mode, const uint32_t *om_src, uint64_t cap, uint64_t &found, bool &capped) -> int {
             build_plan(t, all, t.adj, root, g->label_freq, true, w.plans_h[0], -1, live);
             CU(ctx, cudaMemcpyAsync(w.plans, w.plans_h, sizeof(DevPlan), cudaMemcpyHostToDevice, s));
-            CU(ctx, cudaMemsetAsync(w.st, 0, sizeof(RoundStats), s));
+            int rc2 = clear_search(ctx, w);
+            if (rc2) return rc2;
             P.launches++;
             k_collect_roots<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, om_src, 1u << root, w.roots, w.st);
             CU(ctx, cudaGetLastError());
-            int rc2 = P.read_stats();
-            if (rc2) return rc2;
-            const int64_t nr = w.st_h->n_roots;
-            found = 0;
-            capped = false;
-            if (nr == 0) return CCPM_OK;
             a.om = om_src;
-            a.n_roots = nr;
+            a.n_roots = -1;
             a.heads = 1u << root;
             a.cap = cap;
             a.enum_heads = 1;
             a.om_out = r->om;
             a.eb_out = r->eb;
-            P.launches++;
-            k_expand<<<grid_for(ctx, nr * 32, 256, 8), 256, 0, s>>>(a);
-            CU(ctx, cudaGetLastError());
-            if ((rc2 = P.read_stats())) return rc2;
-            a.n_items = w.st_h->n_items;
-            if (!starve && a.n_items <= w.items_cap && (rc2 = expand_more(ctx, w, a, t.n0, P.launches))) return rc2;
-            CU(ctx, cudaMemsetAsync(w.next_root, 0, sizeof(unsigned long long), s));
-            const bool use_items = a.n_items <= w.items_cap;
-            const int gr = grid_for(ctx, nr * 32, 128, 16);
-            if (use_items) {
-                if ((rc2 = item_passes(ctx, w, a, mode == kMark ? 2 : 1, split, starve, P.launches, P.item_passes))) return rc2;
-            } else if (mode == kMark) {
-                P.launches++;
-                k_final_search<kMark><<<gr, 128, 0, s>>>(a);
-            } else {
-                P.launches++;
-                k_final_search<kCount><<<gr, 128, 0, s>>>(a);
-            }
-            CU(ctx, cudaGetLastError());
-            if ((rc2 = P.read_stats())) return rc2;
-            P.windows += (int64_t)w.st_h->windows;
+            const SearchMode sm{mode == kMark ? 2 : 1, split, starve};
+            if ((rc2 = queue_search(ctx, w, a, sm, t.n0, P.launches))) return rc2;
+            CU(ctx, cudaEventRecord(fev[1], s));
+            // most often the enumeration is over by then and marked everything:
+            // the summary needs no round trip of its own
+            if (mode == kMark && (rc2 = queue_summary())) return rc2;
+            if ((rc2 = read_control(ctx, w))) return rc2;
+            summary_done = mode == kMark && search_complete(w, sm) && w.st_h->n_items <= w.items_cap && !w.st_h->overflow;
+            if (!search_complete(w, sm) && (rc2 = finish_search(ctx, w, a, sm, P.launches))) return rc2;
+            P.windows += (int64_t)(w.st_h->windows + w.st_h->expanded);
             found = w.st_h->matches;
             capped = w.st_h->overflow != 0;
             return CCPM_OK;
@@ -4436,7 +4535,7 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
         } else {
             count_valid = false;
         }
-        CUF(cudaEventRecord(fev[1], s));
+        if (!final_done || !summary_done) CUF(cudaEventRecord(fev[1], s));
         if (!final_done) {
             // the capped enumeration's marks stay: every one belongs to a match
             // found, so the existence searches below skip those (vertex,
@@ -4451,53 +4550,33 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
             // their edges.
             for (int q = 0; q < t.n0; q++) build_plan(t, all, t.adj, q, g->label_freq, true, w.plans_h[q], -1, live);
             CUF(cudaMemcpyAsync(w.plans, w.plans_h, sizeof(DevPlan) * (size_t)t.n0, cudaMemcpyHostToDevice, s));
-            CUF(cudaMemsetAsync(w.st, 0, sizeof(RoundStats), s));
+            RCF(clear_search(ctx, w));
             P.launches++;
             k_collect_roots<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, w.om[P.cur], all, w.roots, w.st);
             CUF(cudaGetLastError());
-            RCF(P.read_stats());
-            int64_t n_roots = w.st_h->n_roots;
-            if (n_roots > 0) {
-                a.om = w.om[P.cur];
-                a.n_roots = n_roots;
-                a.heads = all;
-                a.enum_heads = 0;
-                P.launches++;
-                k_expand<<<grid_for(ctx, n_roots * 32, 256, 8), 256, 0, s>>>(a);
-                CUF(cudaGetLastError());
-                RCF(P.read_stats());
-                a.n_items = w.st_h->n_items;
-                if (!starve && a.n_items <= w.items_cap) RCF(expand_more(ctx, w, a, t.n0, P.launches));
-                if (a.n_items <= w.items_cap) {
-                    RCF(run_items(false));
-                } else {
-                    CUF(cudaMemsetAsync(w.next_root, 0, sizeof(unsigned long long), s));
-                    P.launches++;
-                    k_nlcc_search<<<grid_for(ctx, n_roots * 32, 128, 16), 128, 0, s>>>(a);
-                    CUF(cudaGetLastError());
-                    RCF(P.read_stats());
-                }
-                if (w.st_h->overflow) over = true;
-                P.windows += (int64_t)w.st_h->windows;
-                P.launches++;
-                k_sat_to_omega<<<grid_for(ctx, n_roots, 256, 8), 256, 0, s>>>(w.roots, n_roots, w.sat, w.om[P.cur], r->om);
-                CUF(cudaGetLastError());
-            }
+            a.om = w.om[P.cur];
+            a.n_roots = -1;
+            a.heads = all;
+            a.enum_heads = 0;
+            const SearchMode vm{0, split, starve};
+            RCF(queue_search(ctx, w, a, vm, t.n0, P.launches));
+            RCF(read_control(ctx, w));
+            if (!search_complete(w, vm)) RCF(finish_search(ctx, w, a, vm, P.launches));
+            if (w.st_h->overflow) over = true;
+            P.windows += (int64_t)(w.st_h->windows + w.st_h->expanded);
+            P.launches++;
+            k_sat_to_omega<<<grid_for(ctx, w.st_h->n_roots, 256, 8), 256, 0, s>>>(w.roots, w.st, w.sat, w.om[P.cur], r->om);
+            CUF(cudaGetLastError());
             a.sat_seed = nullptr;
             CUF(cudaEventRecord(fev[2], s));
             // (B) every entry between omega* vertices that no embedding has marked
             // yet: some match maps a template edge onto it?
             std::vector<std::pair<int, int>> oriented;
             for (auto &e : t.edges) { oriented.push_back(e); oriented.push_back({e.second, e.first}); }
-            if (n_roots > 0) {
-                CUF(cudaMemsetAsync(w.st, 0, sizeof(RoundStats), s));
-                P.launches++;
-                k_collect_roots<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, r->om, all, w.roots, w.st);
-                CUF(cudaGetLastError());
-                RCF(P.read_stats());
-                n_roots = w.st_h->n_roots;
-            }
-            for (size_t o0 = 0; n_roots > 0 && o0 < oriented.size(); o0 += 32) {
+            // (the roots are collected with the first edges; -1: the host does not
+            // know their number yet)
+            int64_t n_roots = -1;
+            for (size_t o0 = 0; n_roots != 0 && o0 < oriented.size(); o0 += 32) {
                 EdgeTab tab;
                 std::memset(&tab, 0, sizeof(tab));
                 tab.n = (int)std::min<size_t>(32, oriented.size() - o0);
@@ -4511,41 +4590,42 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
                 // the candidate entries of a range of roots become items; a range
                 // whose items do not fit is halved and made again (the bits marked
                 // so far stay: every one of them is a found match's edge)
-                int64_t span = n_roots;
-                for (int64_t r0 = 0; r0 < n_roots;) {
-                    const int64_t r1 = std::min(n_roots, r0 + span);
-                    CUF(cudaMemsetAsync(w.st, 0, sizeof(RoundStats), s));
+                const SearchMode em{4, split, starve};
+                int64_t span = n_roots, r0 = 0;
+                while (n_roots < 0 || r0 < n_roots) {
+                    const int64_t r1 = n_roots < 0 ? -1 : std::min(n_roots, r0 + span);
+                    RCF(clear_search(ctx, w));
                     a.roots = w.roots + r0;
-                    a.n_roots = r1 - r0;
+                    a.n_roots = n_roots < 0 ? -1 : r1 - r0;
+                    if (n_roots < 0) {
+                        P.launches++;
+                        k_collect_roots<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, r->om, all, w.roots, w.st);
+                        CUF(cudaGetLastError());
+                    }
                     P.launches++;
-                    k_edge_items<<<grid_for(ctx, a.n_roots * 256, 256, 8), 256, 0, s>>>(a, tab);
+                    k_edge_items<<<grid_sms(ctx) * 8, 256, 0, s>>>(a, tab);
                     CUF(cudaGetLastError());
-                    RCF(P.read_stats());
-                    a.n_items = w.st_h->n_items;
-                    if (a.n_items > w.items_cap) {
-                        if (r1 - r0 == 1)
+                    a.n_items = -1;
+                    RCF(queue_passes(ctx, w, a, em, P.launches));
+                    RCF(read_control(ctx, w));
+                    if (n_roots < 0) span = n_roots = w.st_h->n_roots;
+                    const int64_t done_to = r1 < 0 ? n_roots : r1;
+                    if (w.st_h->n_items > w.items_cap) {
+                        if (done_to - r0 == 1)
                             return fail(set_err(ctx, CCPM_EOVERFLOW, "edge pass: one vertex has too many candidate edges"));
-                        span = std::max<int64_t>(1, (r1 - r0) / 2);
+                        span = std::max<int64_t>(1, (done_to - r0) / 2);
                         continue;
                     }
-                    if (a.n_items > 0) {
-                        RCF(run_items(true));
-                        if (w.st_h->overflow) over = true;
-                        P.windows += (int64_t)w.st_h->windows;
-                    }
-                    r0 = r1;
+                    RCF(finish_search(ctx, w, a, em, P.launches));
+                    if (w.st_h->overflow) over = true;
+                    P.windows += (int64_t)w.st_h->windows;
+                    r0 = done_to;
                 }
                 a.roots = w.roots;
-                a.n_roots = n_roots;
             }
             CUF(cudaEventRecord(fev[3], s));
-            CUF(ctx_sync(ctx));
-            cudaEventElapsedTime(&ms_fv, fev[1], fev[2]);
-            cudaEventElapsedTime(&ms_fe, fev[2], fev[3]);
-        } else {
-            CUF(ctx_sync(ctx));
+            existence = true;
         }
-        cudaEventElapsedTime(&ms_fc, fev[0], fev[1]);
         final_done = true;
     }
     if (!final_done) {
@@ -4563,13 +4643,17 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
         CUF(cudaMemcpyAsync(r->om, w.om[P.cur], sizeof(uint32_t) * (size_t)g->n, cudaMemcpyDeviceToDevice, s));
         CUF(cudaMemcpyAsync(r->eb, w.ebits, sizeof(uint32_t) * (size_t)w.words, cudaMemcpyDeviceToDevice, s));
     }
-    CUF(cudaEventRecord(w.ev[3], s));
-    CUF(cudaMemsetAsync(w.cnt, 0, 2 * sizeof(unsigned long long), s));
-    P.launches++;
-    k_count<<<grid_for(ctx, std::max<int64_t>(g->n, w.words), 256, 8), 256, 0, s>>>(g->n, r->om, w.words, r->eb, w.cnt);
-    CUF(cudaGetLastError());
-    CUF(cudaMemcpyAsync(w.cnt_h, w.cnt, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-    CUF(ctx_sync(ctx));
+    if (!summary_done) {
+        RCF(queue_summary());
+        RCF(read_control(ctx, w));
+    }
+    if (opt.run_final) {
+        cudaEventElapsedTime(&ms_fc, fev[0], fev[1]);
+        if (existence) {
+            cudaEventElapsedTime(&ms_fv, fev[1], fev[2]);
+            cudaEventElapsedTime(&ms_fe, fev[2], fev[3]);
+        }
+    }
     float ms_lcc = 0, ms_nlcc = 0, ms_final = 0;
     cudaEventElapsedTime(&ms_lcc, w.ev[0], w.ev[1]);
     cudaEventElapsedTime(&ms_nlcc, w.ev[1], w.ev[2]);
@@ -5103,32 +5187,31 @@ int ccpm_result_matches(ccpm_ctx_t ctx, ccpm_result_t r, ccpm_tmpl_t tm, const c
     LabelMask lm;
     std::memset(&lm, 0, sizeof(lm));
     for (int q = 0; q < t.n0; q++) lm.m[t.labels[q]] |= 1u << q;
-    CUR(cudaMemsetAsync(w.st, 0, sizeof(RoundStats), s));
+    if ((rc = clear_search(ctx, w))) { release(); return rc; }
+    CUR(cudaMemsetAsync(&w.ctl->init, 0, sizeof(RoundStats), s));
     CUR(cudaMemsetAsync(w.ebits, 0, sizeof(uint32_t) * (size_t)(w.words + 1), s));
     k_init<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, g->rp, g->lab, lm, r->om, w.om[0], w.om[1], nullptr, nullptr,
-                                                       0, w.small[0], w.med[0], w.chunk[0], w.acc, w.st, hub_deg,
-                                                       P.short_max, 0u);
+                                                       0, w.small[0], w.med[0], w.chunk[0], w.acc, &w.ctl->init, hub_deg,
+                                                       P.short_max, 0u, nullptr, nullptr, 0);
     CUR(cudaGetLastError());
-    k_live_entries<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, g->rp, g->col, w.om[0], r->eb, w.ebits, w.deg,
-                                                                   w.st);
+    k_live_entries<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, g->rp, g->col, w.om[0], r->eb, w.ebits, w.deg, w.st);
     CUR(cudaGetLastError());
     k_collect_roots<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, w.om[0], 1u << root, w.roots, w.st);
     CUR(cudaGetLastError());
-    CUR(cudaMemcpyAsync(w.st_h, w.st, sizeof(RoundStats), cudaMemcpyDeviceToHost, s));
-    CUR(cudaStreamSynchronize(s));
+    if ((rc = read_control(ctx, w))) { release(); return rc; }
     const int64_t n_roots = w.st_h->n_roots, kept = (int64_t)w.st_h->kept;
-    if (w.st_h->n_hub_slots > (unsigned)w.acc_cap || w.st_h->n_chunk > w.chunk_cap) {
+    const RoundStats &lists = w.ctl_h->init;
+    if (lists.n_hub_slots > (unsigned)w.acc_cap || (int64_t)lists.n_chunk > w.chunk_cap) {
         release();
         return set_err(ctx, CCPM_EOVERFLOW, "hub bookkeeping overflow");
     }
     bool over = false;
     if (n_roots > 0 && kept > 0) {
-        P.n_small = w.st_h->n_small;
-        P.n_med = w.st_h->n_med;
-        P.n_chunk = w.st_h->n_chunk;
+        P.n_small = lists.n_small;
+        P.n_med = lists.n_med;
+        P.n_chunk = lists.n_chunk;
         P.last_kept = kept;
-        if ((rc = P.compact())) { release(); return rc; }
-        CUR(cudaMemsetAsync(w.st, 0, sizeof(RoundStats), s));
+        if ((rc = P.compact()) || (rc = clear_search(ctx, w))) { release(); return rc; }
         SearchArgs a{};
         a.rp = g->rp;
         a.col = g->col;
@@ -5139,7 +5222,6 @@ int ccpm_result_matches(ccpm_ctx_t ctx, ccpm_result_t r, ccpm_tmpl_t tm, const c
         a.om = w.om[0];
         a.roots = w.roots;
         a.n_roots = n_roots;
-        a.next_root = w.next_root;
         a.plans = w.plans;
         a.heads = 1u << root;
         a.sat = w.sat;
@@ -5155,27 +5237,17 @@ int ccpm_result_matches(ccpm_ctx_t ctx, ccpm_result_t r, ccpm_tmpl_t tm, const c
         a.list_count = w.cnt;
         a.vcnt = d_vc;
         a.ecnt = d_ec;
-        int64_t launches = 0, passes = 0;
-        k_expand<<<grid_for(ctx, n_roots * 32, 256, 8), 256, 0, s>>>(a);
-        CUR(cudaGetLastError());
-        CUR(cudaMemcpyAsync(w.st_h, w.st, sizeof(RoundStats), cudaMemcpyDeviceToHost, s));
-        CUR(cudaStreamSynchronize(s));
-        a.n_items = w.st_h->n_items;
-        if (!starve && a.n_items <= w.items_cap && (rc = expand_more(ctx, w, a, t.n0, launches))) { release(); return rc; }
-        CUR(cudaMemsetAsync(w.next_root, 0, sizeof(unsigned long long), s));
-        if (a.n_items <= w.items_cap) {
-            if ((rc = item_passes(ctx, w, a, 3, split, starve, launches, passes))) { release(); return rc; }
-        } else {
-            k_final_search<kList><<<grid_for(ctx, n_roots * 32, 128, 16), 128, 0, s>>>(a);
-            CUR(cudaGetLastError());
+        int64_t launches = 0;
+        const SearchMode mode{3, split, starve};
+        if ((rc = queue_search(ctx, w, a, mode, t.n0, launches)) || (rc = read_control(ctx, w)) ||
+            (!search_complete(w, mode) && (rc = finish_search(ctx, w, a, mode, launches)))) {
+            release();
+            return rc;
         }
-        CUR(cudaMemcpyAsync(w.st_h, w.st, sizeof(RoundStats), cudaMemcpyDeviceToHost, s));
-        CUR(cudaStreamSynchronize(s));
         over = w.st_h->overflow != 0;
     }
-    unsigned long long found = 0;
-    CUR(cudaMemcpyAsync(&found, w.cnt, sizeof(found), cudaMemcpyDeviceToHost, s));
-    CUR(cudaStreamSynchronize(s));
+    // the counters read last are the search's (or show that there was none)
+    const unsigned long long found = n_roots > 0 && kept > 0 ? w.cnt_h[0] : 0ull;
     if (!dst_on_device) {
         const uint64_t rows = std::min<uint64_t>((uint64_t)found, list_cap);
         if (rows) CUR(cudaMemcpyAsync(list, d_list, sizeof(int32_t) * (size_t)(rows * (uint64_t)t.n0), cudaMemcpyDeviceToHost, s));
@@ -5507,7 +5579,7 @@ int lcc_fixpoint_noalloc_body(int device, void *cuda_stream, int64_t n, int64_t 
         if (m_dir & 31) k_set_word<<<1, 1, 0, s>>>(ebits + words - 1, (1u << (uint32_t)(m_dir & 31)) - 1u);
     }
     k_init<<<grid(n, 256), 256, 0, s>>>(n, row_ptr, labels, lm, nullptr, om[0], om[1], nullptr, nullptr, 0, small[0],
-                                        med[0], chunk[0], acc, st, hub, kSmallDeg, 0u);
+                                        med[0], chunk[0], acc, st, hub, kSmallDeg, 0u, nullptr, nullptr, 0);
     NA_CU(cudaGetLastError());
     NA_CU(read_stats());
     if (hs.n_hub_slots > (unsigned)L.acc_cap || (int64_t)hs.n_chunk > L.chunk_cap)
@@ -5544,6 +5616,7 @@ int lcc_fixpoint_noalloc_body(int device, void *cuda_stream, int64_t n, int64_t 
         a.elab = nullptr;
         a.sparse = 0;
         a.prev = nullptr;
+        a.gate = nullptr;
         a.resident_warps = num_sms * 32;
         a.eta_off = 0u;
         a.nw_bytes = 0;
