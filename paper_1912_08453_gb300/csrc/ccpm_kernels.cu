@@ -661,6 +661,40 @@ struct LccTally {
     uint32_t changed = 0, died = 0;
 };
 
+// The round counters of a block's warps, one atomic per counter and block:
+// with a warp each, the thousands of atomics on one address lasted longer than
+// the round itself on small frontiers.  totals: 9 zeroed words of shared memory.
+__device__ __forceinline__ void add_totals(const LccTally &tl, unsigned long long *totals, RoundStats *st) {
+    auto add = [&](int i, unsigned long long x) {
+        x = warp_total(x);
+        if (lane_id() == 0 && x) atomicAdd(&totals[i], x);
+    };
+    add(0, tl.scanned);
+    add(1, tl.rows);
+    add(2, tl.alive);
+    add(3, tl.kept);
+    add(4, tl.rows_next);
+    add(5, tl.changed);
+    add(6, tl.died);
+    add(7, tl.old_kept);
+    add(8, tl.died_rows);
+    __syncthreads();
+    const unsigned long long sum = threadIdx.x < 9 ? totals[threadIdx.x] : 0ull;
+    if (sum) {
+        switch (threadIdx.x) {
+            case 0: atomicAdd(&st->scanned, sum); break;
+            case 1: atomicAdd(&st->row_entries, sum); break;
+            case 2: atomicAdd(&st->alive, sum); break;
+            case 3: atomicAdd(&st->kept, sum); break;
+            case 4: atomicAdd(&st->rows_next, sum); break;
+            case 5: atomicOr(&st->changed, 1u); break;
+            case 6: atomicAdd(&st->died, (unsigned int)sum); break;
+            case 7: atomicAdd(&st->old_kept, sum); break;
+            default: atomicAdd(&st->died_rows, sum); break;
+        }
+    }
+}
+
 // What a round decided for vertex v (one lane): its omega was wv and is now
 // `keep`, `kept` of the `len` entries of its row stay active.  A full round
 // writes omega'; a delta round lists the change (long: the row is longer than
@@ -1056,9 +1090,7 @@ k_lcc_round(LccArgs a, DevTmpl t) {
     // (3) short rows: 32 vertices per warp batch, entries streamed flat
     short_rows<MAXC, MODE>(a, s, slm, cm, srows[wib], gwarp, nwarps, n_small, bs, bg, tl);
 
-    // what is left in the warps' buffers and their totals go out once per block:
-    // with a warp each, the thousands of atomics on one address lasted longer
-    // than the round itself on small frontiers
+    // what is left in the warps' buffers goes out once per block
     __syncthreads();
     if (MODE == kDelta) {
         block_flush(bg, &scnt[3][0], wib);
@@ -1067,36 +1099,412 @@ k_lcc_round(LccArgs a, DevTmpl t) {
         block_flush(bm, &scnt[1][0], wib);
         block_flush(bc, &scnt[2][0], wib);
     }
-    auto add = [&](int i, unsigned long long x) {
-        x = warp_total(x);
-        if (lane == 0 && x) atomicAdd(&totals[i], x);
-    };
-    add(0, tl.scanned);
-    add(1, tl.rows);
-    add(2, tl.alive);
-    add(3, tl.kept);
-    add(4, tl.rows_next);
-    add(5, tl.changed);
-    add(6, tl.died);
-    if (MODE == kDelta) {
-        add(7, tl.old_kept);
-        add(8, tl.died_rows);
+    add_totals(tl, totals, a.st);
+}
+
+// -------------------------------------------------------------------------
+// The first round of a fresh prune (Alg. 3 and the first pass of Alg. 4 in one
+// kernel).  omega_0 is the mask of a vertex's label, so the round needs labels
+// only: the vertices are taken in id order (no frontier list is written and
+// read back), and omega is written once, as the round leaves it, in both
+// buffers.  Only the survivors are listed for the next round.
+//
+// It was bound by instructions: one entry per lane and step, with the row
+// located and reduced every 32 entries, took 5 warp instructions per entry.  A
+// lane now takes four consecutive entries per step (their labels are one
+// 32-bit load), looks each label up in a table of (omega, packed class counts)
+// and votes with a nibble of the bitmap word, and rows are walked by as many
+// lanes as they fill: rows of at most 16 entries by their own lane, up to 64 by
+// 8 lanes (four rows side by side), longer ones by the warp (128 entries per
+// step), those past max(hub_deg, 1024) in pieces by k_first_hubs.  32M vertices,
+// 10^9 entries, 20M vertices initially active: initialisation and first round
+// 5.0 -> 3.0 ms, and the second round, whose lists now hold survivors only, 3.5
+// -> 3.1 ms.
+// -------------------------------------------------------------------------
+
+struct FirstArgs {
+    int64_t n, m;
+    const int64_t *rp;
+    const int32_t *col;
+    const uint8_t *lab;
+    const uint8_t *elab;          // neighbours' labels in entry order (ELAB), readable up to m + 3
+    uint32_t *om0, *om1;
+    void *nw0, *nw1;
+    int nw_bytes;
+    uint32_t *ebits;              // all ones
+    uint32_t *deg;
+    int32_t *small_out, *med_out; // survivors, for the next round
+    ChunkItem *chunk_out;
+    ChunkItem *hub_list;          // pieces of the rows left to k_first_hubs, sizes in `hubs`
+    RoundStats *hubs;
+    HubAcc *acc;
+    RoundStats *st;
+    int hub_deg, short_max;
+    uint32_t eta_off;
+    int col_vec;                  // col is 16-byte aligned
+    LabelMask lm;
+};
+
+constexpr int kFirstLane = 16, kFirstGroup = 64, kFirstWarp = 1024;   // row lengths of the three paths
+
+struct FirstAcc { uint32_t U = 0, cp = 0, nN = 0; };   // union, class counts (four bytes), kept entries
+
+// Table of the first round: label -> omega_0 and, per multiplicity class, 1 in
+// the class's byte if omega_0 meets it.
+__device__ __forceinline__ void first_table(uint2 *lut, const SmemTmpl &s, const LabelMask &lm) {
+    for (int L = threadIdx.x; L < 256; L += blockDim.x) {
+        const uint32_t w = lm.m[L];
+        uint32_t pack = 0;
+        for (int c = 0; c < 4 && c < s.n_cls; c++) pack |= (w & s.cls_mask[c]) ? 1u << (8 * c) : 0u;
+        lut[L] = make_uint2(w, pack);
     }
-    __syncthreads();
-    const unsigned long long sum = threadIdx.x < 9 ? totals[threadIdx.x] : 0ull;
-    if (sum) {
-        switch (threadIdx.x) {
-            case 0: atomicAdd(&a.st->scanned, sum); break;
-            case 1: atomicAdd(&a.st->row_entries, sum); break;
-            case 2: atomicAdd(&a.st->alive, sum); break;
-            case 3: atomicAdd(&a.st->kept, sum); break;
-            case 4: atomicAdd(&a.st->rows_next, sum); break;
-            case 5: atomicOr(&a.st->changed, 1u); break;
-            case 6: atomicAdd(&a.st->died, (unsigned int)sum); break;
-            case 7: atomicAdd(&a.st->old_kept, sum); break;
-            default: atomicAdd(&a.st->died_rows, sum); break;
+}
+
+// Labels of the neighbours at entries e..e+3 (e a multiple of 4), one per byte;
+// those outside [beg, end) are any value.
+template <bool ELAB>
+__device__ __forceinline__ uint32_t labels4(const FirstArgs &a, int64_t e, int64_t beg, int64_t end) {
+    if (ELAB) return __ldcs((const unsigned int *)(a.elab + e));
+    int32_t u[4];
+    if (a.col_vec && e + 4 <= a.m) {
+        const int4 c = __ldcs((const int4 *)(a.col + e));
+        u[0] = c.x; u[1] = c.y; u[2] = c.z; u[3] = c.w;
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; j++) u[j] = e + j >= beg && e + j < end ? __ldcs(a.col + e + j) : 0;
+    }
+    uint32_t labs = 0;
+#pragma unroll
+    for (int j = 0; j < 4; j++)
+        if (e + j >= beg && e + j < end) labs |= (uint32_t)__ldg(a.lab + u[j]) << (8 * j);
+    return labs;
+}
+
+// Bits j of a nibble with e + j in [beg, end).
+__device__ __forceinline__ uint32_t range4(int64_t e, int64_t beg, int64_t end) {
+    const int lo = (int)min((int64_t)4, max((int64_t)0, beg - e)), hi = (int)min((int64_t)4, max((int64_t)0, end - e));
+    return ((1u << hi) - 1u) & ~((1u << lo) - 1u);
+}
+
+// Four entries: the kept ones as a nibble.
+template <int MAXC>
+__device__ __forceinline__ uint32_t take4(uint32_t labs, uint32_t in, uint32_t nbr, const uint2 *lut, FirstAcc &A,
+                                          LccTally &tl) {
+    uint32_t keep = 0, live = 0;
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        const uint2 q = lut[(labs >> (8 * j)) & 255u];
+        const uint32_t w = (in >> j) & 1u ? q.x : 0u;
+        live += w != 0u;
+        if (w & nbr) {
+            A.U |= w;
+            if (MAXC > 0) A.cp += q.y;
+            keep |= 1u << j;
         }
     }
+    const uint32_t k = __popc(keep);
+    A.nN += k;
+    tl.scanned += live;
+    if (k != live) tl.changed = 1u;          // eta eliminates a live entry
+    return keep;
+}
+
+// Store the kept bits of one bitmap word of the row [beg, end).
+__device__ __forceinline__ void store_word(uint32_t *ebits, int64_t wi, int64_t beg, int64_t end, uint32_t kept) {
+    const int64_t e0 = wi << 5;
+    if (e0 >= end || e0 + 32 <= beg) return;
+    if (e0 >= beg && e0 + 32 <= end) { ebits[wi] = kept; return; }
+    uint32_t in = ~0u;                       // shared with a neighbouring row
+    if (e0 < beg) in &= ~0u << (uint32_t)(beg - e0);
+    if (end - e0 < 32) in &= (1u << (uint32_t)(end - e0)) - 1u;
+    if (in & ~kept) atomicAnd(&ebits[wi], ~(in & ~kept));
+}
+
+// The whole warp walks [beg, end); every lane gets the sums.
+template <int MAXC, bool ELAB>
+__device__ __forceinline__ void first_warp(const FirstArgs &a, int64_t beg, int64_t end, uint32_t nbr, const uint2 *lut,
+                                           Partial<MAXC> &p, LccTally &tl) {
+    const int lane = (int)lane_id();
+    const int64_t w0 = beg >> 7;
+    const int nwin = (int)(((end + 127) >> 7) - w0);
+    FirstAcc A;
+    int64_t e = (w0 << 7) + 4 * lane;
+    auto load = [&](int64_t x) { return x < end && x + 4 > beg ? labels4<ELAB>(a, x, beg, end) : 0u; };
+    uint32_t next = load(e);
+    for (int k = 0; k < nwin; k++, e += 128) {
+        const uint32_t labs = next;
+        if (k + 1 < nwin) next = load(e + 128);
+        const uint32_t nib = take4<MAXC>(labs, range4(e, beg, end), nbr, lut, A, tl);
+        uint32_t word = nib << (4 * (lane & 7));
+        word |= __shfl_xor_sync(FULL_MASK, word, 1);
+        word |= __shfl_xor_sync(FULL_MASK, word, 2);
+        word |= __shfl_xor_sync(FULL_MASK, word, 4);
+        if ((lane & 7) == 0) store_word(a.ebits, e >> 5, beg, end, word);
+        if (MAXC > 0 && (k & 31) == 31) {    // before a byte can overflow
+#pragma unroll
+            for (int c = 0; c < MAXC; c++) p.cnt[c] += (A.cp >> (8 * c)) & 255u;
+            A.cp = 0;
+        }
+    }
+    p.U = __reduce_or_sync(FULL_MASK, A.U);
+    p.nN = __reduce_add_sync(FULL_MASK, A.nN);
+#pragma unroll
+    for (int c = 0; c < MAXC; c++) p.cnt[c] = __reduce_add_sync(FULL_MASK, p.cnt[c] + ((A.cp >> (8 * c)) & 255u));
+}
+
+// List a surviving vertex for the next round (all lanes call; `want` lanes list).
+__device__ __forceinline__ void list_survivor(const FirstArgs &a, bool want, int32_t v, int64_t len,
+                                              WarpBuf<int32_t> &bs, WarpBuf<int32_t> &bm) {
+    const int64_t small_max = a.hub_deg < a.short_max ? a.hub_deg : a.short_max;
+    bs.push(want && len <= small_max, v);
+    bm.push(want && len > small_max && len <= a.hub_deg, v);
+    if (want && len > a.hub_deg) {
+        const int nch = (int)((len + a.hub_deg - 1) / a.hub_deg);
+        const int slot = (int)atomicAdd(&a.st->n_hub_slots, 1u);
+        const unsigned int base = atomicAdd(&a.st->n_chunk, (unsigned int)nch);
+        for (int c = 0; c < nch; c++) a.chunk_out[base + c] = ChunkItem{v, c, slot, nch};
+    }
+}
+
+template <int MAXC>
+__device__ __forceinline__ void unpack_classes(uint32_t cp, Partial<MAXC> &p) {
+#pragma unroll
+    for (int c = 0; c < MAXC; c++) p.cnt[c] = (cp >> (8 * c)) & 255u;
+}
+
+template <int MAXC, bool ELAB>
+__global__ void __launch_bounds__(256, 4)
+k_first_round(FirstArgs a, DevTmpl t) {
+    __shared__ SmemTmpl s;
+    __shared__ uint2 lut[256];
+    __shared__ int32_t sbuf[2][8][32];
+    __shared__ int scnt[2][8];
+    __shared__ unsigned long long totals[9];
+    if (threadIdx.x < 9) totals[threadIdx.x] = 0ull;
+    load_tmpl(s, t);
+    const int wib = threadIdx.x >> 5;
+    const int lane = (int)lane_id();
+    if (lane == 0) { scnt[0][wib] = 0; scnt[1][wib] = 0; }
+    __syncthreads();
+    first_table(lut, s, a.lm);
+    __syncthreads();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        // no entries past m: the padding bits of the last word and the guard word stay 0
+        if (a.m & 31) atomicAnd(&a.ebits[a.m >> 5], (1u << (uint32_t)(a.m & 31)) - 1u);
+        a.ebits[(a.m + 31) >> 5] = 0u;
+    }
+    WarpBuf<int32_t> bs{sbuf[0][wib], &scnt[0][wib], a.small_out, &a.st->n_small};
+    WarpBuf<int32_t> bm{sbuf[1][wib], &scnt[1][wib], a.med_out, &a.st->n_med};
+    const int64_t gwarp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    // small graphs: fewer than 32 vertices per warp, so that every warp has some
+    const int per = (int)max((int64_t)1, min((int64_t)32, a.n / nwarps));
+    const int64_t in_warp = max((int64_t)kFirstWarp, (int64_t)a.hub_deg);
+    LccTally tl;
+    for (int64_t v0 = gwarp * per; v0 < a.n; v0 += nwarps * per) {
+        const int64_t v = v0 + lane;
+        const bool mine = lane < per && v < a.n;
+        uint32_t wv = 0u, nbr = 0u, keep = 0u, kept = 0u;
+        int64_t beg = 0, end = 0;
+        if (mine) wv = lut[a.lab[v]].x;
+        if (wv) {
+            beg = a.rp[v];
+            end = a.rp[v + 1];
+            nbr = nbr_mask(wv, s) | a.eta_off;
+        }
+        const int64_t len = end - beg;
+        const bool hub = len > in_warp;
+        // (1) short rows, one lane each
+        if (wv && len > 0 && len <= kFirstLane) {
+            FirstAcc A;
+            uint32_t kb = 0;                                 // kept entries, relative to beg
+            const int64_t e0 = beg & ~(int64_t)3;
+            if (ELAB) {
+                uint32_t labs[5];
+#pragma unroll
+                for (int i = 0; i < 5; i++) labs[i] = e0 + 4 * i < end ? labels4<true>(a, e0 + 4 * i, beg, end) : 0u;
+#pragma unroll
+                for (int i = 0; i < 5; i++) {
+                    const int64_t e = e0 + 4 * i;
+                    if (e < end) {
+                        const uint32_t nib = take4<MAXC>(labs[i], range4(e, beg, end), nbr, lut, A, tl);
+                        kb |= e < beg ? nib >> (int)(beg - e) : nib << (int)(e - beg);
+                    }
+                }
+            } else {
+                for (int64_t e = e0; e < end; e += 4) {
+                    const uint32_t nib = take4<MAXC>(labels4<false>(a, e, beg, end), range4(e, beg, end), nbr, lut, A, tl);
+                    kb |= e < beg ? nib >> (int)(beg - e) : nib << (int)(e - beg);
+                }
+            }
+            Partial<MAXC> p;
+            p.U = A.U;
+            p.nN = A.nN;
+            unpack_classes<MAXC>(A.cp, p);
+            keep = decide<MAXC>(wv, p, s);
+            kept = A.nN;
+            // the bits of a vertex that dies are not read again
+            if (keep) clear_rel(a.ebits, beg, ((1u << (int)len) - 1u) & ~kb);
+        }
+        // (2) rows of up to 64 entries, four at a time, eight lanes each
+        for (uint32_t todo = __ballot_sync(FULL_MASK, wv && len > kFirstLane && len <= kFirstGroup); todo;) {
+            int src[4];
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                src[i] = todo ? __ffs(todo) - 1 : -1;
+                todo &= todo - 1u;
+            }
+            const int g = lane >> 3, j = lane & 7;
+            const int from = g == 0 ? src[0] : g == 1 ? src[1] : g == 2 ? src[2] : src[3];
+            const int f = from < 0 ? 0 : from;
+            const int64_t gb = __shfl_sync(FULL_MASK, beg, f);
+            const int64_t ge0 = __shfl_sync(FULL_MASK, end, f);
+            const int64_t ge = from < 0 ? gb : ge0;          // an empty group: no entry is in range
+            const uint32_t gn = __shfl_sync(FULL_MASK, nbr, f), gw = __shfl_sync(FULL_MASK, wv, f);
+            const int64_t w0 = gb >> 5;
+            uint32_t labs[3], word[3];
+            FirstAcc A;
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                const int64_t e = ((w0 + k) << 5) + 4 * j;
+                labs[k] = e < ge && e + 4 > gb ? labels4<ELAB>(a, e, gb, ge) : 0u;
+            }
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                const int64_t e = ((w0 + k) << 5) + 4 * j;
+                word[k] = take4<MAXC>(labs[k], range4(e, gb, ge), gn, lut, A, tl) << (4 * j);
+            }
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) {
+#pragma unroll
+                for (int k = 0; k < 3; k++) word[k] |= __shfl_xor_sync(FULL_MASK, word[k], o);
+                A.U |= __shfl_xor_sync(FULL_MASK, A.U, o);
+                A.nN += __shfl_xor_sync(FULL_MASK, A.nN, o);
+                if (MAXC > 0) A.cp += __shfl_xor_sync(FULL_MASK, A.cp, o);   // at most 64 per byte
+            }
+            Partial<MAXC> p;
+            p.U = A.U;
+            p.nN = A.nN;
+            unpack_classes<MAXC>(A.cp, p);
+            const uint32_t gk = decide<MAXC>(gw, p, s);
+            if (gk && from >= 0 && j < 3) store_word(a.ebits, w0 + j, gb, ge, j == 0 ? word[0] : j == 1 ? word[1] : word[2]);
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const uint32_t k = __shfl_sync(FULL_MASK, gk, 8 * i), c = __shfl_sync(FULL_MASK, A.nN, 8 * i);
+                if (lane == src[i]) { keep = k; kept = c; }
+            }
+        }
+        // (3) longer rows, the warp together
+        for (uint32_t todo = __ballot_sync(FULL_MASK, wv && len > kFirstGroup && !hub); todo; todo &= todo - 1u) {
+            const int src = __ffs(todo) - 1;
+            Partial<MAXC> p;
+            first_warp<MAXC, ELAB>(a, __shfl_sync(FULL_MASK, beg, src), __shfl_sync(FULL_MASK, end, src),
+                                   __shfl_sync(FULL_MASK, nbr, src), lut, p, tl);
+            const uint32_t k = decide<MAXC>(__shfl_sync(FULL_MASK, wv, src), p, s);
+            if (lane == src) { keep = k; kept = p.nN; }
+        }
+        if (hub) {
+            const int nch = (int)((len + a.hub_deg - 1) / a.hub_deg);
+            const int slot = (int)atomicAdd(&a.hubs->n_hub_slots, 1u);
+            const unsigned int base = atomicAdd(&a.hubs->n_chunk, (unsigned int)nch);
+            for (int c = 0; c < nch; c++) a.hub_list[base + c] = ChunkItem{(int32_t)v, c, slot, nch};
+        } else if (mine) {
+            if (wv) {
+                tl.alive++;
+                tl.rows += (unsigned long long)len;
+                if (keep) { tl.kept += kept; tl.rows_next += (unsigned long long)len; }
+                else tl.died++;
+                if (keep != wv) tl.changed = 1u;
+                a.deg[v] = keep ? kept : 0u;
+            }
+            a.om0[v] = keep;
+            a.om1[v] = keep;
+            store_narrow(a.nw0, a.nw_bytes, v, keep);
+            store_narrow(a.nw1, a.nw_bytes, v, keep);
+        }
+        list_survivor(a, keep != 0u, (int32_t)v, len, bs, bm);
+    }
+    __syncthreads();
+    block_flush(bs, &scnt[0][0], wib);
+    block_flush(bm, &scnt[1][0], wib);
+    add_totals(tl, totals, a.st);
+}
+
+// The first round's long rows, one warp per piece; the last piece of a row
+// decides.
+template <int MAXC, bool ELAB>
+__global__ void __launch_bounds__(256, 4)
+k_first_hubs(FirstArgs a, DevTmpl t) {
+    const int64_t n_piece = a.hubs->n_chunk;
+    if (n_piece == 0) return;
+    __shared__ SmemTmpl s;
+    __shared__ uint2 lut[256];
+    __shared__ int32_t sbuf[2][8][32];
+    __shared__ int scnt[2][8];
+    __shared__ unsigned long long totals[9];
+    if (threadIdx.x < 9) totals[threadIdx.x] = 0ull;
+    load_tmpl(s, t);
+    const int wib = threadIdx.x >> 5;
+    const int lane = (int)lane_id();
+    if (lane == 0) { scnt[0][wib] = 0; scnt[1][wib] = 0; }
+    __syncthreads();
+    first_table(lut, s, a.lm);
+    __syncthreads();
+    WarpBuf<int32_t> bs{sbuf[0][wib], &scnt[0][wib], a.small_out, &a.st->n_small};
+    WarpBuf<int32_t> bm{sbuf[1][wib], &scnt[1][wib], a.med_out, &a.st->n_med};
+    const int64_t gwarp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    LccTally tl;
+    for (int64_t it = gwarp; it < n_piece; it += nwarps) {
+        const ChunkItem ci = a.hub_list[it];
+        const uint32_t wv = lut[a.lab[ci.v]].x;
+        const int64_t rbeg = a.rp[ci.v], rend = a.rp[ci.v + 1];
+        const int64_t beg = rbeg + (int64_t)ci.c * a.hub_deg, end = min(rend, beg + (int64_t)a.hub_deg);
+        Partial<MAXC> p;
+        first_warp<MAXC, ELAB>(a, beg, end, nbr_mask(wv, s) | a.eta_off, lut, p, tl);
+        HubAcc *h = a.acc + ci.slot;
+        unsigned int ticket = 0;
+        if (lane == 0) {
+            if (p.U) atomicOr(&h->U, p.U);
+            if (p.nN) atomicAdd(&h->nN, p.nN);
+#pragma unroll
+            for (int c = 0; c < MAXC; c++)
+                if (p.cnt[c]) atomicAdd(&h->cnt[c], p.cnt[c]);
+            __threadfence();
+            ticket = atomicAdd(&h->done, 1u);
+        }
+        ticket = __shfl_sync(FULL_MASK, ticket, 0);
+        uint32_t keep = 0u;
+        if (ticket == (unsigned int)(ci.nchunks - 1)) {
+            __threadfence();
+            Partial<MAXC> tot;
+            tot.U = atomicOr(&h->U, 0u);
+            tot.nN = atomicAdd(&h->nN, 0u);
+#pragma unroll
+            for (int c = 0; c < MAXC; c++) tot.cnt[c] = atomicAdd(&h->cnt[c], 0u);
+            keep = decide<MAXC>(wv, tot, s);
+            __syncwarp();
+            if (lane == 0) {
+                tl.alive++;
+                tl.rows += (unsigned long long)(rend - rbeg);
+                if (keep) { tl.kept += tot.nN; tl.rows_next += (unsigned long long)(rend - rbeg); }
+                else tl.died++;
+                if (keep != wv) tl.changed = 1u;
+                a.deg[ci.v] = keep ? tot.nN : 0u;
+                a.om0[ci.v] = keep;
+                a.om1[ci.v] = keep;
+                store_narrow(a.nw0, a.nw_bytes, ci.v, keep);
+                store_narrow(a.nw1, a.nw_bytes, ci.v, keep);
+                h->U = 0u; h->nN = 0u; h->flags = 0u; h->done = 0u;
+                for (int c = 0; c < MAXC; c++) h->cnt[c] = 0u;
+            }
+        }
+        list_survivor(a, lane == 0 && keep != 0u, ci.v, rend - rbeg, bs, bm);
+    }
+    __syncthreads();
+    block_flush(bs, &scnt[0][0], wib);
+    block_flush(bm, &scnt[1][0], wib);
+    add_totals(tl, totals, a.st);
 }
 
 // -------------------------------------------------------------------------
@@ -3195,7 +3603,7 @@ int ensure_entry_labels(ccpm_ctx *ctx, ccpm_graph *g) {
     if (g->elab || g->m == 0) return CCPM_OK;
     uint8_t *el = nullptr;
     int rc;
-    if ((rc = dalloc(ctx, &el, (size_t)g->m))) return rc;
+    if ((rc = dalloc(ctx, &el, (size_t)g->m + 4))) return rc;     // read four at a time
     int grid = (int)std::min<int64_t>((g->m + 255) / 256, (int64_t)ctx->num_sms * 8);
     k_gather_labels<<<grid, 256, 0, ctx->stream>>>(g->m, g->col, g->lab, el);
     cudaError_t e = cudaGetLastError();
@@ -3508,6 +3916,58 @@ struct Pipeline {
         return CCPM_OK;
     }
 
+    // Fresh prunes start with k_first_round unless the template has more
+    // multiplicity classes than its packed counts hold.
+    bool first_kernel() const { return dense && from_labels && gen < 0 && maxc <= 4; }
+
+    // The first round of a fresh prune (no initialisation runs before it).
+    int launch_first(RoundStats *slot) {
+        Workspace &w = ctx->ws;
+        FirstArgs a;
+        a.n = g->n;
+        a.m = g->m;
+        a.rp = g->rp;
+        a.col = g->col;
+        a.lab = g->lab;
+        a.elab = elab;
+        a.om0 = w.om[0];
+        a.om1 = w.om[1];
+        a.nw0 = w.nw[0];
+        a.nw1 = w.nw[1];
+        a.nw_bytes = nw_bytes;
+        a.ebits = w.ebits;
+        a.deg = w.deg;
+        a.small_out = w.small[li ^ 1];
+        a.med_out = w.med[li ^ 1];
+        a.chunk_out = w.chunk[li ^ 1];
+        a.hub_list = w.chunk[li];
+        a.hubs = &w.ctl->init;
+        a.acc = w.acc;
+        a.st = slot;
+        a.hub_deg = w.hub_deg;
+        a.short_max = short_max;
+        a.eta_off = eta_off ? ~0u : 0u;
+        a.col_vec = ((uintptr_t)g->col & 15) == 0;
+        a.lm = lm0;
+        launches += 2;
+        lcc_launches++;
+        dense = false;
+        from_labels = false;
+#define CCPM_LAUNCH_FIRST(C, E)                                                                                     \
+    do {                                                                                                            \
+        k_first_round<C, E><<<lcc_grid(ctx, k_first_round<C, E>, g->n), 256, 0, ctx->stream>>>(a, dt);              \
+        k_first_hubs<C, E><<<lcc_grid(ctx, k_first_hubs<C, E>, first_rows / kFirstWarp + 1), 256, 0, ctx->stream>>>(a, dt); \
+    } while (0)
+        if (elab) {
+            if (maxc == 0) CCPM_LAUNCH_FIRST(0, true); else CCPM_LAUNCH_FIRST(4, true);
+        } else {
+            if (maxc == 0) CCPM_LAUNCH_FIRST(0, false); else CCPM_LAUNCH_FIRST(4, false);
+        }
+#undef CCPM_LAUNCH_FIRST
+        CU(ctx, cudaGetLastError());
+        return CCPM_OK;
+    }
+
     // Pass the changes of a round (prev) on: the lists of the delta round whose
     // counters are `slot`.  lists: the round was a full one that read the omega
     // buffer c ^ 1 and left its vertices in the lists l.
@@ -3582,7 +4042,9 @@ struct Pipeline {
                 const RoundStats *prev = i ? ring + i - 1 : src;
                 if (!deltas || full_left > 0) {
                     if (full_left > 0) full_left--;
-                    if ((rc = launch_round(ring + i, prev, i ? nullptr : gate, c, l, false))) return rc;
+                    if (first && i == 0 && first_kernel()) rc = launch_first(ring);
+                    else rc = launch_round(ring + i, prev, i ? nullptr : gate, c, l, false);
+                    if (rc) return rc;
                     n_full++;
                     c ^= 1;
                     l ^= 1;
@@ -4249,7 +4711,7 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
         CUF(cudaMemsetAsync(w.ebits, 0xFF, sizeof(uint32_t) * (size_t)w.words, s));
     }
     CUF(cudaMemsetAsync(&w.ctl->init, 0, sizeof(RoundStats), s));
-    {
+    if (!P.first_kernel() || resume) {
         int grid = grid_for(ctx, g->n, 256, 8);
         P.launches++;
         k_init<<<grid, 256, 0, s>>>(g->n, g->rp, g->lab, lm, resume ? r->om : nullptr, w.om[0], w.om[1], w.nw[0],

@@ -34,21 +34,28 @@ def stars(copies, seed):
 
 
 @pytest.mark.parametrize("graph", ["stars1", "stars8", "rmat12", "rmat17"])
-def test_rounds_equal_the_oracle(graph):
+@pytest.mark.parametrize("offset", [0, 1])
+def test_rounds_equal_the_oracle(graph, offset):
+    """offset: the columns start that many elements past a 16-byte boundary."""
+    import torch
     from paper_1912_08453_gb300 import ccpm
     if graph.startswith("stars"):
         g = stars(int(graph[5:]), 5)
     else:
         g = wl.rmat_graph(int(graph[4:]), seed=9, labels="zipf", n_labels=6)
     ctx = ccpm.Context(0)
-    dev = ccpm.Graph(ctx, g.row_ptr, g.col, g.labels)
+    col = torch.zeros(g.m_dir + offset, dtype=torch.int32, device="cuda:0")[offset:]
+    col.copy_(torch.from_numpy(g.col))
+    torch.cuda.synchronize()
+    dev = ccpm.Graph(ctx, torch.from_numpy(g.row_ptr).cuda(), col, torch.from_numpy(g.labels).cuda())
     for tl, te in TEMPLATES:
         og = oracle.Graph(g.row_ptr, g.col, g.labels)
         omega, active = oracle.init(og, tl, te)
         rounds, scanned = oracle.lcc(og, tl, te, omega, active)
         t = ccpm.Template(ctx, tl, te)
-        for short_rows in (0, 1, 1024):
-            r = ccpm.prune(ctx, dev, t, ccpm.options(lcc_only=1, short_rows=short_rows))
+        for opts in ({}, {"short_rows": 1}, {"short_rows": 1024}, {"hub_degree": 16}, {"hub_degree": 4096},
+                     {"entry_labels": 1}, {"compact": 1}, {"compact": -1}):
+            r = ccpm.prune(ctx, dev, t, ccpm.options(lcc_only=1, **opts))
             np.testing.assert_array_equal(r.omega(), omega)
             np.testing.assert_array_equal(r.edge_bitmap(), oracle.pack_bits(active))
             assert r.phase_rounds()[0] == rounds
