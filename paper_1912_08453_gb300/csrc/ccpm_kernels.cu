@@ -1103,105 +1103,166 @@ k_lcc_round(LccArgs a, DevTmpl t) {
 }
 
 // -------------------------------------------------------------------------
-// The first round of a fresh prune (Alg. 3 and the first pass of Alg. 4 in one
-// kernel).  omega_0 is the mask of a vertex's label, so the round needs labels
-// only: the vertices are taken in id order (no frontier list is written and
-// read back), and omega is written once, as the round leaves it, in both
-// buffers.  Only the survivors are listed for the next round.
+// The first round, and the later ones where the rows are huge (kHugeRows), for
+// templates of at most four multiplicity classes; k_lcc_round above serves the
+// others.
 //
-// It was bound by instructions: one entry per lane and step, with the row
-// located and reduced every 32 entries, took 5 warp instructions per entry.  A
-// lane now takes four consecutive entries per step (their labels are one
-// 32-bit load), looks each label up in a table of (omega, packed class counts)
-// and votes with a nibble of the bitmap word, and rows are walked by as many
-// lanes as they fill: rows of at most 16 entries by their own lane, up to 64 by
-// 8 lanes (four rows side by side), longer ones by the warp (128 entries per
-// step), those past max(hub_deg, 1024) in pieces by k_first_hubs.  32M vertices,
-// 10^9 entries, 20M vertices initially active: initialisation and first round
-// 5.0 -> 3.0 ms, and the second round, whose lists now hold survivors only, 3.5
-// -> 3.1 ms.
+// A lane takes four consecutive entries per step: their edge bits are a nibble
+// of a bitmap word, their columns one 16-byte load, and the four gathers that
+// follow are in flight together.  A neighbour's omega arrives as a byte (its
+// label in the first round, its narrow omega later) that indexes a table of
+// (omega, one byte per class it meets), so class counts are one addition.
+// Rows are walked by as many lanes as they fill: up to 16 entries by their own
+// lane, up to 64 by 8 lanes (four rows side by side), longer ones by the warp.
+//
+// The rounds are bound by the latency of dependent loads (list entry, omega and
+// offsets, bits, columns, neighbours), not by bytes: a warp that walked one row
+// after the other, 32 entries a step, spent 3 to 4 us on a row of 200 entries.
+// long_rows keeps the bits of the next two stretches, the columns of the next
+// step and the gathers of the current one in flight, across rows.
+//
+// The first round of a fresh prune needs labels only (omega_0 is the mask of a
+// vertex's label), so it is one with the initialisation (Alg. 3): k_first_round
+// takes the vertices in id order, with no list written and read back, decides
+// short rows and lists the longer ones for k_rows.  It writes omega as the
+// round leaves it, in both buffers, and lists survivors only.
 // -------------------------------------------------------------------------
 
-struct FirstArgs {
-    int64_t n, m;
+// Where a neighbour's omega comes from: its label in entry order (first round,
+// graphs that have the entry labels), its label (first round), its 1-byte
+// omega, or its 2- or 4-byte omega.
+constexpr int kByEntry = 0, kByLabel = 1, kByByte = 2, kByWord = 3;
+constexpr int kFirst = 3;                    // a round's MODE, beside kFull and kDelta
+
+// Entries in the initially active rows from which k_rows takes the rounds after
+// the first: the second and third round of 32M vertices (6*10^8 such entries)
+// take 3.4 ms with it and 4.4 with k_lcc_round, those of 4M vertices (9*10^7)
+// 0.26 and 0.22, of 3M (4*10^7) 0.18 and 0.16; on 64K vertices a round takes
+// 7.6 and 6.3 us (one chain of latencies, which k_lcc_round keeps shorter).
+constexpr int64_t kHugeRows = (int64_t)1 << 28;
+// ... below which k_first_round walks the longer rows too, with no second
+// kernel over a list of them (64K vertices: 31 against 41 us; 3M: 216 against
+// 197).
+constexpr int64_t kInlineRows = (int64_t)1 << 22;
+
+struct RowArgs {
+    int64_t n, m;                 // m: columns that may be read four at a time
     const int64_t *rp;
     const int32_t *col;
+    int col_vec;                  // col is 16-byte aligned
     const uint8_t *lab;
-    const uint8_t *elab;          // neighbours' labels in entry order (ELAB), readable up to m + 3
-    uint32_t *om0, *om1;
-    void *nw0, *nw1;
+    const uint8_t *elab;          // readable up to entry m + 15
+    const uint32_t *om;           // omega the round reads (kFull, kDelta), and its narrow copy
+    const void *nw;
     int nw_bytes;
-    uint32_t *ebits;              // all ones
-    uint32_t *deg;
-    int32_t *small_out, *med_out; // survivors, for the next round
+    uint32_t *om_out[2];          // omega the round writes: [0] (kFull), both (kFirst)
+    void *nw_out[2];
+    uint32_t *ebits;
+    int guard;                    // kFirst: a word follows the bitmap's last
+    int inline_long;              // kFirst: k_first_round walks rows of up to 1024 entries itself
+    uint32_t *deg;                // entries each evaluated vertex keeps (nullable)
+    uint32_t *dirty;
+    Change *chg;
+    ChangePiece *chg_piece;
+    const int32_t *small_in, *med_in;
+    const ChunkItem *chunk_in;
+    const RoundStats *sizes;      // sizes of these lists (NULL: the next three)
+    int64_t n_small, n_med, n_chunk;
+    const RoundStats *gate;       // the round runs only if these counters say `changed` (nullable)
+    int32_t *small_out, *med_out;
     ChunkItem *chunk_out;
-    ChunkItem *hub_list;          // pieces of the rows left to k_first_hubs, sizes in `hubs`
-    RoundStats *hubs;
+    int32_t *first_med;           // kFirst: the rows k_first_round leaves to k_rows, sizes in first_sizes
+    ChunkItem *first_chunk;
+    RoundStats *first_sizes;
     HubAcc *acc;
     RoundStats *st;
     int hub_deg, short_max;
     uint32_t eta_off;
-    int col_vec;                  // col is 16-byte aligned
     LabelMask lm;
 };
 
-constexpr int kFirstLane = 16, kFirstGroup = 64, kFirstWarp = 1024;   // row lengths of the three paths
+constexpr int kLaneRow = 16, kGroupRow = 64, kWarpRow = 1024;   // row lengths of the three paths
 
-struct FirstAcc { uint32_t U = 0, cp = 0, nN = 0; };   // union, class counts (four bytes), kept entries
+struct RowAcc { uint32_t U = 0, cp = 0, nN = 0; };   // union, class counts (four bytes), kept entries
 
-// Table of the first round: label -> omega_0 and, per multiplicity class, 1 in
-// the class's byte if omega_0 meets it.
-__device__ __forceinline__ void first_table(uint2 *lut, const SmemTmpl &s, const LabelMask &lm) {
-    for (int L = threadIdx.x; L < 256; L += blockDim.x) {
-        const uint32_t w = lm.m[L];
+// byte -> (omega, 1 in the byte of every class it meets)
+template <int F>
+__device__ __forceinline__ void make_table(uint2 *lut, const SmemTmpl &s, const LabelMask &lm) {
+    for (int i = threadIdx.x; i < 256; i += blockDim.x) {
+        const uint32_t w = (F == kByEntry || F == kByLabel) ? lm.m[i] : (uint32_t)i;
         uint32_t pack = 0;
         for (int c = 0; c < 4 && c < s.n_cls; c++) pack |= (w & s.cls_mask[c]) ? 1u << (8 * c) : 0u;
-        lut[L] = make_uint2(w, pack);
+        lut[i] = make_uint2(w, pack);
     }
 }
 
-// Labels of the neighbours at entries e..e+3 (e a multiple of 4), one per byte;
-// those outside [beg, end) are any value.
-template <bool ELAB>
-__device__ __forceinline__ uint32_t labels4(const FirstArgs &a, int64_t e, int64_t beg, int64_t end) {
-    if (ELAB) return __ldcs((const unsigned int *)(a.elab + e));
-    int32_t u[4];
+// Columns of the entries e + j with bit j of nib set (e a multiple of 4).
+__device__ __forceinline__ void quad_cols(const RowArgs &a, int64_t e, uint32_t nib, int32_t (&u)[4]) {
+    u[0] = u[1] = u[2] = u[3] = 0;
+    if (!nib) return;
     if (a.col_vec && e + 4 <= a.m) {
         const int4 c = __ldcs((const int4 *)(a.col + e));
         u[0] = c.x; u[1] = c.y; u[2] = c.z; u[3] = c.w;
     } else {
 #pragma unroll
-        for (int j = 0; j < 4; j++) u[j] = e + j >= beg && e + j < end ? __ldcs(a.col + e + j) : 0;
+        for (int j = 0; j < 4; j++)
+            if ((nib >> j) & 1u) u[j] = __ldcs(a.col + e + j);
     }
-    uint32_t labs = 0;
+}
+
+// What the four entries' neighbours hold: four bytes, or four words.
+template <int F> struct Quad { uint32_t v[F == kByWord ? 4 : 1]; };
+
+template <int F>
+__device__ __forceinline__ Quad<F> quad_gather(const RowArgs &a, uint32_t nib, const int32_t (&u)[4]) {
+    Quad<F> q;
+    uint32_t x[4];
 #pragma unroll
-    for (int j = 0; j < 4; j++)
-        if (e + j >= beg && e + j < end) labs |= (uint32_t)__ldg(a.lab + u[j]) << (8 * j);
-    return labs;
+    for (int j = 0; j < 4; j++) {
+        x[j] = 0u;
+        if ((nib >> j) & 1u) {
+            if (F == kByLabel) x[j] = __ldg(a.lab + u[j]);
+            else if (F == kByByte) x[j] = __ldg((const uint8_t *)a.nw + u[j]);
+            else x[j] = gather_om(a.om, a.nw, a.nw_bytes, u[j]);
+        }
+    }
+    if constexpr (F == kByWord) {
+#pragma unroll
+        for (int j = 0; j < 4; j++) q.v[j] = x[j];
+    } else {
+        q.v[0] = x[0] | (x[1] << 8) | (x[2] << 16) | (x[3] << 24);
+    }
+    return q;
 }
 
-// Bits j of a nibble with e + j in [beg, end).
-__device__ __forceinline__ uint32_t range4(int64_t e, int64_t beg, int64_t end) {
-    const int lo = (int)min((int64_t)4, max((int64_t)0, beg - e)), hi = (int)min((int64_t)4, max((int64_t)0, end - e));
-    return ((1u << hi) - 1u) & ~((1u << lo) - 1u);
-}
-
-// Four entries: the kept ones as a nibble.
-template <int MAXC>
-__device__ __forceinline__ uint32_t take4(uint32_t labs, uint32_t in, uint32_t nbr, const uint2 *lut, FirstAcc &A,
-                                          LccTally &tl) {
+// Four entries (those of nib): the kept ones as a nibble.  Entries without a
+// bit hold an empty omega, except where labels come from a stream (kByEntry).
+template <int MAXC, int F>
+__device__ __forceinline__ uint32_t quad_take(const Quad<F> &q, uint32_t nib, uint32_t nbr, const uint2 *lut,
+                                              const uint32_t (&cm)[4], RowAcc &A, LccTally &tl) {
     uint32_t keep = 0, live = 0;
 #pragma unroll
     for (int j = 0; j < 4; j++) {
-        const uint2 q = lut[(labs >> (8 * j)) & 255u];
-        const uint32_t w = (in >> j) & 1u ? q.x : 0u;
-        live += w != 0u;
+        uint32_t w, pack = 0u;
+        if constexpr (F == kByWord) {
+            w = q.v[j];
+#pragma unroll
+            for (int c = 0; c < MAXC; c++) pack |= (w & cm[c]) ? 1u << (8 * c) : 0u;
+        } else {
+            const uint2 x = lut[(q.v[0] >> (8 * j)) & 255u];
+            w = x.x;
+            pack = x.y;
+            if ((F == kByEntry || F == kByLabel) && !((nib >> j) & 1u)) w = 0u;
+        }
+        if (F != kByByte) live += w != 0u;
         if (w & nbr) {
             A.U |= w;
-            if (MAXC > 0) A.cp += q.y;
+            if (MAXC > 0) A.cp += pack;
             keep |= 1u << j;
         }
     }
+    if (F == kByByte)                        // bytes that are not zero
+        live = __popc((((q.v[0] & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | q.v[0]) & 0x80808080u);
     const uint32_t k = __popc(keep);
     A.nN += k;
     tl.scanned += live;
@@ -1209,52 +1270,369 @@ __device__ __forceinline__ uint32_t take4(uint32_t labs, uint32_t in, uint32_t n
     return keep;
 }
 
-// Store the kept bits of one bitmap word of the row [beg, end).
-__device__ __forceinline__ void store_word(uint32_t *ebits, int64_t wi, int64_t beg, int64_t end, uint32_t kept) {
+// Bits of the word wi that belong to the row [beg, end).
+__device__ __forceinline__ uint32_t word_range(int64_t wi, int64_t beg, int64_t end) {
     const int64_t e0 = wi << 5;
-    if (e0 >= end || e0 + 32 <= beg) return;
-    if (e0 >= beg && e0 + 32 <= end) { ebits[wi] = kept; return; }
-    uint32_t in = ~0u;                       // shared with a neighbouring row
+    if (e0 >= end || e0 + 32 <= beg) return 0u;
+    uint32_t in = ~0u;
     if (e0 < beg) in &= ~0u << (uint32_t)(beg - e0);
     if (end - e0 < 32) in &= (1u << (uint32_t)(end - e0)) - 1u;
-    if (in & ~kept) atomicAnd(&ebits[wi], ~(in & ~kept));
+    return in;
 }
 
-// The whole warp walks [beg, end); every lane gets the sums.
-template <int MAXC, bool ELAB>
-__device__ __forceinline__ void first_warp(const FirstArgs &a, int64_t beg, int64_t end, uint32_t nbr, const uint2 *lut,
-                                           Partial<MAXC> &p, LccTally &tl) {
-    const int lane = (int)lane_id();
-    const int64_t w0 = beg >> 7;
-    const int nwin = (int)(((end + 127) >> 7) - w0);
-    FirstAcc A;
-    int64_t e = (w0 << 7) + 4 * lane;
-    auto load = [&](int64_t x) { return x < end && x + 4 > beg ? labels4<ELAB>(a, x, beg, end) : 0u; };
-    uint32_t next = load(e);
-    for (int k = 0; k < nwin; k++, e += 128) {
-        const uint32_t labs = next;
-        if (k + 1 < nwin) next = load(e + 128);
-        const uint32_t nib = take4<MAXC>(labs, range4(e, beg, end), nbr, lut, A, tl);
-        uint32_t word = nib << (4 * (lane & 7));
-        word |= __shfl_xor_sync(FULL_MASK, word, 1);
-        word |= __shfl_xor_sync(FULL_MASK, word, 2);
-        word |= __shfl_xor_sync(FULL_MASK, word, 4);
-        if ((lane & 7) == 0) store_word(a.ebits, e >> 5, beg, end, word);
-        if (MAXC > 0 && (k & 31) == 31) {    // before a byte can overflow
+// The row's bits `had` of word wi shrink to `kept`.  The bit goes with failing
+// entries and with those whose other end is inactive already.
+__device__ __forceinline__ void store_bits(uint32_t *ebits, int64_t wi, uint32_t in, uint32_t had, uint32_t kept) {
+    if (!(had & ~kept)) return;
+    if (in == ~0u) ebits[wi] = kept;
+    else atomicAnd(&ebits[wi], ~(had & ~kept));          // shared with a neighbouring row
+}
+
+// The row's active bits in word wi.
+template <int MODE>
+__device__ __forceinline__ uint32_t row_word(const RowArgs &a, int64_t wi, int64_t beg, int64_t end) {
+    const uint32_t in = word_range(wi, beg, end);
+    if (MODE == kFirst) return in;
+    return in ? a.ebits[wi] & in : 0u;
+}
+
+template <int MAXC>
+__device__ __forceinline__ void unpack_classes(uint32_t cp, Partial<MAXC> &p) {
 #pragma unroll
-            for (int c = 0; c < MAXC; c++) p.cnt[c] += (A.cp >> (8 * c)) & 255u;
-            A.cp = 0;
+    for (int c = 0; c < MAXC; c++) p.cnt[c] += (cp >> (8 * c)) & 255u;
+}
+
+// Rows of up to 64 entries, one vertex per lane (wv = 0: none): omega' and the
+// number of entries kept.  All lanes call.
+template <int MAXC, int MODE, int F>
+__device__ __forceinline__ void short_batch(const RowArgs &a, const SmemTmpl &s, const uint2 *lut,
+                                            const uint32_t (&cm)[4], uint32_t wv, uint32_t nbr, int64_t beg, int64_t end,
+                                            uint32_t &keep, uint32_t &kept, LccTally &tl) {
+    const int lane = (int)lane_id();
+    const int64_t len = end - beg;
+    // (1) up to 16 entries, by the lane itself
+    if (wv && len > 0 && len <= kLaneRow) {
+        RowAcc A;
+        const int64_t wi = beg >> 5;
+        const uint32_t sh = (uint32_t)(beg & 31), in = (1u << (int)len) - 1u;
+        uint32_t had = in;                               // active entries, relative to beg
+        if (MODE != kFirst) {
+            had = a.ebits[wi] >> sh;
+            if (sh + (uint32_t)len > 32u) had |= a.ebits[wi + 1] << (32 - sh);
+            had &= in;
+        }
+        uint32_t kb = 0;
+        const int64_t e0 = beg & ~(int64_t)3;
+        const int lead = (int)(beg - e0);
+        const uint32_t nibs = had << lead;               // by groups of four entries from e0
+        if (F == kByEntry) {
+            uint32_t labs[5];
+#pragma unroll
+            for (int i = 0; i < 5; i++)
+                labs[i] = e0 + 4 * i < end ? __ldcs((const unsigned int *)(a.elab + e0 + 4 * i)) : 0u;
+#pragma unroll
+            for (int i = 0; i < 5; i++) {
+                Quad<F> q;
+                q.v[0] = labs[i];
+                const uint32_t nib = (nibs >> (4 * i)) & 15u;
+                if (nib) kb |= quad_take<MAXC, F>(q, nib, nbr, lut, cm, A, tl) << (4 * i);
+            }
+        } else {
+            int32_t u[4], nx[4];
+            quad_cols(a, e0, nibs & 15u, u);
+            for (int i = 0; (nibs >> (4 * i)) != 0u; i++) {
+                const uint32_t nib = (nibs >> (4 * i)) & 15u;
+                const Quad<F> q = quad_gather<F>(a, nib, u);
+                quad_cols(a, e0 + 4 * (i + 1), (nibs >> (4 * i + 4)) & 15u, nx);
+                kb |= quad_take<MAXC, F>(q, nib, nbr, lut, cm, A, tl) << (4 * i);
+#pragma unroll
+                for (int j = 0; j < 4; j++) u[j] = nx[j];
+            }
+        }
+        kb >>= lead;
+        Partial<MAXC> p;
+        p.U = A.U;
+        p.nN = A.nN;
+        unpack_classes<MAXC>(A.cp, p);
+        keep = decide<MAXC>(wv, p, s);
+        kept = A.nN;
+        // the bits of a vertex that dies: no round reads them again
+        if (keep) clear_rel(a.ebits, beg, had & ~kb);
+    }
+    // (2) up to 64, four rows at a time, eight lanes each
+    for (uint32_t todo = __ballot_sync(FULL_MASK, wv && len > kLaneRow && len <= kGroupRow); todo;) {
+        int src[4];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            src[i] = todo ? __ffs(todo) - 1 : -1;
+            todo &= todo - 1u;
+        }
+        const int g = lane >> 3, j = lane & 7;
+        const int from = g == 0 ? src[0] : g == 1 ? src[1] : g == 2 ? src[2] : src[3];
+        const int f = from < 0 ? 0 : from;
+        const int64_t gb = __shfl_sync(FULL_MASK, beg, f), ge0 = __shfl_sync(FULL_MASK, end, f);
+        const int64_t ge = from < 0 ? gb : ge0;          // an empty group: no entry is in range
+        const uint32_t gn = __shfl_sync(FULL_MASK, nbr, f), gw = __shfl_sync(FULL_MASK, wv, f);
+        const int64_t w0 = gb >> 5;
+        uint32_t had[3], word[3];
+        Quad<F> q[3];
+        RowAcc A;
+#pragma unroll
+        for (int k = 0; k < 3; k++) had[k] = row_word<MODE>(a, w0 + k, gb, ge);
+        if (F == kByEntry) {
+#pragma unroll
+            for (int k = 0; k < 3; k++)
+                q[k].v[0] = (had[k] >> (4 * j)) & 15u
+                                ? __ldcs((const unsigned int *)(a.elab + ((w0 + k) << 5) + 4 * j)) : 0u;
+        } else {
+            int32_t u[3][4];
+#pragma unroll
+            for (int k = 0; k < 3; k++) quad_cols(a, ((w0 + k) << 5) + 4 * j, (had[k] >> (4 * j)) & 15u, u[k]);
+#pragma unroll
+            for (int k = 0; k < 3; k++) q[k] = quad_gather<F>(a, (had[k] >> (4 * j)) & 15u, u[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; k++)
+            word[k] = quad_take<MAXC, F>(q[k], (had[k] >> (4 * j)) & 15u, gn, lut, cm, A, tl) << (4 * j);
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) {
+#pragma unroll
+            for (int k = 0; k < 3; k++) word[k] |= __shfl_xor_sync(FULL_MASK, word[k], o);
+            A.U |= __shfl_xor_sync(FULL_MASK, A.U, o);
+            A.nN += __shfl_xor_sync(FULL_MASK, A.nN, o);
+            if (MAXC > 0) A.cp += __shfl_xor_sync(FULL_MASK, A.cp, o);   // at most 64 per byte
+        }
+        Partial<MAXC> p;
+        p.U = A.U;
+        p.nN = A.nN;
+        unpack_classes<MAXC>(A.cp, p);
+        const uint32_t gk = decide<MAXC>(gw, p, s);
+        if (gk && from >= 0 && j < 3)
+            store_bits(a.ebits, w0 + j, word_range(w0 + j, gb, ge), j == 0 ? had[0] : j == 1 ? had[1] : had[2],
+                       j == 0 ? word[0] : j == 1 ? word[1] : word[2]);
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const uint32_t k = __shfl_sync(FULL_MASK, gk, 8 * i), c = __shfl_sync(FULL_MASK, A.nN, 8 * i);
+            if (lane == src[i]) { keep = k; kept = c; }
         }
     }
+}
+
+// Row sums over the warp.
+template <int MAXC>
+__device__ __forceinline__ void reduce_row(const RowAcc &A, Partial<MAXC> &p, int n_cls) {
     p.U = __reduce_or_sync(FULL_MASK, A.U);
     p.nN = __reduce_add_sync(FULL_MASK, A.nN);
 #pragma unroll
-    for (int c = 0; c < MAXC; c++) p.cnt[c] = __reduce_add_sync(FULL_MASK, p.cnt[c] + ((A.cp >> (8 * c)) & 255u));
+    for (int c = 0; c < MAXC; c++)
+        if (c < n_cls) p.cnt[c] = __reduce_add_sync(FULL_MASK, p.cnt[c] + ((A.cp >> (8 * c)) & 255u));
 }
 
-// List a surviving vertex for the next round (all lanes call; `want` lanes list).
-__device__ __forceinline__ void list_survivor(const FirstArgs &a, bool want, int32_t v, int64_t len,
-                                              WarpBuf<int32_t> &bs, WarpBuf<int32_t> &bm) {
+// Rows (or pieces of rows) of any length, one per lane of `rows`, walked by the
+// warp one after the other; done(j, sums) is called by all lanes after the row
+// of lane j.  Stretches of 1024 entries (a bitmap word per lane), steps of 128
+// entries that hold an active one.
+template <int MAXC, int MODE, int F, typename D>
+__device__ __forceinline__ void long_rows(const RowArgs &a, int n_cls, const uint2 *lut, const uint32_t (&cm)[4],
+                                          uint32_t rows,
+                                          int64_t beg, int64_t end, uint32_t nbr, LccTally &tl, D &&done) {
+    if (!rows) return;
+    const int lane = (int)lane_id();
+    const int first = __ffs(rows) - 1;
+    auto next_row = [&](int j) {                     // the lane after j that has a row (32: none)
+        const uint32_t rest = j < 31 ? rows >> (j + 1) << (j + 1) : 0u;
+        return rest ? __ffs(rest) - 1 : 32;
+    };
+    RowAcc A;
+    Partial<MAXC> p;
+    int since = 0;                                   // steps since the class bytes were emptied
+    auto finish = [&](int j) {
+        Partial<MAXC> sum = p;
+        reduce_row<MAXC>(A, sum, n_cls);
+        done(j, sum);
+        A = RowAcc();
+        p = Partial<MAXC>();
+        since = 0;
+    };
+    auto spill_classes = [&](int steps, int most) {
+        since += steps;
+        if (MAXC > 0 && since >= most) {             // before a byte can overflow
+            unpack_classes<MAXC>(A.cp, p);
+            A.cp = 0;
+            since = 0;
+        }
+    };
+    if constexpr (F == kByEntry) {
+        // the labels are one contiguous stream: 16 per lane and step
+        int j = first;
+        int64_t b = __shfl_sync(FULL_MASK, beg, j), e = __shfl_sync(FULL_MASK, end, j);
+        int64_t base = b & ~(int64_t)31;
+        auto load = [&](int64_t at, int64_t rb, int64_t re) {
+            const int64_t x = at + 16 * lane;
+            return x < re && x + 16 > rb ? __ldcs((const uint4 *)(a.elab + x)) : make_uint4(0, 0, 0, 0);
+        };
+        uint4 nx = load(base, b, e);
+        while (j < 32) {
+            const uint4 cur = nx;
+            const int64_t cb = b, ce = e, at = base;
+            const int cj = j;
+            base += 512;
+            if (base >= e) {
+                j = next_row(j);
+                if (j < 32) {
+                    b = __shfl_sync(FULL_MASK, beg, j);
+                    e = __shfl_sync(FULL_MASK, end, j);
+                    base = b & ~(int64_t)31;
+                }
+            }
+            if (j < 32) nx = load(base, b, e);
+            const uint32_t rn = __shfl_sync(FULL_MASK, nbr, cj);
+            const int64_t wi = (at >> 5) + (lane >> 1);
+            const uint32_t in = word_range(wi, cb, ce);
+            const uint32_t half = (in >> (16 * (lane & 1))) & 0xFFFFu;
+            uint32_t kept = 0;
+            if (half) {
+                const uint32_t x[4] = {cur.x, cur.y, cur.z, cur.w};
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    Quad<F> q;
+                    q.v[0] = x[i];
+                    kept |= quad_take<MAXC, F>(q, (half >> (4 * i)) & 15u, rn, lut, cm, A, tl) << (4 * i);
+                }
+            }
+            kept <<= 16 * (lane & 1);
+            kept |= __shfl_xor_sync(FULL_MASK, kept, 1);
+            if (!(lane & 1)) store_bits(a.ebits, wi, in, in, kept);
+            spill_classes(1, 15);
+            if (j != cj) finish(cj);
+        }
+        return;
+    } else {
+        // offsets inside a row count from its first bitmap word whose index is a
+        // multiple of 4, so that they fit 32 bits and a lane's four columns
+        // are 16-byte aligned
+        const int64_t my_w0 = (beg >> 7) << 2;
+        const int my_lo = (int)(beg - (my_w0 << 5)), my_hi = (int)(end - (my_w0 << 5));
+        struct Seg { int j, at, hi; uint32_t word; };        // row, first entry of the stretch, row end
+        auto read = [&](Seg &g) {
+            g.word = 0u;
+            if (g.j >= 32) return;
+            g.hi = __shfl_sync(FULL_MASK, my_hi, g.j);
+            const int lo = __shfl_sync(FULL_MASK, my_lo, g.j);
+            const int64_t w0 = __shfl_sync(FULL_MASK, my_w0, g.j);
+            const int e = g.at + 32 * lane;
+            if (e >= g.hi || e + 32 <= lo) return;
+            uint32_t in = ~0u;
+            if (e < lo) in &= ~0u << (lo - e);
+            if (g.hi - e < 32) in &= (1u << (g.hi - e)) - 1u;
+            g.word = MODE == kFirst ? in : a.ebits[w0 + (e >> 5)] & in;
+        };
+        auto after = [&](const Seg &g) {
+            Seg n{g.j, g.at + 1024, g.hi, 0u};
+            if (n.at >= g.hi) { n.j = next_row(g.j); n.at = 0; }
+            return n;
+        };
+        auto steps = [&](const Seg &g) {             // bit 4k: step k holds an active entry
+            uint32_t b = __ballot_sync(FULL_MASK, g.word != 0u);
+            b |= b >> 1;
+            b |= b >> 2;
+            return b & 0x11111111u;
+        };
+        Seg cur{first, 0, 0, 0u};
+        read(cur);
+        Seg n1 = after(cur);
+        read(n1);
+        uint32_t u_nib = 0;                          // the step whose columns are loaded
+        int32_t u[4];
+        bool have = false;
+        auto columns = [&](const Seg &g, int k4) {
+            const uint32_t wd = __shfl_sync(FULL_MASK, g.word, k4 + (lane >> 3));
+            const int64_t w0 = __shfl_sync(FULL_MASK, my_w0, g.j);
+            u_nib = (wd >> (4 * (lane & 7))) & 15u;
+            quad_cols(a, (w0 << 5) + (g.at + 32 * k4 + 4 * lane), u_nib, u);
+            have = true;
+        };
+        for (;;) {
+            Seg n2 = after(n1);
+            read(n2);
+            const uint32_t rn = __shfl_sync(FULL_MASK, nbr, cur.j);
+            for (uint32_t t = steps(cur); t;) {
+                const int k4 = __ffs(t) - 1;
+                t &= t - 1u;
+                if (!have) columns(cur, k4);
+                const uint32_t nib = u_nib;
+                const Quad<F> q = quad_gather<F>(a, nib, u);
+                have = false;
+                if (t) {
+                    columns(cur, __ffs(t) - 1);
+                } else {
+                    const uint32_t tn = steps(n1);
+                    if (tn) columns(n1, __ffs(tn) - 1);
+                }
+                const uint32_t keep = quad_take<MAXC, F>(q, nib, rn, lut, cm, A, tl);
+                if (__any_sync(FULL_MASK, keep != nib)) {
+                    uint32_t kept = keep << (4 * (lane & 7));
+                    kept |= __shfl_xor_sync(FULL_MASK, kept, 1);
+                    kept |= __shfl_xor_sync(FULL_MASK, kept, 2);
+                    kept |= __shfl_xor_sync(FULL_MASK, kept, 4);
+                    const uint32_t had = __shfl_sync(FULL_MASK, cur.word, k4 + (lane >> 3));
+                    const int lo = __shfl_sync(FULL_MASK, my_lo, cur.j);
+                    const int64_t w0 = __shfl_sync(FULL_MASK, my_w0, cur.j);
+                    if ((lane & 7) == 0 && (had & ~kept)) {
+                        const int e = cur.at + 32 * (k4 + (lane >> 3));
+                        uint32_t *p_word = a.ebits + w0 + (e >> 5);
+                        if (e >= lo && e + 32 <= cur.hi) *p_word = kept;
+                        else atomicAnd(p_word, ~(had & ~kept));          // shared with a neighbouring row
+                    }
+                }
+                spill_classes(1, 60);
+            }
+            if (n1.j != cur.j) finish(cur.j);
+            if (n1.j >= 32) break;
+            cur = n1;
+            n1 = n2;
+        }
+    }
+}
+
+// What a round decided for the lane's vertex v: its omega was wv and is now
+// `keep`, `kept` of the `len` entries of its row stay active.
+template <int MODE>
+__device__ __forceinline__ void settle_row(const RowArgs &a, int32_t v, uint32_t wv, uint32_t keep, uint32_t kept,
+                                           int64_t len, LccTally &tl) {
+    tl.alive++;
+    tl.rows += (unsigned long long)len;
+    if (keep) { tl.kept += kept; tl.rows_next += (unsigned long long)len; }
+    else tl.died++;
+    if (keep != wv) tl.changed = 1u;
+    if (MODE == kDelta) {
+        tl.old_kept += a.deg[v];
+        if (keep == 0u) tl.died_rows += (unsigned long long)len;
+        if (keep != wv && len > a.hub_deg) {
+            const unsigned int np = (unsigned int)((len + a.hub_deg - 1) / a.hub_deg);
+            const unsigned int b = atomicAdd(&a.st->n_chg_piece, np);
+            for (unsigned int c = 0; c < np; c++) a.chg_piece[b + c] = ChangePiece{v, (int32_t)c};
+        }
+    }
+    if (a.deg) a.deg[v] = keep ? kept : 0u;
+}
+
+// omega' of the lane's vertex (a vertex that was inactive gets its 0 again: the
+// buffer may still hold what it had before it died).
+template <int MODE>
+__device__ __forceinline__ void write_omega(const RowArgs &a, int64_t v, uint32_t keep) {
+    if (MODE == kDelta) return;
+    a.om_out[0][v] = keep;
+    store_narrow(a.nw_out[0], a.nw_bytes, v, keep);
+    if (MODE == kFirst) {
+        a.om_out[1][v] = keep;
+        store_narrow(a.nw_out[1], a.nw_bytes, v, keep);
+    }
+}
+
+// List a vertex for the next round by its row length (all lanes call).
+__device__ __forceinline__ void list_row(const RowArgs &a, bool want, int32_t v, int64_t len, WarpBuf<int32_t> &bs,
+                                         WarpBuf<int32_t> &bm) {
     const int64_t small_max = a.hub_deg < a.short_max ? a.hub_deg : a.short_max;
     bs.push(want && len <= small_max, v);
     bm.push(want && len > small_max && len <= a.hub_deg, v);
@@ -1266,244 +1644,269 @@ __device__ __forceinline__ void list_survivor(const FirstArgs &a, bool want, int
     }
 }
 
-template <int MAXC>
-__device__ __forceinline__ void unpack_classes(uint32_t cp, Partial<MAXC> &p) {
-#pragma unroll
-    for (int c = 0; c < MAXC; c++) p.cnt[c] = (cp >> (8 * c)) & 255u;
-}
-
-template <int MAXC, bool ELAB>
+// The first round: every vertex in id order.  Rows of more than 64 entries are
+// left to k_rows (those past max(hub_deg, 1024) in pieces of hub_deg).
+template <int MAXC, int F>
 __global__ void __launch_bounds__(256, 4)
-k_first_round(FirstArgs a, DevTmpl t) {
+k_first_round(RowArgs a, DevTmpl t) {
     __shared__ SmemTmpl s;
     __shared__ uint2 lut[256];
-    __shared__ int32_t sbuf[2][8][32];
-    __shared__ int scnt[2][8];
+    __shared__ int32_t sbuf[3][8][32];
+    __shared__ int scnt[3][8];
     __shared__ unsigned long long totals[9];
     if (threadIdx.x < 9) totals[threadIdx.x] = 0ull;
     load_tmpl(s, t);
     const int wib = threadIdx.x >> 5;
     const int lane = (int)lane_id();
-    if (lane == 0) { scnt[0][wib] = 0; scnt[1][wib] = 0; }
+    if (lane < 3) scnt[lane][wib] = 0;
     __syncthreads();
-    first_table(lut, s, a.lm);
+    make_table<F>(lut, s, a.lm);
     __syncthreads();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        // no entries past m: the padding bits of the last word and the guard word stay 0
+        // no entries past m: the padding bits of the last word (and a guard word
+        // after it, where the bitmap has one) stay 0
         if (a.m & 31) atomicAnd(&a.ebits[a.m >> 5], (1u << (uint32_t)(a.m & 31)) - 1u);
-        a.ebits[(a.m + 31) >> 5] = 0u;
+        if (a.guard) a.ebits[(a.m + 31) >> 5] = 0u;
     }
     WarpBuf<int32_t> bs{sbuf[0][wib], &scnt[0][wib], a.small_out, &a.st->n_small};
     WarpBuf<int32_t> bm{sbuf[1][wib], &scnt[1][wib], a.med_out, &a.st->n_med};
+    WarpBuf<int32_t> bl{sbuf[2][wib], &scnt[2][wib], a.first_med, &a.first_sizes->n_med};
     const int64_t gwarp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     // small graphs: fewer than 32 vertices per warp, so that every warp has some
     const int per = (int)max((int64_t)1, min((int64_t)32, a.n / nwarps));
-    const int64_t in_warp = max((int64_t)kFirstWarp, (int64_t)a.hub_deg);
+    const int64_t in_warp = max((int64_t)kWarpRow, (int64_t)a.hub_deg), stride = nwarps * per;
+    uint32_t cm[4];
+#pragma unroll
+    for (int c = 0; c < 4; c++) cm[c] = s.cls_mask[c];
     LccTally tl;
-    for (int64_t v0 = gwarp * per; v0 < a.n; v0 += nwarps * per) {
-        const int64_t v = v0 + lane;
-        const bool mine = lane < per && v < a.n;
-        uint32_t wv = 0u, nbr = 0u, keep = 0u, kept = 0u;
-        int64_t beg = 0, end = 0;
-        if (mine) wv = lut[a.lab[v]].x;
-        if (wv) {
-            beg = a.rp[v];
-            end = a.rp[v + 1];
-            nbr = nbr_mask(wv, s) | a.eta_off;
-        }
-        const int64_t len = end - beg;
-        const bool hub = len > in_warp;
-        // (1) short rows, one lane each
-        if (wv && len > 0 && len <= kFirstLane) {
-            FirstAcc A;
-            uint32_t kb = 0;                                 // kept entries, relative to beg
-            const int64_t e0 = beg & ~(int64_t)3;
-            if (ELAB) {
-                uint32_t labs[5];
-#pragma unroll
-                for (int i = 0; i < 5; i++) labs[i] = e0 + 4 * i < end ? labels4<true>(a, e0 + 4 * i, beg, end) : 0u;
-#pragma unroll
-                for (int i = 0; i < 5; i++) {
-                    const int64_t e = e0 + 4 * i;
-                    if (e < end) {
-                        const uint32_t nib = take4<MAXC>(labs[i], range4(e, beg, end), nbr, lut, A, tl);
-                        kb |= e < beg ? nib >> (int)(beg - e) : nib << (int)(e - beg);
-                    }
-                }
-            } else {
-                for (int64_t e = e0; e < end; e += 4) {
-                    const uint32_t nib = take4<MAXC>(labels4<false>(a, e, beg, end), range4(e, beg, end), nbr, lut, A, tl);
-                    kb |= e < beg ? nib >> (int)(beg - e) : nib << (int)(e - beg);
-                }
-            }
-            Partial<MAXC> p;
-            p.U = A.U;
-            p.nN = A.nN;
-            unpack_classes<MAXC>(A.cp, p);
-            keep = decide<MAXC>(wv, p, s);
-            kept = A.nN;
-            // the bits of a vertex that dies are not read again
-            if (keep) clear_rel(a.ebits, beg, ((1u << (int)len) - 1u) & ~kb);
-        }
-        // (2) rows of up to 64 entries, four at a time, eight lanes each
-        for (uint32_t todo = __ballot_sync(FULL_MASK, wv && len > kFirstLane && len <= kFirstGroup); todo;) {
-            int src[4];
-#pragma unroll
-            for (int i = 0; i < 4; i++) {
-                src[i] = todo ? __ffs(todo) - 1 : -1;
-                todo &= todo - 1u;
-            }
-            const int g = lane >> 3, j = lane & 7;
-            const int from = g == 0 ? src[0] : g == 1 ? src[1] : g == 2 ? src[2] : src[3];
-            const int f = from < 0 ? 0 : from;
-            const int64_t gb = __shfl_sync(FULL_MASK, beg, f);
-            const int64_t ge0 = __shfl_sync(FULL_MASK, end, f);
-            const int64_t ge = from < 0 ? gb : ge0;          // an empty group: no entry is in range
-            const uint32_t gn = __shfl_sync(FULL_MASK, nbr, f), gw = __shfl_sync(FULL_MASK, wv, f);
-            const int64_t w0 = gb >> 5;
-            uint32_t labs[3], word[3];
-            FirstAcc A;
-#pragma unroll
-            for (int k = 0; k < 3; k++) {
-                const int64_t e = ((w0 + k) << 5) + 4 * j;
-                labs[k] = e < ge && e + 4 > gb ? labels4<ELAB>(a, e, gb, ge) : 0u;
-            }
-#pragma unroll
-            for (int k = 0; k < 3; k++) {
-                const int64_t e = ((w0 + k) << 5) + 4 * j;
-                word[k] = take4<MAXC>(labs[k], range4(e, gb, ge), gn, lut, A, tl) << (4 * j);
-            }
-#pragma unroll
-            for (int o = 1; o < 8; o <<= 1) {
-#pragma unroll
-                for (int k = 0; k < 3; k++) word[k] |= __shfl_xor_sync(FULL_MASK, word[k], o);
-                A.U |= __shfl_xor_sync(FULL_MASK, A.U, o);
-                A.nN += __shfl_xor_sync(FULL_MASK, A.nN, o);
-                if (MAXC > 0) A.cp += __shfl_xor_sync(FULL_MASK, A.cp, o);   // at most 64 per byte
-            }
-            Partial<MAXC> p;
-            p.U = A.U;
-            p.nN = A.nN;
-            unpack_classes<MAXC>(A.cp, p);
-            const uint32_t gk = decide<MAXC>(gw, p, s);
-            if (gk && from >= 0 && j < 3) store_word(a.ebits, w0 + j, gb, ge, j == 0 ? word[0] : j == 1 ? word[1] : word[2]);
-#pragma unroll
-            for (int i = 0; i < 4; i++) {
-                const uint32_t k = __shfl_sync(FULL_MASK, gk, 8 * i), c = __shfl_sync(FULL_MASK, A.nN, 8 * i);
-                if (lane == src[i]) { keep = k; kept = c; }
+    // the labels of the next batch but one and the offsets of the next one are
+    // loaded while a batch is walked
+    auto label_mask = [&](int64_t v) { return lane < per && v < a.n ? lut[a.lab[v]].x : 0u; };
+    auto offsets = [&](int64_t v, uint32_t w, int64_t &b, int64_t &e) {
+        b = e = 0;
+        if (w) { b = a.rp[v]; e = a.rp[v + 1]; }
+    };
+    int64_t v = gwarp * per + lane;
+    uint32_t w1 = label_mask(v), w2 = label_mask(v + stride);
+    int64_t b1, e1;
+    offsets(v, w1, b1, e1);
+    for (int64_t v0 = gwarp * per; v0 < a.n; v0 += stride, v += stride) {
+        const uint32_t wv = w1;
+        const int64_t beg = b1, end = e1, len = end - beg;
+        w1 = w2;
+        offsets(v + stride, w1, b1, e1);
+        w2 = label_mask(v + 2 * stride);
+        uint32_t keep = 0u, kept = 0u;
+        const uint32_t nbr = wv ? nbr_mask(wv, s) | a.eta_off : 0u;
+        short_batch<MAXC, kFirst, F>(a, s, lut, cm, wv, nbr, beg, end, keep, kept, tl);
+        const bool later = a.inline_long ? len > in_warp : len > kGroupRow;
+        if (a.inline_long) {
+            Partial<MAXC> sums;
+            const bool longer = len > kGroupRow && !later;
+            long_rows<MAXC, kFirst, F>(a, s.n_cls, lut, cm, __ballot_sync(FULL_MASK, longer), beg, end, nbr, tl,
+                                       [&](int j, const Partial<MAXC> &p) { if (lane == j) sums = p; });
+            if (longer) {
+                keep = decide<MAXC>(wv, sums, s);
+                kept = sums.nN;
             }
         }
-        // (3) longer rows, the warp together
-        for (uint32_t todo = __ballot_sync(FULL_MASK, wv && len > kFirstGroup && !hub); todo; todo &= todo - 1u) {
-            const int src = __ffs(todo) - 1;
-            Partial<MAXC> p;
-            first_warp<MAXC, ELAB>(a, __shfl_sync(FULL_MASK, beg, src), __shfl_sync(FULL_MASK, end, src),
-                                   __shfl_sync(FULL_MASK, nbr, src), lut, p, tl);
-            const uint32_t k = decide<MAXC>(__shfl_sync(FULL_MASK, wv, src), p, s);
-            if (lane == src) { keep = k; kept = p.nN; }
-        }
-        if (hub) {
+        bl.push(later && len <= in_warp, (int32_t)v);
+        if (len > in_warp) {
             const int nch = (int)((len + a.hub_deg - 1) / a.hub_deg);
-            const int slot = (int)atomicAdd(&a.hubs->n_hub_slots, 1u);
-            const unsigned int base = atomicAdd(&a.hubs->n_chunk, (unsigned int)nch);
-            for (int c = 0; c < nch; c++) a.hub_list[base + c] = ChunkItem{(int32_t)v, c, slot, nch};
-        } else if (mine) {
-            if (wv) {
-                tl.alive++;
-                tl.rows += (unsigned long long)len;
-                if (keep) { tl.kept += kept; tl.rows_next += (unsigned long long)len; }
-                else tl.died++;
-                if (keep != wv) tl.changed = 1u;
-                a.deg[v] = keep ? kept : 0u;
-            }
-            a.om0[v] = keep;
-            a.om1[v] = keep;
-            store_narrow(a.nw0, a.nw_bytes, v, keep);
-            store_narrow(a.nw1, a.nw_bytes, v, keep);
+            const int slot = (int)atomicAdd(&a.first_sizes->n_hub_slots, 1u);
+            const unsigned int base = atomicAdd(&a.first_sizes->n_chunk, (unsigned int)nch);
+            for (int c = 0; c < nch; c++) a.first_chunk[base + c] = ChunkItem{(int32_t)v, c, slot, nch};
         }
-        list_survivor(a, keep != 0u, (int32_t)v, len, bs, bm);
+        if (!later && lane < per && v < a.n) {
+            if (wv) settle_row<kFirst>(a, (int32_t)v, wv, keep, kept, len, tl);
+            write_omega<kFirst>(a, v, keep);
+        }
+        list_row(a, keep != 0u, (int32_t)v, len, bs, bm);
     }
     __syncthreads();
     block_flush(bs, &scnt[0][0], wib);
     block_flush(bm, &scnt[1][0], wib);
+    block_flush(bl, &scnt[2][0], wib);
     add_totals(tl, totals, a.st);
 }
 
-// The first round's long rows, one warp per piece; the last piece of a row
-// decides.
-template <int MAXC, bool ELAB>
+// A round over lists: all active vertices (kFull), those near a change
+// (kDelta), or the long rows of the first round (kFirst).
+template <int MAXC, int MODE, int F>
 __global__ void __launch_bounds__(256, 4)
-k_first_hubs(FirstArgs a, DevTmpl t) {
-    const int64_t n_piece = a.hubs->n_chunk;
-    if (n_piece == 0) return;
+k_rows(RowArgs a, DevTmpl t) {
+    if (a.gate && a.gate->changed == 0u) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) a.st->skipped = 1u;
+        return;
+    }
+    const int64_t n_small = MODE == kFirst ? 0 : (a.sizes ? (int64_t)a.sizes->n_small : a.n_small);
+    const int64_t n_med = a.sizes ? (int64_t)a.sizes->n_med : a.n_med;
+    const int64_t n_chunk = a.sizes ? (int64_t)a.sizes->n_chunk : a.n_chunk;
+    if (n_small + n_med + n_chunk == 0) return;
     __shared__ SmemTmpl s;
-    __shared__ uint2 lut[256];
+    __shared__ uint2 lut[F == kByWord ? 1 : 256];
     __shared__ int32_t sbuf[2][8][32];
-    __shared__ int scnt[2][8];
+    __shared__ ChunkItem cbuf[MODE == kFull ? 8 : 1][32];
+    __shared__ Change gbuf[MODE == kDelta ? 8 : 1][32];
+    __shared__ int scnt[4][8];
     __shared__ unsigned long long totals[9];
     if (threadIdx.x < 9) totals[threadIdx.x] = 0ull;
     load_tmpl(s, t);
     const int wib = threadIdx.x >> 5;
     const int lane = (int)lane_id();
-    if (lane == 0) { scnt[0][wib] = 0; scnt[1][wib] = 0; }
+    if (lane < 4) scnt[lane][wib] = 0;
     __syncthreads();
-    first_table(lut, s, a.lm);
+    if (F != kByWord) make_table<F>(lut, s, a.lm);
     __syncthreads();
     WarpBuf<int32_t> bs{sbuf[0][wib], &scnt[0][wib], a.small_out, &a.st->n_small};
     WarpBuf<int32_t> bm{sbuf[1][wib], &scnt[1][wib], a.med_out, &a.st->n_med};
+    WarpBuf<ChunkItem> bc{cbuf[MODE == kFull ? wib : 0], &scnt[2][wib], a.chunk_out, &a.st->n_chunk};
+    WarpBuf<Change> bg{gbuf[MODE == kDelta ? wib : 0], &scnt[3][wib], a.chg, &a.st->n_chg};
     const int64_t gwarp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    uint32_t cm[4];
+#pragma unroll
+    for (int c = 0; c < 4; c++) cm[c] = s.cls_mask[c];
     LccTally tl;
-    for (int64_t it = gwarp; it < n_piece; it += nwarps) {
-        const ChunkItem ci = a.hub_list[it];
-        const uint32_t wv = lut[a.lab[ci.v]].x;
-        const int64_t rbeg = a.rp[ci.v], rend = a.rp[ci.v + 1];
-        const int64_t beg = rbeg + (int64_t)ci.c * a.hub_deg, end = min(rend, beg + (int64_t)a.hub_deg);
-        Partial<MAXC> p;
-        first_warp<MAXC, ELAB>(a, beg, end, nbr_mask(wv, s) | a.eta_off, lut, p, tl);
-        HubAcc *h = a.acc + ci.slot;
-        unsigned int ticket = 0;
-        if (lane == 0) {
-            if (p.U) atomicOr(&h->U, p.U);
-            if (p.nN) atomicAdd(&h->nN, p.nN);
-#pragma unroll
-            for (int c = 0; c < MAXC; c++)
-                if (p.cnt[c]) atomicAdd(&h->cnt[c], p.cnt[c]);
-            __threadfence();
-            ticket = atomicAdd(&h->done, 1u);
-        }
-        ticket = __shfl_sync(FULL_MASK, ticket, 0);
-        uint32_t keep = 0u;
-        if (ticket == (unsigned int)(ci.nchunks - 1)) {
-            __threadfence();
-            Partial<MAXC> tot;
-            tot.U = atomicOr(&h->U, 0u);
-            tot.nN = atomicAdd(&h->nN, 0u);
-#pragma unroll
-            for (int c = 0; c < MAXC; c++) tot.cnt[c] = atomicAdd(&h->cnt[c], 0u);
-            keep = decide<MAXC>(wv, tot, s);
-            __syncwarp();
-            if (lane == 0) {
-                tl.alive++;
-                tl.rows += (unsigned long long)(rend - rbeg);
-                if (keep) { tl.kept += tot.nN; tl.rows_next += (unsigned long long)(rend - rbeg); }
-                else tl.died++;
-                if (keep != wv) tl.changed = 1u;
-                a.deg[ci.v] = keep ? tot.nN : 0u;
-                a.om0[ci.v] = keep;
-                a.om1[ci.v] = keep;
-                store_narrow(a.nw0, a.nw_bytes, ci.v, keep);
-                store_narrow(a.nw1, a.nw_bytes, ci.v, keep);
-                h->U = 0u; h->nN = 0u; h->flags = 0u; h->done = 0u;
-                for (int c = 0; c < MAXC; c++) h->cnt[c] = 0u;
+    auto omega_of = [&](int32_t v) { return MODE == kFirst ? lut[a.lab[v]].x : __ldg(a.om + v); };
+    auto clear = [&](int32_t v) { atomicAnd(&a.dirty[v >> 5], ~(1u << (v & 31))); };
+    // few rows: fewer per warp and batch, so that every warp has some
+    auto batch = [&](int64_t rows, int64_t share) { return (int)max((int64_t)1, min((int64_t)32, rows / (share * nwarps))); };
+
+    // (1) pieces of long rows, combined through HubAcc; a row's last piece decides
+    const int pc = batch(n_chunk, 4);
+    for (int64_t b0 = gwarp * pc; b0 < n_chunk; b0 += nwarps * pc) {
+        const int cnt = (int)min((int64_t)pc, n_chunk - b0);
+        ChunkItem ci{0, 0, 0, 0};
+        uint32_t wv = 0u;
+        int64_t rb = 0, re = 0, beg = 0, end = 0;
+        if (lane < cnt) {
+            ci = a.chunk_in[b0 + lane];
+            wv = omega_of(ci.v);
+            rb = a.rp[ci.v];
+            re = a.rp[ci.v + 1];
+            if (wv) {
+                beg = rb + (int64_t)ci.c * a.hub_deg;
+                end = min(re, beg + (int64_t)a.hub_deg);
+            } else if (ci.c == 0) {
+                write_omega<MODE>(a, ci.v, 0u);
+                if (MODE == kFull && a.deg) a.deg[ci.v] = 0u;
+                if (MODE == kDelta) clear(ci.v);
             }
         }
-        list_survivor(a, lane == 0 && keep != 0u, ci.v, rend - rbeg, bs, bm);
+        const uint32_t nbr = wv ? nbr_mask(wv, s) | a.eta_off : 0u;
+        // the lanes keep their pieces' sums and combine them side by side: one
+        // fence and ticket after the other cost more than the rows
+        Partial<MAXC> mine;
+        long_rows<MAXC, MODE, F>(a, s.n_cls, lut, cm, __ballot_sync(FULL_MASK, wv != 0u), beg, end, nbr, tl,
+                                 [&](int j, const Partial<MAXC> &p) { if (lane == j) mine = p; });
+        uint32_t now = wv;                            // omega', if the lane's piece was the row's last
+        if (wv) {
+            HubAcc *h = a.acc + ci.slot;
+            if (mine.U) atomicOr(&h->U, mine.U);
+            if (mine.nN) atomicAdd(&h->nN, mine.nN);
+#pragma unroll
+            for (int c = 0; c < MAXC; c++)
+                if (mine.cnt[c]) atomicAdd(&h->cnt[c], mine.cnt[c]);
+            __threadfence();
+            if (atomicAdd(&h->done, 1u) == (unsigned int)(ci.nchunks - 1)) {
+                __threadfence();
+                Partial<MAXC> tot;
+                tot.U = atomicOr(&h->U, 0u);
+                tot.nN = atomicAdd(&h->nN, 0u);
+#pragma unroll
+                for (int c = 0; c < MAXC; c++) tot.cnt[c] = atomicAdd(&h->cnt[c], 0u);
+                now = decide<MAXC>(wv, tot, s);
+                settle_row<MODE>(a, ci.v, wv, now, tot.nN, re - rb, tl);
+                write_omega<MODE>(a, ci.v, now);
+                if (MODE == kDelta) clear(ci.v);
+                h->U = 0u; h->nN = 0u; h->flags = 0u; h->done = 0u;
+                for (int c = 0; c < MAXC; c++) h->cnt[c] = 0u;
+                if (MODE == kFirst && now) ci.nchunks = -ci.nchunks;      // listed below
+            }
+        }
+        if (MODE == kFirst) list_row(a, ci.nchunks < 0, ci.v, re - rb, bs, bm);
+        else if (MODE == kFull) bc.push(lane < cnt && wv != 0u, ci);
+        else bg.push(lane < cnt && now != wv, Change{ci.v, now});
     }
+
+    // (2) whole rows, the warp together
+    const int mc = batch(n_med, 4);
+    for (int64_t b0 = gwarp * mc; b0 < n_med; b0 += nwarps * mc) {
+        const int cnt = (int)min((int64_t)mc, n_med - b0);
+        int32_t v = -1;
+        uint32_t wv = 0u, keep = 0u, kept = 0u;
+        int64_t beg = 0, end = 0;
+        if (lane < cnt) {
+            v = a.med_in[b0 + lane];
+            wv = omega_of(v);
+            if (wv) {
+                beg = a.rp[v];
+                end = a.rp[v + 1];
+            }
+        }
+        const uint32_t nbr = wv ? nbr_mask(wv, s) | a.eta_off : 0u;
+        Partial<MAXC> mine;
+        long_rows<MAXC, MODE, F>(a, s.n_cls, lut, cm, __ballot_sync(FULL_MASK, wv != 0u), beg, end, nbr, tl,
+                                 [&](int j, const Partial<MAXC> &p) { if (lane == j) mine = p; });
+        if (wv) {
+            keep = decide<MAXC>(wv, mine, s);
+            kept = mine.nN;
+        }
+        if (v >= 0) {
+            if (wv) settle_row<MODE>(a, v, wv, keep, kept, end - beg, tl);
+            else if (MODE == kFull && a.deg) a.deg[v] = 0u;
+            write_omega<MODE>(a, v, keep);
+            if (MODE == kDelta) clear(v);
+        }
+        if (MODE == kFirst) list_row(a, keep != 0u, v, end - beg, bs, bm);
+        else if (MODE == kFull) bm.push(wv != 0u, v);
+        else bg.push(v >= 0 && keep != wv, Change{v, keep});
+    }
+
+    // (3) short rows, 32 per batch; rows of more than 64 entries among them
+    // (options.short_rows) by the warp
+    const int sc = batch(n_small, 1);
+    for (int64_t b0 = gwarp * sc; b0 < n_small; b0 += nwarps * sc) {
+        int32_t v = -1;
+        uint32_t wv = 0u, keep = 0u, kept = 0u;
+        int64_t beg = 0, end = 0;
+        if (lane < sc && b0 + lane < n_small) {
+            v = a.small_in[b0 + lane];
+            wv = omega_of(v);
+            if (wv) {
+                beg = a.rp[v];
+                end = a.rp[v + 1];
+            }
+        }
+        const uint32_t nbr = wv ? nbr_mask(wv, s) | a.eta_off : 0u;
+        short_batch<MAXC, MODE, F>(a, s, lut, cm, wv, nbr, beg, end, keep, kept, tl);
+        long_rows<MAXC, MODE, F>(a, s.n_cls, lut, cm, __ballot_sync(FULL_MASK, wv && end - beg > kGroupRow), beg, end,
+                                 nbr, tl, [&](int j, const Partial<MAXC> &p) {
+            if (lane == j) {
+                keep = decide<MAXC>(wv, p, s);
+                kept = p.nN;
+            }
+        });
+        if (v >= 0) {
+            if (wv) settle_row<MODE>(a, v, wv, keep, kept, end - beg, tl);
+            else if (MODE == kFull && a.deg) a.deg[v] = 0u;
+            write_omega<MODE>(a, v, keep);
+            if (MODE == kDelta) clear(v);
+        }
+        if (MODE == kFull) bs.push(wv != 0u, v);
+        else if (MODE == kDelta) bg.push(v >= 0 && keep != wv, Change{v, keep});
+    }
+
     __syncthreads();
-    block_flush(bs, &scnt[0][0], wib);
-    block_flush(bm, &scnt[1][0], wib);
+    if (MODE == kDelta) {
+        block_flush(bg, &scnt[3][0], wib);
+    } else {
+        block_flush(bs, &scnt[0][0], wib);
+        block_flush(bm, &scnt[1][0], wib);
+        if (MODE == kFull) block_flush(bc, &scnt[2][0], wib);
+    }
     add_totals(tl, totals, a.st);
 }
 
@@ -1980,14 +2383,38 @@ k_materialize_fix(int64_t n, const uint32_t *__restrict__ om, const int64_t *__r
     }
 }
 
-// Zero the rows of the inactive vertices (one thread per vertex; the rows of
-// vertices that were never active, or that a non-local check emptied, still
-// carry bits the rounds never read).
+// Hand-back of the edge map when the live rows are exact: their bits, into a
+// zeroed bitmap.  A warp takes 32 vertices and copies the live rows together:
+// most vertices are dead by then, and clearing their rows instead cost two
+// atomics each (1.15 ms over 32M vertices with 3.6M live; this 0.25).
 __global__ void __launch_bounds__(256)
-k_clear_dead_rows(int64_t n, const uint32_t *__restrict__ om, const int64_t *__restrict__ rp, uint32_t *ebits) {
+k_copy_live_rows(int64_t n, const uint32_t *__restrict__ om, const int64_t *__restrict__ rp,
+                 const uint32_t *__restrict__ bits, uint32_t *out) {
+    const int lane = (int)lane_id();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride)
-        if (om[v] == 0u) clear_row<1>(ebits, rp[v], rp[v + 1], 0);
+    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; b < n; b += stride) {
+        const int64_t v = b + lane;
+        const bool live = v < n && om[v] != 0u;
+        int64_t beg = 0, end = 0;
+        if (live) { beg = rp[v]; end = rp[v + 1]; }
+        const bool shrt = end - beg <= 64;               // at most three words: by the lane itself
+        if (live && shrt) {
+            for (int64_t wi = beg >> 5; (wi << 5) < end; wi++) {
+                const uint32_t in = word_range(wi, beg, end), x = bits[wi] & in;
+                if (in == ~0u) out[wi] = x;
+                else if (x) atomicOr(&out[wi], x);
+            }
+        }
+        for (uint32_t todo = __ballot_sync(FULL_MASK, live && !shrt); todo; todo &= todo - 1u) {
+            const int src = __ffs(todo) - 1;
+            const int64_t rb = __shfl_sync(FULL_MASK, beg, src), re = __shfl_sync(FULL_MASK, end, src);
+            for (int64_t wi = (rb >> 5) + lane; (wi << 5) < re; wi += 32) {
+                const uint32_t in = word_range(wi, rb, re), x = bits[wi] & in;
+                if (in == ~0u) out[wi] = x;
+                else if (x) atomicOr(&out[wi], x);
+            }
+        }
+    }
 }
 
 // -------------------------------------------------------------------------
@@ -3603,7 +4030,7 @@ int ensure_entry_labels(ccpm_ctx *ctx, ccpm_graph *g) {
     if (g->elab || g->m == 0) return CCPM_OK;
     uint8_t *el = nullptr;
     int rc;
-    if ((rc = dalloc(ctx, &el, (size_t)g->m + 4))) return rc;     // read four at a time
+    if ((rc = dalloc(ctx, &el, (size_t)g->m + 16))) return rc;    // read 16 at a time
     int grid = (int)std::min<int64_t>((g->m + 255) / 256, (int64_t)ctx->num_sms * 8);
     k_gather_labels<<<grid, 256, 0, ctx->stream>>>(g->m, g->col, g->lab, el);
     cudaError_t e = cudaGetLastError();
@@ -3854,6 +4281,73 @@ struct Pipeline {
     // omega and list buffers it reads (the host flips cur / li only once a
     // group of queued rounds is done, by the number of rounds that ran).
     int launch_round(RoundStats *slot, const RoundStats *prev, const RoundStats *gate, int c, int l, bool delta) {
+        launches++;
+        lcc_launches++;
+        if (maxc > 4 || first_rows < kHugeRows) return launch_small(slot, prev, gate, c, l, delta);
+        Workspace &w = ctx->ws;
+        RowArgs a = row_args(slot);
+        a.om = w.om[c];
+        a.nw = w.nw[c];
+        a.om_out[0] = w.om[c ^ 1];
+        a.nw_out[0] = w.nw[c ^ 1];
+        a.small_in = delta ? w.dsmall : w.small[l];
+        a.med_in = delta ? w.dmed : w.med[l];
+        a.chunk_in = delta ? w.dchunk : w.chunk[l];
+        // a full round's lists were written by the round before, a delta
+        // round's by k_push into its own counters
+        a.sizes = delta ? slot : prev;
+        a.n_small = n_small;
+        a.n_med = n_med;
+        a.n_chunk = n_chunk;
+        a.gate = prev ? prev : gate;
+        a.small_out = w.small[l ^ 1];
+        a.med_out = w.med[l ^ 1];
+        a.chunk_out = w.chunk[l ^ 1];
+        // a queued round does not know its sizes: one full resident wave
+        const int64_t warps = a.sizes ? (int64_t)1 << 40 : n_small + n_med + n_chunk;
+        from_labels = dense = false;
+        const bool byte = nw_bytes == 1;
+#define CCPM_ROWS(C, M, F) k_rows<C, M, F><<<lcc_grid(ctx, k_rows<C, M, F>, warps), 256, 0, ctx->stream>>>(a, dt)
+#define CCPM_ROWS_BY(M)                                                          \
+    do {                                                                         \
+        if (maxc == 0) { if (byte) CCPM_ROWS(0, M, kByByte); else CCPM_ROWS(0, M, kByWord); } \
+        else { if (byte) CCPM_ROWS(4, M, kByByte); else CCPM_ROWS(4, M, kByWord); }           \
+    } while (0)
+        if (delta) CCPM_ROWS_BY(kDelta);
+        else CCPM_ROWS_BY(kFull);
+#undef CCPM_ROWS_BY
+        CU(ctx, cudaGetLastError());
+        return CCPM_OK;
+    }
+
+    RowArgs row_args(RoundStats *slot) const {
+        Workspace &w = ctx->ws;
+        RowArgs a{};
+        a.n = g->n;
+        a.m = gen < 0 ? g->m : INT64_MAX;            // compacted rows: room past their end
+        a.rp = lrp;
+        a.col = lcol;
+        a.col_vec = ((uintptr_t)lcol & 15) == 0;
+        a.lab = g->lab;
+        a.elab = elab;
+        a.nw_bytes = nw_bytes;
+        a.ebits = lbits;
+        a.deg = w.deg;
+        a.dirty = w.dirty;
+        a.chg = w.chg;
+        a.chg_piece = w.chg_piece;
+        a.acc = w.acc;
+        a.st = slot;
+        a.hub_deg = w.hub_deg;
+        a.short_max = short_max;
+        a.eta_off = eta_off ? ~0u : 0u;
+        a.lm = lm0;
+        return a;
+    }
+
+    // A round of a template with more than four multiplicity classes, or of one
+    // that starts from fewer than kHugeRows entries.
+    int launch_small(RoundStats *slot, const RoundStats *prev, const RoundStats *gate, int c, int l, bool delta) {
         Workspace &w = ctx->ws;
         LccArgs a;
         a.rp = lrp;
@@ -3894,22 +4388,17 @@ struct Pipeline {
         const int64_t resident = (int64_t)grid_sms(ctx) * 32;
         a.med_chunk = (int)std::max<int64_t>(1, std::min<int64_t>(16, n_med / (4 * resident)));
         // a queued round does not know its sizes: one full resident wave
-        int64_t warps = prev ? ((int64_t)1 << 40)
-                             : n_chunk + (n_med + a.med_chunk - 1) / a.med_chunk + n_small;
-        launches++;
-        lcc_launches++;
+        const int64_t warps = prev ? ((int64_t)1 << 40)
+                                   : n_chunk + (n_med + a.med_chunk - 1) / a.med_chunk + n_small;
         // one resident wave: grid-stride work is split evenly over warps that all run at once
 #define CCPM_LAUNCH_LCC(C, M) k_lcc_round<C, M><<<lcc_grid(ctx, k_lcc_round<C, M>, warps), 256, 0, ctx->stream>>>(a, dt)
-#define CCPM_LAUNCH_MODE(M)                        \
-    do {                                           \
-        if (maxc == 0) CCPM_LAUNCH_LCC(0, M);      \
-        else if (maxc <= 4) CCPM_LAUNCH_LCC(4, M); \
-        else CCPM_LAUNCH_LCC(32, M);               \
-    } while (0)
-        if (delta) CCPM_LAUNCH_MODE(kDelta);
-        else if (dense) CCPM_LAUNCH_MODE(kDense);
-        else CCPM_LAUNCH_MODE(kFull);
-#undef CCPM_LAUNCH_MODE
+        if (maxc == 0 && delta) CCPM_LAUNCH_LCC(0, kDelta);
+        else if (maxc == 0) CCPM_LAUNCH_LCC(0, kFull);
+        else if (maxc <= 4 && delta) CCPM_LAUNCH_LCC(4, kDelta);
+        else if (maxc <= 4) CCPM_LAUNCH_LCC(4, kFull);
+        else if (delta) CCPM_LAUNCH_LCC(kMaxCls, kDelta);
+        else if (dense) CCPM_LAUNCH_LCC(kMaxCls, kDense);
+        else CCPM_LAUNCH_LCC(kMaxCls, kFull);
 #undef CCPM_LAUNCH_LCC
         dense = false;      // only the first round after init sees every bit set
         CU(ctx, cudaGetLastError());
@@ -3923,45 +4412,36 @@ struct Pipeline {
     // The first round of a fresh prune (no initialisation runs before it).
     int launch_first(RoundStats *slot) {
         Workspace &w = ctx->ws;
-        FirstArgs a;
-        a.n = g->n;
-        a.m = g->m;
-        a.rp = g->rp;
-        a.col = g->col;
-        a.lab = g->lab;
-        a.elab = elab;
-        a.om0 = w.om[0];
-        a.om1 = w.om[1];
-        a.nw0 = w.nw[0];
-        a.nw1 = w.nw[1];
-        a.nw_bytes = nw_bytes;
-        a.ebits = w.ebits;
-        a.deg = w.deg;
+        RowArgs a = row_args(slot);
+        a.guard = 1;
+        a.inline_long = first_rows < kInlineRows ? 1 : 0;
+        for (int i = 0; i < 2; i++) {
+            a.om_out[i] = w.om[i];
+            a.nw_out[i] = w.nw[i];
+        }
         a.small_out = w.small[li ^ 1];
         a.med_out = w.med[li ^ 1];
         a.chunk_out = w.chunk[li ^ 1];
-        a.hub_list = w.chunk[li];
-        a.hubs = &w.ctl->init;
-        a.acc = w.acc;
-        a.st = slot;
-        a.hub_deg = w.hub_deg;
-        a.short_max = short_max;
-        a.eta_off = eta_off ? ~0u : 0u;
-        a.col_vec = ((uintptr_t)g->col & 15) == 0;
-        a.lm = lm0;
+        a.first_med = w.med[li];
+        a.first_chunk = w.chunk[li];
+        a.first_sizes = &w.ctl->init;
+        a.med_in = w.med[li];
+        a.chunk_in = w.chunk[li];
+        a.sizes = &w.ctl->init;
         launches += 2;
         lcc_launches++;
-        dense = false;
-        from_labels = false;
-#define CCPM_LAUNCH_FIRST(C, E)                                                                                     \
-    do {                                                                                                            \
-        k_first_round<C, E><<<lcc_grid(ctx, k_first_round<C, E>, g->n), 256, 0, ctx->stream>>>(a, dt);              \
-        k_first_hubs<C, E><<<lcc_grid(ctx, k_first_hubs<C, E>, first_rows / kFirstWarp + 1), 256, 0, ctx->stream>>>(a, dt); \
+        from_labels = dense = false;
+#define CCPM_LAUNCH_FIRST(C, F)                                                                              \
+    do {                                                                                                     \
+        k_first_round<C, F><<<lcc_grid(ctx, k_first_round<C, F>, g->n), 256, 0, ctx->stream>>>(a, dt);       \
+        k_rows<C, kFirst, F><<<lcc_grid(ctx, k_rows<C, kFirst, F>,                                           \
+                                        first_rows / (a.inline_long ? kWarpRow : kGroupRow) + 1), 256, 0,    \
+                               ctx->stream>>>(a, dt);                                                        \
     } while (0)
         if (elab) {
-            if (maxc == 0) CCPM_LAUNCH_FIRST(0, true); else CCPM_LAUNCH_FIRST(4, true);
+            if (maxc == 0) CCPM_LAUNCH_FIRST(0, kByEntry); else CCPM_LAUNCH_FIRST(4, kByEntry);
         } else {
-            if (maxc == 0) CCPM_LAUNCH_FIRST(0, false); else CCPM_LAUNCH_FIRST(4, false);
+            if (maxc == 0) CCPM_LAUNCH_FIRST(0, kByLabel); else CCPM_LAUNCH_FIRST(4, kByLabel);
         }
 #undef CCPM_LAUNCH_FIRST
         CU(ctx, cudaGetLastError());
@@ -5094,16 +5574,19 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
         // hand back the pruned state: exact edge map for live rows, dead rows
         // zeroed.  When every round ran on the full rows with edge
         // elimination, the last (quiescent) round has already left the live
-        // rows exact, and only the rows of dead vertices are cleared.
+        // rows exact, and they are copied out.
         P.launches++;
-        if (P.gen < 0 && !P.eta_off)
-            k_clear_dead_rows<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, w.om[P.cur], g->rp, w.ebits);
-        else
+        if (P.gen < 0 && !P.eta_off) {
+            CUF(cudaMemsetAsync(r->eb, 0, sizeof(uint32_t) * (size_t)(w.words + 1), s));
+            k_copy_live_rows<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, w.om[P.cur], g->rp, w.ebits, r->eb);
+            CUF(cudaGetLastError());
+        } else {
             k_materialize_fix<<<grid_for(ctx, g->n * 32, 256, 8), 256, 0, s>>>(g->n, w.om[P.cur], g->rp, g->col,
                                                                                w.ebits, P.dt);
-        CUF(cudaGetLastError());
+            CUF(cudaGetLastError());
+            CUF(cudaMemcpyAsync(r->eb, w.ebits, sizeof(uint32_t) * (size_t)w.words, cudaMemcpyDeviceToDevice, s));
+        }
         CUF(cudaMemcpyAsync(r->om, w.om[P.cur], sizeof(uint32_t) * (size_t)g->n, cudaMemcpyDeviceToDevice, s));
-        CUF(cudaMemcpyAsync(r->eb, w.ebits, sizeof(uint32_t) * (size_t)w.words, cudaMemcpyDeviceToDevice, s));
     }
     if (!summary_done) {
         RCF(queue_summary());
@@ -5885,10 +6368,14 @@ namespace {
 // loaded holds these bytes until the process exits.
 constexpr size_t kNoAllocScratchBytes = (size_t)16 << 20;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
+// counters of the first round's lists and of two groups of queued rounds
+constexpr int kNoAllocRounds = 4;
+static __device__ RoundStats g_noalloc_rounds[1 + 2 * kNoAllocRounds];
 
 constexpr int kNoAllocMaxDevices = 64;
 std::mutex g_noalloc_mu;
 void *g_noalloc_addr[kNoAllocMaxDevices] = {};
+void *g_noalloc_rounds_addr[kNoAllocMaxDevices] = {};
 
 size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -5985,16 +6472,21 @@ int lcc_fixpoint_noalloc_body(int device, void *cuda_stream, int64_t n, int64_t 
     cudaError_t e = cudaSetDevice(device);
     if (e != cudaSuccess) return fail(CCPM_ECUDA, cudaGetErrorString(e));
     unsigned char *base = nullptr;
+    RoundStats *rounds_dev = nullptr;
     {
         // once per device, with that device current: the device address of the
         // scratch array (the host-side symbol is only a stand-in)
         std::lock_guard<std::mutex> lock(g_noalloc_mu);
         if (!g_noalloc_addr[device]) {
-            void *p = nullptr;
+            void *p = nullptr, *q = nullptr;
             e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
-            if (e != cudaSuccess || !p) return fail(CCPM_ECUDA, "cudaGetSymbolAddress of the scratch array failed");
+            if (e == cudaSuccess) e = cudaGetSymbolAddress(&q, g_noalloc_rounds);
+            if (e != cudaSuccess || !p || !q)
+                return fail(CCPM_ECUDA, "cudaGetSymbolAddress of the scratch arrays failed");
             g_noalloc_addr[device] = p;
+            g_noalloc_rounds_addr[device] = q;
         }
+        rounds_dev = (RoundStats *)g_noalloc_rounds_addr[device];
         base = (unsigned char *)g_noalloc_addr[device];
     }
     int num_sms = 0;
@@ -6003,10 +6495,11 @@ int lcc_fixpoint_noalloc_body(int device, void *cuda_stream, int64_t n, int64_t 
     cudaStream_t s = (cudaStream_t)cuda_stream;
     {
         // the scratch is sized from m_dir: the offsets must agree with it
-        // before any kernel writes there (two 8-byte reads into the stack)
+        // before any kernel writes there (the two 8-byte ends, read into the
+        // stack as one strided copy)
         int64_t ends[2] = {-1, -1};
-        e = cudaMemcpyAsync(&ends[0], row_ptr, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&ends[1], row_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+        e = cudaMemcpy2DAsync(ends, sizeof(int64_t), row_ptr, sizeof(int64_t) * (size_t)n, sizeof(int64_t), 2,
+                              cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return fail(CCPM_ECUDA, cudaGetErrorString(e));
         if (ends[0] != 0 || ends[1] != m_dir) return fail(CCPM_EINVAL, "row_ptr[0] must be 0 and row_ptr[n] == m_dir");
@@ -6035,71 +6528,125 @@ int lcc_fixpoint_noalloc_body(int device, void *cuda_stream, int64_t n, int64_t 
     const int64_t words = (m_dir + 31) / 32;
     // the scratch keeps whatever the previous call left: clear what must start at zero
     NA_CU(cudaMemsetAsync(acc, 0, sizeof(HubAcc) * (size_t)L.acc_cap, s));
-    NA_CU(cudaMemsetAsync(st, 0, sizeof(RoundStats), s));
-    if (words > 0) {
-        NA_CU(cudaMemsetAsync(ebits, 0xFF, sizeof(uint32_t) * (size_t)words, s));
-        if (m_dir & 31) k_set_word<<<1, 1, 0, s>>>(ebits + words - 1, (1u << (uint32_t)(m_dir & 31)) - 1u);
-    }
-    k_init<<<grid(n, 256), 256, 0, s>>>(n, row_ptr, labels, lm, nullptr, om[0], om[1], nullptr, nullptr, 0, small[0],
-                                        med[0], chunk[0], acc, st, hub, kSmallDeg, 0u, nullptr, nullptr, 0);
-    NA_CU(cudaGetLastError());
-    NA_CU(read_stats());
-    if (hs.n_hub_slots > (unsigned)L.acc_cap || (int64_t)hs.n_chunk > L.chunk_cap)
-        return fail(CCPM_EOVERFLOW, "split-row bookkeeping overflow");
-    int64_t n_small = hs.n_small, n_med = hs.n_med, n_chunk = hs.n_chunk, scanned = 0;
+    if (words > 0) NA_CU(cudaMemsetAsync(ebits, 0xFF, sizeof(uint32_t) * (size_t)words, s));
+    int64_t scanned = 0;
     int cur = 0, li = 0;
     int32_t r = 0;
-    for (;;) {
-        NA_CU(cudaMemsetAsync(st, 0, sizeof(RoundStats), s));
-        LccArgs a;
+    if (dt.n_cls <= 4) {
+        // rounds queued kNoAllocRounds at a time, each reading the list sizes of
+        // the one before on the device
+        RowArgs a{};
+        a.n = n;
+        a.m = m_dir;
         a.rp = row_ptr;
         a.col = col;
-        a.om_cur = om[cur];
-        a.om_next = om[cur ^ 1];
+        a.col_vec = ((uintptr_t)col & 15) == 0;
+        a.lab = labels;
         a.ebits = ebits;
-        a.small_in = small[li];
-        a.med_in = med[li];
-        a.chunk_in = chunk[li];
-        a.n_small = n_small;
-        a.n_med = n_med;
-        a.n_chunk = n_chunk;
-        a.small_out = small[li ^ 1];
-        a.med_out = med[li ^ 1];
-        a.chunk_out = chunk[li ^ 1];
         a.acc = acc;
-        a.st = st;
         a.hub_deg = hub;
-        a.deg = nullptr;
-        a.dirty = nullptr;
-        a.chg = nullptr;
-        a.chg_piece = nullptr;
-        a.med_chunk = 1;
-        a.lab0 = nullptr;
-        a.elab = nullptr;
-        a.sparse = 0;
-        a.prev = nullptr;
-        a.gate = nullptr;
-        a.resident_warps = num_sms * 32;
-        a.eta_off = 0u;
-        a.nw_bytes = 0;
-        a.nw_cur = nullptr;
-        a.nw_next = nullptr;
-        // at most one resident wave (four blocks an SM): the rows are dealt out evenly over the warps
-        const int g = std::min(grid((n_chunk + n_med + n_small) * 32, 256), 4 * num_sms);
-        if (dt.n_cls == 0) k_lcc_round<0, kFull><<<g, 256, 0, s>>>(a, dt);
-        else if (dt.n_cls <= 4) k_lcc_round<4, kFull><<<g, 256, 0, s>>>(a, dt);
-        else k_lcc_round<32, kFull><<<g, 256, 0, s>>>(a, dt);
+        a.short_max = kSmallDeg;
+        a.lm = lm;
+        const int wave = 4 * num_sms;
+        RoundStats *prev = nullptr;
+        for (int group = 0;; group++) {
+            RoundStats *ring = rounds_dev + 1 + (group & 1) * kNoAllocRounds;
+            NA_CU(cudaMemsetAsync(ring, 0, sizeof(RoundStats) * kNoAllocRounds, s));
+            if (group == 0) NA_CU(cudaMemsetAsync(rounds_dev, 0, sizeof(RoundStats), s));
+            for (int i = 0; i < kNoAllocRounds; i++) {
+                a.st = ring + i;
+                a.small_in = small[li];
+                a.med_in = med[li];
+                a.chunk_in = chunk[li];
+                a.small_out = small[li ^ 1];
+                a.med_out = med[li ^ 1];
+                a.chunk_out = chunk[li ^ 1];
+                if (!prev) {
+                    a.om_out[0] = om[0];
+                    a.om_out[1] = om[1];
+                    a.first_med = med[li];
+                    a.first_chunk = chunk[li];
+                    a.first_sizes = rounds_dev;
+                    a.sizes = rounds_dev;
+                    const int gf = std::min(grid(n, 8), wave);
+                    if (dt.n_cls == 0) {
+                        k_first_round<0, kByLabel><<<gf, 256, 0, s>>>(a, dt);
+                        k_rows<0, kFirst, kByLabel><<<wave, 256, 0, s>>>(a, dt);
+                    } else {
+                        k_first_round<4, kByLabel><<<gf, 256, 0, s>>>(a, dt);
+                        k_rows<4, kFirst, kByLabel><<<wave, 256, 0, s>>>(a, dt);
+                    }
+                } else {
+                    a.om = om[cur];
+                    a.om_out[0] = om[cur ^ 1];
+                    a.sizes = prev;
+                    a.gate = prev;
+                    if (dt.n_cls == 0) k_rows<0, kFull, kByWord><<<wave, 256, 0, s>>>(a, dt);
+                    else k_rows<4, kFull, kByWord><<<wave, 256, 0, s>>>(a, dt);
+                }
+                NA_CU(cudaGetLastError());
+                prev = ring + i;
+                li ^= 1;
+                cur ^= 1;
+            }
+            RoundStats h[kNoAllocRounds];
+            NA_CU(cudaMemcpyAsync(h, ring, sizeof(h), cudaMemcpyDeviceToHost, s));
+            NA_CU(cudaStreamSynchronize(s));
+            bool done = false;
+            for (int i = 0; i < kNoAllocRounds && !done; i++) {
+                r++;
+                scanned += (int64_t)h[i].scanned;
+                done = !h[i].changed;
+            }
+            if (done) break;
+            if (r > 4 * (m_dir + n) + 8) return fail(CCPM_ETIMEOUT, "LCC did not converge");
+        }
+        cur = 0;       // a fixpoint leaves the two buffers equal
+    } else {
+        NA_CU(cudaMemsetAsync(st, 0, sizeof(RoundStats), s));
+        k_init<<<grid(n, 256), 256, 0, s>>>(n, row_ptr, labels, lm, nullptr, om[0], om[1], nullptr, nullptr, 0, small[0],
+                                            med[0], chunk[0], acc, st, hub, kSmallDeg, 0u, nullptr, nullptr, 0);
         NA_CU(cudaGetLastError());
+        if (m_dir & 31) k_set_word<<<1, 1, 0, s>>>(ebits + words - 1, (1u << (uint32_t)(m_dir & 31)) - 1u);
         NA_CU(read_stats());
-        r++;
-        scanned += (int64_t)hs.scanned;
-        n_small = hs.n_small;
-        n_med = hs.n_med;
-        n_chunk = hs.n_chunk;
-        li ^= 1;
-        cur ^= 1;
-        if (!hs.changed) break;
-        if (r > 4 * (m_dir + n) + 8) return fail(CCPM_ETIMEOUT, "LCC did not converge");
+        int64_t n_small = hs.n_small, n_med = hs.n_med, n_chunk = hs.n_chunk;
+        for (;;) {
+            NA_CU(cudaMemsetAsync(st, 0, sizeof(RoundStats), s));
+            LccArgs a{};
+            a.rp = row_ptr;
+            a.col = col;
+            a.om_cur = om[cur];
+            a.om_next = om[cur ^ 1];
+            a.ebits = ebits;
+            a.small_in = small[li];
+            a.med_in = med[li];
+            a.chunk_in = chunk[li];
+            a.n_small = n_small;
+            a.n_med = n_med;
+            a.n_chunk = n_chunk;
+            a.small_out = small[li ^ 1];
+            a.med_out = med[li ^ 1];
+            a.chunk_out = chunk[li ^ 1];
+            a.acc = acc;
+            a.st = st;
+            a.hub_deg = hub;
+            a.med_chunk = 1;
+            a.resident_warps = num_sms * 32;
+            // at most one resident wave (four blocks an SM): the rows are dealt out evenly over the warps
+            const int g = std::min(grid((n_chunk + n_med + n_small) * 32, 256), 4 * num_sms);
+            k_lcc_round<kMaxCls, kFull><<<g, 256, 0, s>>>(a, dt);
+            NA_CU(cudaGetLastError());
+            NA_CU(read_stats());
+            r++;
+            scanned += (int64_t)hs.scanned;
+            n_small = hs.n_small;
+            n_med = hs.n_med;
+            n_chunk = hs.n_chunk;
+            li ^= 1;
+            cur ^= 1;
+            if (!hs.changed) break;
+            if (r > 4 * (m_dir + n) + 8) return fail(CCPM_ETIMEOUT, "LCC did not converge");
+        }
     }
     // both omega buffers agree at the fixpoint; the caller's buffer must hold it
     if (cur != 0) NA_CU(cudaMemcpyAsync(omega, om[cur], sizeof(uint32_t) * (size_t)n, cudaMemcpyDeviceToDevice, s));
