@@ -11,6 +11,7 @@
 // across the batch are FP32.  The backward products (dW2 = H1^T dZ2,
 // dZ1 = dZ2 W2^T, dW1 = X^T dZ1) round their operands (H1, dZ2, W2, X, dZ1)
 // to BF16 the same way.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -268,13 +269,351 @@ __global__ void k_mlp_adam(float *prm, float *grad, float *m1, float *m2, int st
 }
 
 // Minibatch row indices from a counter-based hash (SplitMix64 finaliser).
+__device__ __forceinline__ int32_t sample_row(int batch, int n, uint64_t seed, int step, int i) {
+    uint64_t z = seed + 0x9E3779B97F4A7C15ull * (uint64_t)((int64_t)step * batch + i + 1);
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    z ^= z >> 31;
+    return (int32_t)(z % (uint64_t)n);
+}
+
 __global__ void k_mlp_sample(int32_t *idx, int batch, int n, uint64_t seed, int step) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < batch; i += gridDim.x * blockDim.x) {
-        uint64_t z = seed + 0x9E3779B97F4A7C15ull * (uint64_t)((int64_t)step * batch + i + 1);
-        z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-        z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-        z ^= z >> 31;
-        idx[i] = (int32_t)(z % (uint64_t)n);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < batch; i += gridDim.x * blockDim.x)
+        idx[i] = sample_row(batch, n, seed, step, i);
+}
+
+// ------------------------------------------------------------- training loop
+//
+// All Adam steps of a training call in one kernel, one thread-block cluster.
+// A step is a chain of small products and reductions, so its time is latency:
+// as three kernels and a memset (sampling, backward over 64-row blocks with
+// atomics into one gradient, Adam) it took 37 us at 256 rows, 28 of them in the
+// backward kernel with its scalar fragment loads.  Here a block holds the weights in
+// shared memory (bf16, as the products want them) and 32 rows at a time; warp w
+// owns columns 8w..8w+7 of both hidden layers, so activations stay in the
+// registers they were computed in and every gradient of those columns ends up
+// in that warp; fragments are loaded with ldmatrix.  The blocks' gradients are
+// summed slice by slice through distributed shared memory, in rank order (so
+// two runs give the same bits), the slice's owner does its Adam step on FP32
+// masters and writes the new weights to all blocks: two cluster barriers a
+// step, 5.9 us.  Always eight blocks, since the Adam step is split over them too:
+// with one block for 32 rows a step took 25 us.
+
+namespace cg = cooperative_groups;
+
+constexpr int TR = 32;             // rows per block and chunk
+constexpr int TTHREADS = 256;      // 8 warps
+constexpr int LDH = HID + 8, LDX = IN + 8;     // row strides: ldmatrix rows on distinct banks
+constexpr int kTrainCluster = 8;   // blocks
+constexpr int kTrainMaxBatch = 4096;   // rows up to which the fused loop is used
+
+struct TrainSmem {
+    alignas(16) __nv_bfloat16 w1[IN * LDH], w2[HID * LDH];
+    alignas(16) __nv_bfloat16 x[TR * LDX], h1[TR * LDH], dz2[TR * LDH], dz1[TR * LDH];
+    float b1[HID], b2[HID], w3[HID], b3;
+    float t[TR], dy[TR];
+    float ypart[TR][HID / 8 + 1];
+    float grad[NPARAM];
+    float corr[2];                 // Adam's bias corrections of this step
+    float sse;
+};
+
+struct TrainArgs {
+    float *prm, *m1, *m2, *sse;
+    const float *X, *T;
+    int N, batch, rows;            // rows: per block
+    int steps, step0, adam0;       // steps of this launch, sampling steps and Adam steps before it
+    uint64_t seed;
+    float lr;
+};
+
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+template <bool TRANS>
+__device__ __forceinline__ void ldm4(uint32_t (&r)[4], const void *p) {
+    if (TRANS)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_addr(p)) : "memory");
+    else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_addr(p)) : "memory");
+}
+template <bool TRANS>
+__device__ __forceinline__ void ldm2(uint32_t (&r)[2], const void *p) {
+    if (TRANS)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];"
+                     : "=r"(r[0]), "=r"(r[1]) : "r"(smem_addr(p)) : "memory");
+    else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];"
+                     : "=r"(r[0]), "=r"(r[1]) : "r"(smem_addr(p)) : "memory");
+}
+__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
+        "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+
+// Fragments of a 16 x 16 A tile / a 16 x 8 B tile.  M: row-major matrix with row
+// stride ld holding A (rows m, columns k) or A^T; B (rows k, columns n) or B^T.
+__device__ __forceinline__ void frag_a(uint32_t (&r)[4], const __nv_bfloat16 *M, int ld, int m0, int k0) {
+    const int l = threadIdx.x & 31;
+    ldm4<false>(r, M + (m0 + (l & 15)) * ld + k0 + 8 * (l >> 4));
+}
+__device__ __forceinline__ void frag_at(uint32_t (&r)[4], const __nv_bfloat16 *M, int ld, int m0, int k0) {
+    const int l = threadIdx.x & 31;     // tiles in the order (m, k), (m + 8, k), (m, k + 8), (m + 8, k + 8)
+    ldm4<true>(r, M + (k0 + (l & 7) + 8 * (l >> 4)) * ld + m0 + 8 * ((l >> 3) & 1));
+}
+__device__ __forceinline__ void frag_b(uint32_t (&r)[2], const __nv_bfloat16 *M, int ld, int k0, int n0) {
+    const int l = threadIdx.x & 15;
+    ldm2<true>(r, M + (k0 + l) * ld + n0);
+}
+__device__ __forceinline__ void frag_bt(uint32_t (&r)[2], const __nv_bfloat16 *M, int ld, int k0, int n0) {
+    const int l = threadIdx.x & 15;
+    ldm2<false>(r, M + (n0 + (l & 7)) * ld + k0 + 8 * (l >> 3));
+}
+
+// Sum over the eight row groups of a fragment column.
+__device__ __forceinline__ float col_sum(float x) {
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
+    return x;
+}
+
+// New value of parameter i in a block's working copy.
+__device__ __forceinline__ void put_param(TrainSmem &S, int i, float v) {
+    if (i < OFF_B1) S.w1[(i / HID) * LDH + i % HID] = __float2bfloat16_rn(v);
+    else if (i < OFF_W2) S.b1[i - OFF_B1] = v;
+    else if (i < OFF_B2) S.w2[((i - OFF_W2) / HID) * LDH + (i - OFF_W2) % HID] = __float2bfloat16_rn(v);
+    else if (i < OFF_W3) S.b2[i - OFF_B2] = v;
+    else if (i < OFF_B3) S.w3[i - OFF_W3] = v;
+    else S.b3 = v;
+}
+
+__global__ void __launch_bounds__(TTHREADS) k_mlp_train(TrainArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    TrainSmem &S = *reinterpret_cast<TrainSmem *>(smem);
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank();
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, g = lane >> 2, tq = lane & 3;
+    const int n0 = 8 * w, c0 = n0 + 2 * tq;              // the warp's columns, this lane's first one
+    // this thread's share of the block's slice of the parameters
+    constexpr int C = kTrainCluster, slice = (NPARAM + C - 1) / C, kOwn = (slice + TTHREADS - 1) / TTHREADS;
+    const int own0 = rank * slice;
+    float p[kOwn], m1[kOwn], m2[kOwn];
+#pragma unroll
+    for (int k = 0; k < kOwn; k++) {
+        const int j = tid + k * TTHREADS, i = own0 + j;
+        p[k] = m1[k] = m2[k] = 0.f;
+        if (j < slice && i < NPARAM) { p[k] = a.prm[i]; m1[k] = a.m1[i]; m2[k] = a.m2[i]; }
+    }
+    for (int i = tid; i < NPARAM; i += TTHREADS) put_param(S, i, a.prm[i]);
+    const int first = rank * a.rows, last = min(a.batch, first + a.rows);     // this block's rows
+    const int chunks = (a.rows + TR - 1) / TR;
+    const float inv_n = 1.f / (float)a.batch;
+    // a chunk's inputs: four features per thread (the first 128), a target per
+    // thread (the next 32), fetched one chunk ahead
+    float4 nx = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto fetch = [&](int step, int chunk) {
+        nx = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (step >= a.steps) return;
+        const int r = tid < 128 ? tid >> 2 : tid - 128, row = first + chunk * TR + r;
+        if (tid >= 128 + TR || row >= last) return;
+        const int src = sample_row(a.batch, a.N, a.seed, a.step0 + step, row);
+        if (tid < 128) nx = *reinterpret_cast<const float4 *>(a.X + (size_t)src * IN + 4 * (tid & 3));
+        else nx.x = a.T[src];
+    };
+    fetch(0, 0);
+    for (int step = 0; step < a.steps; step++) {
+        float gw2[4][4] = {}, gw1[4] = {}, gb1[2] = {}, gb2[2] = {}, gw3[2] = {}, gb3 = 0.f, sse = 0.f;
+        for (int chunk = 0; chunk < chunks; chunk++) {
+            if (tid < 128) {
+                __nv_bfloat16 *d = S.x + (tid >> 2) * LDX + 4 * (tid & 3);
+                d[0] = __float2bfloat16_rn(nx.x);
+                d[1] = __float2bfloat16_rn(nx.y);
+                d[2] = __float2bfloat16_rn(nx.z);
+                d[3] = __float2bfloat16_rn(nx.w);
+            } else if (tid < 128 + TR) {
+                S.t[tid - 128] = nx.x;
+            } else if (tid < 128 + TR + 2 && chunk == 0) {
+                S.corr[tid - 128 - TR] = 1.f - powf(tid == 128 + TR ? 0.9f : 0.999f, (float)(a.adam0 + step + 1));
+            }
+            __syncthreads();
+            if (chunk + 1 < chunks) fetch(step, chunk + 1);
+            else fetch(step + 1, 0);
+            // h1 = relu(X W1 + b1)
+            uint32_t pos1 = 0;                           // z1 > 0, per fragment element
+            {
+                uint32_t b[2];
+                frag_b(b, S.w1, LDH, 0, n0);
+#pragma unroll
+                for (int mt = 0; mt < 2; mt++) {
+                    uint32_t f[4];
+                    float z[4] = {};
+                    frag_a(f, S.x, LDX, 16 * mt, 0);
+                    mma16816(z, f, b);
+#pragma unroll
+                    for (int i = 0; i < 4; i++) {
+                        z[i] += S.b1[c0 + (i & 1)];
+                        if (z[i] > 0.f) pos1 |= 1u << (4 * mt + i);
+                        else z[i] = 0.f;
+                    }
+                    __nv_bfloat16 *h = S.h1 + (16 * mt + g) * LDH + c0;
+                    *reinterpret_cast<__nv_bfloat162 *>(h) = __floats2bfloat162_rn(z[0], z[1]);
+                    *reinterpret_cast<__nv_bfloat162 *>(h + 8 * LDH) = __floats2bfloat162_rn(z[2], z[3]);
+                }
+            }
+            __syncthreads();
+            // z2 = h1 W2 + b2, and the warp's part of y = relu(z2) w3 + b3
+            float z2[2][4] = {};
+#pragma unroll
+            for (int k = 0; k < HID; k += 16) {
+                uint32_t b[2];
+                frag_b(b, S.w2, LDH, k, n0);
+#pragma unroll
+                for (int mt = 0; mt < 2; mt++) {
+                    uint32_t f[4];
+                    frag_a(f, S.h1, LDH, 16 * mt, k);
+                    mma16816(z2[mt], f, b);
+                }
+            }
+#pragma unroll
+            for (int mt = 0; mt < 2; mt++) {
+#pragma unroll
+                for (int i = 0; i < 4; i++) z2[mt][i] += S.b2[c0 + (i & 1)];
+#pragma unroll
+                for (int hrow = 0; hrow < 2; hrow++) {
+                    float y = fmaxf(z2[mt][2 * hrow], 0.f) * S.w3[c0] + fmaxf(z2[mt][2 * hrow + 1], 0.f) * S.w3[c0 + 1];
+                    y += __shfl_xor_sync(0xFFFFFFFFu, y, 1);
+                    y += __shfl_xor_sync(0xFFFFFFFFu, y, 2);
+                    if (tq == 0) S.ypart[16 * mt + 8 * hrow + g][w] = y;
+                }
+            }
+            __syncthreads();
+            if (tid < TR) {
+                float y = S.b3, e = 0.f;
+#pragma unroll
+                for (int i = 0; i < HID / 8; i++) y += S.ypart[tid][i];
+                if (first + chunk * TR + tid < last) e = y - S.t[tid];
+                S.dy[tid] = e * inv_n;
+                sse += e * e;
+                gb3 += e * inv_n;
+            }
+            __syncthreads();
+            // dz2 = dy w3 relu'(z2); gradients of w3 and b2
+#pragma unroll
+            for (int mt = 0; mt < 2; mt++) {
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    const float dy = S.dy[16 * mt + 8 * (i >> 1) + g], z = z2[mt][i];
+                    gw3[i & 1] += dy * fmaxf(z, 0.f);
+                    z2[mt][i] = z > 0.f ? dy * S.w3[c0 + (i & 1)] : 0.f;
+                    gb2[i & 1] += z2[mt][i];
+                }
+                __nv_bfloat16 *d = S.dz2 + (16 * mt + g) * LDH + c0;
+                *reinterpret_cast<__nv_bfloat162 *>(d) = __floats2bfloat162_rn(z2[mt][0], z2[mt][1]);
+                *reinterpret_cast<__nv_bfloat162 *>(d + 8 * LDH) = __floats2bfloat162_rn(z2[mt][2], z2[mt][3]);
+            }
+            __syncthreads();
+            // dz1 = (dz2 W2^T) relu'(z1); dW2 += h1^T dz2
+            float d1[2][4] = {};
+#pragma unroll
+            for (int k = 0; k < HID; k += 16) {
+                uint32_t b[2];
+                frag_bt(b, S.w2, LDH, k, n0);
+#pragma unroll
+                for (int mt = 0; mt < 2; mt++) {
+                    uint32_t f[4];
+                    frag_a(f, S.dz2, LDH, 16 * mt, k);
+                    mma16816(d1[mt], f, b);
+                }
+            }
+#pragma unroll
+            for (int mt = 0; mt < 2; mt++) {
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    if (!((pos1 >> (4 * mt + i)) & 1u)) d1[mt][i] = 0.f;
+                    gb1[i & 1] += d1[mt][i];
+                }
+                __nv_bfloat16 *d = S.dz1 + (16 * mt + g) * LDH + c0;
+                *reinterpret_cast<__nv_bfloat162 *>(d) = __floats2bfloat162_rn(d1[mt][0], d1[mt][1]);
+                *reinterpret_cast<__nv_bfloat162 *>(d + 8 * LDH) = __floats2bfloat162_rn(d1[mt][2], d1[mt][3]);
+            }
+#pragma unroll
+            for (int k = 0; k < TR; k += 16) {
+                uint32_t b[2];
+                frag_b(b, S.dz2, LDH, k, n0);
+#pragma unroll
+                for (int mt = 0; mt < 4; mt++) {
+                    uint32_t f[4];
+                    frag_at(f, S.h1, LDH, 16 * mt, k);
+                    mma16816(gw2[mt], f, b);
+                }
+            }
+            __syncwarp();
+            // dW1 += x^T dz1 (the warp's own columns of dz1)
+#pragma unroll
+            for (int k = 0; k < TR; k += 16) {
+                uint32_t f[4], b[2];
+                frag_at(f, S.x, LDX, 0, k);
+                frag_b(b, S.dz1, LDH, k, n0);
+                mma16816(gw1, f, b);
+            }
+            __syncthreads();                             // x, h1 and dz2 are rewritten by the next chunk
+        }
+        // the block's gradient
+#pragma unroll
+        for (int mt = 0; mt < 4; mt++)
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+                S.grad[OFF_W2 + (16 * mt + 8 * (i >> 1) + g) * HID + c0 + (i & 1)] = gw2[mt][i];
+#pragma unroll
+        for (int i = 0; i < 4; i++) S.grad[OFF_W1 + (8 * (i >> 1) + g) * HID + c0 + (i & 1)] = gw1[i];
+#pragma unroll
+        for (int i = 0; i < 2; i++) {
+            const float s1 = col_sum(gb1[i]), s2 = col_sum(gb2[i]), s3 = col_sum(gw3[i]);
+            if (g == 0) {
+                S.grad[OFF_B1 + c0 + i] = s1;
+                S.grad[OFF_B2 + c0 + i] = s2;
+                S.grad[OFF_W3 + c0 + i] = s3;
+            }
+        }
+        if (w == 0) {                                    // rows were taken by the first 32 threads
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                gb3 += __shfl_xor_sync(0xFFFFFFFFu, gb3, o);
+                sse += __shfl_xor_sync(0xFFFFFFFFu, sse, o);
+            }
+            if (lane == 0) { S.grad[OFF_B3] = gb3; S.sse = sse; }
+        }
+        cluster.sync();
+        // sum the blocks' gradients of this block's slice, Adam step, new weights to all blocks
+        const float corr1 = S.corr[0], corr2 = S.corr[1];
+#pragma unroll
+        for (int k = 0; k < kOwn; k++) {
+            const int j = tid + k * TTHREADS, i = own0 + j;
+            if (j >= slice || i >= NPARAM) break;
+            float gi = 0.f;
+#pragma unroll
+            for (int r = 0; r < C; r++) gi += *cluster.map_shared_rank(&S.grad[i], r);
+            m1[k] = 0.9f * m1[k] + (1.f - 0.9f) * gi;
+            m2[k] = 0.999f * m2[k] + (1.f - 0.999f) * gi * gi;
+            p[k] -= a.lr * (m1[k] / corr1) / (sqrtf(m2[k] / corr2) + 1e-8f);
+#pragma unroll
+            for (int r = 0; r < C; r++) put_param(*cluster.map_shared_rank(&S, r), i, p[k]);
+        }
+        if (step == a.steps - 1 && rank == 0 && tid == 0) {
+            float sum = 0.f;
+            for (int r = 0; r < C; r++) sum += *cluster.map_shared_rank(&S.sse, r);
+            *a.sse = sum;
+        }
+        cluster.sync();
+    }
+#pragma unroll
+    for (int k = 0; k < kOwn; k++) {
+        const int j = tid + k * TTHREADS, i = own0 + j;
+        if (j < slice && i < NPARAM) { a.prm[i] = p[k]; a.m1[i] = m1[k]; a.m2[i] = m2[k]; }
     }
 }
 
@@ -307,15 +646,25 @@ int configure_kernels() {
         return CCPM_ECUDA;
     if (cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwd_smem()) != cudaSuccess)
         return CCPM_ECUDA;
+    if (cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem)) !=
+        cudaSuccess)
+        return CCPM_ECUDA;
     done = true;
     return CCPM_OK;
 }
 
-// Device scratch for one call (X, targets, outputs); freed by the caller.
+// Device scratch for one call (X, targets, sampled rows).
 struct Scratch {
-    float *x = nullptr, *t = nullptr, *y = nullptr;
+    float *x = nullptr, *t = nullptr;
     int32_t *idx = nullptr;
-    ~Scratch() { cudaFree(x); cudaFree(t); cudaFree(y); cudaFree(idx); }
+    ~Scratch() { cudaFree(x); }  // the others lie behind x
+    int alloc(size_t rows, size_t picks) {
+        if (cudaMalloc(&x, sizeof(float) * rows * (IN + 1) + sizeof(int32_t) * picks) != cudaSuccess)
+            return CCPM_ENOMEM;
+        t = x + rows * IN;
+        idx = (int32_t *)(t + rows);
+        return CCPM_OK;
+    }
 };
 
 int tiles(int B) { return (B + ROWS - 1) / ROWS; }
@@ -325,10 +674,8 @@ int tiles(int B) { return (B + ROWS - 1) / ROWS; }
 namespace ccpm {
 
 void mlp_scratch_free(MlpScratch &sc) {
-    cudaFree(sc.dx);
-    cudaFree(sc.dy);
+    cudaFree(sc.dx);             // dy and hy lie behind dx and hx
     if (sc.hx) cudaFreeHost(sc.hx);
-    if (sc.hy) cudaFreeHost(sc.hy);
     sc = MlpScratch{};
 }
 
@@ -342,13 +689,13 @@ int mlp_score(ccpm_mlp *m, int B, const float *host_x, float *host_y, void *stre
     if (B > sc.cap) {
         mlp_scratch_free(sc);
         const int cap = std::max(B, 256);
-        if (cudaMalloc(&sc.dx, sizeof(float) * (size_t)cap * IN) != cudaSuccess ||
-            cudaMalloc(&sc.dy, sizeof(float) * (size_t)cap) != cudaSuccess ||
-            cudaMallocHost(&sc.hx, sizeof(float) * (size_t)cap * IN) != cudaSuccess ||
-            cudaMallocHost(&sc.hy, sizeof(float) * (size_t)cap) != cudaSuccess) {
+        if (cudaMalloc(&sc.dx, sizeof(float) * (size_t)cap * (IN + 1)) != cudaSuccess ||
+            cudaMallocHost(&sc.hx, sizeof(float) * (size_t)cap * (IN + 1)) != cudaSuccess) {
             mlp_scratch_free(sc);
             return CCPM_ENOMEM;
         }
+        sc.dy = sc.dx + (size_t)cap * IN;
+        sc.hy = sc.hx + (size_t)cap * IN;
         sc.cap = cap;
     }
     std::memcpy(sc.hx, host_x, sizeof(float) * (size_t)B * IN);
@@ -383,14 +730,16 @@ int ccpm_mlp_create(ccpm_ctx_t ctx, uint64_t seed, ccpm_mlp_t *out) {
     if (!m) return CCPM_ENOMEM;
     m->device = dev;
     m->stream = (cudaStream_t)ctx_stream_ptr(ctx);
-    if (cudaMalloc(&m->prm, sizeof(float) * NPARAM) != cudaSuccess ||
-        cudaMalloc(&m->grad, sizeof(float) * NPARAM) != cudaSuccess ||
-        cudaMalloc(&m->m1, sizeof(float) * NPARAM) != cudaSuccess ||
-        cudaMalloc(&m->m2, sizeof(float) * NPARAM) != cudaSuccess ||
-        cudaMalloc(&m->sse, sizeof(float)) != cudaSuccess) {
+    // one allocation: each allocation and release costs tens of microseconds,
+    // as much as several training steps
+    if (cudaMalloc(&m->prm, sizeof(float) * (4 * NPARAM + 1)) != cudaSuccess) {
         ccpm_mlp_destroy(m);
         return CCPM_ENOMEM;
     }
+    m->grad = m->prm + NPARAM;
+    m->m1 = m->grad + NPARAM;
+    m->m2 = m->m1 + NPARAM;
+    m->sse = m->m2 + NPARAM;
     // He-uniform initial weights from a SplitMix64 stream, zero biases
     std::vector<float> p(NPARAM, 0.f);
     uint64_t st = seed;
@@ -417,7 +766,7 @@ int ccpm_mlp_create(ccpm_ctx_t ctx, uint64_t seed, ccpm_mlp_t *out) {
 void ccpm_mlp_destroy(ccpm_mlp_t m) {
     if (!m) return;
     cudaSetDevice(m->device);
-    cudaFree(m->prm); cudaFree(m->grad); cudaFree(m->m1); cudaFree(m->m2); cudaFree(m->sse);
+    cudaFree(m->prm);
     ccpm::mlp_scratch_free(m->own);
     delete m;
 }
@@ -426,9 +775,8 @@ int ccpm_mlp_set_params(ccpm_mlp_t m, const float *host_params) {
     if (!m || !host_params) return CCPM_EINVAL;
     if (cudaSetDevice(m->device) != cudaSuccess) return CCPM_ECUDA;
     cudaError_t e = cudaMemcpyAsync(m->prm, host_params, sizeof(float) * NPARAM, cudaMemcpyHostToDevice, m->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(m->grad, 0, sizeof(float) * NPARAM, m->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(m->m1, 0, sizeof(float) * NPARAM, m->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(m->m2, 0, sizeof(float) * NPARAM, m->stream);
+    if (e == cudaSuccess)        // gradient and both moments
+        e = cudaMemsetAsync(m->grad, 0, sizeof(float) * 3 * NPARAM, m->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
     m->adam_step = 0;
     return e == cudaSuccess ? CCPM_OK : CCPM_ECUDA;
@@ -455,9 +803,7 @@ int ccpm_mlp_gradient(ccpm_mlp_t m, int B, const float *host_x, const float *hos
     if (cudaSetDevice(m->device) != cudaSuccess) return CCPM_ECUDA;
     if (configure_kernels()) return CCPM_ECUDA;
     Scratch sc;
-    if (cudaMalloc(&sc.x, sizeof(float) * (size_t)B * IN) != cudaSuccess ||
-        cudaMalloc(&sc.t, sizeof(float) * (size_t)B) != cudaSuccess)
-        return CCPM_ENOMEM;
+    if (sc.alloc((size_t)B, 0)) return CCPM_ENOMEM;
     cudaStream_t s = m->stream;
     cudaError_t e = cudaMemcpyAsync(sc.x, host_x, sizeof(float) * (size_t)B * IN, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(sc.t, host_t, sizeof(float) * (size_t)B, cudaMemcpyHostToDevice, s);
@@ -483,15 +829,50 @@ int ccpm_mlp_train(ccpm_mlp_t m, int N, const float *host_x, const float *host_t
     if (cudaSetDevice(m->device) != cudaSuccess) return CCPM_ECUDA;
     if (configure_kernels()) return CCPM_ECUDA;
     Scratch sc;
-    if (cudaMalloc(&sc.x, sizeof(float) * (size_t)N * IN) != cudaSuccess ||
-        cudaMalloc(&sc.t, sizeof(float) * (size_t)N) != cudaSuccess ||
-        cudaMalloc(&sc.idx, sizeof(int32_t) * (size_t)batch) != cudaSuccess)
-        return CCPM_ENOMEM;
+    if (sc.alloc((size_t)N, (size_t)batch)) return CCPM_ENOMEM;
     cudaStream_t s = m->stream;
     cudaError_t e = cudaMemcpyAsync(sc.x, host_x, sizeof(float) * (size_t)N * IN, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(sc.t, host_t, sizeof(float) * (size_t)N, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(m->grad, 0, sizeof(float) * NPARAM, s);
-    for (int it = 0; it < steps && e == cudaSuccess; it++) {
+    // Up to kTrainMaxBatch every step in one kernel, a few thousand steps a
+    // launch: 5.9 us a step up to 256 rows, 10.6 at 1024, 29 at 4096, 54 at 8192
+    // (a block takes its rows 32 at a time).  The kernels per step, which spread
+    // over the whole GPU, take 37 us up to 4096 rows and 40 at 8192.
+    const bool fused = batch <= kTrainMaxBatch;
+    for (int it = 0; fused && it < steps && e == cudaSuccess;) {
+        const int C = kTrainCluster;      // also where a block gets few rows: the Adam step is split, too
+        TrainArgs a;
+        a.prm = m->prm;
+        a.m1 = m->m1;
+        a.m2 = m->m2;
+        a.sse = m->sse;
+        a.X = sc.x;
+        a.T = sc.t;
+        a.N = N;
+        a.batch = batch;
+        a.rows = (batch + C - 1) / C;
+        a.steps = std::min(steps - it, 4096);
+        a.step0 = it;
+        a.adam0 = m->adam_step;
+        a.seed = seed;
+        a.lr = lr;
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at = {};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = (unsigned)C;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.gridDim = dim3((unsigned)C);
+        cfg.blockDim = dim3(TTHREADS);
+        cfg.dynamicSmemBytes = sizeof(TrainSmem);
+        cfg.stream = s;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, k_mlp_train, a);
+        if (e == cudaSuccess) e = cudaGetLastError();
+        it += a.steps;
+        m->adam_step += a.steps;
+    }
+    for (int it = 0; !fused && it < steps && e == cudaSuccess; it++) {
         e = cudaMemsetAsync(m->sse, 0, sizeof(float), s);
         if (e != cudaSuccess) break;
         k_mlp_sample<<<(batch + 255) / 256, 256, 0, s>>>(sc.idx, batch, N, seed, it);
