@@ -13,15 +13,17 @@
 // of Section 4.1).  With every edge label 0 these are the rules of the 32-bit
 // pipeline.
 //
-// Layout and schedule: one warp per listed vertex (one block per vertex whose
-// row is longer than 1024 entries); its entries are read in windows aligned
-// to the 32-entry words of the edge bitmap, so lane i of a window owns bit i
-// of one word (one broadcast load of the bits, one atomic to clear the
-// failing ones).  Rounds are snapshot rounds over two omega
-// buffers; each round lists the vertices that were active at its start for
-// the next round, which writes 0 for those that died and drops them.  The
-// host reads one small counter block per round.  No kernel waits on another
-// block: every loop is bounded by the list or row it walks.
+// Schedule: rounds are snapshot rounds over two omega buffers, and an entry's
+// bit is read and written only with its own row, so a row that dies is wiped
+// where it dies and the last (quiescent) round leaves omega, the bitmap and the
+// active totals as they are handed back.  The first round reads labels instead
+// of omega and writes the bits that stay; it lists the rows by length for the
+// later rounds, which read their counts on the device: four rounds are queued at
+// a time, and those after the quiescent one return at once.  Rows up to kWShort
+// entries go four to a warp, rows up to kWHub one to a warp, longer ones to
+// blocks in chunks; the block that finishes a row's last chunk decides it.  No
+// kernel waits on another block: every loop is bounded by the list or row it
+// walks.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -40,56 +42,85 @@ constexpr int kWT = 64;        // template vertices
 constexpr int kWEL = 8;        // distinct edge labels one template may use
 constexpr int kWCls = 64;      // label-multiplicity classes (need >= 2)
 constexpr int kWEdges = 2016;  // 64 * 63 / 2
-constexpr int kWHub = 1024;    // rows longer than this are walked by a whole block
+constexpr int kWShort = 32;    // rows up to this go eight lanes each
+constexpr int kWHub = 1024;    // rows longer than this are walked by whole blocks
+constexpr int kWChunk = 8192;  // entries a block takes of one: 1024 for each of its 8 warps
+constexpr int kWTile = 128;    // listed vertices a warp looks through at a time
+constexpr int kWQueue = 4;     // rounds queued per host round trip
+constexpr int kWPush = 4;      // neighbours are marked once at most one active vertex in so many changes
 constexpr unsigned FULL = 0xFFFFFFFFu;
 
 // Template tables of one call (device copy, loaded into shared memory).
 struct __align__(16) WideTab {
     int n0, n_el, n_cls, pad;
-    uint8_t el_index[256];         // graph edge label -> edge-label index j, 0xFF: used by no template edge
+    uint8_t el_index[256];         // graph edge label -> edge-label index j, kWEL: used by no template edge
     uint64_t adj[kWEL][kWT];       // adj[j][q]: template neighbours of q joined by an edge of label index j
     uint64_t cls_mask[kWCls];      // template neighbours of cls_q with one vertex label, joined by label cls_j
     uint32_t cls_need[kWCls];      // their number (at least 2; a class of one is the coverage rule)
+    uint64_t q_cls[kWT];           // the classes of q
     uint8_t cls_q[kWCls];
     uint8_t cls_j[kWCls];
 };
 
-struct WideCounters {
-    unsigned long long n_next;     // vertices listed for the next round (rows up to kWHub entries)
-    unsigned long long n_hub_next; // ... with longer rows
+struct WideRound {
+    unsigned long long n_list;     // short rows listed for the next round
     unsigned long long scanned;    // active entries read (both ends live, bit set)
     unsigned long long alive;      // active vertices read
-    unsigned long long active_v, active_e;   // hand-back totals
-    unsigned int changed;
-    unsigned int pad;
+    unsigned long long moved;      // vertices whose omega changed
+    unsigned int changed;          // anything did
+    unsigned int pushed;           // the neighbours of those vertices are marked
+};
+struct WideState {
+    unsigned long long n_mid, n_hub, n_part; // mid rows, chunks of longer rows, rows of several chunks
+    // r[i + 1]: the i-th of the queued rounds (n_list: of the round after it);
+    // r[0]: the round before them
+    WideRound r[kWQueue + 1];
+};
+
+// A chunk of a long row; part: the row's place for combining its chunks, -1: it
+// has only this one.
+struct WideChunk {
+    int32_t v, part, chunk, chunks;
+};
+struct WidePart {
+    unsigned long long U[kWEL];
+    uint32_t cnt[kWCls];
+    uint32_t nN, chg, done, pad;
 };
 
 struct WideArgs {
+    int64_t n;
     const int64_t *rp;
     const int32_t *col;
+    const uint8_t *lab;
     const uint8_t *el;             // edge label per entry, or NULL (all 0)
+    const uint64_t *lmask;         // 256: the template vertices of a label
     const uint64_t *om_in;
     uint64_t *om_out;
     uint32_t *ebits;
-    const int32_t *list_in;
-    int64_t n_in;
+    uint32_t *deg;                 // active entries of an active vertex after its last evaluation
+    const uint8_t *mark_in;        // vertices to evaluate in this round (value `mark`)
+    uint8_t *mark_out;             // ... and in the next one (value `mark` + 1)
+    uint8_t mark;
+    const int32_t *list_in;        // active vertices with short rows
     int32_t *list_out;
-    const int32_t *hub_in;         // vertices whose rows are longer than kWHub entries
-    int64_t n_hub;
-    int32_t *hub_out;
-    WideCounters *st;
+    int32_t *mid;                  // initially active vertices with longer rows
+    WideChunk *hub;
+    WidePart *part;                // all 0 between rounds
+    WideState *st;
+    int slot;                      // of this round
     const WideTab *tab;
 };
 
 __device__ __forceinline__ uint64_t warp_or64(uint64_t x) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x |= __shfl_xor_sync(FULL, x, o);
-    return x;
+    const uint32_t lo = __reduce_or_sync(FULL, (uint32_t)x), hi = __reduce_or_sync(FULL, (uint32_t)(x >> 32));
+    return ((uint64_t)hi << 32) | lo;
 }
 
-__device__ __forceinline__ unsigned long long warp_sum64(unsigned long long x) {
+// Over the eight lanes of a group.
+__device__ __forceinline__ uint64_t group_or64(uint64_t x) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
+    for (int o = 1; o < 8; o <<= 1) x |= __shfl_xor_sync(FULL, x, o);
     return x;
 }
 
@@ -99,296 +130,739 @@ __device__ __forceinline__ void load_tab(WideTab &dst, const WideTab *src) {
     for (int i = threadIdx.x; i < (int)(sizeof(WideTab) / 4); i += blockDim.x) d[i] = s[i];
 }
 
-// Warp-aggregated append of v (lanes with `take`) to list[*count ...].
-__device__ __forceinline__ void push_list(bool take, int32_t v, int32_t *list, unsigned long long *count) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t act = __ballot_sync(FULL, take);
-    if (!act) return;
-    unsigned long long base = 0;
-    const int leader = __ffs(act) - 1;
-    if (lane == leader) base = atomicAdd(count, (unsigned long long)__popc(act));
-    base = __shfl_sync(FULL, base, leader);
-    if (take) list[base + __popc(act & ((1u << lane) - 1u))] = v;
-}
+// Per-thread totals of a round, and the block's shared memory.
+struct WideAcc {
+    unsigned long long scanned = 0;
+    uint32_t alive = 0, moved = 0;
+    bool changed = false;
+    bool push = false, marked = false;       // this round marks; the round before it did
+};
+struct WideShared {
+    WideTab T;
+    uint64_t lm[256];                        // first round: omega of a label
+    uint64_t w[8][kWTile];                   // a warp's short rows: omega, vertex
+    int32_t v[8][kWTile];
+    uint64_t nb[8][4][kWEL + 1];             // per warp and row: template neighbours of omega(v), by edge label
+    unsigned long long bU[kWEL];             // a long row's results
+    uint32_t bcnt[kWCls];
+    uint32_t bN, bchg;
+    unsigned long long scanned, alive, moved;
+    uint32_t changed, last;
+};
 
-// Alg. 3: omega_0(v) = {q : l(q) = l(v)} in both snapshot buffers; every
-// initially active vertex is listed for the first round, on the list of its
-// row length.
-__global__ void __launch_bounds__(256)
-k_wide_init(int64_t n, const int64_t *__restrict__ rp, const uint8_t *__restrict__ lab,
-            const uint64_t *__restrict__ lmask, uint64_t *om0, uint64_t *om1, int32_t *list, int32_t *hub,
-            WideCounters *st) {
-    __shared__ uint64_t sl[256];
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) sl[i] = lmask[i];
-    __syncthreads();
-    for (int64_t v0 = (int64_t)blockIdx.x * blockDim.x; v0 < n; v0 += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t v = v0 + threadIdx.x;
-        uint64_t w = 0;
-        bool long_row = false;
-        if (v < n) {
-            w = sl[lab[v]];
-            om0[v] = w;
-            om1[v] = w;
-            if (w) long_row = rp[v + 1] - rp[v] > kWHub;
-        }
-        push_list(w != 0 && !long_row, (int32_t)v, list, &st->n_next);
-        push_list(w != 0 && long_row, (int32_t)v, hub, &st->n_hub_next);
+// Rows of at most kWShort entries, eight lanes and four entries a lane each, so
+// that four rows of a warp share its instructions and their loads are in flight
+// together.  A row's bits are one 32-bit word in registers.  Coverage is decided
+// first; only the classes of the vertices that pass it are counted.
+template <bool FIRST, int NEL>
+__device__ __forceinline__ void short_row(const WideArgs &a, WideShared &S, bool has, int32_t v, uint64_t wv,
+                                          WideAcc &acc) {
+    const WideTab &T = S.T;
+    const int lane = threadIdx.x & 31, gl = lane & 7, gb = lane & 24;
+    int64_t beg = 0;
+    int len = 0;
+    if (has) {
+        beg = a.rp[v];
+        len = (int)(a.rp[(int64_t)v + 1] - beg);
     }
-}
-
-// The template neighbours of omega(v) per edge-label index (every lane of
-// the warp gets them).
-__device__ __forceinline__ void nbr_masks(const WideTab &T, uint64_t wv, uint64_t (&nb)[kWEL]) {
-    const int lane = threadIdx.x & 31;
+    const int sh = (int)(beg & 31);
+    uint32_t *const word = a.ebits + (beg >> 5);
+    uint32_t rb = len >= 32 ? FULL : (1u << len) - 1u;
+    if (!FIRST && len > 0) {
+        const uint32_t lo = word[0], hi = sh + len > 32 ? word[1] : 0u;
+        rb &= __funnelshift_r(lo, hi, sh);
+    }
+    int32_t u[4];
+    uint8_t lb[4];
+    uint64_t wu[4];
 #pragma unroll
-    for (int j = 0; j < kWEL; j++) nb[j] = 0;
-    for (int q = lane; q < T.n0; q += 32)
-        if ((wv >> q) & 1ull) {
+    for (int k = 0; k < 4; k++) {
+        const bool act = (rb >> (8 * k + gl)) & 1u;
+        u[k] = act ? a.col[beg + 8 * k + gl] : -1;
+        lb[k] = act && a.el ? a.el[beg + 8 * k + gl] : (uint8_t)0;
+    }
 #pragma unroll
-            for (int j = 0; j < kWEL; j++)
-                if (j < T.n_el) nb[j] |= T.adj[j][q];
-        }
+    for (int k = 0; k < 4; k++) wu[k] = u[k] >= 0 ? (FIRST ? S.lm[a.lab[u[k]]] : a.om_in[u[k]]) : 0ull;
+    // template neighbours of omega(v); each lane takes eight template vertices
+    uint64_t nb[NEL], U[NEL];
 #pragma unroll
-    for (int j = 0; j < kWEL; j++) nb[j] = warp_or64(nb[j]);
-}
-
-// One warp's share of a row: windows first_w, first_w + w_step, ... (each a
-// group of four 32-entry windows aligned to the bitmap words, all loaded
-// before any is used).  Per lane: the unions per edge-label index, the
-// surviving entries, the eta change; per class, the count of surviving
-// entries meeting it is added to cnt[c] by lane 0 (atomically when several
-// warps share cnt).
-__device__ __forceinline__ void scan_windows(const WideArgs &a, const WideTab &T, uint64_t wv,
-                                             const uint64_t (&nb)[kWEL], int64_t beg, int64_t end,
-                                             int64_t first_w, int64_t w_step, uint64_t (&U)[kWEL],
-                                             uint32_t &nN, uint32_t &achg, uint32_t *cnt, bool shared_cnt,
-                                             unsigned long long &scanned) {
-    constexpr int WU = 4;
-    const int lane = threadIdx.x & 31;
-    const int n_cls = T.n_cls;
-    for (int64_t w0 = first_w; (w0 << 5) < end; w0 += w_step) {
-        bool bit[WU];
-        int32_t u[WU];
-        uint8_t lb[WU];
-        uint64_t wn[WU];
+    for (int j = 0; j < NEL; j++) nb[j] = U[j] = 0;
+    const uint32_t mine = (uint32_t)(wv >> (8 * gl)) & 0xFFu;
+    for (uint32_t b = mine; b; b &= b - 1) {
+        const int q = 8 * gl + __ffs(b) - 1;
 #pragma unroll
-        for (int k = 0; k < WU; k++) {
-            const int64_t e = ((w0 + k) << 5) + lane;
-            const uint32_t word = ((w0 + k) << 5) < end ? a.ebits[w0 + k] : 0u;
-            bit[k] = e >= beg && e < end && ((word >> lane) & 1u);
-        }
+        for (int j = 0; j < NEL; j++) nb[j] |= T.adj[j][q];
+    }
+    uint64_t *const snb = S.nb[threadIdx.x >> 5][lane >> 3];
 #pragma unroll
-        for (int k = 0; k < WU; k++) {
-            const int64_t e = ((w0 + k) << 5) + lane;
-            u[k] = bit[k] ? a.col[e] : 0;
-            lb[k] = (bit[k] && a.el) ? a.el[e] : (uint8_t)0;
-        }
+    for (int j = 0; j < NEL; j++) {
+        nb[j] = group_or64(nb[j]);
+        if (gl == j) snb[j] = nb[j];
+    }
+    __syncwarp();
+    uint32_t pm = 0;                         // entries that pass
+    int jk[4];
 #pragma unroll
-        for (int k = 0; k < WU; k++) wn[k] = bit[k] ? a.om_in[u[k]] : 0ull;
+    for (int k = 0; k < 4; k++) {
+        const int j = (int)T.el_index[lb[k]];
+        const bool live = wu[k] != 0, pass = (wu[k] & snb[j]) != 0;
+        if (live) acc.scanned++;
+        if (live && !pass) acc.changed = true;           // eta eliminates an active entry
+        jk[k] = pass ? j : -1;
 #pragma unroll
-        for (int k = 0; k < WU; k++) {
-            if (((w0 + k) << 5) >= end) break;          // past the row (warp-uniform)
-            const uint64_t wu = wn[k];
-            const int j = bit[k] ? (int)T.el_index[lb[k]] : 0xFF;
-            uint64_t m = 0;
+        for (int i = 0; i < NEL; i++)
+            U[i] |= wu[k] & (jk[k] == i ? ~0ull : 0ull);
+        pm |= ((__ballot_sync(FULL, pass) >> gb) & 0xFFu) << (8 * k);
+    }
+    uint64_t keep = 0, open = 0;
+    if (__any_sync(FULL, pm != 0)) {
 #pragma unroll
-            for (int jj = 0; jj < kWEL; jj++)
-                if (j == jj) m = nb[jj];
-            const bool live = bit[k] && wu != 0;     // both ends active: the entry is active
-            const bool pass = live && (wu & m) != 0;
-            scanned += live ? 1ull : 0ull;
-            if (live && !pass) achg = 1;             // eta eliminates an active entry
-            if (pass) {
-                nN++;
+        for (int j = 0; j < NEL; j++) U[j] = group_or64(U[j]);
+        if (pm)
+            for (uint32_t b = mine; b; b &= b - 1) {
+                const int q = 8 * gl + __ffs(b) - 1;
+                bool ok = true;
 #pragma unroll
-                for (int jj = 0; jj < kWEL; jj++)
-                    if (j == jj) U[jj] |= wu;
+                for (int j = 0; j < NEL; j++) ok = ok && !(T.adj[j][q] & ~U[j]);
+                if (ok) {
+                    keep |= 1ull << q;
+                    open |= T.q_cls[q];
+                }
             }
-            // the bit goes with the failing entries and with those whose
-            // other end is inactive already (no change: that entry is inactive)
-            const uint32_t drop = __ballot_sync(FULL, bit[k] && !pass);
-            if (drop && lane == 0) atomicAnd(&a.ebits[w0 + k], ~drop);
-            for (int c = 0; c < n_cls; c++) {
-                if (!((wv >> T.cls_q[c]) & 1ull)) continue;
-                const uint32_t hit = __ballot_sync(FULL, pass && j == (int)T.cls_j[c] && (wu & T.cls_mask[c]) != 0);
-                if (lane == 0 && hit) {
-                    if (shared_cnt) atomicAdd(&cnt[c], (uint32_t)__popc(hit));
-                    else cnt[c] += (uint32_t)__popc(hit);
+        keep = group_or64(keep);
+        if (T.n_cls) open = group_or64(open);
+        while (__any_sync(FULL, open != 0)) {
+            const int c = open ? __ffsll((long long)open) - 1 : 0;
+            const uint64_t cm = T.cls_mask[c];
+            const int cj = T.cls_j[c];
+            uint32_t h = 0;
+#pragma unroll
+            for (int k = 0; k < 4; k++) h += jk[k] == cj && (wu[k] & cm) != 0 ? 1u : 0u;
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) h += __shfl_xor_sync(FULL, h, o);
+            if (open) {
+                open &= open - 1;
+                if (h < T.cls_need[c]) {
+                    keep &= ~(1ull << T.cls_q[c]);
+                    open &= ~T.q_cls[T.cls_q[c]];
                 }
             }
         }
     }
-}
-
-// The vertex rule: q stays iff every template neighbour joined by edge
-// label j lies in U[j] and every class of q has enough distinct neighbours;
-// nothing stays without a surviving entry.
-__device__ __forceinline__ uint64_t decide_wide(const WideTab &T, uint64_t wv, const uint64_t (&U)[kWEL], uint32_t nN,
-                                                const uint32_t *cnt) {
-    uint64_t keep = 0;
-    if (nN == 0) return 0;
-    for (int q = 0; q < T.n0; q++) {
-        if (!((wv >> q) & 1ull)) continue;
-        bool ok = true;
+    if (!has) return;                        // (no warp operation below)
+    if (keep != wv) {
+        acc.changed = true;
+        if (gl == 0) acc.moved++;
+        if (!FIRST && acc.push) {
+            if (gl == 0 && keep) a.mark_out[v] = (uint8_t)(a.mark + 1);
 #pragma unroll
-        for (int j = 0; j < kWEL; j++)
-            if (j < T.n_el && (T.adj[j][q] & ~U[j])) ok = false;
-        for (int c = 0; c < T.n_cls && ok; c++)
-            if (T.cls_q[c] == q && cnt[c] < T.cls_need[c]) ok = false;
-        if (ok) keep |= 1ull << q;
+            for (int k = 0; k < 4; k++)
+                if (jk[k] >= 0) a.mark_out[u[k]] = (uint8_t)(a.mark + 1);
+        }
     }
-    return keep;
+    const uint32_t nbits = keep ? pm : 0u;   // a dead row's bits go at once
+    const uint32_t d = FIRST ? nbits : rb & ~nbits;
+    if (gl == 0) {
+        acc.alive++;
+        a.om_out[v] = keep;
+        a.deg[v] = __popc(pm);
+        const uint32_t lo = d << sh;
+        if (lo) {
+            if (FIRST) atomicOr(word, lo);
+            else atomicAnd(word, ~lo);
+        }
+    } else if (gl == 1 && sh) {
+        const uint32_t hi = d >> (32 - sh);
+        if (hi) {
+            if (FIRST) atomicOr(word + 1, hi);
+            else atomicAnd(word + 1, ~hi);
+        }
+    }
 }
 
-// One snapshot round.  Rows of at most kWHub entries: one warp each.  Longer
-// rows (list hub_in): one block each, its warps taking interleaved window
-// groups, the partial results combined in shared memory.  Every vertex
-// listed at the start of the round is listed again (the next round writes
-// its zero if it died here); a vertex stays on the list of its row length.
-__global__ void __launch_bounds__(256)
-k_wide_round(WideArgs a) {
-    __shared__ WideTab T;
-    __shared__ uint32_t cnt[8][kWCls];
-    __shared__ uint32_t bcnt[kWCls];
-    __shared__ unsigned long long bU[kWEL];
-    __shared__ uint32_t bN, bchg;
-    load_tab(T, a.tab);
-    __syncthreads();
-    const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
+__device__ __forceinline__ void list_chunks(const WideArgs &a, int32_t v) {
+    const int64_t beg = a.rp[v], end = a.rp[(int64_t)v + 1];
+    // chunks start at bitmap words
+    const int chunks = (int)((end - (beg & ~31ll) + kWChunk - 1) / kWChunk);
+    const int part = chunks > 1 ? (int)atomicAdd(&a.st->n_part, 1ull) : -1;
+    const unsigned long long at = atomicAdd(&a.st->n_hub, (unsigned long long)chunks);
+    for (int c = 0; c < chunks; c++) a.hub[at + c] = WideChunk{v, part, c, chunks};
+}
+
+// The listed (first round: all) vertices, 128 to a warp at a time: those that
+// died get their zero in this buffer, the active ones with short rows are listed
+// again and evaluated, and the first round lists the longer rows.
+template <bool FIRST, int NEL>
+__device__ __forceinline__ void short_part(const WideArgs &a, WideShared &S, int64_t n_in, WideAcc &acc) {
+    constexpr int W = kWTile / 32;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int nwb = (int)(blockDim.x >> 5);
-    unsigned long long scanned = 0, alive = 0;
-    unsigned int changed = 0;
-    // (1) rows up to kWHub entries, one warp each
-    for (int64_t i = gw; i < a.n_in; i += nw) {
-        const int32_t v = a.list_in[i];
-        const uint64_t wv = a.om_in[v];
-        if (wv == 0) {
-            // died in the previous round: its zero goes to this buffer too
-            if (lane == 0) a.om_out[v] = 0;
-            continue;
+    const uint32_t lt = (1u << lane) - 1u;
+    for (int64_t base = gw * kWTile; base < n_in; base += nw * kWTile) {
+        int32_t v[W];
+        uint64_t w[W];
+#pragma unroll
+        for (int k = 0; k < W; k++) {
+            const int64_t i = base + 32 * k + lane;
+            v[k] = i < n_in ? (FIRST ? (int32_t)i : a.list_in[i]) : -1;
         }
-        if (lane == 0) alive++;
-        uint64_t nb[kWEL];
-        nbr_masks(T, wv, nb);
-        for (int c = lane; c < T.n_cls; c += 32) cnt[wib][c] = 0;
-        __syncwarp();
-        const int64_t beg = a.rp[v], end = a.rp[(int64_t)v + 1];
-        uint64_t U[kWEL];
 #pragma unroll
-        for (int j = 0; j < kWEL; j++) U[j] = 0;
-        uint32_t nN = 0, achg = 0;
-        scan_windows(a, T, wv, nb, beg, end, beg >> 5, 4, U, nN, achg, cnt[wib], false, scanned);
+        for (int k = 0; k < W; k++) w[k] = v[k] >= 0 ? (FIRST ? S.lm[a.lab[v[k]]] : a.om_in[v[k]]) : 0ull;
+        int len[W];                          // 0: short, 1: mid, 2: hub, -1: not active
 #pragma unroll
-        for (int j = 0; j < kWEL; j++) U[j] = warp_or64(U[j]);
-        nN = __reduce_add_sync(FULL, nN);
-        achg = __reduce_or_sync(FULL, achg);
-        __syncwarp();
-        const uint64_t keep = decide_wide(T, wv, U, nN, cnt[wib]);
-        if (keep != wv || achg) changed = 1;
-        if (lane == 0) {
-            a.om_out[v] = keep;
-            const unsigned long long pos = atomicAdd(&a.st->n_next, 1ull);
-            a.list_out[pos] = v;
-        }
-        __syncwarp();
-    }
-    // (2) longer rows, one block each (block-uniform loop)
-    for (int64_t i = blockIdx.x; i < a.n_hub; i += gridDim.x) {
-        const int32_t v = a.hub_in[i];
-        const uint64_t wv = a.om_in[v];
-        if (wv == 0) {
-            if (threadIdx.x == 0) a.om_out[v] = 0;
-            continue;
-        }
-        if (threadIdx.x == 0) alive++;
-        uint64_t nb[kWEL];
-        nbr_masks(T, wv, nb);
-        for (int c = threadIdx.x; c < T.n_cls; c += blockDim.x) bcnt[c] = 0;
-        if (threadIdx.x < kWEL) bU[threadIdx.x] = 0ull;
-        if (threadIdx.x == 0) { bN = 0; bchg = 0; }
-        __syncthreads();
-        const int64_t beg = a.rp[v], end = a.rp[(int64_t)v + 1];
-        uint64_t U[kWEL];
-#pragma unroll
-        for (int j = 0; j < kWEL; j++) U[j] = 0;
-        uint32_t nN = 0, achg = 0;
-        scan_windows(a, T, wv, nb, beg, end, (beg >> 5) + 4 * wib, 4 * nwb, U, nN, achg, bcnt, true, scanned);
-#pragma unroll
-        for (int j = 0; j < kWEL; j++) U[j] = warp_or64(U[j]);
-        nN = __reduce_add_sync(FULL, nN);
-        achg = __reduce_or_sync(FULL, achg);
-        if (lane == 0) {
-#pragma unroll
-            for (int j = 0; j < kWEL; j++)
-                if (U[j]) atomicOr(&bU[j], (unsigned long long)U[j]);
-            if (nN) atomicAdd(&bN, nN);
-            if (achg) atomicOr(&bchg, 1u);
-        }
-        __syncthreads();
-        if (wib == 0) {
-            uint64_t Ub[kWEL];
-#pragma unroll
-            for (int j = 0; j < kWEL; j++) Ub[j] = bU[j];
-            const uint64_t keep = decide_wide(T, wv, Ub, bN, bcnt);
-            if (keep != wv || bchg) changed = 1;
-            if (lane == 0) {
-                a.om_out[v] = keep;
-                const unsigned long long pos = atomicAdd(&a.st->n_hub_next, 1ull);
-                a.hub_out[pos] = v;
+        for (int k = 0; k < W; k++) {
+            len[k] = w[k] ? 0 : -1;
+            if (FIRST && w[k]) {
+                const int64_t l = a.rp[(int64_t)v[k] + 1] - a.rp[v[k]];
+                len[k] = l <= kWShort ? 0 : l <= kWHub ? 1 : 2;
+            }
+            if (v[k] >= 0 && !w[k]) a.om_out[v[k]] = 0;
+            if (!FIRST && acc.marked && w[k] && a.mark_in[v[k]] != a.mark) {
+                len[k] = 3;                  // nothing near it changed
+                acc.alive++;
+                acc.scanned += a.deg[v[k]];
+                a.om_out[v[k]] = w[k];
             }
         }
-        __syncthreads();                          // bcnt / bU / bN are reused
-    }
-    scanned = warp_sum64(scanned);
-    alive = warp_sum64(alive);
-    changed = __reduce_or_sync(FULL, changed);
-    if (lane == 0) {
-        if (scanned) atomicAdd(&a.st->scanned, scanned);
-        if (alive) atomicAdd(&a.st->alive, alive);
-        if (changed) atomicOr(&a.st->changed, 1u);
+        uint32_t cnt[3] = {0, 0, 0};
+#pragma unroll
+        for (int t = 0; t < (FIRST ? 3 : 1); t++) {
+            uint32_t b[W], total = 0;
+#pragma unroll
+            for (int k = 0; k < W; k++) {
+                b[k] = __ballot_sync(FULL, len[k] == t);
+                total += __popc(b[k]);
+            }
+            cnt[t] = total;                  // (t = 0: rows to evaluate, listed with the skipped ones)
+            if (!FIRST)
+#pragma unroll
+                for (int k = 0; k < W; k++) total += __popc(__ballot_sync(FULL, len[k] == 3));
+            if (!total) continue;
+            if (t == 2) {
+#pragma unroll
+                for (int k = 0; k < W; k++)
+                    if (len[k] == t) list_chunks(a, v[k]);
+                continue;
+            }
+            unsigned long long *const n_out = t == 0 ? &a.st->r[a.slot + 1].n_list : &a.st->n_mid;
+            int32_t *const out = t == 0 ? a.list_out : a.mid;
+            unsigned long long pos = 0;
+            if (lane == 0) pos = atomicAdd(n_out, (unsigned long long)total);
+            pos = __shfl_sync(FULL, pos, 0);
+            uint32_t at = 0;
+#pragma unroll
+            for (int k = 0; k < W; k++) {
+                if (len[k] == t) {
+                    const uint32_t o = at + __popc(b[k] & lt);
+                    out[pos + o] = v[k];
+                    if (t == 0) {
+                        S.v[wib][o] = v[k];
+                        S.w[wib][o] = w[k];
+                    }
+                }
+                at += __popc(b[k]);
+            }
+            if (!FIRST)
+#pragma unroll
+                for (int k = 0; k < W; k++) {
+                    const uint32_t skipped = __ballot_sync(FULL, len[k] == 3);
+                    if (len[k] == 3) out[pos + at + __popc(skipped & lt)] = v[k];
+                    at += __popc(skipped);
+                }
+        }
+        __syncwarp();
+        for (uint32_t i0 = 0; i0 < cnt[0]; i0 += 4) {
+            const uint32_t i = i0 + (lane >> 3);
+            const bool has = i < cnt[0];
+            short_row<FIRST, NEL>(a, S, has, has ? S.v[wib][i] : 0, has ? S.w[wib][i] : 0ull, acc);
+        }
+        __syncwarp();
     }
 }
 
-// Hand-back: an entry keeps its bit only if both of its ends are active
-// (rows of dead vertices and entries to dead neighbours are cleared; so are
-// the rows of vertices that were never active).  Counts the active vertices
-// and entries.
-__global__ void __launch_bounds__(256)
-k_wide_clear(int64_t n, const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
-             const uint64_t *__restrict__ om, uint32_t *ebits, WideCounters *st) {
+// Template vertices of omega(v) whose neighbours all lie in U; their classes.
+template <int NEL>
+__device__ __forceinline__ uint64_t covered(const WideTab &T, uint64_t wv, const uint64_t (&U)[NEL], uint64_t &cls) {
     const int lane = threadIdx.x & 31;
-    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    unsigned long long av = 0, ae = 0;
-    for (int64_t v = gw; v < n; v += nw) {
-        const bool vlive = om[v] != 0;
-        if (lane == 0 && vlive) av++;
-        const int64_t beg = rp[v], end = rp[v + 1];
-        for (int64_t w0 = beg >> 5; (w0 << 5) < end; w0++) {
-            const int64_t e = (w0 << 5) + lane;
-            const uint32_t word = ebits[w0];
-            const bool bit = e >= beg && e < end && ((word >> lane) & 1u);
-            const bool keep = bit && vlive && om[col[e]] != 0;
-            ae += keep ? 1ull : 0ull;
-            const uint32_t drop = __ballot_sync(FULL, bit && !keep);
-            if (drop && lane == 0) atomicAnd(&ebits[w0], ~drop);
+    bool ok[2];
+    uint64_t c = 0;
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        const int q = lane + 32 * h;
+        ok[h] = (wv >> q) & 1ull;
+#pragma unroll
+        for (int j = 0; j < NEL; j++) ok[h] = ok[h] && !(T.adj[j][q] & ~U[j]);
+        if (ok[h]) c |= T.q_cls[q];
+    }
+    cls = T.n_cls ? warp_or64(c) : 0ull;
+    const uint64_t lo = __ballot_sync(FULL, ok[0]), hi = __ballot_sync(FULL, ok[1]);
+    return lo | (hi << 32);
+}
+
+// A longer row, or a chunk of one: its arrays from the bitmap word of its first
+// entry on (`off` entries into it, up to `span`).
+struct WideRow {
+    uint32_t *bits;
+    const int32_t *col;
+    const uint8_t *el;
+    uint32_t off, span;
+};
+__device__ __forceinline__ WideRow row_of(const WideArgs &a, int32_t v) {
+    const int64_t beg = a.rp[v], w = beg >> 5;
+    return WideRow{a.ebits + w, a.col + (w << 5), a.el ? a.el + (w << 5) : nullptr, (uint32_t)(beg & 31),
+                   (uint32_t)(a.rp[(int64_t)v + 1] - (w << 5))};
+}
+__device__ __forceinline__ WideRow chunk_of(const WideArgs &a, const WideChunk &h) {
+    WideRow r = row_of(a, h.v);
+    const uint32_t at = (uint32_t)h.chunk * kWChunk;
+    r.bits += at >> 5;
+    r.col += at;
+    if (r.el) r.el += at;
+    if (h.chunk) r.off = 0;
+    r.span = min(r.span - at, (uint32_t)kWChunk);
+    return r;
+}
+__device__ __forceinline__ uint32_t row_bits(const WideRow &r, uint32_t w) {
+    uint32_t m = FULL;
+    if (w == 0) m <<= r.off;
+    if (r.span - 32 * w < 32) m &= (1u << (r.span - 32 * w)) - 1u;
+    return m;
+}
+
+// Walks the set bits of a row (first round: all its bits), 32 bitmap words at a
+// time, lane i holding word i.  An iteration takes four entries a lane, all loads
+// in flight together; f(bit, wu, j, pass) gets which of them are set, their
+// neighbours' omegas and their edge-label indices, and fills in which of them
+// pass; it returns whether to go on.  Either the lanes take four whole words
+// (coalesced), or, where that is fewer iterations, each lane the next four bits
+// of its own word: after the second round most words hold a bit or two.  UPDATE:
+// the bits become those that passed, with one atomic per changed word.
+template <bool FIRST, bool UPDATE, class F>
+__device__ __forceinline__ void walk(const WideArgs &a, const WideShared &S, const WideRow &r, uint32_t first_w,
+                                     uint32_t w_step, F f) {
+    const int lane = threadIdx.x & 31;
+    bool go = true;
+    for (uint32_t w0 = first_w; go && 32 * w0 < r.span; w0 += w_step) {
+        uint32_t word = 0;
+        if (32 * (w0 + lane) < r.span) {
+            word = row_bits(r, w0 + lane);
+            if (!FIRST) word &= r.bits[w0 + lane];
+        }
+        uint32_t groups = __ballot_sync(FULL, word != 0);
+        groups |= groups >> 1;
+        groups = (groups | (groups >> 2)) & 0x11111111u;
+        if (!groups) continue;
+        const bool own = !FIRST && __reduce_max_sync(FULL, (unsigned)__popc(word)) * 3 <= 8u * __popc(groups);
+        uint32_t left = word, kept = 0;
+        while (go && (own ? __any_sync(FULL, left != 0) : groups != 0)) {
+            const int g = own ? 0 : __ffs(groups) - 1;
+            groups &= groups - 1;
+            bool bit[4];
+            int32_t u[4];
+            uint8_t lb[4];
+            uint32_t at[4];                  // bit of `word` in own mode
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                uint32_t e;
+                if (own) {
+                    at[k] = left & (0u - left);
+                    left ^= at[k];
+                    bit[k] = at[k] != 0;
+                    e = 32 * (w0 + lane) + (31 - __clz(at[k] | 1u));
+                } else {
+                    at[k] = 0;
+                    bit[k] = (__shfl_sync(FULL, word, g + k) >> lane) & 1u;
+                    e = 32 * (w0 + g + k) + lane;
+                }
+                u[k] = bit[k] ? r.col[e] : 0;
+                lb[k] = bit[k] && r.el ? r.el[e] : (uint8_t)0;
+            }
+            uint64_t wu[4];
+            int j[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                wu[k] = bit[k] ? (FIRST ? S.lm[a.lab[u[k]]] : a.om_in[u[k]]) : 0ull;
+                j[k] = (int)S.T.el_index[lb[k]];
+            }
+            bool pass[4];
+            go = f(bit, wu, j, pass);
+            if (UPDATE) {
+                if (own) {
+#pragma unroll
+                    for (int k = 0; k < 4; k++) kept |= pass[k] ? at[k] : 0u;
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 4; k++) {
+                        const uint32_t p = __ballot_sync(FULL, pass[k]);
+                        if (lane == g + k) kept = p;
+                    }
+                }
+            }
+        }
+        if (UPDATE) {
+            if (FIRST && kept) atomicOr(&r.bits[w0 + lane], kept);
+            if (!FIRST && word != kept) atomicAnd(&r.bits[w0 + lane], ~(word & ~kept));
         }
     }
-    av = warp_sum64(av);
-    ae = warp_sum64(ae);
-    if (lane == 0) {
-        if (av) atomicAdd(&st->active_v, av);
-        if (ae) atomicAdd(&st->active_e, ae);
+}
+
+// A warp's share of a longer row.  A class is counted only until it is met,
+// which on long rows is within the first groups, and the unions only until they
+// hold all they can.  The warp that has the whole row to itself (WHOLE) counts
+// classes once coverage is known, and only those of the vertices it leaves: on
+// the entries in its registers if they are all, else on a second walk that ends
+// when they are met.  Lane i holds the counts of classes i and i + 32.
+template <int NEL>
+struct RowScan {
+    uint64_t U[NEL], open, keep;
+    uint32_t nN, c0, c1;
+    bool chg;
+};
+
+template <int NEL>
+__device__ __forceinline__ void count_classes(const WideTab &T, const uint64_t (&wu)[4], const int (&jk)[4],
+                                              RowScan<NEL> &R) {
+    const int lane = threadIdx.x & 31;
+    for (uint64_t o = R.open; o; o &= o - 1) {
+        const int c = __ffsll((long long)o) - 1;
+        const uint64_t cm = T.cls_mask[c];
+        const int cj = T.cls_j[c];
+        uint32_t h = 0;
+#pragma unroll
+        for (int k = 0; k < 4; k++) h += __popc(__ballot_sync(FULL, jk[k] == cj && (wu[k] & cm) != 0));
+        if (lane == (c & 31)) {
+            if (c < 32) R.c0 += h;
+            else R.c1 += h;
+        }
+    }
+    if (R.open) {
+        const uint64_t lo = __ballot_sync(FULL, R.c0 < T.cls_need[lane]);
+        const uint64_t hi = __ballot_sync(FULL, R.c1 < T.cls_need[lane + 32]);
+        R.open &= lo | (hi << 32);
     }
 }
 
-// Every entry's bit set; the bits past the last entry stay 0.
-__global__ void k_wide_fill(int64_t words, int64_t m, uint32_t *ebits) {
-    for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < words; w += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t left = m - (w << 5);
-        ebits[w] = left >= 32 ? FULL : ((1u << (uint32_t)left) - 1u);
+template <bool FIRST, int NEL, bool WHOLE>
+__device__ __forceinline__ void scan_row(const WideArgs &a, WideShared &S, uint64_t wv, const WideRow &r,
+                                         uint32_t first_w, uint32_t w_step, RowScan<NEL> &R, WideAcc &acc) {
+    const WideTab &T = S.T;
+    const int lane = threadIdx.x & 31;
+    uint64_t *const nb = S.nb[threadIdx.x >> 5][0];
+    {
+        uint64_t c = 0, m[NEL];
+#pragma unroll
+        for (int j = 0; j < NEL; j++) m[j] = R.U[j] = 0;
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const int q = lane + 32 * h;
+            if ((wv >> q) & 1ull) {
+                c |= T.q_cls[q];
+#pragma unroll
+                for (int j = 0; j < NEL; j++) m[j] |= T.adj[j][q];
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < NEL; j++) {
+            m[j] = warp_or64(m[j]);
+            if (lane == j) nb[j] = m[j];
+        }
+        __syncwarp();
+        R.open = !WHOLE && T.n_cls ? warp_or64(c) : 0ull;
+    }
+    R.keep = 0;
+    R.nN = R.c0 = R.c1 = 0;
+    R.chg = false;
+    bool full = false;                       // the unions hold all they can
+    uint32_t calls = 0;
+    uint64_t wl[4];                          // the last iteration's entries that pass
+    int jl[4];
+    walk<FIRST, true>(a, S, r, first_w, w_step, [&](const bool (&)[4], const uint64_t (&wu)[4], const int (&j)[4],
+                                                    bool (&pass)[4]) {
+        uint64_t m[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            m[k] = wu[k] & nb[j[k]];
+            const bool live = wu[k] != 0;
+            pass[k] = m[k] != 0;
+            if (live) acc.scanned++;
+            if (live && !pass[k]) R.chg = true;          // eta eliminates an active entry
+            if (pass[k]) R.nN++;
+            wl[k] = wu[k];
+            jl[k] = pass[k] ? j[k] : -1;
+        }
+        if (!full) {
+#pragma unroll
+            for (int k = 0; k < 4; k++)
+#pragma unroll
+                for (int i = 0; i < NEL; i++) R.U[i] |= m[k] & (jl[k] == i ? ~0ull : 0ull);
+            if (calls % 4 == 1) {
+                full = true;
+#pragma unroll
+                for (int i = 0; i < NEL; i++) {
+                    R.U[i] = warp_or64(R.U[i]);
+                    full = full && R.U[i] == nb[i];
+                }
+            }
+        }
+        calls++;
+        if (!WHOLE) count_classes<NEL>(T, wl, jl, R);
+        return true;
+    });
+#pragma unroll
+    for (int j = 0; j < NEL; j++)
+        if (!full) R.U[j] = warp_or64(R.U[j]);
+    R.nN = __reduce_add_sync(FULL, R.nN);
+    R.chg = __any_sync(FULL, R.chg);
+    if (WHOLE && R.nN) {
+        R.keep = covered<NEL>(T, wv, R.U, R.open);
+        if (R.open) {
+            if (calls == 1)
+                count_classes<NEL>(T, wl, jl, R);
+            else
+                walk<FIRST, false>(a, S, r, first_w, w_step, [&](const bool (&)[4], const uint64_t (&wu)[4],
+                                                                 const int (&j)[4], bool (&)[4]) {
+#pragma unroll
+                    for (int k = 0; k < 4; k++) jl[k] = wu[k] & nb[j[k]] ? j[k] : -1;
+                    count_classes<NEL>(T, wu, jl, R);
+                    return R.open != 0;
+                });
+            for (uint64_t o = R.open; o; o &= o - 1) R.keep &= ~(1ull << T.cls_q[__ffsll((long long)o) - 1]);
+        }
+    }
+}
+
+// After a row's omega changed: marks the ends of its entries for the next round
+// (its bits as they were read or are now: those dropped in this round were
+// dropped at their other end, too) and, if it died, wipes its bits.
+__device__ __forceinline__ void row_changed(const WideArgs &a, const WideRow &r, bool mark, bool dead, uint32_t first_w,
+                                            uint32_t w_step) {
+    const int lane = threadIdx.x & 31;
+    const uint8_t next = (uint8_t)(a.mark + 1);
+    for (uint32_t w = first_w; 32 * w < r.span; w += w_step) {
+        uint32_t word[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) word[k] = 32 * (w + k) < r.span ? r.bits[w + k] & row_bits(r, w + k) : 0u;
+        if (mark) {
+            int32_t u[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) u[k] = (word[k] >> lane) & 1u ? r.col[32 * (w + k) + lane] : -1;
+#pragma unroll
+            for (int k = 0; k < 4; k++)
+                if (u[k] >= 0) a.mark_out[u[k]] = next;
+        }
+        if (dead && lane < 4 && 32 * (w + lane) < r.span) atomicAnd(&r.bits[w + lane], ~row_bits(r, w + lane));
+    }
+}
+
+// The longer rows listed by the first round.
+template <bool FIRST, int NEL>
+__device__ __forceinline__ void long_part(const WideArgs &a, WideShared &S, WideAcc &acc) {
+    const WideTab &T = S.T;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, nwb = blockDim.x >> 5;
+    const int64_t n_hub = (int64_t)a.st->n_hub, n_mid = (int64_t)a.st->n_mid;
+    // chunks, one block each (block-uniform loop)
+    for (int64_t i = blockIdx.x; i < n_hub; i += gridDim.x) {
+        const WideChunk h = a.hub[i];
+        const int32_t v = h.v;
+        const uint64_t wv = FIRST ? S.lm[a.lab[v]] : a.om_in[v];
+        const bool skip = !FIRST && acc.marked && a.mark_in[v] != a.mark;
+        if (wv == 0 || skip) {               // dead, or nothing near it changed
+            if (threadIdx.x == 0) a.om_out[v] = wv;
+            if (threadIdx.x == 0 && wv && h.chunk == 0) {
+                acc.alive++;
+                acc.scanned += a.deg[v];
+            }
+            continue;
+        }
+        for (int c = threadIdx.x; c < kWCls; c += blockDim.x) S.bcnt[c] = 0;
+        if (threadIdx.x < kWEL) S.bU[threadIdx.x] = 0ull;
+        if (threadIdx.x == 0) { S.bN = 0; S.bchg = 0; }
+        __syncthreads();
+        RowScan<NEL> R;
+        scan_row<FIRST, NEL, false>(a, S, wv, chunk_of(a, h), 32 * wib, 32 * nwb, R, acc);
+        if (R.c0) atomicAdd(&S.bcnt[lane], R.c0);
+        if (R.c1) atomicAdd(&S.bcnt[lane + 32], R.c1);
+        if (lane == 0) {
+#pragma unroll
+            for (int j = 0; j < NEL; j++)
+                if (R.U[j]) atomicOr(&S.bU[j], (unsigned long long)R.U[j]);
+            if (R.nN) atomicAdd(&S.bN, R.nN);
+            if (R.chg) atomicOr(&S.bchg, 1u);
+        }
+        __syncthreads();
+        if (h.chunks > 1) {
+            // add to the row's totals; the block that is last takes them over
+            // (and leaves zeros for the next round)
+            WidePart &P = a.part[h.part];
+            if (threadIdx.x < kWCls) {
+                const uint32_t c = S.bcnt[threadIdx.x];
+                if (c) atomicAdd(&P.cnt[threadIdx.x], c);
+            } else if (threadIdx.x < kWCls + NEL) {
+                const unsigned long long U = S.bU[threadIdx.x - kWCls];
+                if (U) atomicOr(&P.U[threadIdx.x - kWCls], U);
+            } else if (threadIdx.x == kWCls + kWEL) {
+                if (S.bN) atomicAdd(&P.nN, S.bN);
+                if (S.bchg) atomicOr(&P.chg, 1u);
+            }
+            __threadfence();
+            __syncthreads();
+            if (threadIdx.x == 0) S.last = atomicAdd(&P.done, 1u) + 1 == (uint32_t)h.chunks;
+            __syncthreads();
+            if (!S.last) continue;
+            __threadfence();
+            if (threadIdx.x < kWCls) S.bcnt[threadIdx.x] = atomicExch(&P.cnt[threadIdx.x], 0u);
+            else if (threadIdx.x < kWCls + NEL) S.bU[threadIdx.x - kWCls] = atomicExch(&P.U[threadIdx.x - kWCls], 0ull);
+            else if (threadIdx.x == kWCls + kWEL) {
+                S.bN = atomicExch(&P.nN, 0u);
+                S.bchg = atomicExch(&P.chg, 0u);
+                P.done = 0;
+            }
+            __syncthreads();
+        }
+        uint64_t keep = 0;                   // every warp decides
+        if (S.bN) {
+            uint64_t U[NEL], cls;
+#pragma unroll
+            for (int j = 0; j < NEL; j++) U[j] = S.bU[j];
+            keep = covered<NEL>(T, wv, U, cls);
+            const uint64_t lo = __ballot_sync(FULL, S.bcnt[lane] < T.cls_need[lane]);
+            const uint64_t hi = __ballot_sync(FULL, S.bcnt[lane + 32] < T.cls_need[lane + 32]);
+            for (uint64_t o = cls & (lo | (hi << 32)); o; o &= o - 1)
+                keep &= ~(1ull << T.cls_q[__ffsll((long long)o) - 1]);
+        }
+        if (threadIdx.x == 0) {
+            acc.alive++;
+            a.om_out[v] = keep;
+            a.deg[v] = S.bN;
+            if (keep != wv) acc.moved++;     // its entries: k_wide_hubs
+            if (keep != wv || S.bchg) acc.changed = true;
+        }
+        __syncthreads();                     // bcnt / bU / bN are reused
+    }
+    // one warp each; a warp looks at four listed rows at a time
+    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t i0 = gw * 4; i0 < n_mid; i0 += nw * 4) {
+        int32_t v4 = 0;
+        uint64_t w4 = 0;
+        if (lane < 4 && i0 + lane < n_mid) {
+            v4 = a.mid[i0 + lane];
+            w4 = FIRST ? S.lm[a.lab[v4]] : a.om_in[v4];
+            const bool skip = !FIRST && acc.marked && w4 && a.mark_in[v4] != a.mark;
+            if (!w4 || skip) a.om_out[v4] = w4;
+            if (skip) {
+                acc.alive++;
+                acc.scanned += a.deg[v4];
+                w4 = 0;
+            }
+        }
+        for (uint32_t b = __ballot_sync(FULL, w4 != 0); b; b &= b - 1) {
+            const int l = __ffs(b) - 1;
+            const int32_t v = __shfl_sync(FULL, v4, l);
+            const uint64_t wv = __shfl_sync(FULL, w4, l);
+            const WideRow r = row_of(a, v);
+            RowScan<NEL> R;
+            scan_row<FIRST, NEL, true>(a, S, wv, r, 0, 32, R, acc);
+            const bool mark = !FIRST && acc.push && R.keep != wv, dead = !R.keep && R.nN;
+            if (mark || dead) {
+                __syncwarp();                // after the scan's own bits
+                row_changed(a, r, mark, dead, 0, 4);
+            }
+            if (lane == 0) {
+                acc.alive++;
+                a.om_out[v] = R.keep;
+                a.deg[v] = R.nN;
+                if (R.keep != wv) acc.moved++;
+                if (mark && R.keep) a.mark_out[v] = (uint8_t)(a.mark + 1);
+            }
+            if (R.keep != wv || R.chg) acc.changed = true;
+        }
+    }
+}
+
+// One snapshot round; the first one is two launches, since its longer rows are
+// listed by the pass over the short ones.
+enum { kWFirstShort, kWFirstLong, kWLater };
+
+template <int PART, int NEL>
+__global__ void __launch_bounds__(256, NEL <= 4 ? 4 : 2) k_wide_round(WideArgs a) {
+    constexpr bool FIRST = PART != kWLater;
+    __shared__ WideShared S;
+    const WideRound before = a.st->r[a.slot];
+    if (!FIRST && !before.changed) return;   // the round before was the last
+    const int64_t n_in = PART == kWFirstLong ? 0 : FIRST ? a.n : (int64_t)before.n_list;
+    const int nwb = blockDim.x >> 5;
+    bool work = (int64_t)blockIdx.x * nwb * kWTile < n_in;
+    if (PART != kWFirstShort)
+        work = work || (int64_t)blockIdx.x < (int64_t)a.st->n_hub ||
+               (int64_t)blockIdx.x * nwb * 4 < (int64_t)a.st->n_mid;
+    if (!work) return;
+    load_tab(S.T, a.tab);
+    if (FIRST)
+        for (int i = threadIdx.x; i < 256; i += blockDim.x) S.lm[i] = a.lmask[i];
+    if (threadIdx.x == 0) { S.scanned = S.alive = S.moved = 0; S.changed = 0; }
+    for (int i = threadIdx.x; i < 8 * 4; i += blockDim.x) S.nb[i >> 2][i & 3][kWEL] = 0;
+    __syncthreads();
+    WideAcc acc;
+    if (!FIRST) {
+        // without a change of an omega nothing needs a mark
+        acc.marked = before.pushed || !before.moved;
+        acc.push = acc.marked || before.moved * kWPush < before.alive;
+    }
+    if (PART != kWFirstShort) long_part<FIRST, NEL>(a, S, acc);
+    if (PART != kWFirstLong) short_part<FIRST, NEL>(a, S, n_in, acc);
+    // one atomic per block
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc.scanned += __shfl_xor_sync(FULL, acc.scanned, o);
+    const uint32_t alive = __reduce_add_sync(FULL, acc.alive), moved = __reduce_add_sync(FULL, acc.moved);
+    const bool changed = __any_sync(FULL, acc.changed);
+    if (lane == 0) {
+        if (acc.scanned) atomicAdd(&S.scanned, acc.scanned);
+        if (alive) atomicAdd(&S.alive, (unsigned long long)alive);
+        if (moved) atomicAdd(&S.moved, (unsigned long long)moved);
+        if (changed) atomicOr(&S.changed, 1u);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        WideRound *r = &a.st->r[a.slot + 1];
+        if (S.scanned) atomicAdd(&r->scanned, S.scanned);
+        if (S.alive) atomicAdd(&r->alive, S.alive);
+        if (S.moved) atomicAdd(&r->moved, S.moved);
+        if (acc.push) r->pushed = 1;
+        if (S.changed) atomicOr(&r->changed, 1u);
+    }
+}
+
+// The chunks of rows whose omega changed in this round, a block each: marks and
+// wiping, spread like the round's own work (one block per such row left a tail).
+template <bool FIRST>
+__global__ void __launch_bounds__(256) k_wide_hubs(WideArgs a) {
+    const WideRound &now = a.st->r[a.slot + 1];
+    if (!now.moved) return;
+    const int64_t n_hub = (int64_t)a.st->n_hub;
+    for (int64_t i = blockIdx.x; i < n_hub; i += gridDim.x) {
+        const WideChunk h = a.hub[i];
+        const uint64_t wv = FIRST ? a.lmask[a.lab[h.v]] : a.om_in[h.v], keep = a.om_out[h.v];
+        if (keep == wv) continue;
+        const bool mark = !FIRST && now.pushed;
+        if (mark && threadIdx.x == 0 && keep) a.mark_out[h.v] = (uint8_t)(a.mark + 1);
+        if (mark || !keep)
+            row_changed(a, chunk_of(a, h), mark, !keep, 4 * (threadIdx.x >> 5), 4 * (blockDim.x >> 5));
+    }
+}
+
+template <int NEL>
+void launch_round(const WideArgs &a, bool first, int grid, int hub_grid, cudaStream_t s) {
+    if (first) {
+        k_wide_round<kWFirstShort, NEL><<<grid, 256, 0, s>>>(a);
+        k_wide_round<kWFirstLong, NEL><<<grid, 256, 0, s>>>(a);
+        if (hub_grid) k_wide_hubs<true><<<hub_grid, 256, 0, s>>>(a);
+    } else {
+        k_wide_round<kWLater, NEL><<<grid, 256, 0, s>>>(a);
+        if (hub_grid) k_wide_hubs<false><<<hub_grid, 256, 0, s>>>(a);
     }
 }
 
@@ -455,29 +929,24 @@ int build_tab(int n0, const uint8_t *labels, int m0, const int32_t *edges, const
                 t.cls_need[t.n_cls] = (uint32_t)popc64(grp);
                 t.cls_q[t.n_cls] = (uint8_t)q;
                 t.cls_j[t.n_cls] = (uint8_t)j;
+                t.q_cls[q] |= 1ull << t.n_cls;
                 t.n_cls++;
             }
         }
+    for (uint8_t &j : t.el_index)
+        if (j == 0xFF) j = kWEL;
     std::memset(lmask, 0, sizeof(uint64_t) * 256);
     for (int q = 0; q < n0; q++) lmask[labels[q]] |= 1ull << q;
     return CCPM_OK;
 }
 
-// Device buffers of one call, freed on every return path.
+// Device memory of one call, freed on every return path.  One allocation: ten
+// of them and their releases took 1 ms on a graph of 4M vertices.
 struct WideBufs {
-    WideTab *tab = nullptr;
-    uint64_t *lmask = nullptr;
-    uint64_t *om[2] = {nullptr, nullptr};
-    int32_t *list[2] = {nullptr, nullptr};
-    int32_t *hub[2] = {nullptr, nullptr};
-    uint32_t *bits = nullptr;
-    WideCounters *st = nullptr;
-    WideCounters *st_h = nullptr;
+    char *mem = nullptr;
     cudaEvent_t ev[2] = {nullptr, nullptr};
     ~WideBufs() {
-        cudaFree(tab); cudaFree(lmask); cudaFree(om[0]); cudaFree(om[1]);
-        cudaFree(list[0]); cudaFree(list[1]); cudaFree(hub[0]); cudaFree(hub[1]); cudaFree(bits); cudaFree(st);
-        if (st_h) cudaFreeHost(st_h);
+        cudaFree(mem);
         for (auto e : ev) if (e) cudaEventDestroy(e);
     }
 };
@@ -511,73 +980,97 @@ extern "C" int ccpm_lcc_wide(ccpm_ctx_t ctx, ccpm_graph_t g, int n0, const uint8
         cudaError_t e_ = (call);                 \
         if (e_ != cudaSuccess) return fail(e_, what); \
     } while (0)
-    WCU(cudaMalloc(&B.tab, sizeof(WideTab)), "alloc");
-    WCU(cudaMalloc(&B.lmask, sizeof(lmask)), "alloc");
-    for (int i = 0; i < 2; i++) {
-        WCU(cudaMalloc(&B.om[i], sizeof(uint64_t) * (size_t)std::max<int64_t>(n, 1)), "alloc");
-        WCU(cudaMalloc(&B.list[i], sizeof(int32_t) * (size_t)std::max<int64_t>(n, 1)), "alloc");
-        WCU(cudaMalloc(&B.hub[i], sizeof(int32_t) * (size_t)std::max<int64_t>(n, 1)), "alloc");
-    }
-    WCU(cudaMalloc(&B.bits, sizeof(uint32_t) * (size_t)std::max<int64_t>(words, 1)), "alloc");
-    WCU(cudaMalloc(&B.st, sizeof(WideCounters)), "alloc");
-    WCU(cudaMallocHost(&B.st_h, sizeof(WideCounters)), "alloc");
+    size_t size = 0;
+    auto part = [&](size_t bytes) {
+        const size_t at = size;
+        size += (bytes + 255) / 256 * 256;
+        return at;
+    };
+    // a row of more than k entries takes k + 1 of the m
+    // (a chunked row may take one chunk more, being counted from a bitmap word)
+    const int64_t max_mid = std::min(n, m / (kWShort + 1)), max_rows = std::min(n, m / (kWHub + 1)),
+                  max_hub = m / kWChunk + 2 * max_rows, max_part = std::min(n, m / (kWChunk - 31));
+    const size_t at_tab = part(sizeof(WideTab)), at_lm = part(sizeof(lmask)), at_st = part(sizeof(WideState)),
+                 at_bits = part(sizeof(uint32_t) * (size_t)words), at_om0 = part(sizeof(uint64_t) * (size_t)n),
+                 at_om1 = part(sizeof(uint64_t) * (size_t)n), at_mark0 = part((size_t)n), at_mark1 = part((size_t)n),
+                 at_deg = part(sizeof(uint32_t) * (size_t)n), at_l0 = part(sizeof(int32_t) * (size_t)n),
+                 at_l1 = part(sizeof(int32_t) * (size_t)n), at_mid = part(sizeof(int32_t) * (size_t)max_mid),
+                 at_hub = part(sizeof(WideChunk) * (size_t)max_hub),
+                 at_part = part(sizeof(WidePart) * (size_t)max_part);
+    WCU(cudaMalloc(&B.mem, size), "alloc");
+    uint64_t *const om[2] = {(uint64_t *)(B.mem + at_om0), (uint64_t *)(B.mem + at_om1)};
+    int32_t *const list[2] = {(int32_t *)(B.mem + at_l0), (int32_t *)(B.mem + at_l1)};
+    uint32_t *const bits = (uint32_t *)(B.mem + at_bits);
+    WideState *const st = (WideState *)(B.mem + at_st);
+    WideState sh;
     WCU(cudaEventCreate(&B.ev[0]), "event");
     WCU(cudaEventCreate(&B.ev[1]), "event");
-    WCU(cudaMemcpyAsync(B.tab, &tab, sizeof(WideTab), cudaMemcpyHostToDevice, s), "copy");
-    WCU(cudaMemcpyAsync(B.lmask, lmask, sizeof(lmask), cudaMemcpyHostToDevice, s), "copy");
+    WCU(cudaMemcpyAsync(B.mem + at_tab, &tab, sizeof(WideTab), cudaMemcpyHostToDevice, s), "copy");
+    WCU(cudaMemcpyAsync(B.mem + at_lm, lmask, sizeof(lmask), cudaMemcpyHostToDevice, s), "copy");
     WCU(cudaEventRecord(B.ev[0], s), "event");
-    WCU(cudaMemsetAsync(B.st, 0, sizeof(WideCounters), s), "memset");
-    if (words > 0) {
-        k_wide_fill<<<grid_of(ctx, words, 256, 8), 256, 0, s>>>(words, m, B.bits);
-        WCU(cudaGetLastError(), "launch");
-    }
-    k_wide_init<<<grid_of(ctx, n, 256, 8), 256, 0, s>>>(n, G.rp, G.lab, B.lmask, B.om[0], B.om[1], B.list[0],
-                                                         B.hub[0], B.st);
-    WCU(cudaGetLastError(), "launch");
-    WCU(cudaMemcpyAsync(B.st_h, B.st, sizeof(WideCounters), cudaMemcpyDeviceToHost, s), "copy");
-    WCU(cudaStreamSynchronize(s), "sync");
-    int64_t n_in = (int64_t)B.st_h->n_next, n_hub = (int64_t)B.st_h->n_hub_next;
-    int64_t rounds = 0, scanned = 0, alive = 0;
-    int cur = 0, li = 0;
-    for (;;) {
-        WCU(cudaMemsetAsync(B.st, 0, sizeof(WideCounters), s), "memset");
-        WideArgs a;
-        a.rp = G.rp;
-        a.col = G.col;
-        a.el = G.el;
-        a.om_in = B.om[cur];
-        a.om_out = B.om[cur ^ 1];
-        a.ebits = B.bits;
-        a.list_in = B.list[li];
-        a.n_in = n_in;
-        a.list_out = B.list[li ^ 1];
-        a.hub_in = B.hub[li];
-        a.n_hub = n_hub;
-        a.hub_out = B.hub[li ^ 1];
-        a.st = B.st;
-        a.tab = B.tab;
-        const int grid = std::max(grid_of(ctx, n_in * 32, 256, 8), grid_of(ctx, n_hub * 256, 256, 8));
-        k_wide_round<<<grid, 256, 0, s>>>(a);
-        WCU(cudaGetLastError(), "launch");
-        WCU(cudaMemcpyAsync(B.st_h, B.st, sizeof(WideCounters), cudaMemcpyDeviceToHost, s), "copy");
+    // counters, bits and marks 0; the first round writes om[0] in full, later ones
+    // the listed vertices of the other buffer
+    WCU(cudaMemsetAsync(B.mem + at_st, 0, at_om0 - at_st, s), "memset");
+    WCU(cudaMemsetAsync(B.mem + at_om1, 0, at_deg - at_om1, s), "memset");
+    WideArgs a;
+    a.n = n;
+    a.rp = G.rp;
+    a.col = G.col;
+    a.lab = G.lab;
+    a.el = G.el;
+    a.lmask = (const uint64_t *)(B.mem + at_lm);
+    a.ebits = bits;
+    a.deg = (uint32_t *)(B.mem + at_deg);
+    a.mid = (int32_t *)(B.mem + at_mid);
+    a.hub = (WideChunk *)(B.mem + at_hub);
+    a.part = (WidePart *)(B.mem + at_part);
+    if (max_part) WCU(cudaMemsetAsync(a.part, 0, sizeof(WidePart) * (size_t)max_part, s), "memset");
+    a.st = st;
+    a.tab = (const WideTab *)(B.mem + at_tab);
+    const int grid = std::max(std::max(grid_of(ctx, n, 8 * kWTile, 8), grid_of(ctx, max_mid, 32, 8)),
+                              grid_of(ctx, max_hub, 1, 8));
+    const int hub_grid = max_hub ? grid_of(ctx, max_hub, 1, 8) : 0;
+    uint8_t *const mark[2] = {(uint8_t *)(B.mem + at_mark0), (uint8_t *)(B.mem + at_mark1)};
+    int64_t rounds = 0, scanned = 0, alive = 0, active_v = 0, active_e = 0;
+    for (bool more = true; more;) {
+        if (rounds) {
+            WCU(cudaMemcpyAsync(&st->r[0], &st->r[kWQueue], sizeof(WideRound), cudaMemcpyDeviceToDevice, s), "copy");
+            WCU(cudaMemsetAsync(&st->r[1], 0, sizeof(WideRound) * kWQueue, s), "memset");
+        }
+        for (int i = 0; i < kWQueue; i++) {
+            const int64_t t = rounds + i;
+            a.slot = i;
+            a.mark = (uint8_t)t;             // of one of the last 256 rounds: an older one only costs time
+            a.mark_in = mark[(t + 1) & 1];
+            a.mark_out = mark[t & 1];
+            a.om_in = om[(t + 1) & 1];
+            a.om_out = om[t & 1];
+            a.list_in = list[(t + 1) & 1];
+            a.list_out = list[t & 1];
+            if (tab.n_el <= 1) launch_round<1>(a, t == 0, grid, hub_grid, s);
+            else if (tab.n_el == 2) launch_round<2>(a, t == 0, grid, hub_grid, s);
+            else if (tab.n_el == 3) launch_round<3>(a, t == 0, grid, hub_grid, s);
+            else launch_round<8>(a, t == 0, grid, hub_grid, s);
+            WCU(cudaGetLastError(), "launch");
+        }
+        WCU(cudaMemcpyAsync(&sh, st, sizeof(sh), cudaMemcpyDeviceToHost, s), "copy");
         WCU(cudaStreamSynchronize(s), "sync");
-        rounds++;
-        scanned += (int64_t)B.st_h->scanned;
-        alive += (int64_t)B.st_h->alive;
-        cur ^= 1;                  // omega of the round just run
-        li ^= 1;
-        n_in = (int64_t)B.st_h->n_next;
-        n_hub = (int64_t)B.st_h->n_hub_next;
-        if (!B.st_h->changed) break;
+        for (int i = 0; i < kWQueue && more; i++) {
+            rounds++;
+            const WideRound &r = sh.r[i + 1];
+            scanned += (int64_t)r.scanned;
+            alive += (int64_t)r.alive;
+            more = r.changed != 0;
+            // a round without a change read the active vertices and entries
+            active_v = (int64_t)r.alive;
+            active_e = (int64_t)r.scanned;
+        }
     }
-    WCU(cudaMemsetAsync(B.st, 0, sizeof(WideCounters), s), "memset");
-    k_wide_clear<<<grid_of(ctx, n * 32, 256, 8), 256, 0, s>>>(n, G.rp, G.col, B.om[cur], B.bits, B.st);
-    WCU(cudaGetLastError(), "launch");
     WCU(cudaEventRecord(B.ev[1], s), "event");
     const cudaMemcpyKind kind = out_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-    if (n > 0) WCU(cudaMemcpyAsync(omega, B.om[cur], sizeof(uint64_t) * (size_t)n, kind, s), "copy");
-    if (words > 0) WCU(cudaMemcpyAsync(ebits, B.bits, sizeof(uint32_t) * (size_t)words, kind, s), "copy");
-    WCU(cudaMemcpyAsync(B.st_h, B.st, sizeof(WideCounters), cudaMemcpyDeviceToHost, s), "copy");
+    if (n > 0)
+        WCU(cudaMemcpyAsync(omega, om[(rounds - 1) & 1], sizeof(uint64_t) * (size_t)n, kind, s), "copy");
+    if (words > 0) WCU(cudaMemcpyAsync(ebits, bits, sizeof(uint32_t) * (size_t)words, kind, s), "copy");
     WCU(cudaStreamSynchronize(s), "sync");
 #undef WCU
     if (stats) {
@@ -586,8 +1079,8 @@ extern "C" int ccpm_lcc_wide(ccpm_ctx_t ctx, ccpm_graph_t g, int n0, const uint8
         stats->rounds = rounds;
         stats->edges_scanned = scanned;
         stats->vertices_scanned = alive;
-        stats->active_v = (int64_t)B.st_h->active_v;
-        stats->active_e_dir = (int64_t)B.st_h->active_e;
+        stats->active_v = active_v;
+        stats->active_e_dir = active_e;
         stats->ms = ms;
     }
     return CCPM_OK;
