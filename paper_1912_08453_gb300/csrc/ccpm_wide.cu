@@ -21,9 +21,18 @@
 // later rounds, which read their counts on the device: four rounds are queued at
 // a time, and those after the quiescent one return at once.  Rows up to kWShort
 // entries go four to a warp, rows up to kWHub one to a warp, longer ones to
-// blocks in chunks; the block that finishes a row's last chunk decides it.  No
-// kernel waits on another block: every loop is bounded by the list or row it
-// walks.
+// blocks in chunks; the block that finishes a row's last chunk decides it.  Once
+// few vertices change, their neighbours are marked and a round evaluates only
+// those; the others count as what they read last.  No kernel waits on another
+// block: every loop is bounded by the list or row it walks.
+//
+// Figures: 4M vertices, 124M entries, a sampled template of 48 vertices and 3
+// edge labels; 112M, 40M, 17M, 6M and 6M entries read by the five rounds.  With
+// one warp a row, every window of every row in each round, per-vertex list
+// atomics and a hand-back pass over the bitmap they took 7.2, 4.9, 2.9, 0.7 and
+// 0.5 ms, the hand-back 1.9 and allocations 1 ms.  Now 0.24 + 0.89, 0.89, 0.66,
+// 0.37 and 0.07 ms, and 0.25 for the allocation.  What bounds them: instructions
+// (45 % of the issue slots) and gather latency at 32 warps an SM.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -47,7 +56,7 @@ constexpr int kWHub = 1024;    // rows longer than this are walked by whole bloc
 constexpr int kWChunk = 8192;  // entries a block takes of one: 1024 for each of its 8 warps
 constexpr int kWTile = 128;    // listed vertices a warp looks through at a time
 constexpr int kWQueue = 4;     // rounds queued per host round trip
-constexpr int kWPush = 4;      // neighbours are marked once at most one active vertex in so many changes
+constexpr int kWPush = 4;      // neighbours are marked once less than one active vertex in so many changes
 constexpr unsigned FULL = 0xFFFFFFFFu;
 
 // Template tables of one call (device copy, loaded into shared memory).
@@ -436,7 +445,8 @@ __device__ __forceinline__ uint32_t row_bits(const WideRow &r, uint32_t w) {
 // neighbours' omegas and their edge-label indices, and fills in which of them
 // pass; it returns whether to go on.  Either the lanes take four whole words
 // (coalesced), or, where that is fewer iterations, each lane the next four bits
-// of its own word: after the second round most words hold a bit or two.  UPDATE:
+// of its own word: after the second round most words hold a bit or two (rounds 2
+// to 4: 1.07, 0.98 and 0.65 ms with whole words only, 0.89, 0.66 and 0.37 so).  UPDATE:
 // the bits become those that passed, with one atomic per changed word.
 template <bool FIRST, bool UPDATE, class F>
 __device__ __forceinline__ void walk(const WideArgs &a, const WideShared &S, const WideRow &r, uint32_t first_w,
@@ -786,6 +796,8 @@ __device__ __forceinline__ void long_part(const WideArgs &a, WideShared &S, Wide
 // listed by the pass over the short ones.
 enum { kWFirstShort, kWFirstLong, kWLater };
 
+// Four blocks an SM (64 registers): with 2, 3 and 5 the rounds above took 6.3,
+// 3.7 and 4.1 ms in all instead of 3.2.
 template <int PART, int NEL>
 __global__ void __launch_bounds__(256, NEL <= 4 ? 4 : 2) k_wide_round(WideArgs a) {
     constexpr bool FIRST = PART != kWLater;
@@ -941,7 +953,7 @@ int build_tab(int n0, const uint8_t *labels, int m0, const int32_t *edges, const
 }
 
 // Device memory of one call, freed on every return path.  One allocation: ten
-// of them and their releases took 1 ms on a graph of 4M vertices.
+// of them and their releases took 1 ms on a graph of 4M vertices, this takes 0.25.
 struct WideBufs {
     char *mem = nullptr;
     cudaEvent_t ev[2] = {nullptr, nullptr};
