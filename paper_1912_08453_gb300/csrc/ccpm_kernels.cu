@@ -2221,15 +2221,18 @@ k_compact_fill(CompactArgs a) {
         }
         place_ranked(a, beg, end, gstart + before);
     }
-    // whole rows, 32 list entries per warp step.  A row keeping at most 16
+    // whole rows, up to 32 list entries per warp step.  A row keeping at most 16
     // entries (most of them, once the first round has run) is written by its
     // own lane, one pass per label rank; the others by the whole warp in turn.
+    // Short lists are dealt out over more warps, down to four rows each (and one
+    // slot atomic): 1000 rows, 630 of them long, took 72 us at 32 a step.
     const int64_t n_rows = n_med + n_small;
-    for (int64_t b = gwarp * 32; b < n_rows; b += nwarps * 32) {
+    const int per = (int)max((int64_t)4, min((int64_t)32, n_rows / nwarps));
+    for (int64_t b = gwarp * per; b < n_rows; b += nwarps * per) {
         const int64_t idx = b + lane;
         int32_t vl = -1;
         int64_t beg = 0, end = 0, out = 0, k = 0;
-        if (idx < n_rows) {
+        if (lane < per && idx < n_rows) {
             vl = idx < n_med ? a.med_in[idx] : a.small_in[idx - n_med];
             if (__ldg(a.om + vl) == 0u) vl = -1;
         }
@@ -2780,9 +2783,17 @@ __device__ __forceinline__ void mark_window(const SearchArgs &a, const DevPlan &
 // and mark the vertices and edges of every one / count them and list them.
 constexpr int kExist = 0, kCount = 1, kMark = 2, kList = 3;
 
-// Windows a search scans at least before it hands work on to idle warps, and
-// between its looks at what the other warps do.
-constexpr uint64_t kLook = 16;
+// Windows between a search's looks at what the other warps do, and so at least
+// before it hands work on to idle ones.  A window that marks takes up to 8 us
+// (every match's edges are looked up), one that only asks or counts 1 us, but all
+// warps look at the same two words.  us of a prune with a 6-vertex tree on 5785
+// vertices, of one with a 5-cycle on 16M, and of a listing on 1M, at 16, 8, 4 and
+// 2 windows in every mode: 754, 542, 422, 440; 7917, 7281, 7363, 8018; 1791, 1821,
+// 2085, 2629.  With 4 where marks are made, else 8: 415, 7040 and 1800.  A listing
+// over fewer than kFewItems items hands on at once, the quickest way to more items
+// (9*10^6 entries, 3 roots: 470 -> 370 us); pruning lost by it (415 -> 455 us).
+__host__ __device__ constexpr uint64_t look_windows(int mode) { return mode == kMark ? 4 : 8; }
+constexpr int64_t kFewItems = 1024;
 constexpr int kSpillParts = 32;      // items one open level's untested candidates become, at most
 
 // Hand the rest of a long search to other warps.  Every open level L (d0..d)
@@ -2866,6 +2877,10 @@ __device__ bool search_from(const SearchArgs &a, const DevPlan &P, int d0, WarpS
                             uint32_t part_lo = 0u, uint32_t part_hi = 0u) {
     const int lane = (int)lane_id();
     const int k = P.k;
+    const uint64_t look_every = MODE == kList && a.starve && W.n_items < kFewItems ? 1 : look_windows(MODE);
+    bool pending = false;
+    unsigned int was_stop = 0;
+    unsigned long long was_next = 0;
     uint64_t used = 0;
     unsigned long long pub = (MODE == kCount || MODE == kMark) ? W.pub : 0;   // matches published so far
     if (d0 >= k) {                                  // the placed prefix is already a full map
@@ -2891,15 +2906,28 @@ __device__ bool search_from(const SearchArgs &a, const DevPlan &P, int d0, WarpS
             const int64_t pos = W.pos[d], end = W.end[d];
             if (pos >= end) { d--; continue; }
             if (++used > a.budget) { over = true; return MODE == kExist; }
-            // every kLook windows (marking: and every 128 matches): has another
+            // every few windows (marking: and every 128 matches): has another
             // warp answered this existence question already, has the count run
             // past its cap, are other warps out of work?
-            const bool look = (used & (kLook - 1)) == 0u || (MODE == kMark && matches - pub >= 128u);
+            bool look = (used & (look_every - 1)) == 0u || (MODE == kMark && matches - pub >= 128u);
+            if (MODE == kExist || MODE == kList) {
+                // loaded here, looked at a window later
+                const bool due = pending;
+                pending = look;
+                look = due;
+            }
+            unsigned int seen_stop = was_stop;
+            unsigned long long seen_next = was_next;
+            if ((MODE == kExist || MODE == kList) && pending && lane == 0) {
+                if (MODE == kList) was_stop = *(volatile const unsigned int *)&a.st->overflow;
+                else was_stop = W.done_word ? *(volatile const uint32_t *)W.done_word & W.done_bit : 0u;
+                if (a.starve) was_next = *(volatile const unsigned long long *)&a.ctl->next;
+            }
             if (look) {
                 unsigned int stop = 0, hand = 0;
                 if (lane == 0) {
                     if (MODE == kExist) {
-                        stop = W.done_word && (*(volatile const uint32_t *)W.done_word & W.done_bit);
+                        stop = seen_stop;
                     } else if (MODE == kCount || MODE == kMark) {
                         // counting (and marking) stops as soon as the total passes
                         // the cap: publish this warp's new matches and read the
@@ -2910,10 +2938,11 @@ __device__ bool search_from(const SearchArgs &a, const DevPlan &P, int d0, WarpS
                         W.pub = matches;
                         stop = tot > a.cap || *(volatile const unsigned int *)&a.st->overflow;
                     } else {
-                        stop = matches > a.cap || *(volatile const unsigned int *)&a.st->overflow;
+                        stop = matches > a.cap || seen_stop;
                     }
-                    if (a.starve && used >= kLook)
-                        hand = *(volatile const unsigned long long *)&a.ctl->next >= (unsigned long long)W.n_items;
+                    if (MODE == kCount || MODE == kMark)
+                        seen_next = a.starve && used >= look_every ? *(volatile const unsigned long long *)&a.ctl->next : 0ull;
+                    hand = a.starve && seen_next >= (unsigned long long)W.n_items;
                 }
                 pub = matches;
                 if (__shfl_sync(FULL_MASK, stop, 0)) {
