@@ -113,9 +113,10 @@ typedef struct {
                                    /* 1 = after every round that leaves some, -1 = */
                                    /* never; results are the same in all modes     */
     int      search_split;         /* windows a search scans before it hands its   */
-                                   /* untried candidates to other warps: 0 = the   */
-                                   /* library default (2048), -1 = never; results  */
-                                   /* are the same for every value                 */
+                                   /* untried candidates to other warps even when  */
+                                   /* none is idle (it does so sooner when they    */
+                                   /* are): 0 = the library default (2048), -1 =   */
+                                   /* never; results are the same for every value  */
     int      lcc_only;             /* 1: stop at the first LCC fixpoint (no non-   */
                                    /* local constraint, no final search); the     */
                                    /* result holds that fixpoint                   */

@@ -1,6 +1,6 @@
 """The fused training loop against single steps made of the gradient kernel and
 an Adam update in float64, on the same sampled rows, at the edges of its row
-split (64-row tiles, one to eight blocks with some) and of the rule that selects it.
+split (64-row tiles, one to eight blocks at work) and of the rule that selects it.
 
 Tolerance: both sides round the same operands to BF16, so gradients differ by
 the order of FP32 sums and by the odd activation that rounds to the neighbouring
