@@ -3882,7 +3882,11 @@ struct ccpm_result {
 
 namespace {
 
+// Every CUDA failure is reported through here, so the runtime's record of it is
+// cleared here: left standing, the next call would find it after its first
+// launch and fail for it.
 int set_err(ccpm_ctx *ctx, int code, const std::string &msg) {
+    if (code == CCPM_ENOMEM || code == CCPM_ECUDA) cudaGetLastError();
     if (ctx) ctx->err = msg;
     return code;
 }

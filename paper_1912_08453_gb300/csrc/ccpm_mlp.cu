@@ -663,6 +663,13 @@ int configure_kernels() {
     return CCPM_OK;
 }
 
+// A refused allocation: reported by its own call, and not once more by the
+// check after the next launch.
+int no_memory() {
+    cudaGetLastError();
+    return CCPM_ENOMEM;
+}
+
 // Device scratch for one call (X, targets, sampled rows).
 struct Scratch {
     float *x = nullptr, *t = nullptr;
@@ -670,7 +677,7 @@ struct Scratch {
     ~Scratch() { cudaFree(x); }  // the others lie behind x
     int alloc(size_t rows, size_t picks) {
         if (cudaMalloc(&x, sizeof(float) * rows * (IN + 1) + sizeof(int32_t) * picks) != cudaSuccess)
-            return CCPM_ENOMEM;
+            return no_memory();
         t = x + rows * IN;
         idx = (int32_t *)(t + rows);
         return CCPM_OK;
@@ -702,7 +709,7 @@ int mlp_score(ccpm_mlp *m, int B, const float *host_x, float *host_y, void *stre
         if (cudaMalloc(&sc.dx, sizeof(float) * (size_t)cap * (IN + 1)) != cudaSuccess ||
             cudaMallocHost(&sc.hx, sizeof(float) * (size_t)cap * (IN + 1)) != cudaSuccess) {
             mlp_scratch_free(sc);
-            return CCPM_ENOMEM;
+            return no_memory();
         }
         sc.dy = sc.dx + (size_t)cap * IN;
         sc.hy = sc.hx + (size_t)cap * IN;
@@ -744,7 +751,7 @@ int ccpm_mlp_create(ccpm_ctx_t ctx, uint64_t seed, ccpm_mlp_t *out) {
     // as much as several training steps
     if (cudaMalloc(&m->prm, sizeof(float) * (4 * NPARAM + 1)) != cudaSuccess) {
         ccpm_mlp_destroy(m);
-        return CCPM_ENOMEM;
+        return no_memory();
     }
     m->grad = m->prm + NPARAM;
     m->m1 = m->grad + NPARAM;

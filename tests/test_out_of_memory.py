@@ -1,0 +1,58 @@
+"""A refused allocation is an error of its call and of no other: the next call
+on the same context finds a whole workspace, or makes one, and no stale error."""
+import numpy as np
+import pytest
+
+from paper_1912_08453_gb300 import ccpm
+from paper_1912_08453_gb300 import workloads as wl
+from tests.fake_cuda import fake, fake_library  # noqa: F401
+
+TL, TE = [5, 4, 8, 7, 4, 5], [(0, 1), (1, 2), (1, 3), (3, 4), (3, 5), (2, 3)]
+
+
+@pytest.fixture()
+def env(fake):  # noqa: F811
+    g = wl.rmat_graph(6, seed=3)
+    ctx = ccpm.Context(0)
+    yield fake, g, ctx, ccpm.Graph(ctx, g.row_ptr, g.col, g.labels), ccpm.Template(ctx, TL, TE)
+    ctx.close()
+
+
+def fails_then_works(f, call, attempts):
+    """Refuse the 1st, 2nd, ... allocation of call(k): it reports CCPM_ENOMEM, and
+    the same call then works and touches no missing buffer."""
+    refused = 0
+    for k in range(1, attempts + 1):
+        f.fake_fail_at(k)
+        try:
+            call(k)
+        except ccpm.CcpmError as e:
+            assert e.code == ccpm.CCPM_ENOMEM, (k, str(e))
+            refused += 1
+        else:
+            assert f.fake_allocs() < k, f"allocation {k} was refused, and the call went on"
+        f.fake_fail_at(0)
+        call(k)
+        assert f.fake_bad() == 0, f"after refusing allocation {k}"
+    assert 0 < refused < attempts            # every allocation was refused once
+
+
+def test_wide(env):
+    f, g, ctx, graph, t = env
+    fails_then_works(f, lambda k: ccpm.lcc_wide(ctx, graph, TL, TE), 4)
+
+
+def test_network(env):
+    f, g, ctx, graph, t = env
+    x, y = np.zeros((64, 16), np.float32), np.zeros(64, np.float32)
+
+    def call(k):
+        net = ccpm.Mlp(ctx, seed=1)
+        try:
+            net.train(x, y, steps=2, batch=64)
+            net.gradient(x, y)
+            net.forward(x)
+        finally:
+            net.close()
+
+    fails_then_works(f, call, 8)
