@@ -3772,6 +3772,7 @@ struct Control {
 };
 
 struct Workspace {
+    bool ready = false;              // everything below that ws_make allocates is there
     int64_t n = 0, m = 0, words = 0;
     int hub_deg = 0;
     uint32_t *om[2] = {nullptr, nullptr};
@@ -3965,10 +3966,8 @@ void ws_free(Workspace &w) {
     w = Workspace{};
 }
 
-int ws_ensure(ccpm_ctx *ctx, ccpm_graph *g, int hub_deg) {
+int ws_make(ccpm_ctx *ctx, ccpm_graph *g, int hub_deg) {
     Workspace &w = ctx->ws;
-    if (w.om[0] && w.hub_deg == hub_deg && w.n == g->n && w.m == g->m) return CCPM_OK;
-    ws_free(w);
     w.n = g->n;
     w.m = g->m;
     w.words = (g->m + 31) / 32;
@@ -4011,7 +4010,19 @@ int ws_ensure(ccpm_ctx *ctx, ccpm_graph *g, int hub_deg) {
     CU(ctx, cudaMallocHost((void **)&w.plans_h, kMaxPlans * sizeof(DevPlan)));
     CU(ctx, cudaMemsetAsync(w.acc, 0, sizeof(HubAcc) * (size_t)w.acc_cap, ctx->stream));
     for (auto &e : w.ev) CU(ctx, cudaEventCreate(&e));
+    w.ready = true;
     return CCPM_OK;
+}
+
+// The context's workspace for this graph: all of it, or, if something could not
+// be had, nothing.
+int ws_ensure(ccpm_ctx *ctx, ccpm_graph *g, int hub_deg) {
+    Workspace &w = ctx->ws;
+    if (w.ready && w.hub_deg == hub_deg && w.n == g->n && w.m == g->m) return CCPM_OK;
+    ws_free(w);
+    const int rc = ws_make(ctx, g, hub_deg);
+    if (rc) ws_free(w);
+    return rc;
 }
 
 // Label-grouped copy of the rows: a stable segmented sort of every row by the

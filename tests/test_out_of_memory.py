@@ -37,6 +37,27 @@ def fails_then_works(f, call, attempts):
     assert 0 < refused < attempts            # every allocation was refused once
 
 
+@pytest.mark.parametrize("kind", ["prune", "lcc_only", "matches", "explore", "batch"])
+def test_pruning(env, kind):
+    f, g, ctx, graph, t = env
+    kept = ccpm.prune(ctx, graph, t) if kind == "matches" else None
+
+    def call(k):
+        # another piece length each time: the workspace is made again
+        o = ccpm.options(hub_degree=16 + k, batch_workers=1, lcc_only=int(kind == "lcc_only"))
+        if kind == "matches":
+            kept.matches(t, vertex_counts=True, opts=o)
+        elif kind == "explore":
+            ccpm.explore(ctx, graph, t, 1, o)[1].close()
+        elif kind == "batch":
+            for r in ccpm.prune_batch(ctx, graph, [t], o):
+                r.close()
+        else:
+            ccpm.prune(ctx, graph, t, o).close()
+
+    fails_then_works(f, call, 60)
+
+
 def test_wide(env):
     f, g, ctx, graph, t = env
     fails_then_works(f, lambda k: ccpm.lcc_wide(ctx, graph, TL, TE), 4)
