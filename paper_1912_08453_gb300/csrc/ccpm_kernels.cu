@@ -4599,6 +4599,7 @@ struct Pipeline {
                 return set_err(ctx, CCPM_EOVERFLOW, "hub bookkeeping overflow");
             if (!initial && group == 0 && !w.st_h->changed) {
                 synced = was_synced;                      // the check changed nothing: no round ran
+                lcc_launches -= G;
                 break;
             }
             gate = nullptr;
