@@ -647,11 +647,15 @@ size_t fwd_smem() { return sizeof(FwdSmem); }
 size_t bwd_smem() { return sizeof(BwdSmem); }
 
 int configure_kernels() {
-    // batch workers reach this concurrently: configure once, under a lock
+    // once per device, as the setting belongs to the current device's copy of a
+    // kernel; under a lock, as batch workers reach this concurrently
+    constexpr int kDevices = 64;     // those past it are configured by every call
     static std::mutex mu;
-    static bool done = false;
+    static bool done[kDevices] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return CCPM_ECUDA;
     std::lock_guard<std::mutex> lock(mu);
-    if (done) return CCPM_OK;
+    if (dev < kDevices && done[dev]) return CCPM_OK;
     if (cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fwd_smem()) != cudaSuccess)
         return CCPM_ECUDA;
     if (cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwd_smem()) != cudaSuccess)
@@ -659,7 +663,7 @@ int configure_kernels() {
     if (cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem)) !=
         cudaSuccess)
         return CCPM_ECUDA;
-    done = true;
+    if (dev < kDevices) done[dev] = true;
     return CCPM_OK;
 }
 
