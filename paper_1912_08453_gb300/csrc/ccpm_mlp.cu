@@ -646,16 +646,45 @@ namespace {
 size_t fwd_smem() { return sizeof(FwdSmem); }
 size_t bwd_smem() { return sizeof(BwdSmem); }
 
-int configure_kernels() {
-    // once per device, as the setting belongs to the current device's copy of a
+// The fused loop's launch: one cluster.
+struct TrainLaunch {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute cluster = {};
+    explicit TrainLaunch(cudaStream_t s) {
+        cluster.id = cudaLaunchAttributeClusterDimension;
+        cluster.val.clusterDim.x = (unsigned)kTrainCluster;
+        cluster.val.clusterDim.y = cluster.val.clusterDim.z = 1;
+        cfg.gridDim = dim3((unsigned)kTrainCluster);
+        cfg.blockDim = dim3(TTHREADS);
+        cfg.dynamicSmemBytes = sizeof(TrainSmem);
+        cfg.stream = s;
+        cfg.attrs = &cluster;
+        cfg.numAttrs = 1;
+    }
+    TrainLaunch(const TrainLaunch &) = delete;
+    // Can the current device hold it?  Not where the process is given only some of
+    // the SMs and no eight of them share a cluster's reach.
+    bool fits() const {
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, k_mlp_train, &cfg) == cudaSuccess) return n > 0;
+        cudaGetLastError();
+        return false;
+    }
+};
+
+int configure_kernels(bool *fused = nullptr) {
+    // once per device, as settings belong to the current device's copy of a
     // kernel; under a lock, as batch workers reach this concurrently
     constexpr int kDevices = 64;     // those past it are configured by every call
     static std::mutex mu;
-    static bool done[kDevices] = {};
+    static bool done[kDevices] = {}, fits[kDevices] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return CCPM_ECUDA;
     std::lock_guard<std::mutex> lock(mu);
-    if (dev < kDevices && done[dev]) return CCPM_OK;
+    if (dev < kDevices && done[dev]) {
+        if (fused) *fused = fits[dev];
+        return CCPM_OK;
+    }
     if (cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fwd_smem()) != cudaSuccess)
         return CCPM_ECUDA;
     if (cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwd_smem()) != cudaSuccess)
@@ -663,7 +692,9 @@ int configure_kernels() {
     if (cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem)) !=
         cudaSuccess)
         return CCPM_ECUDA;
-    if (dev < kDevices) done[dev] = true;
+    const bool takes_cluster = TrainLaunch(nullptr).fits();
+    if (fused) *fused = takes_cluster;
+    if (dev < kDevices) { done[dev] = true; fits[dev] = takes_cluster; }
     return CCPM_OK;
 }
 
@@ -848,7 +879,8 @@ int ccpm_mlp_train(ccpm_mlp_t m, int N, const float *host_x, const float *host_t
                    uint64_t seed, float *final_loss) {
     if (!m || N <= 0 || !host_x || !host_t || steps < 0 || batch <= 0) return CCPM_EINVAL;
     if (cudaSetDevice(m->device) != cudaSuccess) return CCPM_ECUDA;
-    if (configure_kernels()) return CCPM_ECUDA;
+    bool fused = false;
+    if (configure_kernels(&fused)) return CCPM_ECUDA;
     Scratch sc;
     if (sc.alloc((size_t)N, (size_t)batch)) return CCPM_ENOMEM;
     cudaStream_t s = m->stream;
@@ -859,7 +891,8 @@ int ccpm_mlp_train(ccpm_mlp_t m, int N, const float *host_x, const float *host_t
     // launch: 8.2 us a step up to 512 rows, 12 at 1024, 35 at 4096, 45 at 8192 (a
     // block takes its rows 64 at a time).  The kernels per step, which spread
     // over the whole GPU, take 37 us up to 4096 rows and 40 at 8192.
-    const bool fused = batch <= kTrainMaxBatch;
+    const TrainLaunch launch(s);
+    fused = fused && batch <= kTrainMaxBatch;
     for (int it = 0; fused && it < steps && e == cudaSuccess;) {
         const int C = kTrainCluster;      // also where a block gets few rows: the Adam step is split, too
         TrainArgs a;
@@ -877,18 +910,7 @@ int ccpm_mlp_train(ccpm_mlp_t m, int N, const float *host_x, const float *host_t
         a.adam0 = m->adam_step;
         a.seed = seed;
         a.lr = lr;
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute at = {};
-        at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim.x = (unsigned)C;
-        at.val.clusterDim.y = at.val.clusterDim.z = 1;
-        cfg.gridDim = dim3((unsigned)C);
-        cfg.blockDim = dim3(TTHREADS);
-        cfg.dynamicSmemBytes = sizeof(TrainSmem);
-        cfg.stream = s;
-        cfg.attrs = &at;
-        cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, k_mlp_train, a);
+        e = cudaLaunchKernelEx(&launch.cfg, k_mlp_train, a);
         if (e == cudaSuccess) e = cudaGetLastError();
         it += a.steps;
         m->adam_step += a.steps;

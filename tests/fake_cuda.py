@@ -3,6 +3,7 @@ kernels do nothing, and allocations, devices and launches fail as a test says.
 For host code whose faults must not be run on a GPU."""
 import ctypes
 import os
+import shutil
 import subprocess
 
 import pytest
@@ -27,11 +28,13 @@ def fake_library(tmp_path_factory):
 
 
 @pytest.fixture()
-def fake(fake_library, monkeypatch):
-    """The fake's controls; ccpm calls the fake library meanwhile."""
-    monkeypatch.setattr(ccpm, "_LIB_PATH", fake_library)
+def fake(fake_library, tmp_path, monkeypatch):
+    """The fake's controls; ccpm calls the fake library meanwhile (a copy of its
+    own for each test: nothing it keeps per process is left from another)."""
+    path = shutil.copy(fake_library, tmp_path)
+    monkeypatch.setattr(ccpm, "_LIB_PATH", path)
     monkeypatch.setattr(ccpm, "lib", ccpm._load())
-    f = ctypes.CDLL(fake_library)
+    f = ctypes.CDLL(path)
     f.fake_limit.argtypes = [ctypes.c_size_t]
     f.fake_fail_at.argtypes = [ctypes.c_long]
     f.fake_calls.argtypes = [ctypes.c_char_p]

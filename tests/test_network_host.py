@@ -21,3 +21,15 @@ def test_every_device_runs_it(fake, batch):  # noqa: F811
         net.close()
         ctx.close()
     assert fake.fake_bad() == 0
+
+
+@pytest.mark.parametrize("batch,clusters,fused", [(64, 1, True), (4096, 1, True), (4097, 1, False), (64, 0, False)])
+def test_training_takes_the_kernels_per_step_without_a_cluster(fake, batch, clusters, fused):  # noqa: F811
+    fake.fake_clusters(clusters)
+    ctx = ccpm.Context(0)
+    net = ccpm.Mlp(ctx, seed=1)
+    net.train(X, Y, steps=3, batch=batch)
+    assert fake.fake_calls(b"k_mlp_train") == int(fused)
+    assert fake.fake_calls(b"k_mlp_backward") == fake.fake_calls(b"k_mlp_adam") == (0 if fused else 3)
+    net.close()
+    ctx.close()
