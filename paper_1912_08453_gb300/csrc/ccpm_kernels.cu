@@ -3830,6 +3830,7 @@ struct ccpm_ctx {
     std::string err;
     Workspace ws;                         // scratch of prunes issued on this context
     std::vector<ccpm_ctx *> workers;      // contexts of concurrent batch workers
+    unsigned long long *label_hist = nullptr;   // counters of a graph load (borrowed arrays)
     cudaEvent_t wait_ev = nullptr;        // batch workers: waits poll this event and yield
     // batch workers: grids are sized for sm_total / min(batch_share, workers
     // busy right now), so the last templates of a batch get the whole GPU back
@@ -4931,6 +4932,7 @@ void ccpm_ctx_destroy(ccpm_ctx_t c) {
     cudaSetDevice(c->device);
     for (ccpm_ctx *wk : c->workers) ccpm_ctx_destroy(wk);
     ws_free(c->ws);
+    cudaFree(c->label_hist);
     if (c->wait_ev) cudaEventDestroy(c->wait_ev);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
     delete c;
@@ -4979,20 +4981,25 @@ int ccpm_graph_load_csr(ccpm_ctx_t ctx, int64_t n, int64_t m, const int64_t *row
         g->rp = const_cast<int64_t *>(row_ptr);
         g->col = const_cast<int32_t *>(col);
         g->lab = const_cast<uint8_t *>(labels);
-        // label counts on the device; the arrays may still be in the making on
-        // the default stream, which the copy of the labels used to wait for
-        unsigned long long *d = nullptr, h[512];
-        cudaError_t e = cudaDeviceSynchronize();
-        if (e == cudaSuccess) e = cudaMalloc((void **)&d, sizeof(h));
-        if (e == cudaSuccess) e = cudaMemsetAsync(d, 0, sizeof(h), ctx->stream);
+        // label counts on the device.  The arrays may still be in the making on the
+        // default stream (or one that waits for it): a copy of one label waits for
+        // these, and for no other stream's work.  The counters stay with the
+        // context, since giving memory back waits for the whole device.
+        uint8_t one;
+        unsigned long long h[512];
+        cudaError_t e = cudaMemcpy(&one, labels, 1, cudaMemcpyDeviceToHost);
+        if (e == cudaSuccess && !ctx->label_hist) e = cudaMalloc((void **)&ctx->label_hist, sizeof(h));
+        if (e == cudaSuccess) e = cudaMemsetAsync(ctx->label_hist, 0, sizeof(h), ctx->stream);
         if (e == cudaSuccess) {
-            k_label_hist<<<grid_for(ctx, n, 256, 8), 256, 0, ctx->stream>>>(n, row_ptr, labels, d);
+            k_label_hist<<<grid_for(ctx, n, 256, 8), 256, 0, ctx->stream>>>(n, row_ptr, labels, ctx->label_hist);
             e = cudaGetLastError();
         }
-        if (e == cudaSuccess) e = cudaMemcpyAsync(h, d, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(h, ctx->label_hist, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-        cudaFree(d);
-        if (e != cudaSuccess) { delete g; return set_err(ctx, CCPM_ECUDA, "graph: label counts"); }
+        if (e != cudaSuccess) {
+            delete g;
+            return set_err(ctx, e == cudaErrorMemoryAllocation ? CCPM_ENOMEM : CCPM_ECUDA, "graph: label counts");
+        }
         for (int L = 0; L < 256; L++) {
             g->label_freq[L] = (int64_t)h[L];
             g->label_rows[L] = (int64_t)h[256 + L];
