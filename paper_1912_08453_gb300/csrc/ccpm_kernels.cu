@@ -3614,6 +3614,7 @@ k_nlcc_apply(const int32_t *__restrict__ roots, const PassCtl *last, int64_t ite
                 died_rows += (unsigned long long)len;
                 died++;
             }
+            if (!chg) continue;                      // no delta rounds follow
             chg[atomicAdd(&st->n_chg, 1u)] = Change{v, nw};
             if (len > hub_deg) {
                 const unsigned int np = (unsigned int)((len + hub_deg - 1) / hub_deg);
@@ -3773,6 +3774,7 @@ struct Control {
 
 struct Workspace {
     bool ready = false;              // everything below that ws_make allocates is there
+    bool lean = false;               // made without what a call can do without (ws_ensure)
     int64_t n = 0, m = 0, words = 0;
     int hub_deg = 0;
     uint32_t *om[2] = {nullptr, nullptr};
@@ -3796,7 +3798,8 @@ struct Workspace {
     RoundStats *st = nullptr, *st_h = nullptr;    // their search counters
     unsigned long long *cnt = nullptr, *cnt_h = nullptr;
     unsigned long long hist_h[kMaxT + 1] = {};    // the latest omega histogram
-    uint32_t *dirty = nullptr;       // delta rounds: one bit per listed vertex, all zero between rounds
+    // delta rounds (NULL where memory is short: no such rounds)
+    uint32_t *dirty = nullptr;       // one bit per listed vertex, all zero between rounds
     int32_t *dsmall = nullptr, *dmed = nullptr;   // their lists
     ChunkItem *dchunk = nullptr;
     Change *chg = nullptr;           // changes of omega not passed on yet
@@ -3967,8 +3970,9 @@ void ws_free(Workspace &w) {
     w = Workspace{};
 }
 
-int ws_make(ccpm_ctx *ctx, ccpm_graph *g, int hub_deg) {
+int ws_make(ccpm_ctx *ctx, ccpm_graph *g, int hub_deg, bool lean) {
     Workspace &w = ctx->ws;
+    w.lean = lean;
     w.n = g->n;
     w.m = g->m;
     w.words = (g->m + 31) / 32;
@@ -3989,10 +3993,10 @@ int ws_make(ccpm_ctx *ctx, ccpm_graph *g, int hub_deg) {
     if ((rc = dalloc(ctx, &w.acc, (size_t)w.acc_cap))) return rc;
     if ((rc = dalloc(ctx, &w.roots, (size_t)g->n))) return rc;
     if ((rc = dalloc(ctx, &w.sat, (size_t)g->n))) return rc;
-    w.items_cap = std::min<int64_t>(std::max<int64_t>(g->m, (int64_t)1 << 22), (int64_t)1 << 24);
+    w.items_cap = std::min<int64_t>(std::max<int64_t>(g->m, (int64_t)1 << 22), (int64_t)1 << 24) >> (lean ? 1 : 0);
     if ((rc = dalloc(ctx, &w.items, (size_t)w.items_cap))) return rc;
     if ((rc = dalloc(ctx, &w.items2, (size_t)kExpandBelow))) return rc;
-    w.spill_cap = std::max<int64_t>(w.items_cap / 4, (int64_t)1 << 20);
+    w.spill_cap = std::max<int64_t>(w.items_cap / 4, (int64_t)1 << (lean ? 19 : 20));
     if ((rc = dalloc(ctx, &w.spill_items, (size_t)w.spill_cap))) return rc;
     if ((rc = dalloc(ctx, &w.plans, (size_t)kMaxPlans))) return rc;
     if ((rc = dalloc(ctx, &w.ctl, 1))) return rc;
@@ -4001,12 +4005,14 @@ int ws_make(ccpm_ctx *ctx, ccpm_graph *g, int hub_deg) {
     w.st_h = &w.ctl_h->st;
     w.cnt = w.ctl->cnt;
     w.cnt_h = w.ctl_h->cnt;
-    if ((rc = dalloc(ctx, &w.dirty, (size_t)g->n / 32 + 1))) return rc;
-    if ((rc = dalloc(ctx, &w.dsmall, (size_t)g->n))) return rc;
-    if ((rc = dalloc(ctx, &w.dmed, (size_t)g->n))) return rc;
-    if ((rc = dalloc(ctx, &w.dchunk, (size_t)w.chunk_cap))) return rc;
-    if ((rc = dalloc(ctx, &w.chg, (size_t)g->n))) return rc;
-    if ((rc = dalloc(ctx, &w.chg_piece, (size_t)w.chunk_cap))) return rc;
+    if (!lean) {
+        if ((rc = dalloc(ctx, &w.dirty, (size_t)g->n / 32 + 1))) return rc;
+        if ((rc = dalloc(ctx, &w.dsmall, (size_t)g->n))) return rc;
+        if ((rc = dalloc(ctx, &w.dmed, (size_t)g->n))) return rc;
+        if ((rc = dalloc(ctx, &w.dchunk, (size_t)w.chunk_cap))) return rc;
+        if ((rc = dalloc(ctx, &w.chg, (size_t)g->n))) return rc;
+        if ((rc = dalloc(ctx, &w.chg_piece, (size_t)w.chunk_cap))) return rc;
+    }
     if ((rc = dalloc(ctx, &w.deg, (size_t)g->n))) return rc;
     CU(ctx, cudaMallocHost((void **)&w.plans_h, kMaxPlans * sizeof(DevPlan)));
     CU(ctx, cudaMemsetAsync(w.acc, 0, sizeof(HubAcc) * (size_t)w.acc_cap, ctx->stream));
@@ -4016,14 +4022,24 @@ int ws_make(ccpm_ctx *ctx, ccpm_graph *g, int hub_deg) {
 }
 
 // The context's workspace for this graph: all of it, or, if something could not
-// be had, nothing.
-int ws_ensure(ccpm_ctx *ctx, ccpm_graph *g, int hub_deg) {
+// be had, nothing.  What a call can do without is left out where memory is short
+// (lean): half of the item lists (searches with more items run one warp per root),
+// and the lists of delta rounds (every round is a full one).  That is 16 B a
+// vertex and up to 0.7 GB less.
+int ws_ensure(ccpm_ctx *ctx, ccpm_graph *g, int hub_deg, bool lean = false) {
     Workspace &w = ctx->ws;
-    if (w.ready && w.hub_deg == hub_deg && w.n == g->n && w.m == g->m) return CCPM_OK;
+    if (w.ready && (w.lean || !lean) && w.hub_deg == hub_deg && w.n == g->n && w.m == g->m) return CCPM_OK;
     ws_free(w);
-    const int rc = ws_make(ctx, g, hub_deg);
+    int rc = ws_make(ctx, g, hub_deg, lean);
     if (rc) ws_free(w);
+    if (rc == CCPM_ENOMEM && !lean) return ws_ensure(ctx, g, hub_deg, true);
     return rc;
+}
+
+// Something beside the workspace did not fit: true if a smaller workspace has
+// taken its place, so that the caller can try again.
+bool ws_shrink(ccpm_ctx *ctx, ccpm_graph *g) {
+    return ctx->ws.ready && !ctx->ws.lean && ws_ensure(ctx, g, ctx->ws.hub_deg, true) == CCPM_OK;
 }
 
 // Label-grouped copy of the rows: a stable segmented sort of every row by the
@@ -4709,7 +4725,9 @@ struct Pipeline {
     // than a few million entries to look over: exploring a clique on 8192
     // vertices took 154 ms with full rounds and 177 with delta rounds, the LCC
     // phase of 32M vertices with 350M entries in the live rows 22.7 and 11.7.
-    bool use_deltas(int64_t rows_now) const { return compact_mode <= 0 && rows_now >= ((int64_t)1 << 22); }
+    bool use_deltas(int64_t rows_now) const {
+        return compact_mode <= 0 && rows_now >= ((int64_t)1 << 22) && !ctx->ws.lean;
+    }
 
     // Frontier of the live vertices over rows rp (the pieces of a long row
     // consecutive and in order); also makes both omega buffers equal.
@@ -5148,7 +5166,7 @@ int ccpm_tmpl_set_order(ccpm_tmpl_t t, int n, const int32_t *order) {
     return CCPM_OK;
 }
 
-int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_options *opt_in, ccpm_result_t *out) {
+static int prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_options *opt_in, ccpm_result_t *out) {
     if (!ctx || !g || !tm || !out) return CCPM_EINVAL;
     if (g->ctx->device != ctx->device) return set_err(ctx, CCPM_EINVAL, "graph lives on another device");
     ccpm_options opt;
@@ -5228,7 +5246,7 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
         if (rc_) return fail(rc_);    \
     } while (0)
 
-    CUF(cudaMemsetAsync(w.dirty, 0, sizeof(uint32_t) * (size_t)(g->n / 32 + 1), s));
+    if (!w.lean) CUF(cudaMemsetAsync(w.dirty, 0, sizeof(uint32_t) * (size_t)(g->n / 32 + 1), s));
     CUF(cudaEventRecord(w.ev[0], s));
     // ---- init (Alg. 3)
     LabelMask lm;
@@ -5699,6 +5717,15 @@ int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_option
 #undef RCF
 }
 
+int ccpm_prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_options *opt_in, ccpm_result_t *out) {
+    const int rc = prune(ctx, g, tm, opt_in, out);
+    // every allocation comes before the result is written: a saved state is still
+    // there to resume from
+    if (rc != CCPM_ENOMEM || !ws_shrink(ctx, g)) return rc;
+    g->prunes--;                                     // one prune
+    return prune(ctx, g, tm, opt_in, out);
+}
+
 // Run the templates tmpls[order[0..)] of a batch on `W` worker contexts, one
 // host thread each, taking templates from a shared counter in that order.
 // Returns the first error.
@@ -5892,6 +5919,18 @@ __global__ void k_or_words(uint32_t *dst, const uint32_t *src, int64_t n) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) dst[i] |= src[i];
 }
 
+// Arrays of a state, between two prunes (the workspace is idle).
+int state_arrays(ccpm_ctx *ctx, ccpm_graph *g, int64_t words, uint32_t **om, uint32_t **eb) {
+    for (;;) {
+        int rc = dalloc(ctx, om, (size_t)g->n);
+        if (!rc && (rc = dalloc(ctx, eb, (size_t)words + 1))) {
+            cudaFree(*om);
+            *om = nullptr;
+        }
+        if (rc != CCPM_ENOMEM || !ws_shrink(ctx, g)) return rc;
+    }
+}
+
 // A result on graph g for template t holding (om, eb) copied from `src`
 // arrays (the candidate set), ready for a resumed prune.
 int result_from(ccpm_ctx *ctx, ccpm_graph *g, const Template &t, const uint32_t *om, const uint32_t *eb,
@@ -5899,9 +5938,8 @@ int result_from(ccpm_ctx *ctx, ccpm_graph *g, const Template &t, const uint32_t 
     ccpm_result *r = new (std::nothrow) ccpm_result();
     if (!r) return set_err(ctx, CCPM_ENOMEM, "result: host allocation");
     r->g = g;
-    int rc;
-    if ((rc = dalloc(ctx, &r->om, (size_t)g->n)) || (rc = dalloc(ctx, &r->eb, (size_t)words + 1))) {
-        cudaFree(r->om); cudaFree(r->eb);
+    const int rc = state_arrays(ctx, g, words, &r->om, &r->eb);
+    if (rc) {
         delete r;
         return rc;
     }
@@ -5967,10 +6005,7 @@ int ccpm_explore(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t base, int max_remov
     // match of every variant
     uint32_t *c_om = nullptr, *c_eb = nullptr;
     int rc;
-    if ((rc = dalloc(ctx, &c_om, (size_t)g->n)) || (rc = dalloc(ctx, &c_eb, (size_t)words + 1))) {
-        cudaFree(c_om); cudaFree(c_eb);
-        return rc;
-    }
+    if ((rc = state_arrays(ctx, g, words, &c_om, &c_eb))) return rc;
     auto cleanup = [&]() { cudaFree(c_om); cudaFree(c_eb); };
     auto fail_c = [&](int code) { cleanup(); return code; };
     if (cudaMemsetAsync(c_om, 0, sizeof(uint32_t) * (size_t)g->n, s) != cudaSuccess ||
@@ -6108,7 +6143,7 @@ int ccpm_result_phase_rounds(ccpm_result_t r, int32_t *dst, int cap) {
     return CCPM_OK;
 }
 
-int ccpm_result_matches(ccpm_ctx_t ctx, ccpm_result_t r, ccpm_tmpl_t tm, const ccpm_options *opt_in,
+static int list_matches(ccpm_ctx_t ctx, ccpm_result_t r, ccpm_tmpl_t tm, const ccpm_options *opt_in,
                         int32_t *list, uint64_t list_cap, uint64_t *vertex_counts, uint64_t *entry_counts,
                         int dst_on_device, uint64_t *n_matches) {
     if (!ctx || !r || !tm || !n_matches || (list_cap > 0 && !list)) return CCPM_EINVAL;
@@ -6261,6 +6296,14 @@ int ccpm_result_matches(ccpm_ctx_t ctx, ccpm_result_t r, ccpm_tmpl_t tm, const c
 
 const uint32_t *ccpm_result_omega_device(ccpm_result_t r) { return r ? r->om : nullptr; }
 const uint32_t *ccpm_result_edge_bitmap_device(ccpm_result_t r) { return r ? r->eb : nullptr; }
+
+int ccpm_result_matches(ccpm_ctx_t ctx, ccpm_result_t r, ccpm_tmpl_t tm, const ccpm_options *opt_in,
+                        int32_t *list, uint64_t list_cap, uint64_t *vertex_counts, uint64_t *entry_counts,
+                        int dst_on_device, uint64_t *n_matches) {
+    const int rc = list_matches(ctx, r, tm, opt_in, list, list_cap, vertex_counts, entry_counts, dst_on_device, n_matches);
+    if (rc != CCPM_ENOMEM || !ws_shrink(ctx, r->g)) return rc;
+    return list_matches(ctx, r, tm, opt_in, list, list_cap, vertex_counts, entry_counts, dst_on_device, n_matches);
+}
 
 int ccpm_graph_batch_workers(ccpm_graph_t g) { return g ? g->tuned_workers : 0; }
 

@@ -21,7 +21,7 @@ std::map<std::string, void *> symbols;
 std::map<std::pair<int, const void *>, int> dyn_smem;     // (device, kernel) -> bytes allowed
 std::map<std::string, long> calls;            // runtime calls and kernels launched, by name
 long n_alloc = 0, fail_at = 0, bad = 0;
-size_t in_use = 0, limit = ~(size_t)0;
+size_t in_use = 0, peak = 0, limit = ~(size_t)0;
 bool clusters = true;
 thread_local int device = 0;
 thread_local cudaError_t last = cudaSuccess;
@@ -41,11 +41,12 @@ cudaError_t note(const char *name, cudaError_t e = cudaSuccess) {
 cudaError_t alloc(void **p, size_t n, bool counts) {
     Lock l(mu);
     *p = nullptr;
-    if (++n_alloc == fail_at || (counts && in_use + n > limit)) return ret(cudaErrorMemoryAllocation);
+    if ((++n_alloc >= fail_at && fail_at) || (counts && in_use + n > limit)) return ret(cudaErrorMemoryAllocation);
     char *q = (char *)std::calloc(n ? n : 1, 1);
     if (!q) return ret(cudaErrorMemoryAllocation);
     blocks[q] = n;
     if (counts) in_use += n;
+    if (in_use > peak) peak = in_use;
     *p = q;
     return cudaSuccess;
 }
@@ -95,12 +96,15 @@ void fake_reset() {
     last = cudaSuccess;
     calls.clear();
 }
+// the k-th allocation from now and all later ones are refused (0: none)
 void fake_fail_at(long k) { Lock l(mu); n_alloc = 0; fail_at = k; }
-void fake_limit(size_t bytes) { Lock l(mu); limit = in_use + bytes; }     // from now on
+// `bytes` more than now; fake_peak: the most from there on
+void fake_limit(size_t bytes) { Lock l(mu); limit = in_use + bytes; peak = in_use; }
 void fake_clusters(int allowed) { clusters = allowed != 0; }
 long fake_allocs() { Lock l(mu); return n_alloc; }
 long fake_bad() { Lock l(mu); return bad; }
 size_t fake_in_use() { Lock l(mu); return in_use; }
+size_t fake_peak() { Lock l(mu); return peak; }
 // calls of a runtime function or launches of kernels whose name contains `what`
 long fake_calls(const char *what) {
     Lock l(mu);

@@ -40,7 +40,7 @@ def fake(fake_library, tmp_path, monkeypatch):
     f.fake_calls.argtypes = [ctypes.c_char_p]
     for name in ("fake_allocs", "fake_bad", "fake_calls"):
         getattr(f, name).restype = ctypes.c_long
-    f.fake_in_use.restype = ctypes.c_size_t
+    f.fake_in_use.restype = f.fake_peak.restype = ctypes.c_size_t
     f.fake_reset()
     yield f
     f.fake_reset()

@@ -19,8 +19,8 @@ def env(fake):  # noqa: F811
 
 
 def fails_then_works(f, call, attempts):
-    """Refuse the 1st, 2nd, ... allocation of call(k): it reports CCPM_ENOMEM, and
-    the same call then works and touches no missing buffer."""
+    """Refuse the 1st, 2nd, ... allocation of call(k), and those after it: it reports
+    CCPM_ENOMEM, and the same call then works and touches no missing buffer."""
     refused = 0
     for k in range(1, attempts + 1):
         f.fake_fail_at(k)
@@ -77,3 +77,43 @@ def test_network(env):
             net.close()
 
     fails_then_works(f, call, 8)
+
+
+@pytest.mark.parametrize("kind", ["prune", "lcc_only", "resume", "matches", "explore"])
+def test_pruning_takes_less_where_memory_is_short(env, kind, monkeypatch):
+    """Half of the item lists (64 B each, 2^22 and 2^20 of them for a small graph)
+    and the lists of delta rounds (16 B a vertex) are wanted, not needed."""
+    f, g, ctx, graph, t = env
+    o = ccpm.options(lcc_only=int(kind == "lcc_only"))
+    state = ccpm.prune(ctx, graph, t, o).export_state()
+    o.resume = int(kind == "resume")
+
+    def need(limit):
+        """The call's peak, on a context of its own and with this much memory."""
+        c = ccpm.Context(0)
+        r = ccpm.state_import(c, graph, t, state) if kind in ("resume", "matches") else None
+        before = f.fake_in_use()
+        f.fake_limit(limit)
+        try:
+            if kind == "matches":
+                monkeypatch.setattr(graph, "ctx", c)      # the context the call runs on
+                r.matches(t, vertex_counts=True, entry_counts=True)
+            elif kind == "explore":
+                r = ccpm.explore(c, graph, t, 1, o)[1]
+            else:
+                r = ccpm.prune(c, graph, t, o, result=r)
+            return f.fake_peak() - before
+        finally:
+            f.fake_limit(1 << 60)
+            if r is not None:
+                r.close()
+            c.close()
+            assert f.fake_bad() == 0
+
+    wanted = need(1 << 60)
+    least = wanted - 32 * (2**22 + 2**20) - 16 * g.n
+    for limit in (wanted, wanted - 1, wanted - 4 * g.n, wanted - 2**20, least):
+        assert need(limit) <= limit
+    with pytest.raises(ccpm.CcpmError) as e:
+        need(least // 2)
+    assert e.value.code == ccpm.CCPM_ENOMEM
