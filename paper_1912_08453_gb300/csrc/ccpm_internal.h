@@ -116,3 +116,7 @@ void build_plan(const Template &t, uint32_t svert, const uint32_t *sadj, int roo
                 const unsigned long long *qlive = nullptr);
 
 }  // namespace ccpm
+
+// For tests: the sizes from which a context's prunes take other round kernels
+// (results are the same), so that small graphs reach all of them.
+extern "C" void ccpm_test_round_limits(ccpm_ctx_t ctx, int64_t huge_rows, int64_t inline_rows, int64_t delta_rows);

@@ -1144,6 +1144,9 @@ constexpr int64_t kHugeRows = (int64_t)1 << 28;
 // kernel over a list of them (64K vertices: 31 against 41 us; 3M: 216 against
 // 197).
 constexpr int64_t kInlineRows = (int64_t)1 << 22;
+// Entries in the live rows from which later rounds evaluate changes only
+// (Pipeline::use_deltas).
+constexpr int64_t kDeltaRows = (int64_t)1 << 22;
 
 struct RowArgs {
     int64_t n, m;                 // m: columns that may be read four at a time
@@ -3833,6 +3836,8 @@ struct ccpm_ctx {
     std::string err;
     Workspace ws;                         // scratch of prunes issued on this context
     std::vector<ccpm_ctx *> workers;      // contexts of concurrent batch workers
+    // row entries from which the LCC rounds go another way; tests lower them
+    int64_t huge_rows = kHugeRows, inline_rows = kInlineRows, delta_rows = kDeltaRows;
     unsigned long long *label_hist = nullptr;   // counters of a graph load (borrowed arrays)
     cudaEvent_t wait_ev = nullptr;        // batch workers: waits poll this event and yield
     // batch workers: grids are sized for sm_total / min(batch_share, workers
@@ -4344,7 +4349,7 @@ struct Pipeline {
     int launch_round(RoundStats *slot, const RoundStats *prev, const RoundStats *gate, int c, int l, bool delta) {
         launches++;
         lcc_launches++;
-        if (maxc > 4 || first_rows < kHugeRows) return launch_small(slot, prev, gate, c, l, delta);
+        if (maxc > 4 || first_rows < ctx->huge_rows) return launch_small(slot, prev, gate, c, l, delta);
         Workspace &w = ctx->ws;
         RowArgs a = row_args(slot);
         a.om = w.om[c];
@@ -4475,7 +4480,7 @@ struct Pipeline {
         Workspace &w = ctx->ws;
         RowArgs a = row_args(slot);
         a.guard = 1;
-        a.inline_long = first_rows < kInlineRows ? 1 : 0;
+        a.inline_long = first_rows < ctx->inline_rows ? 1 : 0;
         for (int i = 0; i < 2; i++) {
             a.om_out[i] = w.om[i];
             a.nw_out[i] = w.nw[i];
@@ -4726,7 +4731,7 @@ struct Pipeline {
     // vertices took 154 ms with full rounds and 177 with delta rounds, the LCC
     // phase of 32M vertices with 350M entries in the live rows 22.7 and 11.7.
     bool use_deltas(int64_t rows_now) const {
-        return compact_mode <= 0 && rows_now >= ((int64_t)1 << 22) && !ctx->ws.lean;
+        return compact_mode <= 0 && rows_now >= ctx->delta_rows && !ctx->ws.lean;
     }
 
     // Frontier of the live vertices over rows rp (the pieces of a long row
@@ -4943,6 +4948,12 @@ int ccpm_ctx_create(int device, void *stream, ccpm_ctx_t *out) {
     }
     *out = c;
     return CCPM_OK;
+}
+
+void ccpm_test_round_limits(ccpm_ctx_t c, int64_t huge_rows, int64_t inline_rows, int64_t delta_rows) {
+    c->huge_rows = huge_rows;
+    c->inline_rows = inline_rows;
+    c->delta_rows = delta_rows;
 }
 
 void ccpm_ctx_destroy(ccpm_ctx_t c) {
