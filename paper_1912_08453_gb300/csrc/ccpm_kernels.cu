@@ -1103,9 +1103,9 @@ k_lcc_round(LccArgs a, DevTmpl t) {
 }
 
 // -------------------------------------------------------------------------
-// The first round, and the later ones where the rows are huge (kHugeRows), for
-// templates of at most four multiplicity classes; k_lcc_round above serves the
-// others.
+// The first round of templates with at most four multiplicity classes, and their
+// later ones where the rows are huge and omega fits a byte (kHugeRows);
+// k_lcc_round above serves the others.
 //
 // A lane takes four consecutive entries per step: their edge bits are a nibble
 // of a bitmap word, their columns one 16-byte load, and the four gathers that
@@ -1130,15 +1130,26 @@ k_lcc_round(LccArgs a, DevTmpl t) {
 
 // Where a neighbour's omega comes from: its label in entry order (first round,
 // graphs that have the entry labels), its label (first round), its 1-byte
-// omega, or its 2- or 4-byte omega.
+// omega, or omega itself (allocation-free LCC, which keeps no narrow copy).
 constexpr int kByEntry = 0, kByLabel = 1, kByByte = 2, kByWord = 3;
 constexpr int kFirst = 3;                    // a round's MODE, beside kFull and kDelta
 
 // Entries in the initially active rows from which k_rows takes the rounds after
-// the first: the second and third round of 32M vertices (6*10^8 such entries)
-// take 3.4 ms with it and 4.4 with k_lcc_round, those of 4M vertices (9*10^7)
-// 0.26 and 0.22, of 3M (4*10^7) 0.18 and 0.16; on 64K vertices a round takes
-// 7.6 and 6.3 us (one chain of latencies, which k_lcc_round keeps shorter).
+// the first, where omega fits a byte (templates of up to 8 vertices).  ms of
+// these rounds with k_rows and with k_lcc_round, Zipf labels, 30 entries a vertex:
+//   vertices               8M (142M entries)   32M (570M entries)
+//   8, two classes         1.09   1.41         4.12   5.13
+//   8, three classes       0.81   1.05         2.83   3.85
+//   7, three classes       0.92   1.00         3.22   3.52
+//   5, no class            0.66   0.68         2.54   2.44
+//   9, two classes         1.36   1.27         5.62   5.00
+//   12, three classes      1.57   1.50         6.77   5.71
+// 13 templates of up to 8 vertices at 32M: 0.92 to 1.36 times as fast, 1.12 on
+// average.  A wider omega leaves k_rows without its table by bytes: slower at
+// every size.  The line itself is not sharp: at 36M entries (2M vertices) 0.45 against 0.52
+// with two classes and 0.21 against 0.17 without (8M entries); degree labels, 3M
+// vertices (40M entries), 0.18 against 0.16; on 64K vertices a round takes 7.6
+// against 6.3 us (one chain of latencies, which k_lcc_round keeps shorter).
 constexpr int64_t kHugeRows = (int64_t)1 << 28;
 // ... below which k_first_round walks the longer rows too, with no second
 // kernel over a list of them (64K vertices: 31 against 41 us; 3M: 216 against
@@ -1226,7 +1237,7 @@ __device__ __forceinline__ Quad<F> quad_gather(const RowArgs &a, uint32_t nib, c
         if ((nib >> j) & 1u) {
             if (F == kByLabel) x[j] = __ldg(a.lab + u[j]);
             else if (F == kByByte) x[j] = __ldg((const uint8_t *)a.nw + u[j]);
-            else x[j] = gather_om(a.om, a.nw, a.nw_bytes, u[j]);
+            else x[j] = __ldg(a.om + u[j]);
         }
     }
     if constexpr (F == kByWord) {
@@ -4349,7 +4360,8 @@ struct Pipeline {
     int launch_round(RoundStats *slot, const RoundStats *prev, const RoundStats *gate, int c, int l, bool delta) {
         launches++;
         lcc_launches++;
-        if (maxc > 4 || first_rows < ctx->huge_rows) return launch_small(slot, prev, gate, c, l, delta);
+        if (maxc > 4 || nw_bytes != 1 || first_rows < ctx->huge_rows)
+            return launch_small(slot, prev, gate, c, l, delta);
         Workspace &w = ctx->ws;
         RowArgs a = row_args(slot);
         a.om = w.om[c];
@@ -4372,16 +4384,11 @@ struct Pipeline {
         // a queued round does not know its sizes: one full resident wave
         const int64_t warps = a.sizes ? (int64_t)1 << 40 : n_small + n_med + n_chunk;
         from_labels = dense = false;
-        const bool byte = nw_bytes == 1;
-#define CCPM_ROWS(C, M, F) k_rows<C, M, F><<<lcc_grid(ctx, k_rows<C, M, F>, warps), 256, 0, ctx->stream>>>(a, dt)
-#define CCPM_ROWS_BY(M)                                                          \
-    do {                                                                         \
-        if (maxc == 0) { if (byte) CCPM_ROWS(0, M, kByByte); else CCPM_ROWS(0, M, kByWord); } \
-        else { if (byte) CCPM_ROWS(4, M, kByByte); else CCPM_ROWS(4, M, kByWord); }           \
-    } while (0)
-        if (delta) CCPM_ROWS_BY(kDelta);
-        else CCPM_ROWS_BY(kFull);
-#undef CCPM_ROWS_BY
+#define CCPM_ROWS(C, M) \
+    k_rows<C, M, kByByte><<<lcc_grid(ctx, k_rows<C, M, kByByte>, warps), 256, 0, ctx->stream>>>(a, dt)
+        if (maxc == 0) { if (delta) CCPM_ROWS(0, kDelta); else CCPM_ROWS(0, kFull); }
+        else { if (delta) CCPM_ROWS(4, kDelta); else CCPM_ROWS(4, kFull); }
+#undef CCPM_ROWS
         CU(ctx, cudaGetLastError());
         return CCPM_OK;
     }
@@ -4411,8 +4418,8 @@ struct Pipeline {
         return a;
     }
 
-    // A round of a template with more than four multiplicity classes, or of one
-    // that starts from fewer than kHugeRows entries.
+    // A round of a template with more than eight vertices or four multiplicity
+    // classes, or of one that starts from fewer than kHugeRows entries.
     int launch_small(RoundStats *slot, const RoundStats *prev, const RoundStats *gate, int c, int l, bool delta) {
         Workspace &w = ctx->ws;
         LccArgs a;

@@ -169,7 +169,11 @@ cudaError_t cudaGetDevice(int *d) { *d = device; return cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr, int) { *v = 8; return cudaSuccess; }
 cudaError_t cudaDeviceSynchronize() { return note("cudaDeviceSynchronize"); }
 cudaError_t cudaGetLastError() { const cudaError_t e = last; last = cudaSuccess; return e; }
-const char *cudaGetErrorString(cudaError_t e) { return e == cudaSuccess ? "no error" : "fake error"; }
+const char *cudaGetErrorString(cudaError_t e) {
+    thread_local std::string s;
+    s = "fake error " + std::to_string((int)e);
+    return s.c_str();
+}
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { *s = (cudaStream_t)1; return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return note("cudaStreamSynchronize"); }

@@ -30,7 +30,8 @@ def fake_library(tmp_path_factory):
 @pytest.fixture()
 def fake(fake_library, tmp_path, monkeypatch):
     """The fake's controls; ccpm calls the fake library meanwhile (a copy of its
-    own for each test: nothing it keeps per process is left from another)."""
+    own for each test: nothing it keeps per process is left from another).  A test
+    closes what it made, so that no handle of the fake reaches the real library."""
     path = shutil.copy(fake_library, tmp_path)
     monkeypatch.setattr(ccpm, "_LIB_PATH", path)
     monkeypatch.setattr(ccpm, "lib", ccpm._load())

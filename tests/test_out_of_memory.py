@@ -14,8 +14,10 @@ TL, TE = [5, 4, 8, 7, 4, 5], [(0, 1), (1, 2), (1, 3), (3, 4), (3, 5), (2, 3)]
 def env(fake):  # noqa: F811
     g = wl.rmat_graph(6, seed=3)
     ctx = ccpm.Context(0)
-    yield fake, g, ctx, ccpm.Graph(ctx, g.row_ptr, g.col, g.labels), ccpm.Template(ctx, TL, TE)
-    ctx.close()
+    graph, t = ccpm.Graph(ctx, g.row_ptr, g.col, g.labels), ccpm.Template(ctx, TL, TE)
+    yield fake, g, ctx, graph, t
+    for x in (t, graph, ctx):            # before the library is the real one again
+        x.close()
 
 
 def fails_then_works(f, call, attempts):
@@ -40,7 +42,7 @@ def fails_then_works(f, call, attempts):
 @pytest.mark.parametrize("kind", ["prune", "lcc_only", "matches", "explore", "batch"])
 def test_pruning(env, kind):
     f, g, ctx, graph, t = env
-    kept = ccpm.prune(ctx, graph, t) if kind == "matches" else None
+    kept = ccpm.prune(ctx, graph, t)
 
     def call(k):
         # another piece length each time: the workspace is made again
@@ -56,6 +58,7 @@ def test_pruning(env, kind):
             ccpm.prune(ctx, graph, t, o).close()
 
     fails_then_works(f, call, 60)
+    kept.close()
 
 
 def test_wide(env):
@@ -85,7 +88,9 @@ def test_pruning_takes_less_where_memory_is_short(env, kind, monkeypatch):
     and the lists of delta rounds (16 B a vertex) are wanted, not needed."""
     f, g, ctx, graph, t = env
     o = ccpm.options(lcc_only=int(kind == "lcc_only"))
-    state = ccpm.prune(ctx, graph, t, o).export_state()
+    first = ccpm.prune(ctx, graph, t, o)
+    state = first.export_state()
+    first.close()
     o.resume = int(kind == "resume")
 
     def need(limit):
