@@ -6024,8 +6024,9 @@ int ccpm_explore(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t base, int max_remov
     uint32_t *c_om = nullptr, *c_eb = nullptr;
     int rc;
     if ((rc = state_arrays(ctx, g, words, &c_om, &c_eb))) return rc;
+    ccpm_result *made = nullptr;         // the union, if this call made it
     auto cleanup = [&]() { cudaFree(c_om); cudaFree(c_eb); };
-    auto fail_c = [&](int code) { cleanup(); return code; };
+    auto fail_c = [&](int code) { cleanup(); ccpm_result_destroy(made); return code; };
     if (cudaMemsetAsync(c_om, 0, sizeof(uint32_t) * (size_t)g->n, s) != cudaSuccess ||
         cudaMemsetAsync(c_eb, 0, sizeof(uint32_t) * (size_t)(words + 1), s) != cudaSuccess)
         return fail_c(set_err(ctx, CCPM_ECUDA, "explore: memset"));
@@ -6057,7 +6058,8 @@ int ccpm_explore(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t base, int max_remov
     ccpm_result *u = *out;
     if (u && u->g != g) return fail_c(set_err(ctx, CCPM_EINVAL, "explore: result was made for another graph"));
     if (!u) {
-        if ((rc = result_from(ctx, g, B, c_om, c_eb, words, &u))) return fail_c(rc);
+        if ((rc = result_from(ctx, g, B, c_om, c_eb, words, &made))) return fail_c(rc);
+        u = made;
     }
     u->tmpl_fp = tmpl_fingerprint(B);
     u->phase_rounds.clear();

@@ -44,4 +44,4 @@ def fake(fake_library, tmp_path, monkeypatch):
     f.fake_in_use.restype = f.fake_peak.restype = ctypes.c_size_t
     f.fake_reset()
     yield f
-    f.fake_reset()
+    assert f.fake_in_use() == 0, "device memory left behind"
