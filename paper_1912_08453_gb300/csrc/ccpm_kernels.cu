@@ -4321,7 +4321,6 @@ struct Pipeline {
     int64_t rows = 0, alive = 0, launches = 0, lcc_launches = 0;
     int64_t alg_bytes = 0, kernel_bytes = 0, first_entries = 0, lcc_rounds_run = 0;
     double ms_first = 0.0;
-    int rc_compact = 0;
     double ms_lcc_kernel = 0.0;
     double ms_search_kernel = 0.0;
     int64_t search_launches = 0, nlcc_entries = 0;
@@ -4685,7 +4684,7 @@ struct Pipeline {
                 return set_err(ctx, CCPM_ETIMEOUT, "LCC did not converge");
             src = ring + G - 1;
             if (compact_mode > 0 && want_compact()) {
-                if ((rc_compact = compact())) return rc_compact;
+                if ((rc = compact())) return rc;
                 src = nullptr;            // rebuilt lists: their sizes are the host's
             }
         }
@@ -5503,16 +5502,13 @@ static int prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_opti
         a.items_cap = w.items_cap;
         // the final enumeration keeps the background label frequencies (measured
         // faster than ordering by live candidates there)
-        const unsigned long long *live = nullptr;
         int root = 0;
-        for (int q = 1; q < t.n0; q++) {
-            const bool fewer = live ? live[q] < live[root] : g->label_freq[t.labels[q]] < g->label_freq[t.labels[root]];
-            if (fewer) root = q;
-        }
+        for (int q = 1; q < t.n0; q++)
+            if (g->label_freq[t.labels[q]] < g->label_freq[t.labels[root]]) root = q;
         // one pass over every match from roots of `root`: count (mode kCount) or
         // count and mark (kMark); returns overflow of the cap
         auto count_pass = [&](int mode, const uint32_t *om_src, uint64_t cap, uint64_t &found, bool &capped) -> int {
-            build_plan(t, all, t.adj, root, g->label_freq, true, w.plans_h[0], -1, live);
+            build_plan(t, all, t.adj, root, g->label_freq, true, w.plans_h[0]);
             CU(ctx, cudaMemcpyAsync(w.plans, w.plans_h, sizeof(DevPlan), cudaMemcpyHostToDevice, s));
             int rc2 = clear_search(ctx, w);
             if (rc2) return rc2;
@@ -5578,7 +5574,7 @@ static int prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_opti
             // (A) every (v, q): some match has phi(q) = v?  Found embeddings also
             // satisfy the other (vertex, template vertex) pairs they place and mark
             // their edges.
-            for (int q = 0; q < t.n0; q++) build_plan(t, all, t.adj, q, g->label_freq, true, w.plans_h[q], -1, live);
+            for (int q = 0; q < t.n0; q++) build_plan(t, all, t.adj, q, g->label_freq, true, w.plans_h[q]);
             CUF(cudaMemcpyAsync(w.plans, w.plans_h, sizeof(DevPlan) * (size_t)t.n0, cudaMemcpyHostToDevice, s));
             RCF(clear_search(ctx, w));
             P.launches++;
@@ -5613,7 +5609,7 @@ static int prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_opti
                 for (int o = 0; o < tab.n; o++) {
                     tab.a[o] = (int8_t)oriented[o0 + (size_t)o].first;
                     tab.b[o] = (int8_t)oriented[o0 + (size_t)o].second;
-                    build_plan(t, all, t.adj, tab.a[o], g->label_freq, true, w.plans_h[o], tab.b[o], live);
+                    build_plan(t, all, t.adj, tab.a[o], g->label_freq, true, w.plans_h[o], tab.b[o]);
                 }
                 CUF(cudaMemcpyAsync(w.plans, w.plans_h, sizeof(DevPlan) * (size_t)tab.n, cudaMemcpyHostToDevice, s));
                 a.om = r->om;

@@ -441,9 +441,9 @@ __device__ __forceinline__ uint32_t row_bits(const WideRow &r, uint32_t w) {
 
 // Walks the set bits of a row (first round: all its bits), 32 bitmap words at a
 // time, lane i holding word i.  An iteration takes four entries a lane, all loads
-// in flight together; f(bit, wu, j, pass) gets which of them are set, their
-// neighbours' omegas and their edge-label indices, and fills in which of them
-// pass; it returns whether to go on.  Either the lanes take four whole words
+// in flight together; f(wu, j, pass) gets their neighbours' omegas (0 where there
+// is no entry) and their edge-label indices, and fills in which of them pass; it
+// returns whether to go on.  Either the lanes take four whole words
 // (coalesced), or, where that is fewer iterations, each lane the next four bits
 // of its own word: after the second round most words hold a bit or two (rounds 2
 // to 4: 1.07, 0.98 and 0.65 ms with whole words only, 0.89, 0.66 and 0.37 so).  UPDATE:
@@ -496,7 +496,7 @@ __device__ __forceinline__ void walk(const WideArgs &a, const WideShared &S, con
                 j[k] = (int)S.T.el_index[lb[k]];
             }
             bool pass[4];
-            go = f(bit, wu, j, pass);
+            go = f(wu, j, pass);
             if (UPDATE) {
                 if (own) {
 #pragma unroll
@@ -588,8 +588,7 @@ __device__ __forceinline__ void scan_row(const WideArgs &a, WideShared &S, uint6
     uint32_t calls = 0;
     uint64_t wl[4];                          // the last iteration's entries that pass
     int jl[4];
-    walk<FIRST, true>(a, S, r, first_w, w_step, [&](const bool (&)[4], const uint64_t (&wu)[4], const int (&j)[4],
-                                                    bool (&pass)[4]) {
+    walk<FIRST, true>(a, S, r, first_w, w_step, [&](const uint64_t (&wu)[4], const int (&j)[4], bool (&pass)[4]) {
         uint64_t m[4];
 #pragma unroll
         for (int k = 0; k < 4; k++) {
@@ -631,8 +630,8 @@ __device__ __forceinline__ void scan_row(const WideArgs &a, WideShared &S, uint6
             if (calls == 1)
                 count_classes<NEL>(T, wl, jl, R);
             else
-                walk<FIRST, false>(a, S, r, first_w, w_step, [&](const bool (&)[4], const uint64_t (&wu)[4],
-                                                                 const int (&j)[4], bool (&)[4]) {
+                walk<FIRST, false>(a, S, r, first_w, w_step, [&](const uint64_t (&wu)[4], const int (&j)[4],
+                                                                 bool (&)[4]) {
 #pragma unroll
                     for (int k = 0; k < 4; k++) jl[k] = wu[k] & nb[j[k]] ? j[k] : -1;
                     count_classes<NEL>(T, wu, jl, R);
