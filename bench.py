@@ -240,15 +240,25 @@ def roofline(kernel, alg_bytes, ms, n_launch, workload, extra=None):
 
 
 def lcc_roofline(counts, workload):
-    """k_lcc_round over every round of the given prunes.  Algorithmic bytes
-    per round: 8.25 per active entry M_a + 16 per active vertex n_a."""
-    return roofline("k_lcc_round", sum(c["lcc_alg_bytes"] for c in counts),
-                    sum(c["ms_lcc_kernel"] for c in counts), sum(c["lcc_launches"] for c in counts), workload,
-                    {"M_a": sum(c["edges_scanned_lcc"] for c in counts),
+    """The LCC rounds of the given prunes.  Algorithmic bytes per round: 8.25
+    per active entry M_a + 16 per active vertex n_a of the state the round
+    finds.  A later round over large rows evaluates only the vertices near a
+    change, so it reads less than that: read_gbs counts what the kernels
+    evaluate (24 B per vertex, 4.125 per entry of its row, 4 per active entry)."""
+    ms = sum(c["ms_lcc_kernel"] for c in counts)
+    rounds = sum(c["lcc_launches"] for c in counts)
+    read = sum(c["lcc_kernel_bytes"] for c in counts)
+    read_gbs = (read / 1e9) / (ms / 1e3) if ms > 0 else 0.0
+    return roofline("LCC rounds", sum(c["lcc_alg_bytes"] for c in counts), ms, rounds, workload,
+                    {"kernels": "k_first_round, k_rows, k_push, k_lcc_round (a round is one or two of them; launches "
+                                "counts rounds)",
+                     "M_a": sum(c["edges_scanned_lcc"] for c in counts),
                      "n_a": sum(c["lcc_active_vertices"] for c in counts),
                      "R": sum(c["lcc_row_entries"] for c in counts),
-                     "kernel_bytes_per_launch": sum(c["lcc_kernel_bytes"] for c in counts) /
-                     max(sum(c["lcc_launches"] for c in counts), 1)})
+                     "kernel_bytes_per_launch": read / max(rounds, 1),
+                     "read_gbs": read_gbs, "read_frac": read_gbs / measured_peak_hbm()[0],
+                     "note": "achieved counts every active entry of each round's state; read_gbs only those that the "
+                             "round evaluates"})
 
 
 def lcc_first_round(counts):

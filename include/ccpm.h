@@ -171,26 +171,33 @@ typedef struct {
     int64_t  edges_scanned_lcc;    /* sum over LCC rounds of active CSR entries   */
     int64_t  edges_scanned_search; /* CSR entries examined by NLCC + final search */
     double   ms_total, ms_lcc, ms_nlcc, ms_final;   /* device time per stage     */
-    /* measurement of the LCC round kernel (CUDA events around each launch on
-     * the context stream) and the traffic the method itself needs per round
-     * (Alg. 4 over n_a active vertices and M_a active CSR entries):
+    /* measurement of the LCC rounds (CUDA events around each group of queued
+     * rounds on the context stream; a round is one or two kernels) and the
+     * traffic the method itself needs per round (Alg. 4 over n_a active
+     * vertices and M_a active CSR entries):
      *   16 B per active vertex (two 4-byte row offsets, omega read and write)
      * + 8.25 B per active entry (column index, gather of the neighbour's
-     *   omega, read and write of its edge bit)                              */
-    int64_t  lcc_launches;
+     *   omega, read and write of its edge bit).
+     * n_a and M_a (edges_scanned_lcc, lcc_active_vertices, lcc_row_entries)
+     * describe the state each round finds: a later round over large rows
+     * evaluates only the vertices near a change and takes the others' entries
+     * from their last evaluation, so it reads less (lcc_kernel_bytes)       */
+    int64_t  lcc_launches;         /* rounds that ran (= lcc_rounds_total)      */
     double   ms_lcc_kernel;
     int64_t  lcc_alg_bytes;        /* sum over rounds of 8.25 M_a + 16 n_a      */
     int64_t  lcc_row_entries;      /* CSR entries in rows of active vertices  */
     int64_t  lcc_active_vertices;  /* active vertices, summed over rounds      */
     int64_t  kernel_launches;      /* all kernels this call launched          */
     int64_t  lcc_compactions;      /* row compactions (K4) between LCC rounds */
-    double   ms_search_kernel;     /* device time of the NLCC search kernels  */
-    int64_t  search_launches;      /* their launches                          */
-    int64_t  search_entries_nlcc;  /* row entries those kernels examined      */
+    double   ms_search_kernel;     /* device time of the NLCC searches: item  */
+                                   /* lists and passes (and the host round    */
+                                   /* trips of those with more passes than    */
+                                   /* are queued at a time)                   */
+    int64_t  search_launches;      /* their number                            */
+    int64_t  search_entries_nlcc;  /* row entries the passes examined         */
     /* what the kernel itself reads and writes per round: 24 B per vertex it
      * evaluates (two int64 offsets, omega read and write) + 4.125 B per entry
-     * of such a row (column index, edge bit) + 4 B per active entry (gather);
-     * later rounds over large rows evaluate only the vertices near a change   */
+     * of such a row (column index, edge bit) + 4 B per active entry (gather)  */
     int64_t  lcc_kernel_bytes;
     int64_t  lcc_first_entries;    /* M_a of the first round after init       */
     double   ms_lcc_first;         /* device time of that round               */

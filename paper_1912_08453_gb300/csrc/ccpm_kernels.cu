@@ -2403,7 +2403,7 @@ k_materialize_fix(int64_t n, const uint32_t *__restrict__ om, const int64_t *__r
 // Hand-back of the edge map when the live rows are exact: their bits, into a
 // zeroed bitmap.  A warp takes 32 vertices and copies the live rows together:
 // most vertices are dead by then, and clearing their rows instead cost two
-// atomics each (1.15 ms over 32M vertices with 3.6M live; this 0.25).
+// atomics each (1.15 ms over 32M vertices with 3.6M live; this 0.40).
 __global__ void __launch_bounds__(256)
 k_copy_live_rows(int64_t n, const uint32_t *__restrict__ om, const int64_t *__restrict__ rp,
                  const uint32_t *__restrict__ bits, uint32_t *out) {
@@ -2819,8 +2819,8 @@ constexpr int kSpillParts = 32;      // items one open level's untested candidat
 // microsecond or more), so a pass lasts as long as its longest search.  Handing
 // on only after 2048 windows, 16M vertices / 5*10^8 entries / 5-cycle template:
 // 50 ms in 10 passes of k_nlcc_items and 18.6 ms in 3 of k_edge_search; handing
-// on when the list is empty: 2.1 ms in 32 passes and 0.5 ms in 8 (the whole
-// prune 75.7 -> 7.7 ms; a batch of 24 templates on 4M vertices 105 -> 27 ms).
+// on when the list is empty: 2.0 ms in 40 passes and 0.5 ms in 8 (the whole
+// prune 78.6 -> 5.9 ms; a batch of 24 templates on 4M vertices 105 -> 23 ms).
 // Returns false (the search goes on where it is) when the list is full.
 // Reservations only ever add to the counter: the successful ones are exactly
 // those ending at or below the capacity, and they fill the list up to the
@@ -5201,8 +5201,9 @@ static int prune(ccpm_ctx_t ctx, ccpm_graph_t g, ccpm_tmpl_t tm, const ccpm_opti
     // a caller's own budget counts windows as one search scans them: no handing
     // on to idle warps, which would restart its count.  Those searches are
     // spread up front instead (expand_more: a kernel and a host round trip per
-    // level), which is slower where both work: 8.3 against 7.7 ms on the 5-cycle
-    // template over 16M vertices, 32 against 27 ms for a batch over 4M
+    // level) and handed on after `split` windows only, which is slower where both
+    // work: a prune with the 5-cycle template over 16M vertices 43.6 against 5.8
+    // ms, a batch of 24 templates over 4M 35 against 20
     const bool starve = opt.search_split >= 0 && opt.search_budget == 0;
     int rc = ws_ensure(ctx, g, hub_deg);
     if (rc) return rc;
@@ -6174,11 +6175,7 @@ static int list_matches(ccpm_ctx_t ctx, ccpm_result_t r, ccpm_tmpl_t tm, const c
     const int hub_deg = opt.hub_degree > 0 ? std::min(opt.hub_degree, kMaxHubDeg) : kDefaultHubDeg;
     const uint64_t budget = opt.search_budget ? opt.search_budget : ~0ull;
     const uint64_t split = opt.search_split < 0 ? 0 : (opt.search_split == 0 ? kSpillAfter : (uint64_t)opt.search_split);
-    // a caller's own budget counts windows as one search scans them: no handing
-    // on to idle warps, which would restart its count.  Those searches are
-    // spread up front instead (expand_more: a kernel and a host round trip per
-    // level), which is slower where both work: 8.3 against 7.7 ms on the 5-cycle
-    // template over 16M vertices, 32 against 27 ms for a batch over 4M
+    // as for a prune: with a caller's own budget, no handing on to idle warps
     const bool starve = opt.search_split >= 0 && opt.search_budget == 0;
     int rc = ws_ensure(ctx, g, hub_deg);
     if (rc) return rc;

@@ -890,7 +890,7 @@ int ccpm_mlp_train(ccpm_mlp_t m, int N, const float *host_x, const float *host_t
     // Up to kTrainMaxBatch every step in one kernel, a few thousand steps a
     // launch: 8.2 us a step up to 512 rows, 12 at 1024, 35 at 4096, 45 at 8192 (a
     // block takes its rows 64 at a time).  The kernels per step, which spread
-    // over the whole GPU, take 37 us up to 4096 rows and 40 at 8192.
+    // over the whole GPU, take 37 to 40 us up to 4096 rows and 41 at 8192.
     const TrainLaunch launch(s);
     fused = fused && batch <= kTrainMaxBatch;
     for (int it = 0; fused && it < steps && e == cudaSuccess;) {
