@@ -3880,6 +3880,7 @@ struct ccpm_graph {
     int tuned_split = 0, tuned_short = 0, tuned_hub = 0, tuned_share = 0;
     double tuned_ms = 0.0;        // the chosen setting's time on the tuning slice
     std::atomic<int> prunes{0};   // prunes started on this graph
+    std::atomic<int> listings{0};
     std::atomic<bool> lrows_ready{false};   // lcol/nlab built (read without the lock)
     uint8_t *elab = nullptr;      // label of each entry's neighbour, CSR order (built on first use)
     uint8_t *edge_lab = nullptr;  // edge label of each entry (ccpm_graph_set_edge_labels), or none
@@ -6160,6 +6161,48 @@ int ccpm_result_phase_rounds(ccpm_result_t r, int32_t *dst, int cap) {
     return CCPM_OK;
 }
 
+// Does a listing copy the result's entries into rows of their own (K4) before it
+// searches?  Otherwise it reads the label-grouped copy of the graph's rows.  The
+// copy costs some 0.1 ms and several passes over all vertices; on the graph's rows
+// a label group holds entries outside the result, and partial maps run over edges
+// outside it.  us without / with the copy (list of 1000, no counts):
+//   result entries, template, graph                      without     with
+//      17,300  triangle, Zipf labels, 32M vertices           224    1,396
+//     179,272  triangle, Zipf labels, 32M                    366    1,601
+//     117,340  triangle, Zipf labels, 16M                    268      976
+//      26,920  5-cycle, Zipf labels, 1M                      724      767
+//     149,792  4-cycle, Zipf labels, 4M                    1,099    1,388
+//      14,130  two 4-cycles sharing a path, 100 labels, 1M 3,738    2,401
+//       2,284  4-cycle + triangle, degree labels, 1M         172      278
+//      10,294  the same, 22K                                 598      688
+//      22,478  the same, 26K                               2,085    1,372
+//     117,320  the same, 80K                              14,683    2,963
+//     879,814  the same, 1M                              266,655    1,716
+//     486,850  tree, degree labels, 1M                     2,098    2,338
+// What makes the difference is the length of the groups: past a window (32
+// entries) on average, as under hubs that carry their degree as label, every step
+// of a search reads several.  With shorter ones the copy was worse in 207 of 231
+// results of 2 to 940,000 entries and at most 1.6 times as fast, with three
+// template vertices always worse.  Results that no final search made may hold many
+// entries that no match uses; they are copied, unless they are small.  The first
+// listing of a graph whose rows are not grouped yet copies, too: grouping them
+// pays off from the second on.
+constexpr int64_t kCopyEntries = (int64_t)1 << 14;
+
+static bool listing_copies(ccpm_graph *g, const ccpm_result *r, const Template &t) {
+    if (!g->lrows_ready.load() && g->listings == 0) return true;
+    if (r->counts.active_e_dir < kCopyEntries || t.n0 <= 3) return false;
+    if (!r->counts.count_valid) return true;
+    for (auto &e : t.edges)
+        for (int x : {e.first, e.second}) {
+            const int y = x == e.first ? e.second : e.first;
+            // mean row of label(x) times the share of entries that lead to label(y)
+            const double row = (double)g->label_rows[t.labels[x]] / (double)std::max<int64_t>(g->label_freq[t.labels[x]], 1);
+            if (row * (double)g->label_rows[t.labels[y]] > 32.0 * (double)g->m) return true;
+        }
+    return false;
+}
+
 static int list_matches(ccpm_ctx_t ctx, ccpm_result_t r, ccpm_tmpl_t tm, const ccpm_options *opt_in,
                         int32_t *list, uint64_t list_cap, uint64_t *vertex_counts, uint64_t *entry_counts,
                         int dst_on_device, uint64_t *n_matches) {
@@ -6216,12 +6259,9 @@ static int list_matches(ccpm_ctx_t ctx, ccpm_result_t r, ccpm_tmpl_t tm, const c
     const uint32_t all = t.n0 == 32 ? 0xFFFFFFFFu : ((1u << t.n0) - 1u);
     build_plan(t, all, t.adj, root, g->label_freq, true, w.plans_h[0], -1, nullptr);
     CUR(cudaMemcpyAsync(w.plans, w.plans_h, sizeof(DevPlan), cudaMemcpyHostToDevice, s));
-    // every match lies inside the result's vertices and entries: the search
-    // reads rows that hold nothing else, label group by label group from a
-    // directory.  Over the graph's own rows nearly every candidate scanned is
-    // outside the result and every group is found by two binary searches:
-    // 340,000 matches of a 4-cycle with a triangle (1M vertices, 3*10^7
-    // entries) took 261 ms there and take 1.8 ms here, 0.3 ms of it the copy
+    // every match lies inside the result's vertices and entries: the search reads
+    // rows that hold nothing else, label group by label group from a directory, or
+    // where that does not pay the graph's own grouped rows
     Pipeline P;
     P.ctx = ctx;
     P.g = g;
@@ -6229,44 +6269,51 @@ static int list_matches(ccpm_ctx_t ctx, ccpm_result_t r, ccpm_tmpl_t tm, const c
     P.lrp = g->rp;
     P.lcol = g->col;
     P.lbits = w.ebits;
-    LabelMask lm;
-    std::memset(&lm, 0, sizeof(lm));
-    for (int q = 0; q < t.n0; q++) lm.m[t.labels[q]] |= 1u << q;
+    const uint32_t *om = r->om;
     if ((rc = clear_search(ctx, w))) { release(); return rc; }
-    CUR(cudaMemsetAsync(&w.ctl->init, 0, sizeof(RoundStats), s));
-    CUR(cudaMemsetAsync(w.ebits, 0, sizeof(uint32_t) * (size_t)(w.words + 1), s));
-    k_init<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, g->rp, g->lab, lm, r->om, w.om[0], w.om[1], nullptr, nullptr,
-                                                       0, w.small[0], w.med[0], w.chunk[0], w.acc, &w.ctl->init, hub_deg,
-                                                       P.short_max, 0u, nullptr, nullptr, 0);
-    CUR(cudaGetLastError());
-    k_live_entries<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, g->rp, g->col, w.om[0], r->eb, w.ebits, w.deg, w.st);
-    CUR(cudaGetLastError());
-    k_collect_roots<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, w.om[0], 1u << root, w.roots, w.st);
-    CUR(cudaGetLastError());
-    if ((rc = read_control(ctx, w))) { release(); return rc; }
-    const int64_t n_roots = w.st_h->n_roots, kept = (int64_t)w.st_h->kept;
-    const RoundStats &lists = w.ctl_h->init;
-    if (lists.n_hub_slots > (unsigned)w.acc_cap || (int64_t)lists.n_chunk > w.chunk_cap) {
-        release();
-        return set_err(ctx, CCPM_EOVERFLOW, "hub bookkeeping overflow");
-    }
-    bool over = false;
-    if (n_roots > 0 && kept > 0) {
+    bool any = true;                      // something to search, as far as the host knows
+    const bool copies = listing_copies(g, r, t);
+    g->listings++;
+    if (copies || ensure_label_rows(ctx, g)) {
+        om = w.om[0];
+        LabelMask lm;
+        std::memset(&lm, 0, sizeof(lm));
+        for (int q = 0; q < t.n0; q++) lm.m[t.labels[q]] |= 1u << q;
+        CUR(cudaMemsetAsync(&w.ctl->init, 0, sizeof(RoundStats), s));
+        CUR(cudaMemsetAsync(w.ebits, 0, sizeof(uint32_t) * (size_t)(w.words + 1), s));
+        k_init<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, g->rp, g->lab, lm, r->om, w.om[0], w.om[1], nullptr,
+                                                           nullptr, 0, w.small[0], w.med[0], w.chunk[0], w.acc,
+                                                           &w.ctl->init, hub_deg, P.short_max, 0u, nullptr, nullptr, 0);
+        CUR(cudaGetLastError());
+        k_live_entries<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, g->rp, g->col, om, r->eb, w.ebits, w.deg, w.st);
+        CUR(cudaGetLastError());
+        if ((rc = read_control(ctx, w))) { release(); return rc; }
+        const RoundStats &lists = w.ctl_h->init;
+        if (lists.n_hub_slots > (unsigned)w.acc_cap || (int64_t)lists.n_chunk > w.chunk_cap) {
+            release();
+            return set_err(ctx, CCPM_EOVERFLOW, "hub bookkeeping overflow");
+        }
         P.n_small = lists.n_small;
         P.n_med = lists.n_med;
         P.n_chunk = lists.n_chunk;
-        P.last_kept = kept;
-        if ((rc = P.compact()) || (rc = clear_search(ctx, w))) { release(); return rc; }
+        P.last_kept = (int64_t)w.st_h->kept;
+        any = P.last_kept > 0;
+        if (any && ((rc = P.compact()) || (rc = clear_search(ctx, w)))) { release(); return rc; }
+    }
+    bool over = false;
+    if (any) {
+        k_collect_roots<<<grid_for(ctx, g->n, 256, 8), 256, 0, s>>>(g->n, om, 1u << root, w.roots, w.st);
+        CUR(cudaGetLastError());
         SearchArgs a{};
         a.rp = g->rp;
         a.col = g->col;
-        a.rl = P.lrp;
-        a.lcol = P.lcol;
-        a.nlab = P.lnlab;
+        a.rl = P.gen >= 0 ? P.lrp : g->rp;
+        a.lcol = P.gen >= 0 ? P.lcol : g->lcol;
+        a.nlab = P.gen >= 0 ? P.lnlab : g->nlab;
         P.directory(a);
-        a.om = w.om[0];
+        a.om = om;
         a.roots = w.roots;
-        a.n_roots = n_roots;
+        a.n_roots = -1;
         a.plans = w.plans;
         a.heads = 1u << root;
         a.sat = w.sat;
@@ -6292,7 +6339,7 @@ static int list_matches(ccpm_ctx_t ctx, ccpm_result_t r, ccpm_tmpl_t tm, const c
         over = w.st_h->overflow != 0;
     }
     // the counters read last are the search's (or show that there was none)
-    const unsigned long long found = n_roots > 0 && kept > 0 ? w.cnt_h[0] : 0ull;
+    const unsigned long long found = any ? w.cnt_h[0] : 0ull;
     if (!dst_on_device) {
         const uint64_t rows = std::min<uint64_t>((uint64_t)found, list_cap);
         if (rows) CUR(cudaMemcpyAsync(list, d_list, sizeof(int32_t) * (size_t)(rows * (uint64_t)t.n0), cudaMemcpyDeviceToHost, s));
