@@ -3850,6 +3850,7 @@ struct ccpm_ctx {
     // row entries from which the LCC rounds go another way; tests lower them
     int64_t huge_rows = kHugeRows, inline_rows = kInlineRows, delta_rows = kDeltaRows;
     unsigned long long *label_hist = nullptr;   // counters of a graph load (borrowed arrays)
+    cudaEvent_t load_ev = nullptr;        // ... and the default stream's state before it
     cudaEvent_t wait_ev = nullptr;        // batch workers: waits poll this event and yield
     // batch workers: grids are sized for sm_total / min(batch_share, workers
     // busy right now), so the last templates of a batch get the whole GPU back
@@ -4969,6 +4970,7 @@ void ccpm_ctx_destroy(ccpm_ctx_t c) {
     for (ccpm_ctx *wk : c->workers) ccpm_ctx_destroy(wk);
     ws_free(c->ws);
     cudaFree(c->label_hist);
+    if (c->load_ev) cudaEventDestroy(c->load_ev);
     if (c->wait_ev) cudaEventDestroy(c->wait_ev);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
     delete c;
@@ -5018,13 +5020,15 @@ int ccpm_graph_load_csr(ccpm_ctx_t ctx, int64_t n, int64_t m, const int64_t *row
         g->col = const_cast<int32_t *>(col);
         g->lab = const_cast<uint8_t *>(labels);
         // label counts on the device.  The arrays may still be in the making on the
-        // default stream (or one that waits for it): a copy of one label waits for
-        // these, and for no other stream's work.  The counters stay with the
-        // context, since giving memory back waits for the whole device.
-        uint8_t one;
+        // default stream (or one that waits for it): the count waits for these, and
+        // for no other stream's work.  Event and counters stay with the context,
+        // since giving memory back waits for the whole device.
         unsigned long long h[512];
-        cudaError_t e = cudaMemcpy(&one, labels, 1, cudaMemcpyDeviceToHost);
+        cudaError_t e = cudaSuccess;
+        if (!ctx->load_ev) e = cudaEventCreateWithFlags(&ctx->load_ev, cudaEventDisableTiming);
         if (e == cudaSuccess && !ctx->label_hist) e = cudaMalloc((void **)&ctx->label_hist, sizeof(h));
+        if (e == cudaSuccess) e = cudaEventRecord(ctx->load_ev, nullptr);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->stream, ctx->load_ev, 0);
         if (e == cudaSuccess) e = cudaMemsetAsync(ctx->label_hist, 0, sizeof(h), ctx->stream);
         if (e == cudaSuccess) {
             k_label_hist<<<grid_for(ctx, n, 256, 8), 256, 0, ctx->stream>>>(n, row_ptr, labels, ctx->label_hist);
