@@ -1237,7 +1237,7 @@ __device__ __forceinline__ Quad<F> quad_gather(const RowArgs &a, uint32_t nib, c
         if ((nib >> j) & 1u) {
             if (F == kByLabel) x[j] = __ldg(a.lab + u[j]);
             else if (F == kByByte) x[j] = __ldg((const uint8_t *)a.nw + u[j]);
-            else x[j] = __ldg(a.om + u[j]);
+            else x[j] = gather_om(a.om, a.nw, a.nw_bytes, u[j]);
         }
     }
     if constexpr (F == kByWord) {
