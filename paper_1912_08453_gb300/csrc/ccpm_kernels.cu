@@ -4138,7 +4138,15 @@ int expand_more(ccpm_ctx *ctx, Workspace &w, SearchArgs &a, int max_depth, int64
         CU(ctx, cudaMemcpyAsync(w.st_h, w.st, sizeof(RoundStats), cudaMemcpyDeviceToHost, ctx->stream));
         CU(ctx, ctx_sync(ctx));
         const unsigned int n2 = w.st_h->n_items;
-        if ((int64_t)n2 > w.items_cap) return set_err(ctx, CCPM_EOVERFLOW, "search items overflow");
+        if ((int64_t)n2 > w.items_cap) {
+            // more than fit: the items stay at the level they were at
+            w.st_h->n_items = (unsigned int)a.n_items;
+            CU(ctx, cudaMemcpyAsync(w.items, w.items2, sizeof(SearchItem) * (size_t)a.n_items, cudaMemcpyDeviceToDevice,
+                                    ctx->stream));
+            CU(ctx, cudaMemcpyAsync(&w.st->n_items, &w.st_h->n_items, sizeof(unsigned int), cudaMemcpyHostToDevice,
+                                    ctx->stream));
+            return CCPM_OK;
+        }
         a.n_items = n2;
     }
     return CCPM_OK;
